@@ -20,6 +20,7 @@
 #include <cstdio>
 
 #include "fosb_internal.h"
+#include "sauter_schwab.cuh"
 
 namespace fosb {
 
@@ -27,12 +28,19 @@ __constant__ double c_bary[6][3];
 __constant__ double c_w[6];
 __constant__ double c_glx[16];
 __constant__ double c_glw[16];
+__constant__ double c_ss_series[kSsTerms][6];  // see make_ss_series
+__device__ double g_ss_table[kSsFields * kSsRegions * kSsMaxNss * kSsMaxNss * kSsMaxNss];
 
 void upload_rules(const Rules& r) {
   cudaMemcpyToSymbol(c_bary, r.bary, sizeof(r.bary));
   cudaMemcpyToSymbol(c_w, r.w, sizeof(r.w));
   cudaMemcpyToSymbol(c_glx, r.glx, sizeof(r.glx));
   cudaMemcpyToSymbol(c_glw, r.glw, sizeof(r.glw));
+  const std::vector<double> tab = make_ss_table(r);
+  cudaMemcpyToSymbol(g_ss_table, tab.data(), tab.size() * sizeof(double));
+  double c[kSsTerms][6];
+  make_ss_series(r, c);
+  cudaMemcpyToSymbol(c_ss_series, c, sizeof(c));
 }
 
 namespace {
@@ -204,84 +212,112 @@ __global__ void __launch_bounds__(256) efie_regular_kernel(DevMesh m, double k, 
 }
 
 // ------------------------------------------------------------------ singular pairs
-// One CTA of 128 threads per touching pair; the Sauter-Schwab 4-cube points are split
-// over the threads, the moments reduced through shared memory.  FP64 throughout.
-// chi(u) - P0 = u1 (P1 - P0) + u2 (P2 - P1), with the edge vectors E[0] = P1 - P0 and
-// E[1] = P2 - P1 formed once per pair
-__device__ __forceinline__ void chi_rel(const double E[2][3], double u1, double u2, double out[3]) {
-#pragma unroll
-  for (int c = 0; c < 3; ++c) out[c] = fma(u1, E[0][c], u2 * E[1][c]);
-}
+// Touching pairs by Sauter-Schwab, FP64, one warp per pair.  Every point of the 4-cube rule is
+// (x, y) = xi (xh, yh) with (xh, yh) fixed by the three coordinates e1..e3 and the region, so
+// with rh = |xh - yh| and phi = k rh the n_ss points along xi share one distance and
+//   sum_a w_a xi_a^3 xi_a^m exp(ik xi_a rh)/(xi_a rh) = S_m(phi) / rh,
+//   S_m(phi) = sum_a w_a xi_a^{2+m} exp(i phi xi_a),   m = 0, 1, 2 (moments of 1, x or y, x.y).
+// S_m is a power series in phi whose coefficients are the rule's own moments (c_ss_series): the
+// same quadrature, without a sine, cosine or square root per point.  The moments are gathered in
+// the reference coordinates (u of x, v of y), whose values and products come from g_ss_table.
+// Bound by the FP64 pipe (one warp instruction per 16 clocks and SM): about 95 FP64
+// instructions per 5 points against 77 per point when every point had its own 1/r and
+// exp(ikr).  At T = 20480, n_ss = 5, k = 4: 9.2 ms, 46.0 ms before; at T = 320, k = 1 the whole
+// assembly call takes 0.32 ms, 1.14 ms before.
+// The series up to here (its rounding is then below 6e-16 of |S_m|, 8e-16 at phase 4; 15 terms);
+// larger phases, which only meshes with edges beyond about half a wavelength reach, take sincos per point.
+constexpr double kSsMaxPhase = 3.0;
 
-// exp(i th) for 0 <= th <= 64 in FP64: Cody-Waite reduction th = n pi/2 + d (pi/2 split in
-// three parts, the first with 33 significant bits so that n times it is exact), |d| <= pi/4,
-// and the Taylor series of sin d / d to d^16 and of cos d to d^18 (truncation below 2e-20
-// relative), then the quadrant n mod 4.  Larger phases, which no touching pair of a resolved
-// mesh reaches, fall back to sincos.
-__device__ __forceinline__ void ss_expi(double th, double& c, double& s) {
-  if (!(th <= 64.0)) {
-    sincos(th, &s, &c);
-    return;
+// Number of phi^2 powers for phases up to ph: the first J with ph^{2J}/(2J)! < 2^-56 (the
+// moments' decay only helps), at most kSsTerms, which covers kSsMaxPhase.
+__device__ __forceinline__ int ss_terms(float ph) {
+  const float p2 = ph * ph;
+  float t = 1.f;
+  int J = 0;
+  while (J < kSsTerms && t > 1.3e-17f) {
+    t *= p2 / float((2 * J + 1) * (2 * J + 2));
+    ++J;
   }
-  const double n = rint(th * 0.6366197723675814);
-  const double d = fma(-n, 3.5215598651832e-27, fma(-n, 6.077100506506192e-11, fma(-n, 1.5707963267341256, th)));
-  const double d2 = d * d;
-  // sin d / d = sum_i (-d2)^i / (2i + 1)!,  cos d = sum_i (-d2)^i / (2i)!
-  double ps = 1.0 / 355687428096000.0;          // 1/17!
-  ps = fma(ps, -d2, 1.0 / 1307674368000.0);     // 1/15!
-  ps = fma(ps, -d2, 1.0 / 6227020800.0);        // 1/13!
-  ps = fma(ps, -d2, 1.0 / 39916800.0);          // 1/11!
-  ps = fma(ps, -d2, 1.0 / 362880.0);            // 1/9!
-  ps = fma(ps, -d2, 1.0 / 5040.0);              // 1/7!
-  ps = fma(ps, -d2, 1.0 / 120.0);               // 1/5!
-  ps = fma(ps, -d2, 1.0 / 6.0);                 // 1/3!
-  ps = fma(ps, -d2, 1.0);
-  double pc = 1.0 / 6402373705728000.0;         // 1/18!
-  pc = fma(pc, -d2, 1.0 / 20922789888000.0);    // 1/16!
-  pc = fma(pc, -d2, 1.0 / 87178291200.0);       // 1/14!
-  pc = fma(pc, -d2, 1.0 / 479001600.0);         // 1/12!
-  pc = fma(pc, -d2, 1.0 / 3628800.0);           // 1/10!
-  pc = fma(pc, -d2, 1.0 / 40320.0);             // 1/8!
-  pc = fma(pc, -d2, 1.0 / 720.0);               // 1/6!
-  pc = fma(pc, -d2, 1.0 / 24.0);                // 1/4!
-  pc = fma(pc, -d2, 0.5);                       // 1/2!
-  pc = fma(pc, -d2, 1.0);
-  const double sd = d * ps, cd = pc;
-  // sin(d + q pi/2), cos(d + q pi/2) for q = n mod 4
-  const int q = int(n) & 3;
-  s = q == 0 ? sd : (q == 1 ? cd : (q == 2 ? -sd : -cd));
-  c = q == 0 ? cd : (q == 1 ? -sd : (q == 2 ? -cd : sd));
+  return J;
 }
 
-__device__ __forceinline__ void ss_accumulate(double k, const double x[3], const double y[3], double w, double acc[16]) {
-  const double dx = x[0] - y[0], dy = x[1] - y[1], dz = x[2] - y[2];
-  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  // 1/r from a float seed and two Newton steps in FP64, y <- y (3 - r2 y^2) / 2:
-  // about 22, then 44, then full significant bits
-  double yr = double(rsqrtf(float(r2)));
-  yr = yr * fma(-0.5 * r2, yr * yr, 1.5);
-  yr = yr * fma(-0.5 * r2, yr * yr, 1.5);
-  double sn, cs;
-  ss_expi(k * (r2 * yr), cs, sn);
-  const double g = w * yr;
-  const double gr = cs * g, gi = sn * g;
-  acc[0] += gr;
-  acc[1] += gi;
+// The moment sums of one lane: I0, then u1, u2, v1, v2, then u1v1, u1v2, u2v1, u2v2 (complex).
+template <int KIND>
+__device__ __forceinline__ void ss_moments(double k, int nss, int J, const double (&EP)[2][3], const double (&EQ)[2][3],
+                                           int lane, double (&acc)[18]) {
+  const int n3 = nss * nss * nss, stride = kSsRegions * n3;
+  const int first = KIND == 3 ? 0 : (KIND == 2 ? 6 : 11), count = (KIND == 3 ? 6 : (KIND == 2 ? 5 : 2)) * n3;
+  const double* tab = g_ss_table + first * n3;
+  for (int idx = lane; idx < count; idx += 32) {
+    auto T = [&](int f) { return __ldg(tab + f * stride + idx); };
+    const double u1 = T(0), u2 = T(1), v1 = T(2), v2 = T(3);
+    double d[3];
+    if constexpr (KIND == 3) {  // EQ = EP: the coordinate differences are in the table
+      const double a = T(9), b = T(10);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    acc[2 + 2 * c] += gr * x[c];
-    acc[3 + 2 * c] += gi * x[c];
-    acc[8 + 2 * c] += gr * y[c];
-    acc[9 + 2 * c] += gi * y[c];
+      for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], b * EP[1][c]);
+    } else if constexpr (KIND == 2) {  // EQ[0] = EP[0], the shared edge
+      const double a = T(9);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], fma(u2, EP[1][c], -v2 * EQ[1][c]));
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        d[c] = fma(u1, EP[0][c], fma(u2, EP[1][c], fma(-v1, EQ[0][c], -v2 * EQ[1][c])));
+    }
+    const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+    const double rinv = ss_rsqrt(r2);
+    const double phi = k * (r2 * rinv);
+    double sr[3], si[3];
+    if (J > 0) {
+      const double p2 = phi * phi;
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        sr[m] = c_ss_series[J - 1][m];
+        si[m] = c_ss_series[J - 1][3 + m];
+      }
+      for (int j = J - 2; j >= 0; --j)
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          sr[m] = fma(sr[m], p2, c_ss_series[j][m]);
+          si[m] = fma(si[m], p2, c_ss_series[j][3 + m]);
+        }
+#pragma unroll
+      for (int m = 0; m < 3; ++m) si[m] *= phi;
+    } else {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) sr[m] = si[m] = 0.0;
+      for (int a = 0; a < nss; ++a) {
+        const double xi = c_glx[a];
+        double sn, cs, w = c_glw[a] * xi * xi;
+        sincos(phi * xi, &sn, &cs);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          sr[m] = fma(w, cs, sr[m]);
+          si[m] = fma(w, sn, si[m]);
+          w *= xi;
+        }
+      }
+    }
+    const double g = T(4) * rinv;
+    acc[0] = fma(g, sr[0], acc[0]);
+    acc[1] = fma(g, si[0], acc[1]);
+    const double ar = g * sr[1], ai = g * si[1], br = g * sr[2], bi = g * si[2];
+    const double uv[4] = {u1, u2, v1, v2};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double p = T(5 + q);
+      acc[2 + 2 * q] = fma(uv[q], ar, acc[2 + 2 * q]);
+      acc[3 + 2 * q] = fma(uv[q], ai, acc[3 + 2 * q]);
+      acc[10 + 2 * q] = fma(p, br, acc[10 + 2 * q]);
+      acc[11 + 2 * q] = fma(p, bi, acc[11 + 2 * q]);
+    }
   }
-  double xy = x[0] * y[0] + x[1] * y[1] + x[2] * y[2];
-  acc[14] += gr * xy;
-  acc[15] += gi * xy;
 }
 
-// One touching pair (index pair of m.touch) by one warp: the lanes share the Sauter-Schwab
-// 4-cube points, a butterfly reduction leaves the 16 moments in every lane, and lanes 0-8
-// form one entry each of the 3 x 3 RWG block and add it (and its mirror) into Z.
+// One touching pair (index pair of m.touch) by one warp: the lanes share the points, a halving
+// reduction and a broadcast leave the moments in every lane, and lanes 0-8 form one entry each
+// of the 3 x 3 RWG block and add it (and its mirror) into Z.
 template <typename OutT>
 __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int nss, OutT* Z, int64_t ldz, int64_t pair) {
   const int lane = threadIdx.x & 31;
@@ -295,7 +331,7 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
       P[a][c] = m.verts[3 * tp.p[a] + c];
       Q[a][c] = m.verts[3 * tp.q[a] + c];
     }
-  // P0 == Q0 for every touching kind, so x - y = (x - P0) - (y - Q0) exactly.
+  // P0 == Q0 for every touching kind; x - P0 = u1 EP[0] + u2 EP[1] and the same for y
   double EP[2][3], EQ[2][3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -304,65 +340,20 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
     EQ[0][c] = Q[1][c] - Q[0][c];
     EQ[1][c] = Q[2][c] - Q[1][c];
   }
-  const int n2 = nss * nss, n4 = n2 * n2;
-  double acc[16];
+  const float ph = ss_phase_bound(k, EP, EQ);
+  const int J = ph <= float(kSsMaxPhase) ? ss_terms(ph) : 0;
+  double acc[18];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = 0.0;
-  for (int idx = lane; idx < n4; idx += 32) {
-    int a = idx / (n2 * nss), b = (idx / n2) % nss, c = (idx / nss) % nss, d = idx % nss;
-    double xi = c_glx[a], e1 = c_glx[b], e2 = c_glx[c], e3 = c_glx[d];
-    double w4 = c_glw[a] * c_glw[b] * c_glw[c] * c_glw[d];
-    double x[3], y[3];
-    if (tp.kind == 3) {
-      double w = w4 * xi * xi * xi * e1 * e1 * e2;
-      const double s[6][4] = {
-          {xi, xi * (1 - e1 + e1 * e2), xi * (1 - e1 * e2 * e3), xi * (1 - e1)},
-          {xi * (1 - e1 * e2 * e3), xi * (1 - e1), xi, xi * (1 - e1 + e1 * e2)},
-          {xi, xi * e1 * (1 - e2 + e2 * e3), xi * (1 - e1 * e2), xi * e1 * (1 - e2)},
-          {xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * (1 - e2 + e2 * e3)},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * (1 - e2)},
-          {xi, xi * e1 * (1 - e2), xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3)}};
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        chi_rel(EP, s[j][0], s[j][1], x);
-        chi_rel(EQ, s[j][2], s[j][3], y);
-        ss_accumulate(k, x, y, w, acc);
-      }
-    } else if (tp.kind == 2) {
-      double w0 = w4 * xi * xi * xi * e1 * e1, w1 = w0 * e2;
-      const double s[5][5] = {
-          {xi, xi * e1 * e3, xi * (1 - e1 * e2), xi * e1 * (1 - e2), w0},
-          {xi, xi * e1, xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), w1},
-          {xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * e2 * e3, w1},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), xi, xi * e1, w1},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * e2, w1}};
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        chi_rel(EP, s[j][0], s[j][1], x);
-        chi_rel(EQ, s[j][2], s[j][3], y);
-        ss_accumulate(k, x, y, s[j][4], acc);
-      }
-    } else {
-      double w = w4 * xi * xi * xi * e2;
-      chi_rel(EP, xi, xi * e1, x);
-      chi_rel(EQ, xi * e2, xi * e2 * e3, y);
-      ss_accumulate(k, x, y, w, acc);
-      chi_rel(EP, xi * e2, xi * e2 * e3, x);
-      chi_rel(EQ, xi, xi * e1, y);
-      ss_accumulate(k, x, y, w, acc);
-    }
-  }
-  // butterfly reduction: every lane ends with the 16 sums
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-  }
+  for (int i = 0; i < 18; ++i) acc[i] = 0.0;
+  if (tp.kind == 3) ss_moments<3>(k, nss, J, EP, EQ, lane, acc);
+  else if (tp.kind == 2) ss_moments<2>(k, nss, J, EP, EQ, lane, acc);
+  else ss_moments<1>(k, nss, J, EP, EQ, lane, acc);
+  ss_warp_sum<18>(acc, lane);
   if (lane >= 9) return;
   // lane = 3 i + j: entry (i, j) of the block,
   //   A_ij = c_i c'_j [XY - q_j.X - p_i.Y + (p_i.q_j) I0],  Phi_ij = d_i d'_j I0,
   //   Z_ij += -ik A_ij + (i/k) Phi_ij,
-  // with p_i, q_j the opposite vertices relative to P0 = Q0
+  // with p_i, q_j the opposite vertices relative to P0 = Q0 and X = EP.u, Y = EQ.v, XY = u EP.EQ v
   const int i = lane / 3, j = lane % 3;
   const int t1 = tp.t1, t2 = tp.t2;
   const double jac = 4.0 * m.tri_area[t1] * m.tri_area[t2] * kInv4Pi;
@@ -373,21 +364,26 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
     pi_[c] = m.verts[3 * a + c] - P[0][c];
     qj[c] = m.verts[3 * b + c] - Q[0][c];
   }
-  double mo[16];
+  auto dot = [](const double (&x)[3], const double (&y)[3]) { return fma(x[0], y[0], fma(x[1], y[1], x[2] * y[2])); };
+  const double pq = dot(pi_, qj);
+  double ar = pq * acc[0], ai = pq * acc[1];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) mo[q] = acc[q] * jac;
-  const double qXr = qj[0] * mo[2] + qj[1] * mo[4] + qj[2] * mo[6];
-  const double qXi = qj[0] * mo[3] + qj[1] * mo[5] + qj[2] * mo[7];
-  const double pYr = pi_[0] * mo[8] + pi_[1] * mo[10] + pi_[2] * mo[12];
-  const double pYi = pi_[0] * mo[9] + pi_[1] * mo[11] + pi_[2] * mo[13];
-  const double pq = pi_[0] * qj[0] + pi_[1] * qj[1] + pi_[2] * qj[2];
-  const double ar = mo[14] - qXr - pYr + pq * mo[0];
-  const double ai = mo[15] - qXi - pYi + pq * mo[1];
-  const double cc = m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j];
-  const double dk = m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j] * kinv;
+  for (int s = 0; s < 2; ++s) {
+    const double qe = dot(qj, EP[s]), pf = dot(pi_, EQ[s]);
+    ar -= fma(qe, acc[2 + 2 * s], pf * acc[6 + 2 * s]);
+    ai -= fma(qe, acc[3 + 2 * s], pf * acc[7 + 2 * s]);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const double ef = dot(EP[s], EQ[t]);
+      ar = fma(ef, acc[10 + 4 * s + 2 * t], ar);
+      ai = fma(ef, acc[11 + 4 * s + 2 * t], ai);
+    }
+  }
+  const double cc = jac * m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j];
+  const double dk = jac * m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j] * kinv;
   // -ik (ar + i ai) = k ai - i k ar;  (i/k) dd (I0r + i I0i) = -(dd/k) I0i + i (dd/k) I0r
-  const double zr = k * cc * ai - dk * mo[1];
-  const double zi = -k * cc * ar + dk * mo[0];
+  const double zr = k * cc * ai - dk * acc[1];
+  const double zi = -k * cc * ar + dk * acc[0];
   const int e1 = m.tri_edge[3 * t1 + i], e2 = m.tri_edge[3 * t2 + j];
   atomic_add_c(Z + 2 * (int64_t(e1) * ldz + e2), zr, zi);
   if (t1 != t2) atomic_add_c(Z + 2 * (int64_t(e2) * ldz + e1), zr, zi);
