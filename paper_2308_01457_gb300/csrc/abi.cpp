@@ -306,9 +306,10 @@ fosb_status fosb_assemble_efie(fosb_mesh mesh, double k, const fosb_quad_opts* o
   FOSB_TRY(ensure_rules(nss));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const size_t elem = is_c64(prec) ? 8 : 16;
-  FOSB_CUDA(cudaMemset2DAsync(Z, ldz * elem, 0, N * elem, N, s));
+  FOSB_CUDA(zero_lower(Z, N, ldz, is_c64(prec), s));
   FOSB_CUDA(launch_assemble_regular(mesh->d, k, arith, Z, ldz, s));
   FOSB_CUDA(launch_assemble_singular(mesh->d, k, nss, is_c64(prec), Z, ldz, s));
+  FOSB_CUDA(mirror_lower(Z, N, ldz, is_c64(prec), s));
   if (n_inc > 0) {
     // copied from a pageable buffer of our own: cudaMemcpyAsync returns once the bytes are
     // staged, so the call needs no synchronisation whatever memory the caller's `inc` is in

@@ -5,9 +5,10 @@
 // right-hand side (Section III) and the covariance-kernel product used by the
 // second-moment system (Section IV).
 //
-// Work decomposition of the regular (vertex-disjoint) triangle pairs: one thread per
-// ordered triangle pair (t1, t2); a warp holds one test triangle t1 (uniform loads) and
-// 32 consecutive trial triangles t2 (coalesced loads).  Each thread accumulates the
+// Z is complex symmetric, so triangle pairs are unordered and fill the lower triangle of Z;
+// mirror_lower_kernel writes the upper one.  Work decomposition of the regular
+// (vertex-disjoint) pairs: one thread per pair t1 < t2; a warp holds one test triangle t1
+// (uniform loads) and 32 consecutive trial triangles t2 (coalesced loads).  Each thread accumulates the
 // eight complex moments
 //     I0 = sum w G,  X = sum w G (x - o1),  Y = sum w G (y - o2),  XY = sum w G (x - o1).(y - o2)
 // over the 6 x 6 point pairs (o1, o2 = first vertices: no cancellation), forms the
@@ -20,6 +21,7 @@
 #include <cstdio>
 
 #include "fosb_internal.h"
+#include "pair_tiles.cuh"
 #include "sauter_schwab.cuh"
 
 namespace fosb {
@@ -64,14 +66,14 @@ __device__ __forceinline__ void atomic_add_c(float* p, double re, double im) {
   atomicAdd(p + 1, float(im));
 }
 
-// Forms the 3 x 3 block from the moments and adds it to Z (or its transpose).
+// Forms the 3 x 3 block from the moments and adds it to the lower triangle of Z.
 //   A_ij = c_i c'_j [XY - q_j.X - p_i.Y + (p_i.q_j) I0],  Phi_ij = d_i d'_j I0,
 //   Z_ij += -ik A_ij - 1/(ik) Phi_ij = -ik A_ij + (i/k) Phi_ij
 // with p_i, q_j the opposite vertices relative to the origins o1, o2.
 template <typename OutT>
 __device__ void scatter_block(double k, const double* m /*16 moments*/, const double p[3][3], const double q[3][3],
                               const double c1[3], const double d1[3], const double c2[3], const double d2[3],
-                              const int e1[3], const int e2[3], OutT* Z, int64_t ldz, bool also_transpose) {
+                              const int e1[3], const int e2[3], OutT* Z, int64_t ldz) {
   const double i0r = m[0], i0i = m[1];
   for (int i = 0; i < 3; ++i) {
     // p_i . X and p_i . Y
@@ -89,8 +91,7 @@ __device__ void scatter_block(double k, const double* m /*16 moments*/, const do
       // -ik (ar + i ai) = k ai - i k ar ;  (i/k) dd (i0r + i i0i) = -(dd/k) i0i + i (dd/k) i0r
       double zr = k * cc * ai - (dd / k) * i0i;
       double zi = -k * cc * ar + (dd / k) * i0r;
-      atomic_add_c(Z + 2 * (int64_t(e1[i]) * ldz + e2[j]), zr, zi);
-      if (also_transpose) atomic_add_c(Z + 2 * (int64_t(e2[j]) * ldz + e1[i]), zr, zi);
+      atomic_add_c(Z + 2 * lower_at(e1[i], e2[j], ldz), zr, zi);
     }
   }
 }
@@ -108,9 +109,10 @@ __device__ __forceinline__ bool shares_vertex(const int a[3], const int b[3]) {
 // R = double (FP64) or float (FP32 path).  OutT = double (complex128 Z) or float.
 template <typename R, typename OutT>
 __global__ void __launch_bounds__(256) efie_regular_kernel(DevMesh m, double k, OutT* Z, int64_t ldz) {
-  const int64_t t1 = int64_t(blockIdx.y) * 8 + (threadIdx.x >> 5);
-  const int64_t t2 = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (t1 >= m.nt || t2 >= m.nt) return;
+  int64_t rg, cb;
+  if (!pair_tile(m.nt, 8, blockIdx.y, blockIdx.x, rg, cb)) return;
+  const int64_t t1 = rg * 8 + (threadIdx.x >> 5), t2 = cb * 32 + (threadIdx.x & 31);
+  if (t1 >= m.nt || t2 >= m.nt || t1 >= t2) return;
   int v1[3], v2[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(256) efie_regular_kernel(DevMesh m, double k, 
     e1[i] = m.tri_edge[3 * t1 + i];
     e2[i] = m.tri_edge[3 * t2 + i];
   }
-  scatter_block(k, mom, p, q, c1, d1, c2, d2, e1, e2, Z, ldz, false);
+  scatter_block(k, mom, p, q, c1, d1, c2, d2, e1, e2, Z, ldz);
 }
 
 // ------------------------------------------------------------------ singular pairs
@@ -317,7 +319,7 @@ __device__ __forceinline__ void ss_moments(double k, int nss, int J, const doubl
 
 // One touching pair (index pair of m.touch) by one warp: the lanes share the points, a halving
 // reduction and a broadcast leave the moments in every lane, and lanes 0-8 form one entry each
-// of the 3 x 3 RWG block and add it (and its mirror) into Z.
+// of the 3 x 3 RWG block and add it into the lower triangle of Z.
 template <typename OutT>
 __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int nss, OutT* Z, int64_t ldz, int64_t pair) {
   const int lane = threadIdx.x & 31;
@@ -384,9 +386,12 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
   // -ik (ar + i ai) = k ai - i k ar;  (i/k) dd (I0r + i I0i) = -(dd/k) I0i + i (dd/k) I0r
   const double zr = k * cc * ai - dk * acc[1];
   const double zi = -k * cc * ar + dk * acc[0];
+  // an ordered pair (t1, t2) stands for (t2, t1) too: both meet on the diagonal, and an identical
+  // pair's block holds both of an entry's halves already
   const int e1 = m.tri_edge[3 * t1 + i], e2 = m.tri_edge[3 * t2 + j];
-  atomic_add_c(Z + 2 * (int64_t(e1) * ldz + e2), zr, zi);
-  if (t1 != t2) atomic_add_c(Z + 2 * (int64_t(e2) * ldz + e1), zr, zi);
+  if (t1 == t2 && e1 < e2) return;
+  const double f = t1 != t2 && e1 == e2 ? 2.0 : 1.0;
+  atomic_add_c(Z + 2 * lower_at(e1, e2, ldz), f * zr, f * zi);
 }
 
 // four touching pairs per 128-thread CTA, one per warp
@@ -427,6 +432,43 @@ __global__ void __launch_bounds__(128) efie_singular_batched_kernel(const BatchI
   if (w >= pairs) return;
   const BatchItem& it = items[batch_find(items, nitems, w, false)];
   singular_pair(it.m, it.k, nss, it.Z, it.ldz, w - it.pair_start);
+}
+
+// ------------------------------------------------------------------ the two triangles of Z
+// Zeroes the lower triangle: a CTA per rows y and n - 1 - y (n + 1 entries together).  Scalars
+// (T = double or float), so a matrix aligned to its scalar is enough.
+template <typename T>
+__global__ void __launch_bounds__(256) zero_lower_kernel(T* Z, int64_t n, int64_t ldz) {
+  for (int h = 0; h < 2; ++h) {
+    const int64_t row = h == 0 ? int64_t(blockIdx.x) : n - 1 - int64_t(blockIdx.x);
+    if (h == 1 && row == int64_t(blockIdx.x)) return;
+    T* z = Z + 2 * row * ldz;
+    for (int64_t c = threadIdx.x; c < 2 * (row + 1); c += 256) z[c] = T(0);
+  }
+}
+
+// Z[c][r] = Z[r][c] for r > c, 32 x 32 tiles through shared memory.  The 66-scalar pitch puts the
+// transposed reads of a warp (16 rows x 2 parts) in different banks.  HBM-bound: half of Z read,
+// half written.  With the unordered pairs the assembly of T = 20480 takes 119 ms, 229 ms with ordered ones.
+constexpr int kMirrorTile = 32;
+template <typename T>
+__global__ void __launch_bounds__(256) mirror_lower_kernel(T* Z, int64_t n, int64_t ldz) {
+  __shared__ T tile[kMirrorTile][2 * kMirrorTile + 2];
+  int64_t rt, ct;
+  if (!lower_tile((n + kMirrorTile - 1) / kMirrorTile, blockIdx.y, blockIdx.x, rt, ct)) return;
+  const int64_t r0 = rt * kMirrorTile, c0 = ct * kMirrorTile;
+  const int l = threadIdx.x & 63, w = threadIdx.x >> 6;
+#pragma unroll
+  for (int q = 0; q < kMirrorTile; q += 4) {
+    const int64_t r = r0 + q + w, c = c0 + (l >> 1);
+    if (r < n && c <= r) tile[q + w][l] = Z[2 * (r * ldz + c) + (l & 1)];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kMirrorTile; q += 4) {
+    const int64_t r = r0 + (l >> 1), c = c0 + q + w;
+    if (r < n && c < r) Z[2 * (c * ldz + r) + (l & 1)] = tile[l >> 1][2 * (q + w) + (l & 1)];
+  }
 }
 
 // ------------------------------------------------------------------ right-hand side
@@ -603,15 +645,29 @@ inline unsigned blocks_for(int64_t n, int bs) { return unsigned((n + bs - 1) / b
 }  // namespace
 
 cudaError_t launch_assemble_regular(const DevMesh& m, double k, int arith, void* Z, int64_t ldz, cudaStream_t s) {
-  dim3 grid(blocks_for(m.nt, 32), blocks_for(m.nt, 8));
-  ProfScope prof("asm_regular", s, 36.0 * (double(m.nt) * double(m.nt) - double(2 * m.ntouch - m.nt)));
-  if (arith == FOSB_ASM_FP64) {
+  ProfScope prof("asm_regular", s, regular_point_pairs(m));
+  if (arith == FOSB_ASM_FF) return launch_efie_regular_ff(m, k, static_cast<double*>(Z), ldz, s);
+  dim3 grid(unsigned(pair_tiles_width(m.nt)), unsigned(pair_tiles_rows(m.nt, 8)));
+  if (arith == FOSB_ASM_FP64)
     efie_regular_kernel<double, double><<<grid, 256, 0, s>>>(m, k, static_cast<double*>(Z), ldz);
-  } else if (arith == FOSB_ASM_FF) {
-    return launch_efie_regular_ff(m, k, static_cast<double*>(Z), ldz, s);
-  } else {
+  else
     efie_regular_kernel<float, float><<<grid, 256, 0, s>>>(m, k, static_cast<float*>(Z), ldz);
-  }
+  return launched();
+}
+
+cudaError_t zero_lower(void* Z, int64_t n, int64_t ldz, bool c64, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  if (c64) zero_lower_kernel<float><<<unsigned((n + 1) / 2), 256, 0, s>>>(static_cast<float*>(Z), n, ldz);
+  else zero_lower_kernel<double><<<unsigned((n + 1) / 2), 256, 0, s>>>(static_cast<double*>(Z), n, ldz);
+  return launched();
+}
+
+cudaError_t mirror_lower(void* Z, int64_t n, int64_t ldz, bool c64, cudaStream_t s) {
+  if (n == 0) return cudaSuccess;
+  const int64_t C = (n + kMirrorTile - 1) / kMirrorTile;
+  const dim3 grid(unsigned(C + 1), unsigned((C + 1) / 2));
+  if (c64) mirror_lower_kernel<float><<<grid, 256, 0, s>>>(static_cast<float*>(Z), n, ldz);
+  else mirror_lower_kernel<double><<<grid, 256, 0, s>>>(static_cast<double*>(Z), n, ldz);
   return launched();
 }
 

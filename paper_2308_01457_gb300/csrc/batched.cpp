@@ -124,8 +124,7 @@ fosb_status fosb_assemble_efie_batched(int64_t nbatch, const fosb_mesh* meshes, 
   }
   auto zero_all = [&]() -> cudaError_t {
     for (int i = 0; i < n; ++i) {
-      const int64_t N = dm[i]->ne;
-      cudaError_t e = cudaMemset2DAsync(dZ[i], ldz[i] * 16, 0, N * 16, N, s);
+      const cudaError_t e = zero_lower(dZ[i], dm[i]->ne, ldz[i], false, s);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -183,6 +182,7 @@ fosb_status fosb_assemble_efie_batched(int64_t nbatch, const fosb_mesh* meshes, 
   }
   FOSB_CUDA(launch_singular_rhs_batched(dm.data(), k, dZ.data(), ldz, db.data(), ldb_v.data(), dinc.data(), ninc.data(),
                                         n, nss, base + reg_bytes, s));
+  for (int i = 0; i < n; ++i) FOSB_CUDA(mirror_lower(dZ[i], dm[i]->ne, ldz[i], false, s));
   if (chosen) {
     chosen->warps = arith == FOSB_ASM_FF ? shape.warps : 0;
     chosen->ctas_per_sm = arith == FOSB_ASM_FF ? shape.min_ctas : 0;

@@ -16,7 +16,8 @@
 //   mu_ab = sum_pq w_p w_q lambda_pa beta_qb G0(x_p, y_q)
 // determines the RWG block exactly (with P_a, Q_b the vertices):
 //   Z_ij = (s_i l_i s'_j l'_j / (4 pi)) [ -(ik/4) sum_ab mu_ab (P_a - P_i).(Q_b - Q_j) + (i/k) sum_ab mu_ab ],
-// which is formed in float-float and added to the complex128 Z with FP64 atomics.
+// which is formed in float-float and added to the lower triangle of the complex128 Z with FP64
+// atomics; pairs are unordered (t1 < t2), the upper triangle is mirrored afterwards.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,6 +25,7 @@
 #include <vector>
 
 #include "fosb_internal.h"
+#include "pair_tiles.cuh"
 
 namespace fosb {
 namespace {
@@ -100,8 +102,9 @@ struct FFConst {
   float c1, c2, c3, inv_c;  // pi/64 = c1 + c2 + c3 (c1, c2 with <= 14 significant bits); 64/pi
 };
 
-__device__ __forceinline__ ff ldff(const float* base, int64_t nt, int f, int64_t t) {
-  return {base[int64_t(f) * nt + t], base[int64_t(f + 1) * nt + t]};
+// (32-bit indices: a dense Z on this card has fewer than 2^17 triangles, 60 nt < 2^31)
+__device__ __forceinline__ ff ldff(const float* base, int nt, int f, int t) {
+  return {base[f * nt + t], base[(f + 1) * nt + t]};
 }
 
 // exp(i theta) for theta = th + tl >= 0, |j| < 1024, table in shared memory
@@ -130,8 +133,8 @@ __device__ __forceinline__ void expi_ff(ff theta, const FFConst& C, const float 
   cs = ff_add(ff_mul(Cc, cd), ff_neg(ff_mul(S, sd)));
 }
 
-// One regular point pair block: test triangle t1, trial triangle t2 (t1, t2 < m.nt); adds the
-// 3 x 3 RWG block into Z unless the triangles touch.  tab: the sin/cos table in shared memory.
+// One regular point pair block: test triangle t1, trial triangle t2 (t1 < t2 < m.nt); adds the
+// 3 x 3 RWG block into the lower triangle of Z unless the triangles touch.  tab: the sin/cos table in shared memory.
 // MFIO: also the block of the MFIO of the dielectric (PMCHWT) system, into ZK (same ldz):
 //   K_ij = -int int (x - y).(f_j(y) x f_i(x)) g,  g = exp(ikr)(ikr - 1)/(4 pi r^3).
 // With a = x - p_i, b = y - q_j, (x - y).(b x a) = (p_i - q_j).(b x a) is bilinear in the
@@ -140,8 +143,8 @@ __device__ __forceinline__ void expi_ff(ff theta, const FFConst& C, const float 
 // gives K_ij = -(s_i l_i s'_j l'_j / (16 pi)) sum_ab nu_ab (p_i - q_j).((Q_b - q_j) x (P_a - p_i)).
 template <bool MFIO>
 __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst& C, double* Z, double* ZK,
-                                                int64_t ldz, int64_t t1, int64_t t2, const float (*tab)[4]) {
-  const int64_t nt = m.nt;
+                                                int64_t ldz, int t1, int t2, const float (*tab)[4]) {
+  const int nt = int(m.nt);
   int v1[3], v2[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -319,7 +322,7 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
       const ff zr = ff_add(ff_mul(C.k4, V.i), ff_neg(ff_mul(C.kinv, I0.i)));
       const ff zi = ff_add(ff_mul(C.kinv, I0.r), ff_neg(ff_mul(C.k4, V.r)));
       const ff sig = ff_mul(ff_mul(sl1[i], sl2[j]), C.inv4pi);
-      double* dst = Z + 2 * (int64_t(e1[i]) * ldz + e2[j]);
+      double* dst = Z + 2 * lower_at(e1[i], e2[j], ldz);
       atomicAdd(dst, to_d(ff_mul(sig, zr)));
       atomicAdd(dst + 1, to_d(ff_mul(sig, zi)));
     }
@@ -382,7 +385,7 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
         // K_ij = -(s_i l_i s'_j l'_j / (16 pi)) V
         const ff sig = ff_mul(ff_mul(sl1[i], sl2[j]), C.inv4pi);
         const float q4 = -0.25f;
-        double* dst = ZK + 2 * (int64_t(e1[i]) * ldz + e2[j]);
+        double* dst = ZK + 2 * lower_at(e1[i], e2[j], ldz);
         atomicAdd(dst, to_d(ff_mul(sig, V.r)) * q4);
         atomicAdd(dst + 1, to_d(ff_mul(sig, V.i)) * q4);
       }
@@ -391,29 +394,31 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
 }
 
 __global__ void __launch_bounds__(128) efie_regular_ff_kernel(DevMesh m, FFConst C, double* Z, int64_t ldz) {
+  int64_t rg, cb;
+  if (!pair_tile(m.nt, 4, blockIdx.y, blockIdx.x, rg, cb)) return;
   __shared__ float tab[128][4];
   for (int e = threadIdx.x; e < 128 * 4; e += blockDim.x) tab[e >> 2][e & 3] = c_sctab[e >> 2][e & 3];
   __syncthreads();
-  const int64_t t1 = int64_t(blockIdx.y) * 4 + (threadIdx.x >> 5);
-  const int64_t t2 = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (t1 >= m.nt || t2 >= m.nt) return;
+  const int t1 = int(rg) * 4 + (threadIdx.x >> 5), t2 = int(cb) * 32 + (threadIdx.x & 31);
+  if (t2 >= int(m.nt) || t1 >= t2) return;
   regular_ff_pair<false>(m, C, Z, nullptr, ldz, t1, t2, tab);
 }
 
 // Dielectric (PMCHWT) system: the EFIO block into ZT and the MFIO block into ZK.
 __global__ void __launch_bounds__(128, 3) pmchwt_regular_ff_kernel(DevMesh m, FFConst C, double* ZT, double* ZK,
                                                                 int64_t ldz) {
+  int64_t rg, cb;
+  if (!pair_tile(m.nt, 4, blockIdx.y, blockIdx.x, rg, cb)) return;
   __shared__ float tab[128][4];
   for (int e = threadIdx.x; e < 128 * 4; e += blockDim.x) tab[e >> 2][e & 3] = c_sctab[e >> 2][e & 3];
   __syncthreads();
-  const int64_t t1 = int64_t(blockIdx.y) * 4 + (threadIdx.x >> 5);
-  const int64_t t2 = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (t1 >= m.nt || t2 >= m.nt) return;
+  const int t1 = int(rg) * 4 + (threadIdx.x >> 5), t2 = int(cb) * 32 + (threadIdx.x & 31);
+  if (t2 >= int(m.nt) || t1 >= t2) return;
   regular_ff_pair<true>(m, C, ZT, ZK, ldz, t1, t2, tab);
 }
 
 // Batched form: one persistent launch over the tiles of many meshes.  Tile w of the batch
-// (WARPS test triangles x 32 trial triangles) belongs to the item with the largest
+// (WARPS test triangles x 32 trial triangles, pair_tiles.cuh) belongs to the item with the largest
 // tile_start <= w; CTAs take tiles from a device ticket until the batch is exhausted, so
 // meshes of uneven size share the GPU without per-mesh launches.
 struct FFBatchItem {
@@ -421,7 +426,7 @@ struct FFBatchItem {
   FFConst C;
   double* Z;
   int64_t ldz;
-  int64_t tiles_x;     // ceil(nt / 32)
+  int64_t tiles_x;     // pair_tiles_width(nt)
   int64_t tile_start;  // first tile of this item in the batch
 };
 
@@ -462,8 +467,10 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) efie_regular_ff_batched_kern
     }
     const int64_t local = w - s_item.tile_start;
     const int64_t ty = local / s_item.tiles_x, tx = local - ty * s_item.tiles_x;
-    const int64_t t1 = ty * WARPS + (threadIdx.x >> 5), t2 = tx * 32 + (threadIdx.x & 31);
-    if (t1 < s_item.m.nt && t2 < s_item.m.nt)
+    int64_t rg, cb;
+    const bool any = pair_tile(s_item.m.nt, WARPS, ty, tx, rg, cb);
+    const int t1 = int(rg) * WARPS + (threadIdx.x >> 5), t2 = int(cb) * 32 + (threadIdx.x & 31);
+    if (any && t2 < int(s_item.m.nt) && t1 < t2)
       regular_ff_pair<false>(s_item.m, s_item.C, s_item.Z, nullptr, s_item.ldz, t1, t2, tab);
     __syncthreads();  // s_tile / s_item are rewritten by the next ticket
   }
@@ -528,8 +535,8 @@ FFConst make_ff_const(double k) {
 cudaError_t launch_efie_regular_ff(const DevMesh& m, double k, double* Z, int64_t ldz, cudaStream_t s) {
   if (k * m.diameter >= ff_max_phase()) return cudaErrorInvalidValue;
   const FFConst C = make_ff_const(k);
-  dim3 grid(cdiv(m.nt, 32), cdiv(m.nt, 4));
-  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  if (cdiv(m.nt, 4) > 65535u) return cudaErrorInvalidValue;
+  const dim3 grid(unsigned(pair_tiles_width(m.nt)), unsigned(pair_tiles_rows(m.nt, 4)));
   efie_regular_ff_kernel<<<grid, 128, 0, s>>>(m, C, Z, ldz);
   return launched();
 }
@@ -539,8 +546,8 @@ cudaError_t launch_efie_regular_ff(const DevMesh& m, double k, double* Z, int64_
 cudaError_t launch_pmchwt_regular_ff(const DevMesh& m, double k, double* ZT, double* ZK, int64_t ldz, cudaStream_t s) {
   if (k * m.diameter >= ff_max_phase()) return cudaErrorInvalidValue;
   const FFConst C = make_ff_const(k);
-  dim3 grid(cdiv(m.nt, 32), cdiv(m.nt, 4));
-  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  if (cdiv(m.nt, 4) > 65535u) return cudaErrorInvalidValue;
+  const dim3 grid(unsigned(pair_tiles_width(m.nt)), unsigned(pair_tiles_rows(m.nt, 4)));
   pmchwt_regular_ff_kernel<<<grid, 128, 0, s>>>(m, C, ZT, ZK, ldz);
   return launched();
 }
@@ -567,9 +574,9 @@ cudaError_t launch_efie_regular_ff_batched(const DevMesh* const* meshes, const d
     items[i].C = make_ff_const(ks[i]);
     items[i].Z = Z[i];
     items[i].ldz = ldz[i];
-    items[i].tiles_x = (m.nt + 31) / 32;
+    items[i].tiles_x = pair_tiles_width(m.nt);
     items[i].tile_start = total;
-    total += items[i].tiles_x * ((m.nt + warps - 1) / warps);
+    total += items[i].tiles_x * pair_tiles_rows(m.nt, warps);
   }
   const size_t need = 256 + sizeof(FFBatchItem) * size_t(nmesh);
   if (scratch_bytes < need) return cudaErrorInvalidValue;
@@ -583,7 +590,7 @@ cudaError_t launch_efie_regular_ff_batched(const DevMesh* const* meshes, const d
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, warps * 32, 0);
   double pairs = 0.0;
-  for (int i = 0; i < nmesh; ++i) pairs += 36.0 * double(meshes[i]->nt) * double(meshes[i]->nt);
+  for (int i = 0; i < nmesh; ++i) pairs += regular_point_pairs(*meshes[i]);
   ProfScope prof("asm_regular", s, pairs);
   kern<<<unsigned(nsm * std::max(occ, 1)), warps * 32, 0, s>>>(d_items, nmesh, total, ticket);
   return launched();

@@ -146,7 +146,14 @@ struct Rules {
 Rules make_rules(int nss);
 
 // ---------------------------------------------------------------- kernels (launchers)
-// Assembly
+// Assembly: the pair kernels fill the lower triangle of the complex symmetric Z (zero_lower
+// before them), mirror_lower writes the upper one; n x n, complex64 or complex128.
+cudaError_t zero_lower(void* Z, int64_t n, int64_t ldz, bool c64, cudaStream_t s);
+cudaError_t mirror_lower(void* Z, int64_t n, int64_t ldz, bool c64, cudaStream_t s);
+// Point pairs of the vertex-disjoint unordered triangle pairs (the work of the regular kernels).
+inline double regular_point_pairs(const DevMesh& m) {
+  return 36.0 * (0.5 * double(m.nt) * double(m.nt + 1) - double(m.ntouch));
+}
 cudaError_t launch_assemble_regular(const DevMesh& m, double k, int arith, void* Z, int64_t ldz, cudaStream_t s);
 cudaError_t launch_assemble_singular(const DevMesh& m, double k, int nss, bool fp32_out, void* Z, int64_t ldz,
                                      cudaStream_t s);
@@ -165,7 +172,8 @@ cudaError_t launch_adjoint_pairs(const DevMesh& m, double k, int nss, const doub
 cudaError_t launch_adjoint_planewave(const DevMesh& m, double k, int64_t ncols, const double* d_pw, const double* wgt,
                                      int64_t ldw, double* grad, cudaStream_t s);
 cudaError_t launch_efie_regular_ff(const DevMesh& m, double k, double* Z, int64_t ldz, cudaStream_t s);
-// PMCHWT regular pairs in float-float for one wavenumber: EFIO blocks into ZT, MFIO blocks into ZK.
+// PMCHWT regular pairs in float-float for one wavenumber: EFIO blocks into ZT, MFIO blocks into
+// ZK (the lower triangles of both).
 cudaError_t launch_pmchwt_regular_ff(const DevMesh& m, double k, double* ZT, double* ZK, int64_t ldz, cudaStream_t s);
 
 // Far field

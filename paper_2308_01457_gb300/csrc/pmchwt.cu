@@ -16,9 +16,9 @@
 // Work decomposition.  One launch per wavenumber computes, for every triangle pair, the
 // EFIO and the MFIO 3 x 3 blocks from one set of point-pair evaluations (r, exp(ikr)) and
 // adds them with FP64 atomics into two N x N blocks of Z: K into the (1,1) block for both
-// wavenumbers, T_0 into the (1,2) block and T_1, as scratch, into the (2,2) block.  A final
-// pass rewrites every entry: (1,2) = T_0 + eta T_1, (2,1) = -T_0 - T_1/eta, (2,2) = (1,1).
-// So a triangle pair costs 18 complex atomics per wavenumber, the same as the PEC EFIE.
+// wavenumbers, T_0 into the (1,2) block and T_1, as scratch, into the (2,2) block.  T and K are
+// symmetric, so pairs are unordered and only the lower triangles are filled; a final pass
+// writes every entry: (1,2) = T_0 + eta T_1, (2,1) = -T_0 - T_1/eta, (2,2) = (1,1), mirrored.
 // The regular pairs run in FP64 here (FOSB_ASM_FP64) or in float-float on the FP32 pipe
 // (FOSB_ASM_FF, pmchwt_regular_ff_kernel in ff_assemble.cu, from barycentric moment
 // matrices); the touching pairs always run in FP64 here.
@@ -40,6 +40,7 @@
 #include <vector>
 
 #include "fosb_internal.h"
+#include "pair_tiles.cuh"
 
 namespace fosb {
 namespace {
@@ -101,13 +102,14 @@ __device__ __forceinline__ bool pm_shares_vertex(const int a[3], const int b[3])
 }
 
 // ------------------------------------------------------------------ regular pairs
-// One thread per ordered vertex-disjoint triangle pair (t1 test, t2 trial); a warp holds one
-// test triangle and 32 consecutive trial triangles.  FP64.
+// One thread per unordered vertex-disjoint triangle pair t1 < t2; a warp holds one test triangle
+// and 32 consecutive trial triangles.  FP64.
 __global__ void __launch_bounds__(256) pmchwt_regular_kernel(DevMesh m, double k, double* ZT, double* ZK,
                                                              int64_t ldz) {
-  const int64_t t1 = int64_t(blockIdx.y) * 8 + (threadIdx.x >> 5);
-  const int64_t t2 = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (t1 >= m.nt || t2 >= m.nt) return;
+  int64_t rg, cb;
+  if (!pair_tile(m.nt, 8, blockIdx.y, blockIdx.x, rg, cb)) return;
+  const int64_t t1 = rg * 8 + (threadIdx.x >> 5), t2 = cb * 32 + (threadIdx.x & 31);
+  if (t1 >= m.nt || t2 >= m.nt || t1 >= t2) return;
   int v1[3], v2[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(256) pmchwt_regular_kernel(DevMesh m, double k
 #pragma unroll
     for (int c = 0; c < 3; ++c) p[c] = m.verts[3 * v1[i] + c] - o1[c];
     const double c1 = m.tri_coef[3 * t1 + i], d1 = m.tri_div[3 * t1 + i];
-    const int64_t row = m.tri_edge[3 * t1 + i];
+    const int row = m.tri_edge[3 * t1 + i];
 #pragma unroll 1
     for (int j = 0; j < 3; ++j) {
       double q[3];
@@ -208,7 +210,7 @@ __global__ void __launch_bounds__(256) pmchwt_regular_kernel(DevMesh m, double k
       for (int c = 0; c < 3; ++c) q[c] = m.verts[3 * v2[j] + c] - o2[c];
       double tr, ti, kr, ki;
       pair_entry(k, e, h, p, q, D, c1 * m.tri_coef[3 * t2 + j], d1 * m.tri_div[3 * t2 + j], tr, ti, kr, ki);
-      const int64_t off = 2 * (row * ldz + m.tri_edge[3 * t2 + j]);
+      const int64_t off = 2 * lower_at(row, m.tri_edge[3 * t2 + j], ldz);
       atomic_add_z(ZT + off, tr, ti);
       atomic_add_z(ZK + off, kr, ki);
     }
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(256) pmchwt_regular_kernel(DevMesh m, double k
 // points (Sauter & Schwab, Boundary Element Methods, Section 5.2: six maps for identical,
 // five for edge-adjacent, two for vertex-adjacent pairs), a butterfly reduction leaves the
 // 36 moments in every lane, and lanes 0-8 form one entry each of the two 3 x 3 blocks and
-// add it and its mirror (both blocks are symmetric under exchanging the triangles).
+// add it into the lower triangles (both blocks are symmetric under exchanging the triangles).
 __device__ __forceinline__ void pm_chi(const double E[2][3], double u1, double u2, double out[3]) {
 #pragma unroll
   for (int c = 0; c < 3; ++c) out[c] = fma(u1, E[0][c], u2 * E[1][c]);
@@ -362,28 +364,62 @@ __global__ void __launch_bounds__(128) pmchwt_singular_kernel(DevMesh m, double 
   pair_entry(k, acc, acc + 16, p, q, D, m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j],
              m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j], tr, ti, kr, ki);
   if (!mfio) kr = ki = 0.0;
-  const int64_t e1 = m.tri_edge[3 * t1 + i], e2 = m.tri_edge[3 * t2 + j];
-  atomic_add_z(ZT + 2 * (e1 * ldz + e2), tr, ti);
-  atomic_add_z(ZK + 2 * (e1 * ldz + e2), kr, ki);
-  if (t1 != t2) {
-    atomic_add_z(ZT + 2 * (e2 * ldz + e1), tr, ti);
-    atomic_add_z(ZK + 2 * (e2 * ldz + e1), kr, ki);
-  }
+  // (t1, t2) stands for (t2, t1) too: both meet on the diagonal, and an identical pair's block
+  // holds both of an entry's halves already
+  const int e1 = m.tri_edge[3 * t1 + i], e2 = m.tri_edge[3 * t2 + j];
+  if (t1 == t2 && e1 < e2) return;
+  const double f = t1 != t2 && e1 == e2 ? 2.0 : 1.0;
+  const int64_t off = 2 * lower_at(e1, e2, ldz);
+  atomic_add_z(ZT + off, f * tr, f * ti);
+  atomic_add_z(ZK + off, f * kr, f * ki);
 }
 
 // ------------------------------------------------------------------ block combination
-// (1,2) = T_0 + eta T_1, (2,1) = -T_0 - T_1/eta, (2,2) = (1,1); T_0 in (1,2), T_1 in (2,2).
-__global__ void pmchwt_combine_kernel(int64_t N, double eta, double2* Z, int64_t ldz) {
-  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= N * N) return;
-  const int64_t r = e / N, c = e % N;
-  const double2 kk = Z[r * ldz + c];
-  const double2 t0 = Z[r * ldz + N + c];
-  const double2 t1 = Z[(N + r) * ldz + N + c];
+// (1,2) = T_0 + eta T_1, (2,1) = -T_0 - T_1/eta, (2,2) = (1,1); T_0 in (1,2), T_1 in (2,2), all
+// three read from their lower triangles and every block written in full: 32 x 32 tiles, the
+// mirrored half through shared memory.
+constexpr int kCombTile = 32;
+__global__ void __launch_bounds__(256) pmchwt_combine_kernel(int64_t N, double eta, double* Z, int64_t ldz) {
+  __shared__ double tile[kCombTile][2 * kCombTile + 2];
+  int64_t rt, ct;
+  if (!lower_tile((N + kCombTile - 1) / kCombTile, blockIdx.y, blockIdx.x, rt, ct)) return;
+  const int64_t r0 = rt * kCombTile, c0 = ct * kCombTile;
+  const int l = threadIdx.x & 63, w = threadIdx.x >> 6;
+  double* z12 = Z + 2 * N;
+  double* z21 = Z + 2 * N * ldz;
+  double* z22 = z21 + 2 * N;
   const double ie = 1.0 / eta;
-  Z[r * ldz + N + c] = make_double2(t0.x + eta * t1.x, t0.y + eta * t1.y);
-  Z[(N + r) * ldz + c] = make_double2(-t0.x - ie * t1.x, -t0.y - ie * t1.y);
-  Z[(N + r) * ldz + N + c] = kk;
+  double v[3][kCombTile / 4];  // K, the (1,2) and the (2,1) entry
+#pragma unroll
+  for (int q = 0; q < kCombTile / 4; ++q) {
+    const int64_t r = r0 + 4 * q + w, c = c0 + (l >> 1), at = 2 * (r * ldz + c) + (l & 1);
+    if (r < N && c <= r) {
+      const double t0 = z12[at], t1 = z22[at];
+      v[0][q] = Z[at];
+      v[1][q] = t0 + eta * t1;
+      v[2][q] = -t0 - ie * t1;
+      z12[at] = v[1][q];
+      z21[at] = v[2][q];
+      z22[at] = v[0][q];
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kCombTile / 4; ++q) tile[4 * q + w][l] = v[b][q];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kCombTile / 4; ++q) {
+      const int64_t r = r0 + (l >> 1), c = c0 + 4 * q + w, at = 2 * (c * ldz + r) + (l & 1);
+      if (r < N && c < r) {
+        const double x = tile[l >> 1][2 * (4 * q + w) + (l & 1)];
+        if (b == 0) Z[at] = z22[at] = x;
+        else if (b == 1) z12[at] = x;
+        else z21[at] = x;
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------------------ far field
@@ -431,12 +467,12 @@ inline unsigned pm_blocks(int64_t n, int bs) { return unsigned((n + bs - 1) / bs
 cudaError_t assemble_pmchwt_one_k(const DevMesh& d, double k, int nss, int arith, double* ZT, double* ZK,
                                   int64_t ldz, cudaStream_t s) {
   {
-    ProfScope prof("pmchwt_regular", s, 36.0 * (double(d.nt) * double(d.nt) - double(2 * d.ntouch - d.nt)));
+    ProfScope prof("pmchwt_regular", s, regular_point_pairs(d));
     cudaError_t e;
     if (arith == FOSB_ASM_FF) {
       e = launch_pmchwt_regular_ff(d, k, ZT, ZK, ldz, s);
     } else {
-      dim3 grid(pm_blocks(d.nt, 32), pm_blocks(d.nt, 8));
+      const dim3 grid(unsigned(pair_tiles_width(d.nt)), unsigned(pair_tiles_rows(d.nt, 8)));
       pmchwt_regular_kernel<<<grid, 256, 0, s>>>(d, k, ZT, ZK, ldz);
       e = launched();
     }
@@ -495,10 +531,11 @@ fosb_status fosb_assemble_pmchwt(fosb_mesh mesh, double k0, double eps_r, double
   double* z11 = z;
   double* z12 = z + 2 * N;
   double* z22 = z + 2 * (N * ldz + N);
-  FOSB_CUDA(cudaMemset2DAsync(Z, ldz * 16, 0, 2 * N * 16, 2 * N, s));
+  for (double* block : {z11, z12, z22}) FOSB_CUDA(zero_lower(block, N, ldz, false, s));
   FOSB_CUDA(assemble_pmchwt_one_k(mesh->d, k0, nss, arith, z12, z11, ldz, s));
   FOSB_CUDA(assemble_pmchwt_one_k(mesh->d, k1, nss, arith, z22, z11, ldz, s));
-  pmchwt_combine_kernel<<<pm_blocks(N * N, 256), 256, 0, s>>>(N, eta, static_cast<double2*>(Z), ldz);
+  const int64_t C = (N + kCombTile - 1) / kCombTile;
+  pmchwt_combine_kernel<<<dim3(unsigned(C + 1), unsigned((C + 1) / 2)), 256, 0, s>>>(N, eta, z, ldz);
   FOSB_CUDA(launched());
   if (n_inc > 0) {
     // rows d, Re p, Im p for the Dirichlet data and d, Re(d x p), Im(d x p) for the Neumann
