@@ -45,6 +45,11 @@ void upload_rules(const Rules& r) {
   cudaMemcpyToSymbol(c_ss_series, c, sizeof(c));
 }
 
+const double* ss_table_device() {
+  void* p = nullptr;
+  return cudaGetSymbolAddress(&p, g_ss_table) == cudaSuccess ? static_cast<const double*>(p) : nullptr;
+}
+
 namespace {
 
 constexpr double kInv4Pi = 0.07957747154594767;  // 1/(4 pi)
@@ -226,50 +231,17 @@ __global__ void __launch_bounds__(256) efie_regular_kernel(DevMesh m, double k, 
 // instructions per 5 points against 77 per point when every point had its own 1/r and
 // exp(ikr).  At T = 20480, n_ss = 5, k = 4: 9.2 ms, 46.0 ms before; at T = 320, k = 1 the whole
 // assembly call takes 0.32 ms, 1.14 ms before.
-// The series up to here (its rounding is then below 6e-16 of |S_m|, 8e-16 at phase 4; 15 terms);
-// larger phases, which only meshes with edges beyond about half a wavelength reach, take sincos per point.
-constexpr double kSsMaxPhase = 3.0;
-
-// Number of phi^2 powers for phases up to ph: the first J with ph^{2J}/(2J)! < 2^-56 (the
-// moments' decay only helps), at most kSsTerms, which covers kSsMaxPhase.
-__device__ __forceinline__ int ss_terms(float ph) {
-  const float p2 = ph * ph;
-  float t = 1.f;
-  int J = 0;
-  while (J < kSsTerms && t > 1.3e-17f) {
-    t *= p2 / float((2 * J + 1) * (2 * J + 2));
-    ++J;
-  }
-  return J;
-}
-
 // The moment sums of one lane: I0, then u1, u2, v1, v2, then u1v1, u1v2, u2v1, u2v2 (complex).
 template <int KIND>
 __device__ __forceinline__ void ss_moments(double k, int nss, int J, const double (&EP)[2][3], const double (&EQ)[2][3],
                                            int lane, double (&acc)[18]) {
-  const int n3 = nss * nss * nss, stride = kSsRegions * n3;
-  const int first = KIND == 3 ? 0 : (KIND == 2 ? 6 : 11), count = (KIND == 3 ? 6 : (KIND == 2 ? 5 : 2)) * n3;
-  const double* tab = g_ss_table + first * n3;
+  const int n3 = nss * nss * nss, stride = kSsRegions * n3, count = ss_regions<KIND>() * n3;
+  const double* tab = g_ss_table + ss_first_region<KIND>() * n3;
   for (int idx = lane; idx < count; idx += 32) {
     auto T = [&](int f) { return __ldg(tab + f * stride + idx); };
-    const double u1 = T(0), u2 = T(1), v1 = T(2), v2 = T(3);
-    double d[3];
-    if constexpr (KIND == 3) {  // EQ = EP: the coordinate differences are in the table
-      const double a = T(9), b = T(10);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], b * EP[1][c]);
-    } else if constexpr (KIND == 2) {  // EQ[0] = EP[0], the shared edge
-      const double a = T(9);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], fma(u2, EP[1][c], -v2 * EQ[1][c]));
-    } else {
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        d[c] = fma(u1, EP[0][c], fma(u2, EP[1][c], fma(-v1, EQ[0][c], -v2 * EQ[1][c])));
-    }
-    const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
-    const double rinv = ss_rsqrt(r2);
-    const double phi = k * (r2 * rinv);
+    const double uv[4] = {T(0), T(1), T(2), T(3)};
+    double rinv, phi;
+    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, rinv, phi);
     double sr[3], si[3];
     if (J > 0) {
       const double p2 = phi * phi;
@@ -305,7 +277,6 @@ __device__ __forceinline__ void ss_moments(double k, int nss, int J, const doubl
     acc[0] = fma(g, sr[0], acc[0]);
     acc[1] = fma(g, si[0], acc[1]);
     const double ar = g * sr[1], ai = g * si[1], br = g * sr[2], bi = g * si[2];
-    const double uv[4] = {u1, u2, v1, v2};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const double p = T(5 + q);
@@ -342,8 +313,7 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
     EQ[0][c] = Q[1][c] - Q[0][c];
     EQ[1][c] = Q[2][c] - Q[1][c];
   }
-  const float ph = ss_phase_bound(k, EP, EQ);
-  const int J = ph <= float(kSsMaxPhase) ? ss_terms(ph) : 0;
+  const int J = ss_terms(ss_phase_bound(k, EP, EQ));
   double acc[18];
 #pragma unroll
   for (int i = 0; i < 18; ++i) acc[i] = 0.0;
@@ -355,7 +325,7 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
   // lane = 3 i + j: entry (i, j) of the block,
   //   A_ij = c_i c'_j [XY - q_j.X - p_i.Y + (p_i.q_j) I0],  Phi_ij = d_i d'_j I0,
   //   Z_ij += -ik A_ij + (i/k) Phi_ij,
-  // with p_i, q_j the opposite vertices relative to P0 = Q0 and X = EP.u, Y = EQ.v, XY = u EP.EQ v
+  // with p_i, q_j the opposite vertices relative to P0 = Q0
   const int i = lane / 3, j = lane % 3;
   const int t1 = tp.t1, t2 = tp.t2;
   const double jac = 4.0 * m.tri_area[t1] * m.tri_area[t2] * kInv4Pi;
@@ -366,21 +336,8 @@ __device__ __forceinline__ void singular_pair(const DevMesh& m, double k, int ns
     pi_[c] = m.verts[3 * a + c] - P[0][c];
     qj[c] = m.verts[3 * b + c] - Q[0][c];
   }
-  auto dot = [](const double (&x)[3], const double (&y)[3]) { return fma(x[0], y[0], fma(x[1], y[1], x[2] * y[2])); };
-  const double pq = dot(pi_, qj);
-  double ar = pq * acc[0], ai = pq * acc[1];
-#pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    const double qe = dot(qj, EP[s]), pf = dot(pi_, EQ[s]);
-    ar -= fma(qe, acc[2 + 2 * s], pf * acc[6 + 2 * s]);
-    ai -= fma(qe, acc[3 + 2 * s], pf * acc[7 + 2 * s]);
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const double ef = dot(EP[s], EQ[t]);
-      ar = fma(ef, acc[10 + 4 * s + 2 * t], ar);
-      ai = fma(ef, acc[11 + 4 * s + 2 * t], ai);
-    }
-  }
+  double ar, ai;
+  ss_efio_entry(acc, EP, EQ, pi_, qj, ar, ai);
   const double cc = jac * m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j];
   const double dk = jac * m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j] * kinv;
   // -ik (ar + i ai) = k ai - i k ar;  (i/k) dd (I0r + i I0i) = -(dd/k) I0i + i (dd/k) I0r

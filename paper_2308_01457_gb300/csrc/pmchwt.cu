@@ -41,6 +41,7 @@
 
 #include "fosb_internal.h"
 #include "pair_tiles.cuh"
+#include "sauter_schwab.cuh"
 
 namespace fosb {
 namespace {
@@ -49,6 +50,7 @@ __constant__ double c_pm_bary[6][3];
 __constant__ double c_pm_w[6];
 __constant__ double c_pm_glx[16];
 __constant__ double c_pm_glw[16];
+__constant__ double c_pm_series[kSsTerms][10];  // make_ss_series, then make_ss_series_mfio
 
 constexpr double kInv4PiPm = 0.07957747154594767;  // 1/(4 pi)
 
@@ -218,58 +220,91 @@ __global__ void __launch_bounds__(256) pmchwt_regular_kernel(DevMesh m, double k
 }
 
 // ------------------------------------------------------------------ singular pairs
-// One touching pair per warp (four per CTA): the lanes share the Sauter-Schwab 4-cube
-// points (Sauter & Schwab, Boundary Element Methods, Section 5.2: six maps for identical,
-// five for edge-adjacent, two for vertex-adjacent pairs), a butterfly reduction leaves the
-// 36 moments in every lane, and lanes 0-8 form one entry each of the two 3 x 3 blocks and
-// add it into the lower triangles (both blocks are symmetric under exchanging the triangles).
-__device__ __forceinline__ void pm_chi(const double E[2][3], double u1, double u2, double out[3]) {
+// One touching pair per warp (four per CTA), FP64, Sauter-Schwab in the form (x, y) = xi (xh, yh)
+// (Sauter & Schwab, Boundary Element Methods, Section 5.2; see efie_singular_kernel): the n_ss
+// points along xi share rh = |xh - yh| and phi = k rh, and their sums are power series in phi:
+//   EFIO:  S_m / rh,     S_m = sum_a w_a xi_a^{2+m} exp(i phi xi_a), m = 0 (I0), 1 (X, Y), 2 (XY);
+//   MFIO:  Q_m / rh^3,   Q_m = sum_a w_a xi_a^m (i phi xi_a - 1) exp(i phi xi_a), m = 1, 2.
+// With D = 0 the MFIO entry needs neither J0 nor the full JX, JY: (p - q).(q x p) = 0 and
+//   K_ij = -c_i c'_j [(p - q).JYX + (p x q).(JY - JX)].
+// Moments in the reference coordinates (u, v) as for the EFIE; identical pairs skip the MFIO.
+// Bound by the FP64 pipe.  At T = 5120, n_ss = 5, both wavenumbers: 8.0 ms, 29.3 ms with every point by itself.
+template <int KIND>
+__device__ __forceinline__ void pm_moments(const double* __restrict__ table, double k, int nss, int J,
+                                           const double (&EP)[2][3], const double (&EQ)[2][3], int lane,
+                                           double (&e)[18], double (&h)[16]) {
+  constexpr bool MFIO = KIND != 3;
+  constexpr int NS = MFIO ? 10 : 6;
+  const int n3 = nss * nss * nss, stride = kSsRegions * n3, count = ss_regions<KIND>() * n3;
+  const double* tab = table + ss_first_region<KIND>() * n3;
+  for (int idx = lane; idx < count; idx += 32) {
+    auto T = [&](int f) { return __ldg(tab + f * stride + idx); };
+    const double uv[4] = {T(0), T(1), T(2), T(3)};
+    double rinv, phi;
+    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, rinv, phi);
+    // s: Re S_0..2, Im S_0..2, Re Q_1..2, Im Q_1..2
+    double s[NS];
+    if (J > 0) {
+      const double p2 = phi * phi;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) out[c] = fma(u1, E[0][c], u2 * E[1][c]);
+      for (int i = 0; i < NS; ++i) s[i] = c_pm_series[J - 1][i];
+      for (int j = J - 2; j >= 0; --j)
+#pragma unroll
+        for (int i = 0; i < NS; ++i) s[i] = fma(s[i], p2, c_pm_series[j][i]);
+#pragma unroll
+      for (int i = 3; i < 6; ++i) s[i] *= phi;
+#pragma unroll
+      for (int i = 8; i < NS; ++i) s[i] *= phi;
+    } else {
+#pragma unroll
+      for (int i = 0; i < NS; ++i) s[i] = 0.0;
+      for (int a = 0; a < nss; ++a) {
+        const double xi = c_pm_glx[a], px = phi * xi;
+        double sn, cs, w = c_pm_glw[a] * xi;
+        sincos(px, &sn, &cs);
+        const double hr = -cs - px * sn, hi = px * cs - sn;
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          if (MFIO && m < 2) {
+            s[(MFIO ? 6 : 0) + m] += w * hr;
+            s[(MFIO ? 8 : 0) + m] += w * hi;
+          }
+          w *= xi;
+          s[m] += w * cs;
+          s[3 + m] += w * sn;
+        }
+      }
+    }
+    const double g = T(4) * rinv, g3 = g * (rinv * rinv);
+    e[0] = fma(g, s[0], e[0]);
+    e[1] = fma(g, s[3], e[1]);
+    const double ar = g * s[1], ai = g * s[4], br = g * s[2], bi = g * s[5];
+    double cr = 0, ci = 0, dr = 0, di = 0;
+    if constexpr (MFIO) {
+      cr = g3 * s[6];
+      ci = g3 * s[8];
+      dr = g3 * s[7];
+      di = g3 * s[9];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double p = T(5 + q);
+      e[2 + 2 * q] = fma(uv[q], ar, e[2 + 2 * q]);
+      e[3 + 2 * q] = fma(uv[q], ai, e[3 + 2 * q]);
+      e[10 + 2 * q] = fma(p, br, e[10 + 2 * q]);
+      e[11 + 2 * q] = fma(p, bi, e[11 + 2 * q]);
+      if constexpr (MFIO) {
+        h[2 * q] = fma(uv[q], cr, h[2 * q]);
+        h[1 + 2 * q] = fma(uv[q], ci, h[1 + 2 * q]);
+        h[8 + 2 * q] = fma(p, dr, h[8 + 2 * q]);
+        h[9 + 2 * q] = fma(p, di, h[9 + 2 * q]);
+      }
+    }
+  }
 }
 
-__device__ __forceinline__ void pm_accumulate(double k, bool mfio, const double x[3], const double y[3], double w,
-                                              double acc[36]) {
-  const double dx = x[0] - y[0], dy = x[1] - y[1], dz = x[2] - y[2];
-  const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-  const double rinv = rsqrt(r2);
-  const double r = r2 * rinv;
-  double sn, cs;
-  sincos(k * r, &sn, &cs);
-  const double g = w * rinv;
-  const double gr = cs * g, gi = sn * g;
-  acc[0] += gr;
-  acc[1] += gi;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    acc[2 + 2 * c] += gr * x[c];
-    acc[3 + 2 * c] += gi * x[c];
-    acc[8 + 2 * c] += gr * y[c];
-    acc[9 + 2 * c] += gi * y[c];
-  }
-  const double xy = x[0] * y[0] + x[1] * y[1] + x[2] * y[2];
-  acc[14] += gr * xy;
-  acc[15] += gi * xy;
-  if (!mfio) return;
-  const double kr = k * r, rinv2 = rinv * rinv;
-  const double hr = (-gr - gi * kr) * rinv2, hi = (gr * kr - gi) * rinv2;
-  double* h = acc + 16;
-  h[0] += hr;
-  h[1] += hi;
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
-    const double yx = y[c1] * x[c2] - y[c2] * x[c1];  // (y x x)_c
-    h[2 + 2 * c] += hr * x[c];
-    h[3 + 2 * c] += hi * x[c];
-    h[8 + 2 * c] += hr * y[c];
-    h[9 + 2 * c] += hi * y[c];
-    h[14 + 2 * c] += hr * yx;
-    h[15 + 2 * c] += hi * yx;
-  }
-}
-
-__global__ void __launch_bounds__(128) pmchwt_singular_kernel(DevMesh m, double k, int nss, double* ZT, double* ZK,
+__global__ void __launch_bounds__(128) pmchwt_singular_kernel(DevMesh m, double k, int nss,
+                                                              const double* __restrict__ table, double* ZT, double* ZK,
                                                               int64_t ldz) {
   const int64_t pair = int64_t(blockIdx.x) * 4 + (threadIdx.x >> 5);
   if (pair >= m.ntouch) return;
@@ -293,77 +328,67 @@ __global__ void __launch_bounds__(128) pmchwt_singular_kernel(DevMesh m, double 
     EQ[0][c] = Q[1][c] - Q[0][c];
     EQ[1][c] = Q[2][c] - Q[1][c];
   }
-  const int n2 = nss * nss, n4 = n2 * n2;
-  double acc[36];
+  // one more term than the EFIO alone: the MFIO's coefficients carry a factor 2j - 1
+  const int J = ss_terms(ss_phase_bound(k, EP, EQ));
+  const int terms = J > 0 ? min(J + 1, kSsTerms) : 0;
+  double e[18], h[16];
 #pragma unroll
-  for (int i = 0; i < 36; ++i) acc[i] = 0.0;
-  for (int idx = lane; idx < n4; idx += 32) {
-    const int a = idx / (n2 * nss), b = (idx / n2) % nss, c = (idx / nss) % nss, d = idx % nss;
-    const double xi = c_pm_glx[a], e1 = c_pm_glx[b], e2 = c_pm_glx[c], e3 = c_pm_glx[d];
-    const double w4 = c_pm_glw[a] * c_pm_glw[b] * c_pm_glw[c] * c_pm_glw[d];
-    double x[3], y[3];
-    if (tp.kind == 3) {
-      const double w = w4 * xi * xi * xi * e1 * e1 * e2;
-      const double s[6][4] = {
-          {xi, xi * (1 - e1 + e1 * e2), xi * (1 - e1 * e2 * e3), xi * (1 - e1)},
-          {xi * (1 - e1 * e2 * e3), xi * (1 - e1), xi, xi * (1 - e1 + e1 * e2)},
-          {xi, xi * e1 * (1 - e2 + e2 * e3), xi * (1 - e1 * e2), xi * e1 * (1 - e2)},
-          {xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * (1 - e2 + e2 * e3)},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * (1 - e2)},
-          {xi, xi * e1 * (1 - e2), xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3)}};
+  for (int i = 0; i < 18; ++i) e[i] = 0.0;
 #pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        pm_chi(EP, s[j][0], s[j][1], x);
-        pm_chi(EQ, s[j][2], s[j][3], y);
-        pm_accumulate(k, false, x, y, w, acc);
-      }
-    } else if (tp.kind == 2) {
-      const double w0 = w4 * xi * xi * xi * e1 * e1, w1 = w0 * e2;
-      const double s[5][5] = {
-          {xi, xi * e1 * e3, xi * (1 - e1 * e2), xi * e1 * (1 - e2), w0},
-          {xi, xi * e1, xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), w1},
-          {xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * e2 * e3, w1},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), xi, xi * e1, w1},
-          {xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * e2, w1}};
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        pm_chi(EP, s[j][0], s[j][1], x);
-        pm_chi(EQ, s[j][2], s[j][3], y);
-        pm_accumulate(k, true, x, y, s[j][4], acc);
-      }
-    } else {
-      const double w = w4 * xi * xi * xi * e2;
-      pm_chi(EP, xi, xi * e1, x);
-      pm_chi(EQ, xi * e2, xi * e2 * e3, y);
-      pm_accumulate(k, true, x, y, w, acc);
-      pm_chi(EP, xi * e2, xi * e2 * e3, x);
-      pm_chi(EQ, xi, xi * e1, y);
-      pm_accumulate(k, true, x, y, w, acc);
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < 36; ++i) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-  }
+  for (int i = 0; i < 16; ++i) h[i] = 0.0;
+  if (tp.kind == 3) pm_moments<3>(table, k, nss, terms, EP, EQ, lane, e, h);
+  else if (tp.kind == 2) pm_moments<2>(table, k, nss, terms, EP, EQ, lane, e, h);
+  else pm_moments<1>(table, k, nss, terms, EP, EQ, lane, e, h);
+  ss_warp_sum<18>(e, lane);
+  if (mfio) ss_warp_sum<16>(h, lane);
   if (lane >= 9) return;
   const int i = lane / 3, j = lane % 3;
   const int t1 = tp.t1, t2 = tp.t2;
   const double jac = 4.0 * m.tri_area[t1] * m.tri_area[t2] * kInv4PiPm;
-#pragma unroll
-  for (int q = 0; q < 36; ++q) acc[q] *= jac;
   const int va = m.tris[3 * t1 + i], vb = m.tris[3 * t2 + j];
   double p[3], q[3];
-  const double D[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     p[c] = m.verts[3 * va + c] - P[0][c];
     q[c] = m.verts[3 * vb + c] - Q[0][c];
   }
-  double tr, ti, kr, ki;
-  pair_entry(k, acc, acc + 16, p, q, D, m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j],
-             m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j], tr, ti, kr, ki);
-  if (!mfio) kr = ki = 0.0;
+  const double cc = jac * m.tri_coef[3 * t1 + i] * m.tri_coef[3 * t2 + j];
+  const double dk = jac * m.tri_div[3 * t1 + i] * m.tri_div[3 * t2 + j] / k;
+  double ar, ai;
+  ss_efio_entry(e, EP, EQ, p, q, ar, ai);
+  // -ik cc (ar + i ai) + (i/k) dd I0
+  const double tr = k * cc * ai - dk * e[1];
+  const double ti = -k * cc * ar + dk * e[0];
+  double kr = 0.0, ki = 0.0;
+  if (mfio) {
+    // h: u1, u2, v1, v2 (MFIO moments of x, y), then u_s v_t; JYX = sum_st (EQ_t x EP_s) u_s v_t
+    double d[3], x[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+      d[c] = p[c] - q[c];
+      x[c] = p[c1] * q[c2] - p[c2] * q[c1];
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const double xe = ss_dot(x, EP[s]), xf = ss_dot(x, EQ[s]);
+      kr += xf * h[4 + 2 * s] - xe * h[2 * s];
+      ki += xf * h[5 + 2 * s] - xe * h[1 + 2 * s];
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        double dfe = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int c1 = (c + 1) % 3, c2 = (c + 2) % 3;
+          dfe += d[c] * (EQ[t][c1] * EP[s][c2] - EQ[t][c2] * EP[s][c1]);
+        }
+        kr += dfe * h[8 + 4 * s + 2 * t];
+        ki += dfe * h[9 + 4 * s + 2 * t];
+      }
+    }
+    kr *= -cc;
+    ki *= -cc;
+  }
   // (t1, t2) stands for (t2, t1) too: both meet on the diagonal, and an identical pair's block
   // holds both of an entry's halves already
   const int e1 = m.tri_edge[3 * t1 + i], e2 = m.tri_edge[3 * t2 + j];
@@ -480,7 +505,9 @@ cudaError_t assemble_pmchwt_one_k(const DevMesh& d, double k, int nss, int arith
   }
   if (d.ntouch == 0) return cudaSuccess;
   ProfScope prof("pmchwt_singular", s, double(d.ntouch));
-  pmchwt_singular_kernel<<<pm_blocks(d.ntouch, 4), 128, 0, s>>>(d, k, nss, ZT, ZK, ldz);
+  const double* table = ss_table_device();
+  if (!table) return cudaErrorInvalidSymbol;
+  pmchwt_singular_kernel<<<pm_blocks(d.ntouch, 4), 128, 0, s>>>(d, k, nss, table, ZT, ZK, ldz);
   return launched();
 }
 
@@ -491,6 +518,12 @@ void upload_rules_pmchwt(const Rules& r) {
   cudaMemcpyToSymbol(c_pm_w, r.w, sizeof(r.w));
   cudaMemcpyToSymbol(c_pm_glx, r.glx, sizeof(r.glx));
   cudaMemcpyToSymbol(c_pm_glw, r.glw, sizeof(r.glw));
+  double e[kSsTerms][6], h[kSsTerms][4], c[kSsTerms][10];
+  make_ss_series(r, e);
+  make_ss_series_mfio(r, h);
+  for (int j = 0; j < kSsTerms; ++j)
+    for (int i = 0; i < 10; ++i) c[j][i] = i < 6 ? e[j][i] : h[j][i - 6];
+  cudaMemcpyToSymbol(c_pm_series, c, sizeof(c));
 }
 
 }  // namespace fosb

@@ -78,6 +78,29 @@ inline void make_ss_series(const Rules& r, double (&c)[kSsTerms][6]) {
   }
 }
 
+// The same for Q_m(phi) = sum_a w_a xi_a^m (i phi xi_a - 1) exp(i phi xi_a), m = 1, 2, the xi sums of
+// exp(ikr)(ikr - 1)/r^3: Re Q_m = sum_j (-1)^j (2j-1)/(2j)! M_{m+2j} phi^{2j} (c[j][m-1]) and
+// Im Q_m = phi sum_j (-1)^j 2j/(2j+1)! M_{m+2j+1} phi^{2j} (c[j][1+m]).
+inline void make_ss_series_mfio(const Rules& r, double (&c)[kSsTerms][4]) {
+  auto moment = [&](int n) {
+    long double s = 0;
+    for (int a = 0; a < r.nss; ++a) s += (long double)r.glw[a] * std::pow((long double)r.glx[a], n);
+    return s;
+  };
+  long double fact = 1;  // (2j)!
+  for (int j = 0; j < kSsTerms; ++j) {
+    if (j > 0) fact *= (long double)(2 * j - 1) * (2 * j);
+    const long double sg = j & 1 ? -1 : 1;
+    for (int m = 1; m <= 2; ++m) {
+      c[j][m - 1] = double(sg * (2 * j - 1) * moment(m + 2 * j) / fact);
+      c[j][1 + m] = double(sg * 2 * j * moment(m + 1 + 2 * j) / (fact * (2 * j + 1)));
+    }
+  }
+}
+
+// The table on the current device (assemble.cu), nullptr if it cannot be had.
+const double* ss_table_device();
+
 // 1/sqrt(x) for a normal x > 0: the hardware's FP64 seed (about 20 bits) and one third-order step,
 // y <- y + y e (1/2 + 3/8 e) with e = 1 - x y^2, which leaves an error of order e^3.
 __device__ __forceinline__ double ss_rsqrt(double x) {
@@ -107,6 +130,83 @@ __device__ __forceinline__ float ss_phase_bound(double k, const double (&EP)[2][
       m2 = fmaxf(m2, x * x + y * y + z * z);
     }
   return float(k) * sqrtf(m2) * 1.0001f;
+}
+
+// The series up to here (its rounding is then below 6e-16 of |S_m|, 8e-16 at phase 4; 15 terms);
+// larger phases, which only meshes with edges beyond about half a wavelength reach, take sincos per point.
+constexpr double kSsMaxPhase = 3.0;
+
+// Number of phi^2 powers for phases up to ph: the first J with ph^{2J}/(2J)! < 2^-56 (the
+// moments' decay only helps), at most kSsTerms; 0 above kSsMaxPhase.
+__device__ __forceinline__ int ss_terms(float ph) {
+  if (!(ph <= float(kSsMaxPhase))) return 0;
+  const float p2 = ph * ph;
+  float t = 1.f;
+  int J = 0;
+  while (J < kSsTerms && t > 1.3e-17f) {
+    t *= p2 / float((2 * J + 1) * (2 * J + 2));
+    ++J;
+  }
+  return J;
+}
+
+// First region and number of regions of a kind of touching pair (3 identical, 2 edge, 1 vertex).
+template <int KIND>
+__device__ __forceinline__ constexpr int ss_first_region() {
+  return KIND == 3 ? 0 : (KIND == 2 ? 6 : 11);
+}
+template <int KIND>
+__device__ __forceinline__ constexpr int ss_regions() {
+  return KIND == 3 ? 6 : (KIND == 2 ? 5 : 2);
+}
+
+// Distance and phase of one point of the table (field f at tab[f * stride]): 1/rh and k rh.
+template <int KIND>
+__device__ __forceinline__ void ss_distance(const double* tab, int stride, const double (&uv)[4],
+                                            const double (&EP)[2][3], const double (&EQ)[2][3], double k,
+                                            double& rinv, double& phi) {
+  double d[3];
+  if constexpr (KIND == 3) {  // EQ = EP: the coordinate differences are in the table
+    const double a = __ldg(tab + 9 * stride), b = __ldg(tab + 10 * stride);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], b * EP[1][c]);
+  } else if constexpr (KIND == 2) {  // EQ[0] = EP[0], the shared edge
+    const double a = __ldg(tab + 9 * stride);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) d[c] = fma(a, EP[0][c], fma(uv[1], EP[1][c], -uv[3] * EQ[1][c]));
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      d[c] = fma(uv[0], EP[0][c], fma(uv[1], EP[1][c], fma(-uv[2], EQ[0][c], -uv[3] * EQ[1][c])));
+  }
+  const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+  rinv = ss_rsqrt(r2);
+  phi = k * (r2 * rinv);
+}
+
+__device__ __forceinline__ double ss_dot(const double (&x)[3], const double (&y)[3]) {
+  return fma(x[0], y[0], fma(x[1], y[1], x[2] * y[2]));
+}
+
+// XY - q.X - p.Y + (p.q) I0 from the reference moments (I0, u1, u2, v1, v2, u1v1, u1v2, u2v1, u2v2;
+// complex): X = EP.u, Y = EQ.v, XY = u EP.EQ v.
+__device__ __forceinline__ void ss_efio_entry(const double* mom, const double (&EP)[2][3], const double (&EQ)[2][3],
+                                              const double (&p)[3], const double (&q)[3], double& ar, double& ai) {
+  const double pq = ss_dot(p, q);
+  ar = pq * mom[0];
+  ai = pq * mom[1];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const double qe = ss_dot(q, EP[s]), pf = ss_dot(p, EQ[s]);
+    ar -= fma(qe, mom[2 + 2 * s], pf * mom[6 + 2 * s]);
+    ai -= fma(qe, mom[3 + 2 * s], pf * mom[7 + 2 * s]);
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const double ef = ss_dot(EP[s], EQ[t]);
+      ar = fma(ef, mom[10 + 4 * s + 2 * t], ar);
+      ai = fma(ef, mom[11 + 4 * s + 2 * t], ai);
+    }
+  }
 }
 
 // acc[i] summed over the warp's lanes, left in every lane.  Halving: each step a lane keeps one

@@ -27,3 +27,23 @@ def test_touching_pairs_match_oracle_at_every_phase(k, n_ss):
     F.assemble_efie(m, k, Z, n_ss=n_ss)
     Zo = O.assemble_z(om, k, n_ss)
     assert np.abs(Z.cpu().numpy() - Zo).max() <= 1e-12 * np.abs(Zo).max()
+
+
+@pytest.mark.parametrize("k0,n_ss", [(0.05, 5), (1.0, 12), (2.0, 1), (2.4, 5), (8.0, 3)])
+def test_pmchwt_touching_pairs_match_oracle_at_every_phase(k0, n_ss):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2308_01457_gb300 as F
+
+    F.build.build()
+    sm = S.ellipsoid(0, (1.0, 0.7, 1.2))
+    m, om = F.mesh_create(sm.verts, sm.tris, sm.vnormals), O.from_synth(sm)
+    N = m.n_edges
+    Z = torch.empty((2 * N, 2 * N), dtype=torch.complex128, device="cuda:0")
+    F.assemble_pmchwt(m, k0, 1.7, 1.0, Z, n_ss=n_ss)
+    Zo = O.assemble_pmchwt(om, k0, 1.7, 1.0, n_ss)
+    for r in range(2):
+        for c in range(2):
+            zo = Zo[r * N:(r + 1) * N, c * N:(c + 1) * N]
+            zg = Z[r * N:(r + 1) * N, c * N:(c + 1) * N].cpu().numpy()
+            assert np.abs(zg - zo).max() <= 1e-12 * np.abs(zo).max()
