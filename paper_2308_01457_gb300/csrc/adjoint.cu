@@ -20,6 +20,9 @@
 #include <cuda_runtime.h>
 
 #include "fosb_internal.h"
+#include "fp64_phase.cuh"
+#include "pair_tiles.cuh"
+#include "sauter_schwab.cuh"
 
 namespace fosb {
 
@@ -28,8 +31,16 @@ __constant__ double c_bary[6][3];
 __constant__ double c_w[6];
 __constant__ double c_glx[16];
 __constant__ double c_glw[16];
+__constant__ double c_wbary[6][3];         // w_q bary_qb
+__constant__ double c_phase[kPhaseTab][2];  // make_phase_table
 
 void upload_rules_adjoint(const Rules& r) {
+  double wb[6][3], ph[kPhaseTab][2];
+  for (int q = 0; q < 6; ++q)
+    for (int b = 0; b < 3; ++b) wb[q][b] = r.w[q] * r.bary[q][b];
+  cudaMemcpyToSymbol(c_wbary, wb, sizeof(wb));
+  make_phase_table(ph);
+  cudaMemcpyToSymbol(c_phase, ph, sizeof(ph));
   cudaMemcpyToSymbol(c_bary, r.bary, sizeof(r.bary));
   cudaMemcpyToSymbol(c_w, r.w, sizeof(r.w));
   cudaMemcpyToSymbol(c_glx, r.glx, sizeof(r.glx));
@@ -199,64 +210,280 @@ __device__ __forceinline__ void add_grad(double* grad, int v, const double g[3],
 }
 
 // ------------------------------------------------------------------ regular pairs
-__global__ void __launch_bounds__(128) adjoint_regular_kernel(DevMesh m, double k, const double* lam, const double* U,
-                                                              int64_t ld, int64_t nrhs, double* grad) {
-  const int64_t t1 = int64_t(blockIdx.y) * 4 + (threadIdx.x >> 5);
-  const int64_t t2 = int64_t(blockIdx.x) * 32 + (threadIdx.x & 31);
-  if (t1 >= m.nt || t2 >= m.nt) return;
-  int v1[3], v2[3], e1[3], e2[3];
-  double sl1[3], sl2[3], l1[3], l2[3], V1[3][3], V2[3][3];
-  tri_edge_data(m, t1, v1, e1, sl1, l1, V1);
-  tri_edge_data(m, t2, v2, e2, sl2, l2, V2);
-  bool touch = false;
+// Unordered pairs t1 < t2 with the symmetrised W_jk (lambda u + u lambda).  H is bilinear in the
+// barycentric coordinates, H = sum_ab lambda_a beta_b H_ab with H_ab = H(P_a, Q_b), and everything
+// linear in G follows from the moments mu_ab = sum_pq w lambda_pa beta_qb G: only the real vector
+// F d = w Re(G'/r H) d is summed per point.  Bound by the FP64 pipe: about 53 instructions per
+// point pair and 1200 per triangle pair (576 of them the W_jk of 8 columns), against 143 and
+// 1000 per ordered pair with every term summed per point.  T = 5120, 8 columns: 92.7 ms, 310.7 ms before.
+
+// imaginary part of a b
+__device__ __forceinline__ double cx_mul_im(Cx a, Cx b) { return fma(a.r, b.i, a.i * b.r); }
+__device__ __forceinline__ Cx cx_axpy(double s, Cx a, Cx b) { return {fma(s, a.r, b.r), fma(s, a.i, b.i)}; }
+
+// One side's G-linear and explicit gradient terms, accumulated into g (vertex gradients of this
+// side).  X: this side's vertices relative to vertex 0, r_j / wq_j: sum_k W_jk and sum_k W_jk Q_k
+// over the other side, mo_a = sum_b mu_ab, moq_a = sum_b mu_ab Q_b, U = sum W Q_k, MX / MO: sum of
+// mu X_a / mu Q_b, MXO the sum of mu X_a.Q_b.
+//   points:   dJ/dx = mik4 G (S y - U)          -> (k/4) Im(S moq_a - U mo_a)
+//   vertices: dJ/dX_j = (ik/4)(r_j MO - wq_j I0) -> -(k/4) Im(...)
+//   lengths:  l_j dJ/dl_j = sum_k W_jk K_jk, K_jk = -(ik/4)(MXO - Q_k.MX - X_j.MO + X_j.Q_k I0) + (i/k) I0.
+__device__ __forceinline__ void adjoint_side(double k4, double kinv, Cx S, Cx I0, Cx MXO, const Cx (&MX)[3],
+                                             const Cx (&MO)[3], const Cx (&U)[3], const Cx (&r)[3],
+                                             const Cx (&wq)[3][3], const Cx (&mo)[3], const Cx (&moq)[3][3],
+                                             const double (&X)[3][3], double (&g)[3][3]) {
+#pragma unroll
   for (int a = 0; a < 3; ++a)
-    for (int b = 0; b < 3; ++b) touch |= v1[a] == v2[b];
-  if (touch) return;
-  double P[3][3], Q[3][3], D[3];
-  for (int a = 0; a < 3; ++a)
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      P[a][d] = V1[a][d] - V1[0][d];
-      Q[a][d] = V2[a][d] - V2[0][d];
+      double im = cx_mul_im(S, moq[a][d]) - cx_mul_im(U[d], mo[a]);
+      im -= cx_mul_im(r[a], MO[d]) - cx_mul_im(wq[a][d], I0);
+      g[a][d] = fma(k4, im, g[a][d]);
     }
-  for (int d = 0; d < 3; ++d) D[d] = V1[0][d] - V2[0][d];
-  PairCoef pc;
-  load_w(lam, U, ld, nrhs, e1, e2, sl1, sl2, false, pc);
-  make_coef(P, Q, pc);
-  PairAcc A;
-  A.I0 = A.Mxy = Cx{0, 0};
-  for (int d = 0; d < 3; ++d) A.Mx[d] = A.My[d] = Cx{0, 0};
-  double xq[6][3], yq[6][3];
-  for (int q = 0; q < 6; ++q)
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    Cx t = MXO, xq = {0.0, 0.0};
+    double im = 0.0;
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      xq[q][d] = m.tri_qp[18 * t1 + 3 * q + d] - V1[0][d];
-      yq[q][d] = m.tri_qp[18 * t2 + 3 * q + d] - V2[0][d];
-      A.gx[q][d] = A.gy[q][d] = 0.0;
-    }
-  for (int p = 0; p < 6; ++p)
-    for (int q = 0; q < 6; ++q) {
-      double dv[3] = {D[0] + xq[p][0] - yq[q][0], D[1] + xq[p][1] - yq[q][1], D[2] + xq[p][2] - yq[q][2]};
-      point_pair(k, pc, xq[p], yq[q], dv, c_w[p] * c_w[q] * kInv4Pi, A.gx[p], A.gy[q], A);
-    }
-  double gP[3][3], gQ[3][3], gl1[3], gl2[3];
-  explicit_terms(k, pc, A, P, Q, l1, l2, gP, gQ, gl1, gl2);
-  double g1[3][3], g2[3][3];
-  for (int a = 0; a < 3; ++a)
-    for (int d = 0; d < 3; ++d) {
-      double s1 = gP[a][d], s2 = gQ[a][d];
-      for (int q = 0; q < 6; ++q) {
-        s1 += c_bary[q][a] * A.gx[q][d];
-        s2 += c_bary[q][a] * A.gy[q][d];
+      if (j > 0) {
+        t = cx_axpy(-X[j][d], MO[d], t);
+        xq = cx_axpy(X[j][d], wq[j][d], xq);
       }
-      g1[a][d] = s1;
-      g2[a][d] = s2;
+      im -= cx_mul_im(wq[j][d], MX[d]);
     }
-  chain_lengths(V1, l1, gl1, g1);
-  chain_lengths(V2, l2, gl2, g2);
-  // J_Z enters the objective with a minus sign
-  for (int a = 0; a < 3; ++a) {
-    add_grad(grad, v1[a], g1[a], -1.0);
-    add_grad(grad, v2[a], g2[a], -1.0);
+    im += cx_mul_im(r[j], t);
+    if (j > 0) im += cx_mul_im(xq, I0);
+    const double lk = fma(k4, im, -kinv * cx_mul_im(r[j], I0));  // l_j dJ/dl_j
+    const int a = (j + 1) % 3, b = (j + 2) % 3;
+    double e[3], l2 = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      e[d] = X[b][d] - X[a][d];
+      l2 = fma(e[d], e[d], l2);
+    }
+    const double rl = ss_rsqrt(l2), f = lk * (rl * rl);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      g[b][d] = fma(f, e[d], g[b][d]);
+      g[a][d] = fma(-f, e[d], g[a][d]);
+    }
   }
+}
+
+__global__ void __launch_bounds__(128) adjoint_regular_kernel(DevMesh m, double k, const double* __restrict__ lam,
+                                                              const double* __restrict__ U, int64_t ld, int64_t nrhs,
+                                                              double* grad) {
+  __shared__ double2 tab[kPhaseTab];
+  int64_t rg, cb;
+  if (!pair_tile(m.nt, 4, blockIdx.y, blockIdx.x, rg, cb)) return;
+  tab[threadIdx.x] = make_double2(c_phase[threadIdx.x][0], c_phase[threadIdx.x][1]);
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t t1 = rg * 4 + (threadIdx.x >> 5);
+  int64_t t2 = cb * 32 + lane;
+  if (t1 >= m.nt) return;  // the whole warp
+  bool live = t2 < m.nt && t1 < t2;
+  int v1[3], v2[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) v1[a] = m.tris[3 * t1 + a];
+  if (live) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      v2[a] = m.tris[3 * t2 + a];
+      live = live && v2[a] != v1[0] && v2[a] != v1[1] && v2[a] != v1[2];
+    }
+  }
+  if (!__any_sync(0xffffffffu, live)) return;
+  double g1[3][3] = {};
+  if (live) {
+    double P[3][3], Q[3][3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        P[a][d] = m.verts[3 * v1[a] + d] - m.verts[3 * v1[0] + d];
+        Q[a][d] = m.verts[3 * v2[a] + d] - m.verts[3 * v2[0] + d];
+      }
+    // W_jk = s_j l_j s'_k l'_k/(4 pi) sum_i (lambda_j u_k + u_j lambda_k)
+    Cx W[3][3] = {};
+    {
+      int64_t o1[3], o2[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        o1[j] = m.tri_edge[3 * t1 + j] * ld;
+        o2[j] = m.tri_edge[3 * t2 + j] * ld;
+      }
+      const Cx* L = reinterpret_cast<const Cx*>(lam);
+      const Cx* Uc = reinterpret_cast<const Cx*>(U);
+#pragma unroll 1
+      for (int64_t i = 0; i < nrhs; ++i) {
+        Cx a[3], b[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          a[j] = L[o1[j] + i];
+          b[j] = Uc[o1[j] + i];
+        }
+#pragma unroll
+        for (int kk = 0; kk < 3; ++kk) {
+          const Cx c = Uc[o2[kk] + i], d = L[o2[kk] + i];
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            Cx& w = W[j][kk];
+            w.r = fma(a[j].r, c.r, fma(-a[j].i, c.i, fma(b[j].r, d.r, fma(-b[j].i, d.i, w.r))));
+            w.i = fma(a[j].r, c.i, fma(a[j].i, c.r, fma(b[j].r, d.i, fma(b[j].i, d.r, w.i))));
+          }
+        }
+      }
+      const double A1 = 2.0 * m.tri_area[t1] * kInv4Pi, A2 = 2.0 * m.tri_area[t2];
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int kk = 0; kk < 3; ++kk) W[j][kk] = W[j][kk] * ((A1 * m.tri_coef[3 * t1 + j]) * (A2 * m.tri_coef[3 * t2 + kk]));
+    }
+    // sums over one side and the vertex values H_ab
+    Cx rj[3], ck[3], S = {0.0, 0.0}, c = {0.0, 0.0}, Us[3] = {}, Vs[3] = {};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      rj[j] = W[j][0] + W[j][1] + W[j][2];
+      ck[j] = W[0][j] + W[1][j] + W[2][j];
+      S = S + rj[j];
+    }
+#pragma unroll
+    for (int j = 1; j < 3; ++j)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        Us[d] = cx_axpy(Q[j][d], ck[j], Us[d]);
+        Vs[d] = cx_axpy(P[j][d], rj[j], Vs[d]);
+      }
+    double pq[3][3] = {};
+#pragma unroll
+    for (int a = 1; a < 3; ++a)
+#pragma unroll
+      for (int b = 1; b < 3; ++b) {
+        pq[a][b] = ss_dot(P[a], Q[b]);
+        c = cx_axpy(pq[a][b], W[a][b], c);
+      }
+    const double k4 = 0.25 * k, kinv = 1.0 / k;
+    Cx H[3][3];
+    {
+      Cx pu[3] = {}, vq[3] = {};
+#pragma unroll
+      for (int a = 1; a < 3; ++a)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          pu[a] = cx_axpy(P[a][d], Us[d], pu[a]);
+          vq[a] = cx_axpy(Q[a][d], Vs[d], vq[a]);
+        }
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          const Cx B = cx_axpy(pq[a][b], S, c - pu[a] - vq[b]);
+          H[a][b] = {fma(k4, B.i, -kinv * S.i), fma(-k4, B.r, kinv * S.r)};  // -(ik/4) B + (i/k) S
+        }
+    }
+    // the point loop: mu and the real F d sums
+    const double* xq = m.tri_qp + 18 * t1;
+    const double* yq = m.tri_qp + 18 * t2;
+    double gy[6][3] = {};
+    Cx mu[3][3] = {};
+#pragma unroll 1
+    for (int p = 0; p < 6; ++p) {
+      const double x0 = xq[3 * p], x1 = xq[3 * p + 1], x2 = xq[3 * p + 2];
+      Cx T[3] = {}, A[3] = {};
+      double gx[3] = {};
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int a = 0; a < 3; ++a) T[b] = cx_axpy(c_wbary[p][a], H[a][b], T[b]);
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        const double d[3] = {x0 - yq[3 * q], x1 - yq[3 * q + 1], x2 - yq[3 * q + 2]};
+        const double r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
+        const double rinv = ss_rsqrt(r2), kr = k * (r2 * rinv);
+        double cs, sn;
+        expi_table(kr, tab, cs, sn);
+        const Cx G = {cs * rinv, sn * rinv};
+        Cx h = {0.0, 0.0};  // w_p w_q H
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+          A[b] = cx_axpy(c_wbary[q][b], G, A[b]);
+          h = cx_axpy(c_wbary[q][b], T[b], h);
+        }
+        // F = Re(G (ikr - 1) H)/r^2
+        const double hr = fma(kr, h.i, h.r), hi = fma(-kr, h.r, h.i);  // -(ikr - 1) H
+        const double F = (rinv * rinv) * fma(G.i, hi, -G.r * hr);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          gx[e] = fma(F, d[e], gx[e]);
+          gy[q][e] = fma(-F, d[e], gy[q][e]);
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) mu[a][b] = cx_axpy(c_wbary[p][a], A[b], mu[a][b]);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) g1[a][e] = fma(c_bary[p][a], gx[e], g1[a][e]);
+      }
+    }
+    double g2[3][3] = {};
+#pragma unroll
+    for (int q = 0; q < 6; ++q)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) g2[b][e] = fma(c_bary[q][b], gy[q][e], g2[b][e]);
+    // moments of G
+    Cx m1[3], m2[3], I0 = {0.0, 0.0}, MP[3] = {}, MQ[3] = {}, MPQ = {0.0, 0.0}, mq[3][3] = {}, mp[3][3] = {};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      m1[a] = mu[a][0] + mu[a][1] + mu[a][2];
+      m2[a] = mu[0][a] + mu[1][a] + mu[2][a];
+      I0 = I0 + m1[a];
+#pragma unroll
+      for (int b = 1; b < 3; ++b)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          mq[a][d] = cx_axpy(Q[b][d], mu[a][b], mq[a][d]);
+          mp[a][d] = cx_axpy(P[b][d], mu[b][a], mp[a][d]);
+        }
+    }
+#pragma unroll
+    for (int a = 1; a < 3; ++a)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        MP[d] = cx_axpy(P[a][d], m1[a], MP[d]);
+        MQ[d] = cx_axpy(Q[a][d], m2[a], MQ[d]);
+        MPQ = cx_axpy(P[a][d], mq[a][d], MPQ);
+      }
+    Cx wq[3][3] = {}, wp[3][3] = {};
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int b = 1; b < 3; ++b)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          wq[j][d] = cx_axpy(Q[b][d], W[j][b], wq[j][d]);
+          wp[j][d] = cx_axpy(P[b][d], W[b][j], wp[j][d]);
+        }
+    adjoint_side(k4, kinv, S, I0, MPQ, MP, MQ, Us, rj, wq, m1, mq, P, g1);
+    adjoint_side(k4, kinv, S, I0, MPQ, MQ, MP, Vs, ck, wp, m2, mp, Q, g2);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) add_grad(grad, v2[a], g2[a], -1.0);  // J_Z enters the objective with a minus sign
+  }
+  // t1 is the warp's: one addition per vertex coordinate
+  double s[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) s[i] = g1[i / 3][i % 3];
+  ss_warp_sum<9>(s, lane);
+  if (lane == 0)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const double g[3] = {s[3 * a], s[3 * a + 1], s[3 * a + 2]};
+      add_grad(grad, v1[a], g, -1.0);
+    }
 }
 
 // ------------------------------------------------------------------ touching pairs
@@ -445,8 +672,8 @@ inline unsigned cdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); }
 
 cudaError_t launch_adjoint_pairs(const DevMesh& m, double k, int nss, const double* lam, const double* U, int64_t ld,
                                  int64_t nrhs, double* grad, cudaStream_t s) {
-  dim3 grid(cdiv(m.nt, 32), cdiv(m.nt, 4));
-  if (grid.y > 65535u) return cudaErrorInvalidValue;
+  if (cdiv(m.nt, 4) > 65535u) return cudaErrorInvalidValue;
+  const dim3 grid(unsigned(pair_tiles_width(m.nt)), unsigned(pair_tiles_rows(m.nt, 4)));
   adjoint_regular_kernel<<<grid, 128, 0, s>>>(m, k, lam, U, ld, nrhs, grad);
   note_launches(1);
   if (m.ntouch > 0) {

@@ -222,6 +222,7 @@ __device__ __forceinline__ void ss_warp_sum(double (&acc)[NV], int lane) {
     const bool up = lane & h;
 #pragma unroll
     for (int i = 0; i < h; ++i) {
+      if (i >= NV) continue;  // zero in every lane
       const double keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
       v[i] = keep + __shfl_xor_sync(0xffffffffu, give, h);
     }
