@@ -33,6 +33,7 @@ __constant__ double c_glx[16];
 __constant__ double c_glw[16];
 __constant__ double c_wbary[6][3];         // w_q bary_qb
 __constant__ double c_phase[kPhaseTab][2];  // make_phase_table
+__constant__ double c_adj_series[kSsTerms][14];  // make_ss_series, then make_ss_series_mfio
 
 void upload_rules_adjoint(const Rules& r) {
   double wb[6][3], ph[kPhaseTab][2];
@@ -41,6 +42,12 @@ void upload_rules_adjoint(const Rules& r) {
   cudaMemcpyToSymbol(c_wbary, wb, sizeof(wb));
   make_phase_table(ph);
   cudaMemcpyToSymbol(c_phase, ph, sizeof(ph));
+  double se[kSsTerms][6], sh[kSsTerms][8], sc[kSsTerms][14];
+  make_ss_series(r, se);
+  make_ss_series_mfio<4>(r, sh);
+  for (int j = 0; j < kSsTerms; ++j)
+    for (int i = 0; i < 14; ++i) sc[j][i] = i < 6 ? se[j][i] : sh[j][i - 6];
+  cudaMemcpyToSymbol(c_adj_series, sc, sizeof(sc));
   cudaMemcpyToSymbol(c_bary, r.bary, sizeof(r.bary));
   cudaMemcpyToSymbol(c_w, r.w, sizeof(r.w));
   cudaMemcpyToSymbol(c_glx, r.glx, sizeof(r.glx));
@@ -58,123 +65,6 @@ __device__ __forceinline__ Cx operator+(Cx a, Cx b) { return {a.r + b.r, a.i + b
 __device__ __forceinline__ Cx operator-(Cx a, Cx b) { return {a.r - b.r, a.i - b.i}; }
 __device__ __forceinline__ Cx operator*(Cx a, Cx b) { return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r}; }
 __device__ __forceinline__ Cx operator*(Cx a, double s) { return {a.r * s, a.i * s}; }
-
-// Per-pair state: the coefficient matrix W (already scaled by s s' l l'), origins and the
-// local (origin-relative) opposite vertices of both triangles.
-struct PairCoef {
-  Cx W[3][3];
-  Cx S, U[3], V[3], c;
-};
-
-__device__ void make_coef(const double P[3][3], const double Q[3][3], PairCoef& pc) {
-  pc.S = {0, 0};
-  pc.c = {0, 0};
-  for (int d = 0; d < 3; ++d) pc.U[d] = pc.V[d] = Cx{0, 0};
-  for (int j = 0; j < 3; ++j)
-    for (int k = 0; k < 3; ++k) {
-      Cx w = pc.W[j][k];
-      pc.S = pc.S + w;
-      double pq = P[j][0] * Q[k][0] + P[j][1] * Q[k][1] + P[j][2] * Q[k][2];
-      pc.c = pc.c + w * pq;
-      for (int d = 0; d < 3; ++d) {
-        pc.U[d] = pc.U[d] + w * Q[k][d];
-        pc.V[d] = pc.V[d] + w * P[j][d];
-      }
-    }
-}
-
-// Accumulators of one pair: real gradients at the points and complex moments.
-struct PairAcc {
-  double gx[6][3], gy[6][3];   // regular: per test / trial point
-  Cx I0, Mx[3], My[3], Mxy;
-};
-
-// One point pair: x, y local coordinates (x - o1, y - o2), dvec = x - y (absolute),
-// weight w (includes the 1/(4 pi) of G).  Returns the real gradient contributions with
-// respect to x and y and adds the moments.
-__device__ __forceinline__ void point_pair(double k, const PairCoef& pc, const double x[3], const double y[3],
-                                           const double dvec[3], double w, double gx[3], double gy[3],
-                                           PairAcc& A) {
-  double r2 = dvec[0] * dvec[0] + dvec[1] * dvec[1] + dvec[2] * dvec[2];
-  double rinv = rsqrt(r2);
-  double r = r2 * rinv;
-  double sn, cs;
-  sincos(k * r, &sn, &cs);
-  Cx G = {cs * rinv * w, sn * rinv * w};
-  Cx Gp_over_r = G * Cx{-rinv * rinv, k * rinv};  // G'(r)/r = G (ik - 1/r)/r
-  double xy = x[0] * y[0] + x[1] * y[1] + x[2] * y[2];
-  Cx xU = pc.U[0] * x[0] + pc.U[1] * x[1] + pc.U[2] * x[2];
-  Cx Vy = pc.V[0] * y[0] + pc.V[1] * y[1] + pc.V[2] * y[2];
-  Cx B = pc.S * xy - xU - Vy + pc.c;
-  const Cx mik4 = {0.0, -0.25 * k};
-  Cx H = mik4 * B + Cx{0.0, 1.0 / k} * pc.S;
-  Cx GH = Gp_over_r * H;
-  Cx Gm = G * mik4;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    Cx dHx = pc.S * y[d] - pc.U[d];  // (S y - U)
-    Cx dHy = pc.S * x[d] - pc.V[d];  // (S x - V)
-    gx[d] += GH.r * dvec[d] + (Gm * dHx).r;
-    gy[d] += -GH.r * dvec[d] + (Gm * dHy).r;
-  }
-  A.I0 = A.I0 + G;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    A.Mx[d] = A.Mx[d] + G * x[d];
-    A.My[d] = A.My[d] + G * y[d];
-  }
-  A.Mxy = A.Mxy + G * xy;
-}
-
-// Explicit (non point) terms of one pair: opposite vertices and edge lengths.
-//   dJ/dP_j = (ik/4) sum_k W_jk (My - Q_k I0),  dJ/dQ_k = (ik/4) sum_j W_jk (Mx - P_j I0),
-//   dJ/dl_j = sum_k W_jk K_jk / l_j,  K_jk = -(ik/4)(Mxy - Q_k.Mx - P_j.My + P_j.Q_k I0) + (i/k) I0.
-__device__ void explicit_terms(double k, const PairCoef& pc, const PairAcc& A, const double P[3][3],
-                               const double Q[3][3], const double l1[3], const double l2[3], double gP[3][3],
-                               double gQ[3][3], double gl1[3], double gl2[3]) {
-  const Cx ik4 = {0.0, 0.25 * k};
-  for (int j = 0; j < 3; ++j) {
-    gl1[j] = gl2[j] = 0.0;
-    for (int d = 0; d < 3; ++d) gP[j][d] = gQ[j][d] = 0.0;
-  }
-  for (int j = 0; j < 3; ++j)
-    for (int kk = 0; kk < 3; ++kk) {
-      Cx w = pc.W[j][kk];
-      Cx wik = w * ik4;
-      for (int d = 0; d < 3; ++d) {
-        gP[j][d] += (wik * (A.My[d] - A.I0 * Q[kk][d])).r;
-        gQ[kk][d] += (wik * (A.Mx[d] - A.I0 * P[j][d])).r;
-      }
-      Cx QMx = A.Mx[0] * Q[kk][0] + A.Mx[1] * Q[kk][1] + A.Mx[2] * Q[kk][2];
-      Cx PMy = A.My[0] * P[j][0] + A.My[1] * P[j][1] + A.My[2] * P[j][2];
-      double pq = P[j][0] * Q[kk][0] + P[j][1] * Q[kk][1] + P[j][2] * Q[kk][2];
-      Cx K = Cx{0.0, -0.25 * k} * (A.Mxy - QMx - PMy + A.I0 * pq) + Cx{0.0, 1.0 / k} * A.I0;
-      double v = (w * K).r;
-      gl1[j] += v / l1[j];
-      gl2[kk] += v / l2[kk];
-    }
-}
-
-// W_jk = s_j s'_k l_j l'_k sum_i lambda[e1_j, i] u[e2_k, i] (+ the mirrored term for
-// touching pairs whose transpose block is not evaluated separately).
-__device__ void load_w(const double* lam, const double* U, int64_t ld, int64_t m, const int e1[3], const int e2[3],
-                       const double sl1[3], const double sl2[3], bool mirror, PairCoef& pc) {
-  for (int j = 0; j < 3; ++j)
-    for (int kk = 0; kk < 3; ++kk) {
-      Cx acc = {0, 0};
-      for (int64_t i = 0; i < m; ++i) {
-        Cx a = {lam[2 * (e1[j] * ld + i)], lam[2 * (e1[j] * ld + i) + 1]};
-        Cx b = {U[2 * (e2[kk] * ld + i)], U[2 * (e2[kk] * ld + i) + 1]};
-        acc = acc + a * b;
-        if (mirror) {
-          Cx a2 = {lam[2 * (e2[kk] * ld + i)], lam[2 * (e2[kk] * ld + i) + 1]};
-          Cx b2 = {U[2 * (e1[j] * ld + i)], U[2 * (e1[j] * ld + i) + 1]};
-          acc = acc + a2 * b2;
-        }
-      }
-      pc.W[j][kk] = acc * (sl1[j] * sl2[kk]);
-    }
-}
 
 __device__ __forceinline__ void tri_edge_data(const DevMesh& m, int64_t t, int v[3], int e[3], double sl[3],
                                               double l[3], double V[3][3]) {
@@ -487,139 +377,277 @@ __global__ void __launch_bounds__(128) adjoint_regular_kernel(DevMesh m, double 
 }
 
 // ------------------------------------------------------------------ touching pairs
-// One CTA (128 threads) per touching pair (t1 <= t2), Sauter-Schwab points in the
-// orientation of the assembly; gradients at the points are chained immediately to the
-// permuted vertices through the barycentric weights of chi.
-__device__ __forceinline__ void chi_bary(double u1, double u2, double a[3]) {
-  a[0] = 1.0 - u1;
-  a[1] = u1 - u2;
-  a[2] = u2;
+// One touching pair (t1 <= t2) per warp, Sauter-Schwab in the form (x, y) = xi (xh, yh) with the
+// xi sums as power series in phi = k |xh - yh| (see efie_singular_kernel).  With the moments of G
+// in the reference coordinates and H along xi a quadratic h0 + xi h1 + xi^2 h2, the sums of F d
+// and of xi F d (chained to the vertices through u and v) are
+//   F_0 = Re(Q_1 h0 + Q_2 h1 + Q_3 h2)/rh^3, F_1 = Re(Q_2 h0 + Q_3 h1 + Q_4 h2)/rh^3,
+//   Q_m = sum_a w_a xi_a^m (i phi xi_a - 1) exp(i phi xi_a).
+// Bound by the FP64 pipe: about 185 instructions per 5 points against 145 per point.  T = 5120,
+// n_ss = 5, 8 columns: 7.8 ms, 39.3 ms before.
+template <int KIND>
+__device__ __forceinline__ void adjoint_ss_moments(const double* __restrict__ table, double k, int nss, int J,
+                                                   const double (&EP)[2][3], const double (&EQ)[2][3], Cx h0,
+                                                   const Cx (&hu)[4], const Cx (&huv)[4], int lane, double (&e)[18],
+                                                   double (&f)[15]) {
+  const int n3 = nss * nss * nss, stride = kSsRegions * n3, count = ss_regions<KIND>() * n3;
+  const double* tab = table + ss_first_region<KIND>() * n3;
+  for (int idx = lane; idx < count; idx += 32) {
+    auto T = [&](int q) { return __ldg(tab + q * stride + idx); };
+    const double uv[4] = {T(0), T(1), T(2), T(3)};
+    double d[3], rinv, phi;
+    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, d, rinv, phi);
+    // Re S_0..2, Im S_0..2, Re Q_1..4, Im Q_1..4
+    double s[14];
+    if (J > 0) {
+      const double p2 = phi * phi;
+#pragma unroll
+      for (int i = 0; i < 14; ++i) s[i] = c_adj_series[J - 1][i];
+      for (int j = J - 2; j >= 0; --j)
+#pragma unroll
+        for (int i = 0; i < 14; ++i) s[i] = fma(s[i], p2, c_adj_series[j][i]);
+#pragma unroll
+      for (int i = 3; i < 6; ++i) s[i] *= phi;
+#pragma unroll
+      for (int i = 10; i < 14; ++i) s[i] *= phi;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 14; ++i) s[i] = 0.0;
+      for (int a = 0; a < nss; ++a) {
+        const double xi = c_glx[a], px = phi * xi;
+        double sn, cs, w = c_glw[a];
+        sincos(px, &sn, &cs);
+        const double hr = -cs - px * sn, hi = px * cs - sn;
+#pragma unroll
+        for (int m = 1; m <= 4; ++m) {
+          w *= xi;
+          s[5 + m] += w * hr;
+          s[9 + m] += w * hi;
+          if (m >= 2) {
+            s[m - 2] += w * cs;
+            s[m + 1] += w * sn;
+          }
+        }
+      }
+    }
+    const double g = T(4) * rinv, g3 = g * (rinv * rinv);
+    Cx h1 = {0.0, 0.0}, h2 = {0.0, 0.0};
+    e[0] = fma(g, s[0], e[0]);
+    e[1] = fma(g, s[3], e[1]);
+    const double ar = g * s[1], ai = g * s[4], br = g * s[2], bi = g * s[5];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double p = T(5 + q);
+      e[2 + 2 * q] = fma(uv[q], ar, e[2 + 2 * q]);
+      e[3 + 2 * q] = fma(uv[q], ai, e[3 + 2 * q]);
+      e[10 + 2 * q] = fma(p, br, e[10 + 2 * q]);
+      e[11 + 2 * q] = fma(p, bi, e[11 + 2 * q]);
+      h1 = cx_axpy(uv[q], hu[q], h1);
+      h2 = cx_axpy(p, huv[q], h2);
+    }
+    double F[2];
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+      F[m] = g3 * (fma(s[6 + m], h0.r, -s[10 + m] * h0.i) + fma(s[7 + m], h1.r, -s[11 + m] * h1.i) +
+                   fma(s[8 + m], h2.r, -s[12 + m] * h2.i));
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[c] = fma(F[0], d[c], f[c]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double fq = F[1] * uv[q];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[3 + 3 * q + c] = fma(fq, d[c], f[3 + 3 * q + c]);
+    }
+  }
 }
 
-__global__ void __launch_bounds__(128) adjoint_singular_kernel(DevMesh m, double k, int nss, const double* lam,
-                                                               const double* U, int64_t ld, int64_t nrhs,
+__global__ void __launch_bounds__(128) adjoint_singular_kernel(DevMesh m, double k, int nss,
+                                                               const double* __restrict__ table,
+                                                               const double* __restrict__ lam,
+                                                               const double* __restrict__ U, int64_t ld, int64_t nrhs,
                                                                double* grad) {
-  const TouchPair tp = m.touch[blockIdx.x];
-  const int t1 = tp.t1, t2 = tp.t2;
-  int v1[3], v2[3], e1[3], e2[3];
-  double sl1[3], sl2[3], l1[3], l2[3], V1[3][3], V2[3][3];
-  tri_edge_data(m, t1, v1, e1, sl1, l1, V1);
-  tri_edge_data(m, t2, v2, e2, sl2, l2, V2);
-  double Pp[3][3], Qp[3][3];  // permuted vertices (Sauter-Schwab order), absolute
-  for (int a = 0; a < 3; ++a)
-    for (int d = 0; d < 3; ++d) {
-      Pp[a][d] = m.verts[3 * tp.p[a] + d];
-      Qp[a][d] = m.verts[3 * tp.q[a] + d];
+  const int64_t pair = int64_t(blockIdx.x) * 4 + (threadIdx.x >> 5);
+  if (pair >= m.ntouch) return;
+  const int lane = threadIdx.x & 31;
+  const TouchPair tp = m.touch[pair];
+  const int64_t t1 = tp.t1, t2 = tp.t2;
+  double EP[2][3], EQ[2][3], X1[3][3], X2[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double o = m.verts[3 * tp.p[0] + c];  // the shared vertex P0 = Q0
+    EP[0][c] = m.verts[3 * tp.p[1] + c] - o;
+    EP[1][c] = m.verts[3 * tp.p[2] + c] - m.verts[3 * tp.p[1] + c];
+    EQ[0][c] = m.verts[3 * tp.q[1] + c] - o;
+    EQ[1][c] = m.verts[3 * tp.q[2] + c] - m.verts[3 * tp.q[1] + c];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      X1[a][c] = m.verts[3 * m.tris[3 * t1 + a] + c] - o;
+      X2[a][c] = m.verts[3 * m.tris[3 * t2 + a] + c] - o;
     }
-  // local coordinates relative to the shared vertex Pp[0] == Qp[0]
-  double P[3][3], Q[3][3];
-  for (int a = 0; a < 3; ++a)
-    for (int d = 0; d < 3; ++d) {
-      P[a][d] = V1[a][d] - Pp[0][d];
-      Q[a][d] = V2[a][d] - Qp[0][d];
+  }
+  // W_jk = s_j l_j s'_k l'_k 4/(4 pi) sum_i (lambda_j u_k [+ u_j lambda_k unless t1 = t2]), one entry
+  // per lane 0-8; the 4 is the reference weights' Jacobian 2A 2A'/(A A')
+  Cx W[3][3];
+  {
+    const int j = lane < 9 ? lane / 3 : 0, kk = lane < 9 ? lane % 3 : 0;
+    const int64_t o1 = m.tri_edge[3 * t1 + j] * ld, o2 = m.tri_edge[3 * t2 + kk] * ld;
+    const Cx* L = reinterpret_cast<const Cx*>(lam);
+    const Cx* Uc = reinterpret_cast<const Cx*>(U);
+    Cx w = {0.0, 0.0};
+    const double mir = t1 != t2 ? 1.0 : 0.0;
+    for (int64_t i = 0; i < nrhs; ++i) {
+      const Cx a = L[o1 + i], b = Uc[o2 + i], c = Uc[o1 + i] * mir, d = L[o2 + i];
+      w = w + a * b + c * d;
     }
-  PairCoef pc;
-  load_w(lam, U, ld, nrhs, e1, e2, sl1, sl2, t1 != t2, pc);
-  make_coef(P, Q, pc);
-  PairAcc A;
-  A.I0 = A.Mxy = Cx{0, 0};
-  for (int d = 0; d < 3; ++d) A.Mx[d] = A.My[d] = Cx{0, 0};
-  double gp[3][3] = {}, gq[3][3] = {};  // gradients w.r.t. the permuted vertices
-  const int n2 = nss * nss, n4 = n2 * n2;
-  auto visit = [&](double u1, double u2, double w1, double w2, double wt) {
-    double ax[3], ay[3], x[3], y[3], dv[3];
-    chi_bary(u1, u2, ax);
-    chi_bary(w1, w2, ay);
-    for (int d = 0; d < 3; ++d) {
-      x[d] = u1 * (Pp[1][d] - Pp[0][d]) + u2 * (Pp[2][d] - Pp[1][d]);
-      y[d] = w1 * (Qp[1][d] - Qp[0][d]) + w2 * (Qp[2][d] - Qp[1][d]);
-      dv[d] = x[d] - y[d];
-    }
-    double gx[3] = {0, 0, 0}, gy[3] = {0, 0, 0};
-    point_pair(k, pc, x, y, dv, 4.0 * wt * kInv4Pi, gx, gy, A);
+    const double sc = (2.0 * m.tri_area[t1] * m.tri_coef[3 * t1 + j]) * (2.0 * m.tri_area[t2] * m.tri_coef[3 * t2 + kk]);
+    w = w * (4.0 * kInv4Pi * sc);
+#pragma unroll
     for (int a = 0; a < 3; ++a)
-      for (int d = 0; d < 3; ++d) {
-        gp[a][d] += ax[a] * gx[d];
-        gq[a][d] += ay[a] * gy[d];
+#pragma unroll
+      for (int b = 0; b < 3; ++b)
+        W[a][b] = {__shfl_sync(0xffffffffu, w.r, 3 * a + b), __shfl_sync(0xffffffffu, w.i, 3 * a + b)};
+  }
+  const double k4 = 0.25 * k, kinv = 1.0 / k;
+  Cx S = {0.0, 0.0}, c0 = {0.0, 0.0}, Us[3] = {}, Vs[3] = {};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const Cx r = W[j][0] + W[j][1] + W[j][2], c = W[0][j] + W[1][j] + W[2][j];
+    S = S + r;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      Us[d] = cx_axpy(X2[j][d], c, Us[d]);
+      Vs[d] = cx_axpy(X1[j][d], r, Vs[d]);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) c0 = cx_axpy(ss_dot(X1[j], X2[b]), W[j][b], c0);
+  }
+  // H(xi xh, xi yh) = h0 + xi h1 + xi^2 h2 with h1 linear in (u, v) and h2 in the products u v
+  const Cx h0 = {fma(k4, c0.i, -kinv * S.i), fma(-k4, c0.r, kinv * S.r)};
+  Cx hu[4], huv[4];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    Cx eu = {0.0, 0.0}, fv = {0.0, 0.0};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      eu = cx_axpy(EP[s][d], Us[d], eu);
+      fv = cx_axpy(EQ[s][d], Vs[d], fv);
+    }
+    hu[s] = {-k4 * eu.i, k4 * eu.r};  // (ik/4) E_s.U
+    hu[2 + s] = {-k4 * fv.i, k4 * fv.r};
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      const double ef = k4 * ss_dot(EP[s], EQ[t]);
+      huv[2 * s + t] = {ef * S.i, -ef * S.r};  // -(ik/4) S E_s.F_t
+    }
+  }
+  const int J = ss_terms(ss_phase_bound(k, EP, EQ));
+  const int terms = J > 0 ? min(J + 1, kSsTerms) : 0;  // the Q series carry a factor 2j - 1
+  double e[18], f[15];
+#pragma unroll
+  for (int i = 0; i < 18; ++i) e[i] = 0.0;
+#pragma unroll
+  for (int i = 0; i < 15; ++i) f[i] = 0.0;
+  if (tp.kind == 3) adjoint_ss_moments<3>(table, k, nss, terms, EP, EQ, h0, hu, huv, lane, e, f);
+  else if (tp.kind == 2) adjoint_ss_moments<2>(table, k, nss, terms, EP, EQ, h0, hu, huv, lane, e, f);
+  else adjoint_ss_moments<1>(table, k, nss, terms, EP, EQ, h0, hu, huv, lane, e, f);
+  ss_warp_sum<18>(e, lane);
+  ss_warp_sum<15>(f, lane);
+  if (lane >= 2) return;
+  // Lane 0 takes t1's side, lane 1 t2's, the same formulas with the sides exchanged: X, E this
+  // side's vertices and edge vectors, O, Eo the other's, Wk this side's index first.
+  const bool sw = lane == 1;
+  auto pick = [&](double a, double b) { return sw ? b : a; };
+  double X[3][3], O[3][3], E[2][3], Eo[2][3];
+  Cx Wk[3][3], Ux[3], Mi[3], Mo[3], Mp[3][3];  // moments: this side's basis (1, u1, u2), the other's, products
+  double g[3][3];                            // point gradients along the basis (F part)
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      X[a][d] = pick(X1[a][d], X2[a][d]);
+      O[a][d] = pick(X2[a][d], X1[a][d]);
+      if (a < 2) {
+        E[a][d] = pick(EP[a][d], EQ[a][d]);
+        Eo[a][d] = pick(EQ[a][d], EP[a][d]);
       }
-  };
-  for (int idx = threadIdx.x; idx < n4; idx += blockDim.x) {
-    int a = idx / (n2 * nss), b = (idx / n2) % nss, c = (idx / nss) % nss, d = idx % nss;
-    double xi = c_glx[a], e1 = c_glx[b], e2 = c_glx[c], e3 = c_glx[d];
-    double w4 = c_glw[a] * c_glw[b] * c_glw[c] * c_glw[d];
-    if (tp.kind == 3) {
-      double w = w4 * xi * xi * xi * e1 * e1 * e2;
-      visit(xi, xi * (1 - e1 + e1 * e2), xi * (1 - e1 * e2 * e3), xi * (1 - e1), w);
-      visit(xi * (1 - e1 * e2 * e3), xi * (1 - e1), xi, xi * (1 - e1 + e1 * e2), w);
-      visit(xi, xi * e1 * (1 - e2 + e2 * e3), xi * (1 - e1 * e2), xi * e1 * (1 - e2), w);
-      visit(xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * (1 - e2 + e2 * e3), w);
-      visit(xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * (1 - e2), w);
-      visit(xi, xi * e1 * (1 - e2), xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), w);
-    } else if (tp.kind == 2) {
-      double w0 = w4 * xi * xi * xi * e1 * e1, w1 = w0 * e2;
-      visit(xi, xi * e1 * e3, xi * (1 - e1 * e2), xi * e1 * (1 - e2), w0);
-      visit(xi, xi * e1, xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), w1);
-      visit(xi * (1 - e1 * e2), xi * e1 * (1 - e2), xi, xi * e1 * e2 * e3, w1);
-      visit(xi * (1 - e1 * e2 * e3), xi * e1 * e2 * (1 - e3), xi, xi * e1, w1);
-      visit(xi * (1 - e1 * e2 * e3), xi * e1 * (1 - e2 * e3), xi, xi * e1 * e2, w1);
-    } else {
-      double w = w4 * xi * xi * xi * e2;
-      visit(xi, xi * e1, xi * e2, xi * e2 * e3, w);
-      visit(xi * e2, xi * e2 * e3, xi, xi * e1, w);
+      Wk[a][d] = {pick(W[a][d].r, W[d][a].r), pick(W[a][d].i, W[d][a].i)};
+      g[a][d] = a == 0 ? pick(f[d], -f[d]) : pick(f[3 * a + d], -f[6 + 3 * a + d]);
     }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) Ux[d] = {pick(Us[d].r, Vs[d].r), pick(Us[d].i, Vs[d].i)};
+  const Cx I0 = {e[0], e[1]};
+  Mi[0] = Mo[0] = Mp[0][0] = I0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    Mi[1 + s] = {pick(e[2 + 2 * s], e[6 + 2 * s]), pick(e[3 + 2 * s], e[7 + 2 * s])};
+    Mo[1 + s] = {pick(e[6 + 2 * s], e[2 + 2 * s]), pick(e[7 + 2 * s], e[3 + 2 * s])};
+    Mp[1 + s][0] = Mi[1 + s];
+    Mp[0][1 + s] = Mo[1 + s];
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      Mp[1 + s][1 + t] = {pick(e[10 + 4 * s + 2 * t], e[10 + 4 * t + 2 * s]),
+                          pick(e[11 + 4 * s + 2 * t], e[11 + 4 * t + 2 * s])};
   }
-  // block reduction: 18 + 18 point-chained reals and the 16 moment reals
-  __shared__ double red[4][52];
-  double vals[52];
-  int o = 0;
-  for (int a = 0; a < 3; ++a)
+  // point gradients linear in G: (k/4) Im(S sum phi_i G y - U sum phi_i G), phi = (1, u1, u2)
+  Cx My[3] = {}, Mx[3] = {}, Mxy = {0.0, 0.0};
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-      vals[o++] = gp[a][d];
-      vals[o++] = gq[a][d];
+      Cx y = {0.0, 0.0};
+#pragma unroll
+      for (int t = 0; t < 2; ++t) y = cx_axpy(Eo[t][d], Mp[i][1 + t], y);
+      g[i][d] = fma(k4, cx_mul_im(S, y) - cx_mul_im(Ux[d], Mp[i][0]), g[i][d]);
+      if (i == 0) My[d] = y;
+      else {
+        Mx[d] = cx_axpy(E[i - 1][d], Mi[i], Mx[d]);
+        Mxy = cx_axpy(E[i - 1][d], y, Mxy);
+      }
     }
-  vals[o++] = A.I0.r; vals[o++] = A.I0.i; vals[o++] = A.Mxy.r; vals[o++] = A.Mxy.i;
-  for (int d = 0; d < 3; ++d) {
-    vals[o++] = A.Mx[d].r; vals[o++] = A.Mx[d].i; vals[o++] = A.My[d].r; vals[o++] = A.My[d].i;
-  }
-  for (int i = 0; i < 52; ++i) {
-    double v = vals[i];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    vals[i] = v;
-  }
-  if ((threadIdx.x & 31) == 0)
-    for (int i = 0; i < 52; ++i) red[threadIdx.x >> 5][i] = vals[i];
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  for (int i = 0; i < 52; ++i) vals[i] = red[0][i] + red[1][i] + red[2][i] + red[3][i];
-  o = 0;
-  for (int a = 0; a < 3; ++a)
-    for (int d = 0; d < 3; ++d) {
-      gp[a][d] = vals[o++];
-      gq[a][d] = vals[o++];
-    }
-  A.I0 = {vals[o], vals[o + 1]}; o += 2;
-  A.Mxy = {vals[o], vals[o + 1]}; o += 2;
-  for (int d = 0; d < 3; ++d) {
-    A.Mx[d] = {vals[o], vals[o + 1]};
-    A.My[d] = {vals[o + 2], vals[o + 3]};
-    o += 4;
-  }
-  double gP[3][3], gQ[3][3], gl1[3], gl2[3];
-  explicit_terms(k, pc, A, P, Q, l1, l2, gP, gQ, gl1, gl2);
-  double g1[3][3], g2[3][3];
-  for (int a = 0; a < 3; ++a)
-    for (int d = 0; d < 3; ++d) {
-      g1[a][d] = gP[a][d];
-      g2[a][d] = gQ[a][d];
-    }
-  chain_lengths(V1, l1, gl1, g1);
-  chain_lengths(V2, l2, gl2, g2);
+  // J_Z enters the objective with a minus sign; x = P0 (1 - u1) + P1 (u1 - u2) + P2 u2
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    add_grad(grad, v1[a], g1[a], -1.0);
-    add_grad(grad, v2[a], g2[a], -1.0);
-    add_grad(grad, tp.p[a], gp[a], -1.0);
-    add_grad(grad, tp.q[a], gq[a], -1.0);
+    double ga[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) ga[d] = a < 2 ? g[a][d] - g[a + 1][d] : g[a][d];
+    add_grad(grad, sw ? tp.q[a] : tp.p[a], ga, -1.0);
   }
+  // opposite vertices and edge lengths (adjoint_side's formulas)
+  double gv[3][3] = {};
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const Cx r = Wk[j][0] + Wk[j][1] + Wk[j][2];
+    Cx t = Mxy, xq = {0.0, 0.0};
+    double im = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      Cx wq = {0.0, 0.0};
+#pragma unroll
+      for (int b = 0; b < 3; ++b) wq = cx_axpy(O[b][d], Wk[j][b], wq);
+      gv[j][d] = fma(-k4, cx_mul_im(r, My[d]) - cx_mul_im(wq, I0), gv[j][d]);
+      t = cx_axpy(-X[j][d], My[d], t);
+      xq = cx_axpy(X[j][d], wq, xq);
+      im -= cx_mul_im(wq, Mx[d]);
+    }
+    im += cx_mul_im(r, t) + cx_mul_im(xq, I0);
+    const double lk = fma(k4, im, -kinv * cx_mul_im(r, I0));
+    const int a = (j + 1) % 3, b = (j + 2) % 3;
+    double ev[3], l2 = 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      ev[d] = X[b][d] - X[a][d];
+      l2 = fma(ev[d], ev[d], l2);
+    }
+    const double rl = ss_rsqrt(l2), fl = lk * (rl * rl);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      gv[b][d] = fma(fl, ev[d], gv[b][d]);
+      gv[a][d] = fma(-fl, ev[d], gv[a][d]);
+    }
+  }
+  const int64_t tt = sw ? t2 : t1;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) add_grad(grad, m.tris[3 * tt + a], gv[a], -1.0);
 }
 
 // ------------------------------------------------------------------ plane-wave moments
@@ -677,7 +705,9 @@ cudaError_t launch_adjoint_pairs(const DevMesh& m, double k, int nss, const doub
   adjoint_regular_kernel<<<grid, 128, 0, s>>>(m, k, lam, U, ld, nrhs, grad);
   note_launches(1);
   if (m.ntouch > 0) {
-    adjoint_singular_kernel<<<unsigned(m.ntouch), 128, 0, s>>>(m, k, nss, lam, U, ld, nrhs, grad);
+    const double* table = ss_table_device();
+    if (!table) return cudaErrorInvalidSymbol;
+    adjoint_singular_kernel<<<cdiv(m.ntouch, 4), 128, 0, s>>>(m, k, nss, table, lam, U, ld, nrhs, grad);
     note_launches(1);
   }
   return cudaGetLastError();

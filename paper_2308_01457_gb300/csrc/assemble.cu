@@ -350,8 +350,8 @@ __device__ __forceinline__ void ss_moments(double k, int nss, int J, const doubl
   for (int idx = lane; idx < count; idx += 32) {
     auto T = [&](int f) { return __ldg(tab + f * stride + idx); };
     const double uv[4] = {T(0), T(1), T(2), T(3)};
-    double rinv, phi;
-    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, rinv, phi);
+    double d[3], rinv, phi;
+    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, d, rinv, phi);
     double sr[3], si[3];
     if (J > 0) {
       const double p2 = phi * phi;

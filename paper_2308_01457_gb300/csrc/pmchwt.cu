@@ -240,8 +240,8 @@ __device__ __forceinline__ void pm_moments(const double* __restrict__ table, dou
   for (int idx = lane; idx < count; idx += 32) {
     auto T = [&](int f) { return __ldg(tab + f * stride + idx); };
     const double uv[4] = {T(0), T(1), T(2), T(3)};
-    double rinv, phi;
-    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, rinv, phi);
+    double d[3], rinv, phi;
+    ss_distance<KIND>(tab + idx, stride, uv, EP, EQ, k, d, rinv, phi);
     // s: Re S_0..2, Im S_0..2, Re Q_1..2, Im Q_1..2
     double s[NS];
     if (J > 0) {
@@ -520,7 +520,7 @@ void upload_rules_pmchwt(const Rules& r) {
   cudaMemcpyToSymbol(c_pm_glw, r.glw, sizeof(r.glw));
   double e[kSsTerms][6], h[kSsTerms][4], c[kSsTerms][10];
   make_ss_series(r, e);
-  make_ss_series_mfio(r, h);
+  make_ss_series_mfio<2>(r, h);
   for (int j = 0; j < kSsTerms; ++j)
     for (int i = 0; i < 10; ++i) c[j][i] = i < 6 ? e[j][i] : h[j][i - 6];
   cudaMemcpyToSymbol(c_pm_series, c, sizeof(c));

@@ -78,10 +78,11 @@ inline void make_ss_series(const Rules& r, double (&c)[kSsTerms][6]) {
   }
 }
 
-// The same for Q_m(phi) = sum_a w_a xi_a^m (i phi xi_a - 1) exp(i phi xi_a), m = 1, 2, the xi sums of
-// exp(ikr)(ikr - 1)/r^3: Re Q_m = sum_j (-1)^j (2j-1)/(2j)! M_{m+2j} phi^{2j} (c[j][m-1]) and
-// Im Q_m = phi sum_j (-1)^j 2j/(2j+1)! M_{m+2j+1} phi^{2j} (c[j][1+m]).
-inline void make_ss_series_mfio(const Rules& r, double (&c)[kSsTerms][4]) {
+// The same for Q_m(phi) = sum_a w_a xi_a^m (i phi xi_a - 1) exp(i phi xi_a), m = 1 .. MM, the xi sums
+// of exp(ikr)(ikr - 1)/r^3: Re Q_m = sum_j (-1)^j (2j-1)/(2j)! M_{m+2j} phi^{2j} (c[j][m-1]) and
+// Im Q_m = phi sum_j (-1)^j 2j/(2j+1)! M_{m+2j+1} phi^{2j} (c[j][MM+m-1]).
+template <int MM>
+inline void make_ss_series_mfio(const Rules& r, double (&c)[kSsTerms][2 * MM]) {
   auto moment = [&](int n) {
     long double s = 0;
     for (int a = 0; a < r.nss; ++a) s += (long double)r.glw[a] * std::pow((long double)r.glx[a], n);
@@ -91,9 +92,9 @@ inline void make_ss_series_mfio(const Rules& r, double (&c)[kSsTerms][4]) {
   for (int j = 0; j < kSsTerms; ++j) {
     if (j > 0) fact *= (long double)(2 * j - 1) * (2 * j);
     const long double sg = j & 1 ? -1 : 1;
-    for (int m = 1; m <= 2; ++m) {
+    for (int m = 1; m <= MM; ++m) {
       c[j][m - 1] = double(sg * (2 * j - 1) * moment(m + 2 * j) / fact);
-      c[j][1 + m] = double(sg * 2 * j * moment(m + 1 + 2 * j) / (fact * (2 * j + 1)));
+      c[j][MM + m - 1] = double(sg * 2 * j * moment(m + 1 + 2 * j) / (fact * (2 * j + 1)));
     }
   }
 }
@@ -160,12 +161,12 @@ __device__ __forceinline__ constexpr int ss_regions() {
   return KIND == 3 ? 6 : (KIND == 2 ? 5 : 2);
 }
 
-// Distance and phase of one point of the table (field f at tab[f * stride]): 1/rh and k rh.
+// Difference xh - yh, distance and phase of one point of the table (field f at tab[f * stride]):
+// 1/rh and k rh.
 template <int KIND>
 __device__ __forceinline__ void ss_distance(const double* tab, int stride, const double (&uv)[4],
                                             const double (&EP)[2][3], const double (&EQ)[2][3], double k,
-                                            double& rinv, double& phi) {
-  double d[3];
+                                            double (&d)[3], double& rinv, double& phi) {
   if constexpr (KIND == 3) {  // EQ = EP: the coordinate differences are in the table
     const double a = __ldg(tab + 9 * stride), b = __ldg(tab + 10 * stride);
 #pragma unroll
