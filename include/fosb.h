@@ -182,8 +182,8 @@ fosb_status fosb_assemble_efie(fosb_mesh mesh, double k, const fosb_quad_opts* o
 /* ---- A5: LU factorisation -----------------------------------------------------------
  * P Z = L U.  complex128 factors (FOSB_FP64): partial pivoting (largest |Re| + |Im|, ties to
  * the lowest row).  complex64 factors (FOSB_MIXED, FOSB_FP32): 256-column blocks of 64-column
- * panels whose pivot rows a tournament chooses (leaves of 256 rows and a fan-in-4 tree, each
- * choosing by partial pivoting with the magnitudes compared on their top 15 mantissa bits).
+ * panels whose pivot rows a tournament chooses (up to 2048 rows per leaf and up to 32 leaves per
+ * merge, each choosing by partial pivoting with the magnitudes compared on their top 15 mantissa bits).
  *   Z    : device, n x n row-major (complex128 for FP64/MIXED, complex64 for FP32);
  *          read, not modified.  For FOSB_MIXED the handle keeps a NON-owning reference
  *          to Z for the FP64 residuals: Z must stay alive and unchanged until

@@ -209,14 +209,17 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   }
   std::vector<double> bn, xn, rn;
   FOSB_TRY(col_norms(Bsrc, n, nrhs, ldbs, nb.as<double>(), bn, s));
-  // x0
-  FOSB_CUDA(convert_c128_to_c64(Bsrc, n, nrhs, ldbs, d.p, nrhs, s));
-  FOSB_CUDA(getrs<float>(lu->lu, n, n, lu->ipiv, d.p, nrhs, nrhs, s, lu->d_status, lu->dinv));
-  FOSB_CUDA(convert_c64_to_c128(d.p, n, nrhs, nrhs, X, ldx, s));
+  auto first_iterate = [&]() -> fosb_status {
+    FOSB_CUDA(convert_c128_to_c64(Bsrc, n, nrhs, ldbs, d.p, nrhs, s));
+    FOSB_CUDA(getrs<float>(lu->lu, n, n, lu->ipiv, d.p, nrhs, nrhs, s, lu->d_status, lu->dinv));
+    FOSB_CUDA(convert_c64_to_c128(d.p, n, nrhs, nrhs, X, ldx, s));
+    return FOSB_OK;
+  };
+  FOSB_TRY(first_iterate());
   const int solver = ropt ? ropt->solver : FOSB_REFINE_AUTO;
   if (solver < FOSB_REFINE_AUTO || solver > FOSB_REFINE_GMRES)
     return fail(FOSB_ERR_INVALID_ARG, "fosb_solve: unknown refinement solver");
-  double prev = INFINITY, prev2 = INFINITY, berr = INFINITY;
+  double prev = INFINITY, prev2 = INFINITY, berr = INFINITY, res = INFINITY, res0 = INFINITY;
   int it = 0;
   for (; solver != FOSB_REFINE_GMRES;) {
     FOSB_CUDA(copy_matrix(Bsrc, n, nrhs, ldbs, r.p, nrhs, 16, s));
@@ -227,11 +230,13 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
                              lu->zff));
     FOSB_TRY(col_norms(r.p, n, nrhs, nrhs, nb.as<double>(), rn, s));
     FOSB_TRY(col_norms(X, n, nrhs, ldx, nb.as<double>(), xn, s));
-    berr = 0.0;
+    berr = res = 0.0;
     for (int64_t c = 0; c < nrhs; ++c) {
       double den = lu->znorm_inf * xn[c] + bn[c];
       berr = std::max(berr, den > 0 ? rn[c] / den : 0.0);
+      res = std::max(res, bn[c] > 0 ? rn[c] / bn[c] : rn[c]);
     }
+    if (it == 0) res0 = res;
     if (berr <= tol || it >= max_iters) break;
     if (berr >= prev && prev >= prev2) break;  // no decrease over two steps
     if (berr < 1e-13 && berr > 0.5 * prev) break;  // at the rounding floor: progress has stalled
@@ -243,7 +248,11 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
     ++it;
   }
   if (solver == FOSB_REFINE_GMRES || (solver == FOSB_REFINE_AUTO && !(berr <= tol) && !(berr <= 1e-13))) {
-    // GMRES-IR column by column for the columns refinement left above the tolerance
+    // GMRES-IR column by column for the columns refinement left above the tolerance, from the
+    // first iterate again where refinement diverged (by the residual: the backward error stays
+    // small as x grows): its last iterate can be off by any power of kappa u_32, which would cost
+    // GMRES-IR its outer steps
+    if (solver == FOSB_REFINE_AUTO && !(res <= res0)) FOSB_TRY(first_iterate());
     Scratch xc(s);
     FOSB_CUDA(xc.alloc(16 * n));
     berr = 0.0;
@@ -375,25 +384,29 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
                                      : getrf<float>(lu->lu, n, n, lu->ipiv, lu->d_status, s);
   if (st != FOSB_OK) return cleanup(st);
   int status = 0;
-  std::vector<int32_t> ipiv(n);
+  std::vector<int32_t> ipiv(prec == FOSB_FP64 ? n : 0);
   if ((e = cudaMemcpyAsync(&status, lu->d_status, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
-      (e = cudaMemcpyAsync(ipiv.data(), lu->ipiv, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s)) ||
+      (prec == FOSB_FP64 &&
+       (e = cudaMemcpyAsync(ipiv.data(), lu->ipiv, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s))) ||
       (e = cudaStreamSynchronize(s)))
     return cleanup(cuda_fail(e, "fosb_factor: status"));
   if (status == FOSB_ERR_TIMEOUT) return cleanup(fail(FOSB_ERR_TIMEOUT, "fosb_factor: panel grid barrier timed out"));
   if (status == FOSB_ERR_SINGULAR) return cleanup(fail(FOSB_ERR_SINGULAR, "fosb_factor: zero pivot"));
-  // compose the row interchanges into one permutation: (P b)[i] = b[perm[i]]
-  std::vector<int32_t> perm(n);
-  for (int64_t i = 0; i < n; ++i) perm[i] = int32_t(i);
-  for (int64_t i = 0; i < n; ++i) {
-    int32_t p = ipiv[i];
-    if (p < 0 || p >= n) return cleanup(fail(FOSB_ERR_CUDA, "fosb_factor: corrupt pivot"));
-    std::swap(perm[i], perm[p]);
+  if (prec == FOSB_FP64) {
+    // compose the row interchanges into one permutation: (P b)[i] = b[perm[i]] (complex64 factors
+    // come with it)
+    std::vector<int32_t> perm(n);
+    for (int64_t i = 0; i < n; ++i) perm[i] = int32_t(i);
+    for (int64_t i = 0; i < n; ++i) {
+      int32_t p = ipiv[i];
+      if (p < 0 || p >= n) return cleanup(fail(FOSB_ERR_CUDA, "fosb_factor: corrupt pivot"));
+      std::swap(perm[i], perm[p]);
+    }
+    // stream-ordered (a plain cudaMemcpy would also wait for the legacy default stream's work);
+    // perm is pageable, so the call returns once it is staged
+    if ((e = cudaMemcpyAsync(lu->ipiv, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s)))
+      return cleanup(cuda_fail(e, "fosb_factor: permutation"));
   }
-  // stream-ordered (a plain cudaMemcpy would also wait for the legacy default stream's work);
-  // perm is pageable, so the call returns once it is staged
-  if ((e = cudaMemcpyAsync(lu->ipiv, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, s)))
-    return cleanup(cuda_fail(e, "fosb_factor: permutation"));
   if (prec != FOSB_FP64) {  // inverted diagonal blocks for the streaming triangular sweeps
     if ((e = cudaMalloc(&lu->dinv, tri_block_inverses_bytes(n))) != cudaSuccess ||
         (e = tri_block_inverses_c64(lu->lu, n, n, lu->dinv, s)) != cudaSuccess)

@@ -119,7 +119,7 @@ struct fosb_lu_s {
   int prec = 0;
   int64_t n = 0;
   void* lu = nullptr;          // n x n factors (complex128 for FP64, complex64 otherwise), row-major ld = n
-  int32_t* ipiv = nullptr;     // n pivots (row swapped with i at step i), device
+  int32_t* ipiv = nullptr;     // composed row permutation, device
   const void* zref = nullptr;  // MIXED: non-owning complex128 Z for residuals
   int64_t ldz = 0;
   void* zff = nullptr;         // MIXED: (hi, lo) float split of Z (n x n float4) for the residual GEMMs
@@ -233,22 +233,27 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha_re, double alp
 // dst (rows x cols float4, ldd) = (hi, lo) float split of the complex128 src
 cudaError_t split_ff(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                      cudaStream_t s);
+// ipiv: complex128 the interchanges (row i was swapped with ipiv[i] at step i), complex64 the
+// composed permutation ((P A)[i] = A[ipiv[i]]).
 template <typename T>
 fosb_status getrf(void* A, int64_t n, int64_t lda, int32_t* ipiv, int* d_status, cudaStream_t s);
 size_t getrf_scratch_bytes(int64_t max_ctas, bool c128);
 // Tournament-pivoting factorisation of one complex64 panel (m x jb at Ap, jb <= 64, m >= jb)
-// with scratch of tslu_scratch_bytes(n_max) bytes (n_max >= m); writes ipiv[0..jb) as
-// absolute rows (row_base + panel row) and permutes the panel's own rows.
+// with scratch of tslu_scratch_bytes(n_max) bytes (n_max >= m): permutes the panel's own rows
+// and leaves the moves in the scratch for tslu_swap.
 size_t tslu_scratch_bytes(int64_t n_max);
-cudaError_t tslu_panel(void* Ap, int64_t m, int jb, int64_t lda, int32_t* ipiv, int64_t row_base, void* scratch,
-                       int64_t n_max, int* d_status, cudaStream_t s);
+cudaError_t tslu_identity(int32_t* perm, int64_t n, cudaStream_t s);  // perm[i] = i
+cudaError_t tslu_panel(void* Ap, int64_t m, int jb, int64_t lda, void* scratch, int64_t n_max, int* d_status,
+                       cudaStream_t s);
 // X (jb x ncols, leading dimension ldx) := L^{-1} X, L the unit lower jb x jb block at D
 // (leading dimension ldd), complex64, jb <= 64: a thread per column (tslu.cu).
 cudaError_t tri_lower_unit_cols(const void* D, int64_t ldd, int jb, void* X, int64_t ldx, int64_t ncols,
                                 cudaStream_t s);
 // The row interchanges of the last tslu_panel on the same scratch, applied to the columns
-// of the n-column matrix A outside the panel's columns [j0, j0 + jb) (rows from j0 on).
-cudaError_t tslu_swap(void* A, int64_t n, int64_t lda, int64_t j0, int jb, const void* scratch, cudaStream_t s);
+// of the n-column matrix A outside the panel's columns [j0, j0 + jb) (rows from j0 on) and to
+// the composed permutation perm ((P A)[i] = A[perm[i]]).
+cudaError_t tslu_swap(void* A, int64_t n, int64_t lda, int64_t j0, int jb, const void* scratch, int32_t* perm,
+                      cudaStream_t s);
 template <typename T>
 fosb_status getrf_external_scratch(void* A, int64_t n, int64_t lda, int32_t* ipiv, int* d_status, void* scratch,
                                    int64_t max_ctas, cudaStream_t s);

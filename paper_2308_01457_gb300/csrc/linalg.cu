@@ -1278,6 +1278,7 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
     cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tslu_scr), tslu_scratch_bytes(n), s);
     if (e == cudaSuccess) e = cudaMallocAsync(&ws_a, update_split_a_bytes(n), s);
     if (e == cudaSuccess) e = cudaMallocAsync(&ws_b, update_split_b_bytes(n), s);
+    if (e == cudaSuccess) e = tslu_identity(ipiv, n, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(scratch, s);
       if (tslu_scr) cudaFreeAsync(tslu_scr, s);
@@ -1289,13 +1290,13 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
   auto panel_step = [&](int64_t j0, int jb) -> cudaError_t {
     cudaError_t e;
     if constexpr (sizeof(T) == 4)
-      e = tslu_panel(A + j0 * lda + j0, n - j0, jb, lda, ipiv + j0, j0, tslu_scr, n, d_status, s);
+      e = tslu_panel(A + j0 * lda + j0, n - j0, jb, lda, tslu_scr, n, d_status, s);
     else
       e = launch_panel<T>(A + j0 * lda + j0, n - j0, jb, lda, ipiv + j0, j0, scr, arrivals, cand_data, rowj,
                           d_status, int64_t(G_cap), nsm, s);
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) {
-      return tslu_swap(A, n, lda, j0, jb, tslu_scr, s);  // the panel's permutation as row moves
+      return tslu_swap(A, n, lda, j0, jb, tslu_scr, ipiv, s);  // the panel's permutation as row moves
     } else {
       laswp_kernel<T><<<cdiv(n, 256), 256, 0, s>>>(A, n, lda, j0, jb, ipiv);
       note_launches(2);  // panel + row swaps
