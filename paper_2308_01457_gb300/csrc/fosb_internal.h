@@ -246,7 +246,7 @@ cudaError_t tslu_identity(int32_t* perm, int64_t n, cudaStream_t s);  // perm[i]
 cudaError_t tslu_panel(void* Ap, int64_t m, int jb, int64_t lda, void* scratch, int64_t n_max, int* d_status,
                        cudaStream_t s);
 // X (jb x ncols, leading dimension ldx) := L^{-1} X, L the unit lower jb x jb block at D
-// (leading dimension ldd), complex64, jb <= 64: a thread per column (tslu.cu).
+// (leading dimension ldd), complex64, jb <= 64 (tslu.cu).
 cudaError_t tri_lower_unit_cols(const void* D, int64_t ldd, int jb, void* X, int64_t ldx, int64_t ncols,
                                 cudaStream_t s);
 // The row interchanges of the last tslu_panel on the same scratch, applied to the columns
