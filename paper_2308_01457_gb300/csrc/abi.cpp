@@ -194,7 +194,8 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   const int max_iters = ropt ? ropt->max_iters : 10;
   // default: the FP64 residual floor grows like sqrt(n) eps; stop at 8 sqrt(n) eps (>= 64 eps)
   const double eps = std::ldexp(1.0, -52);
-  const double tol = (ropt && ropt->tol > 0) ? ropt->tol : std::max(64.0, 8.0 * std::sqrt(double(n))) * eps;
+  const bool own_tol = !(ropt && ropt->tol > 0);
+  const double tol = own_tol ? std::max(64.0, 8.0 * std::sqrt(double(n))) * eps : ropt->tol;
   Scratch r(s), d(s), bkeep(s), nb(s);
   FOSB_CUDA(r.alloc(sizeof(double) * 2 * n * nrhs));
   FOSB_CUDA(d.alloc(sizeof(float) * 2 * n * nrhs));
@@ -237,6 +238,16 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       res = std::max(res, bn[c] > 0 ? rn[c] / bn[c] : rn[c]);
     }
     if (it == 0) res0 = res;
+    if (berr <= tol && own_tol && berr > 0.25 * tol && it < max_iters) {
+      // just below the default tolerance, whose last factor of 4 is above the rounding floor: the
+      // correction that this residual gives is worth its sweep (a better factorisation may stop a
+      // step earlier and must not end further off)
+      FOSB_CUDA(convert_c128_to_c64(r.p, n, nrhs, nrhs, d.p, nrhs, s));
+      FOSB_CUDA(getrs<float>(lu->lu, n, n, lu->ipiv, d.p, nrhs, nrhs, s, lu->d_status, lu->dinv));
+      FOSB_CUDA(axpy_c64_into_c128(d.p, n, nrhs, nrhs, X, ldx, s));
+      ++it;
+      break;
+    }
     if (berr <= tol || it >= max_iters) break;
     if (berr >= prev && prev >= prev2) break;  // no decrease over two steps
     if (berr < 1e-13 && berr > 0.5 * prev) break;  // at the rounding floor: progress has stalled

@@ -1,13 +1,22 @@
 // Trailing update C -= A B of the blocked complex64 LU on the tcgen05 tensor cores, fed by
-// bulk copies of operands split once per block (3xTF32: x = x_b + x_s, x_b = tf32(x),
-//   x y ~ x_b y_b + x_b y_s + x_s y_b).
+// bulk copies of operands split once per block into two fp16 values per real number.
+//
+// The split.  Every row i of A and column j of B is scaled by a power of two that brings its
+// largest |Re|, |Im| into [2^14, 2^15), and x s = x_h + x_l with x_h = fp16(x s), x_l = fp16(x s - x_h):
+//   x y ~ x_h y_h + x_h y_l + x_l y_h,
+// accumulated in FP32 and scaled back exactly.  fp16 carries 11 significand bits as TF32 does, so
+// the pair holds 22 bits like the 3xTF32 split (down to 2^-18 of the row's largest value, below
+// that the error is 2^-40 of it), and one MMA covers 16 values of k instead of 8: half the tensor time.
+// Error against 64 bits at K = 256, normwise: 1.9e-6 (3xTF32 3.6e-6) on uniform operands, on operands graded
+// over six decades inside their rows and on ones scaled by row and column over as many: half as
+// many accumulations in the tensor core.
 //
 // Split once, copied many times.  A (L21, M x K) and B (U12, K x N) are each split by one
 // pass per column block (K <= 256) into the exact shared-memory image the MMAs read: for every
-// 128-row (or 128-column) tile and 8-wide k-slab, 4 KB "parts" in the canonical no-swizzle
+// 128-row (or 128-column) tile and 16-wide k-slab, 4 KB "parts" in the canonical no-swizzle
 // K-major layout (8-row x 16-byte core matrices; 128 B between the two core matrices of a
-// slab, 256 B between 8-row groups).  Per slab, A has 4 parts (Re_b, Re_s, Im_b, Im_s) and
-// B has 6: big [Br_b | Bi_b | -Br_b] then small [Br_s | Bi_s | -Br_s].  A tile's stage is
+// slab, 256 B between 8-row groups).  Per slab, A has 4 parts (Re_h, Re_l, Im_h, Im_l) and
+// B has 6: high [Br_h | Bi_h | -Br_h] then low [Br_l | Bi_l | -Br_l].  A tile's stage is
 // then two plain cp.async.bulk copies (16 KB + 24 KB): no per-CTA split, no scattered
 // shared-memory stores, and a 3-deep ring that hides the L2 latency.
 //
@@ -15,8 +24,8 @@
 // tile in 256 TMEM columns, and B is read through two 256-row windows of the contiguous
 // parts:  [Br | Bi] (at Br) and [Bi | -Br] (at Bi), so
 //   D += A_r [Br | Bi] + (-A_i) [Bi | -Br] = [Ar Br - Ai Bi | Ar Bi + Ai Br]
-// (the -A_i by the instruction's negate-A bit): 6 MMAs of 128 x 256 x 8 per slab instead of
-// 12 of 128 x 128 x 8, with half the B-operand reads per useful flop.
+// (the -A_i by the instruction's negate-A bit): 6 MMAs of 128 x 256 x 16 per slab instead of
+// 12 of 128 x 128 x 16, with half the B-operand reads per useful flop.
 //
 // Roles (persistent, one CTA per SM, tiles in super-rows of 16 row tiles for L2 reuse):
 //   warp 0  producer: per slab waits empty[s], expect_tx 40 KB, two bulk copies;
@@ -27,6 +36,7 @@
 //           subtracted in place, and the half is stored with coalesced 16-byte writes.
 // Every wait is bounded; a time-out sets the status word and an abort flag, the MMA thread
 // drains its MMAs and the producer waits for its copies in flight before TMEM is freed.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -38,9 +48,10 @@ namespace fosb {
 namespace {
 
 constexpr int U_TM = 128, U_TN = 128;          // tile: 128 rows x 128 complex columns
-constexpr int U_KB = kLuBlock;                 // largest k extent of a split block (32 slabs)
-constexpr int U_SLABS = U_KB / 8;
-constexpr int U_PART = 4096;                   // one 128 x 8 tf32 part
+constexpr int U_KB = kLuBlock;                 // largest k extent of a split block (16 slabs)
+constexpr int U_KS = 16;                       // k values per slab
+constexpr int U_SLABS = U_KB / U_KS;
+constexpr int U_PART = 4096;                   // one 128 x 16 fp16 part
 constexpr int U_ABYTES = 4 * U_PART;           // A parts of one slab
 constexpr int U_BBYTES = 6 * U_PART;           // B parts of one slab
 constexpr int U_STAGE = U_ABYTES + U_BBYTES;   // 40 KB
@@ -55,28 +66,23 @@ constexpr long long U_SPIN = 1ll << 24;
 static_assert(U_SMEM <= 227 * 1024, "stages and drain tile exceed shared memory");
 
 __device__ __forceinline__ uint32_t su32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-__device__ __forceinline__ float tf32r(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-// byte offset of element (row, k8) of a part: 8-row groups 256 B apart, k halves 128 B apart
-__host__ __device__ __forceinline__ int part_off(int row, int k8) {
-  return (row >> 3) * 256 + (k8 >> 2) * 128 + (row & 7) * 16 + (k8 & 3) * 4;
+// byte offset of element (row, k), k < 16, of a part: 8-row groups 256 B apart, k halves 128 B apart
+__host__ __device__ __forceinline__ int part_off(int row, int k) {
+  return (row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2;
 }
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   return uint64_t((addr >> 4) & 0x3FFF) | (uint64_t(128 >> 4) << 16) | (uint64_t(256 >> 4) << 32) |
          (uint64_t(1) << 46);
 }
-// kind::tf32: D f32, A/B tf32, K-major, N = 256, M = 128, optional negate-A (bit 13)
+// kind::f16: D f32 (bits 4-5 = 1), A and B fp16 (bits 7-9, 10-12 = 0), K-major, N = 256, M = 128,
+// optional negate-A (bit 13)
 __host__ __device__ constexpr uint32_t u_idesc(bool neg_a) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | (neg_a ? (1u << 13) : 0u) | (uint32_t(256 >> 3) << 17) |
-         (uint32_t(U_TM >> 4) << 24);
+  return (1u << 4) | (neg_a ? (1u << 13) : 0u) | (uint32_t(256 >> 3) << 17) | (uint32_t(U_TM >> 4) << 24);
 }
 __device__ __forceinline__ void u_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 __device__ __forceinline__ bool u_wait(uint32_t mbar, uint32_t parity) {
@@ -131,42 +137,129 @@ __device__ __forceinline__ void u_cp_commit() { asm volatile("cp.async.commit_gr
 __device__ __forceinline__ void u_cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // ---------------------------------------------------------------- splits
-// A (M x K, lda), K <= 256 in nslab = ceil(K / 8) slabs: out[(rt * nslab + s) * 16 KB + p * 4 KB +
-// part_off(r, k8)], parts Re_b, Re_s, Im_b, Im_s; zero outside M x K.  One thread per (row, k)
-// of the padded tile grid.
-__global__ void split_a_kernel(int64_t M, int K, int nslab, const float2* __restrict__ A, int64_t lda,
-                               float* __restrict__ out, int64_t rows_pad) {
-  const int kp = nslab * 8;
-  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= rows_pad * kp) return;
-  const int64_t row = e / kp;
-  const int k = int(e % kp);
-  const float2 v = (row < M && k < K) ? A[row * lda + k] : make_float2(0.f, 0.f);
-  const float rb = tf32r(v.x), ib = tf32r(v.y);
-  float* base = out + ((row / U_TM) * nslab + k / 8) * (U_ABYTES / 4) + part_off(int(row % U_TM), k & 7) / 4;
-  base[0 * U_PART / 4] = rb;
-  base[1 * U_PART / 4] = tf32r(v.x - rb);
-  base[2 * U_PART / 4] = ib;
-  base[3 * U_PART / 4] = tf32r(v.y - ib);
+// Power of two that brings a row's or column's largest |Re|, |Im| (as a float bit pattern) into
+// [2^14, 2^15), and its inverse: exponents kept inside the normal range (both exact), one for
+// zero and for what is not finite.
+__device__ __forceinline__ float split_scale(unsigned mb, float& inv) {
+  const int e = int(mb >> 23);  // biased; 0 for zero and subnormals
+  const int sh = (e == 0 || e == 255) ? 0 : max(-110, min(110, 14 + 127 - e));
+  inv = __uint_as_float(unsigned(127 - sh) << 23);
+  return __uint_as_float(unsigned(127 + sh) << 23);
 }
-// B (K x N, ldb), K <= 256: out[(ct * nslab + s) * 24 KB + p * 4 KB + part_off(c, k8)], parts
-// Br_b, Bi_b, -Br_b, Br_s, Bi_s, -Br_s; zero outside K x N.  Threads run along N (coalesced).
-__global__ void split_b_kernel(int64_t N, int K, int nslab, const float2* __restrict__ B, int64_t ldb,
-                               float* __restrict__ out, int64_t cols_pad) {
-  const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= cols_pad * nslab * 8) return;
-  const int k = int(e / cols_pad);
-  const int64_t col = e % cols_pad;
-  const float2 v = (col < N && k < K) ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
-  const float rb = tf32r(v.x), ib = tf32r(v.y);
-  const float rs = tf32r(v.x - rb), is = tf32r(v.y - ib);
-  float* base = out + ((col / U_TN) * nslab + k / 8) * (U_BBYTES / 4) + part_off(int(col % U_TN), k & 7) / 4;
-  base[0 * U_PART / 4] = rb;
-  base[1 * U_PART / 4] = ib;
-  base[2 * U_PART / 4] = -rb;
-  base[3 * U_PART / 4] = rs;
-  base[4 * U_PART / 4] = is;
-  base[5 * U_PART / 4] = -rs;
+// fp16 pair of 8 scaled values, packed for two 16-byte stores
+__device__ __forceinline__ void split8(const float (&x)[8], float s, uint4& hi, uint4& lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float a = x[2 * i] * s, b = x[2 * i + 1] * s;
+    const __half2 hh = __floats2half2_rn(a, b);
+    const float2 back = __half22float2(hh);
+    const __half2 ll = __floats2half2_rn(a - back.x, b - back.y);
+    h[i] = *reinterpret_cast<const uint32_t*>(&hh);
+    l[i] = *reinterpret_cast<const uint32_t*>(&ll);
+  }
+  hi = make_uint4(h[0], h[1], h[2], h[3]);
+  lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+__device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint4 neg8(uint4 v) {
+  return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+}
+
+// A (M x K, lda), K <= 256 in nslab = ceil(K / 16) slabs: out[(rt * nslab + s) * 16 KB + p * 4 KB +
+// part_off(r, k)], parts Re_h, Re_l, Im_h, Im_l; zero outside M x K; inv[row] the inverse scales.  A warp per
+// 8 rows: lane (row, group) takes every fourth group of 8 values of k, first for the row's largest
+// value, then (from the cache) for the split; 8 rows' 16-byte stores are 128 contiguous bytes.
+__global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nslab, const float2* __restrict__ A,
+                                                      int64_t lda, unsigned char* __restrict__ out,
+                                                      float* __restrict__ inv, int64_t rows_pad) {
+  const int lane = threadIdx.x & 31;
+  const int64_t row = (int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5)) * 8 + (lane & 7);
+  if (row >= rows_pad) return;  // (rows_pad is a multiple of 128: whole warps)
+  const float2* a = A + row * lda;
+  const bool ok = row < M;
+  unsigned mb = 0;
+  for (int g = lane >> 3; g < 2 * nslab; g += 4) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * g + i;
+      const float2 v = ok && k < K ? a[k] : make_float2(0.f, 0.f);
+      mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
+    }
+  }
+  mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, 8));
+  mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, 16));
+  float is;
+  const float s = split_scale(mb, is);
+  if (lane < 8) inv[row] = is;
+  unsigned char* base = out + (row / U_TM) * nslab * int64_t(U_ABYTES);
+  for (int g = lane >> 3; g < 2 * nslab; g += 4) {
+    float re[8], im[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * g + i;
+      const float2 v = ok && k < K ? a[k] : make_float2(0.f, 0.f);
+      re[i] = v.x;
+      im[i] = v.y;
+    }
+    uint4 rh, rl, ih, il;
+    split8(re, s, rh, rl);
+    split8(im, s, ih, il);
+    unsigned char* o = base + (g >> 1) * int64_t(U_ABYTES) + part_off(int(row % U_TM), (g & 1) * 8);
+    *reinterpret_cast<uint4*>(o) = rh;
+    *reinterpret_cast<uint4*>(o + U_PART) = rl;
+    *reinterpret_cast<uint4*>(o + 2 * U_PART) = ih;
+    *reinterpret_cast<uint4*>(o + 3 * U_PART) = il;
+  }
+}
+// B (K x N, ldb), K <= 256: out[(ct * nslab + s) * 24 KB + p * 4 KB + part_off(c, k)], parts
+// Br_h, Bi_h, -Br_h, Br_l, Bi_l, -Br_l; zero outside K x N; inv[col] the inverse scales.  A CTA per
+// 32 columns, lanes along the columns (coalesced), the warps sharing the groups of 8 values of k, first for the
+// columns' largest values, then for the split.
+__global__ void __launch_bounds__(256) split_b_kernel(int64_t N, int K, int nslab, const float2* __restrict__ B,
+                                                      int64_t ldb, unsigned char* __restrict__ out,
+                                                      float* __restrict__ inv) {
+  __shared__ unsigned s_mb[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t col = int64_t(blockIdx.x) * 32 + lane;
+  const bool ok = col < N;
+  unsigned mb = 0;
+  for (int g = warp; g < 2 * nslab; g += 8) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * g + i;
+      const float2 v = ok && k < K ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
+      mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
+    }
+  }
+  s_mb[warp][lane] = mb;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) mb = max(mb, s_mb[w][lane]);
+  float is;
+  const float s = split_scale(mb, is);
+  if (warp == 0) inv[col] = is;
+  unsigned char* base = out + (col / U_TN) * nslab * int64_t(U_BBYTES);
+  for (int g = warp; g < 2 * nslab; g += 8) {
+    float re[8], im[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * g + i;
+      const float2 v = ok && k < K ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
+      re[i] = v.x;
+      im[i] = v.y;
+    }
+    uint4 rh, rl, ih, il;
+    split8(re, s, rh, rl);
+    split8(im, s, ih, il);
+    unsigned char* o = base + (g >> 1) * int64_t(U_BBYTES) + part_off(int(col % U_TN), (g & 1) * 8);
+    *reinterpret_cast<uint4*>(o) = rh;
+    *reinterpret_cast<uint4*>(o + U_PART) = ih;
+    *reinterpret_cast<uint4*>(o + 2 * U_PART) = neg8(rh);
+    *reinterpret_cast<uint4*>(o + 3 * U_PART) = rl;
+    *reinterpret_cast<uint4*>(o + 4 * U_PART) = il;
+    *reinterpret_cast<uint4*>(o + 5 * U_PART) = neg8(rl);
+  }
 }
 
 // tile index -> (row tile, column tile): super-rows of U_GROUP row tiles, columns inside
@@ -181,7 +274,8 @@ __device__ __forceinline__ void tile_rc(int64_t tile, int64_t RT, int64_t CT, in
 // ---------------------------------------------------------------- the update
 __global__ void __launch_bounds__(U_THREADS, 1)
     cgemm_update_split_kernel(int64_t M, int64_t N, int nslab, const unsigned char* __restrict__ As,
-                              const unsigned char* __restrict__ Bs, float2* __restrict__ C, int64_t ldc, int* status,
+                              const unsigned char* __restrict__ Bs, const float* __restrict__ inv_a,
+                              const float* __restrict__ inv_b, float2* __restrict__ C, int64_t ldc, int* status,
                               int vec_ok) {
   extern __shared__ unsigned char u_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(u_raw) + 1023) & ~uintptr_t(1023));
@@ -190,6 +284,7 @@ __global__ void __launch_bounds__(U_THREADS, 1)
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
   __shared__ volatile int epi_stop;
+  __shared__ float s_inv_b[U_TN];  // the tile's column scales
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t RT = (M + U_TM - 1) / U_TM, CT = (N + U_TN - 1) / U_TN, tiles = RT * CT;
   if (warp == 0) {
@@ -307,6 +402,8 @@ __global__ void __launch_bounds__(U_THREADS, 1)
       tile_rc(tile, RT, CT, rt, ct);
       const int64_t row0 = rt * U_TM, col0 = ct * U_TN;
       const uint32_t d = tmem + uint32_t(b) * 256 + (uint32_t(lane_base) << 16);
+      const float sa = -inv_a[row0 + r_local];
+      s_inv_b[et] = inv_b[col0 + et];  // read after the barrier below; the last tile's reads are behind one
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         if (vec_ok) {
@@ -347,10 +444,12 @@ __global__ void __launch_bounds__(U_THREADS, 1)
           for (int j = 0; j < 32; j += 2) {
             float4* p = reinterpret_cast<float4*>(&sE[u_piece(r_local, cs * 16 + (j >> 1))]);
             float4 c4 = vec_ok ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
-            c4.x -= __uint_as_float(vr[j]);
-            c4.y -= __uint_as_float(vi[j]);
-            c4.z -= __uint_as_float(vr[j + 1]);
-            c4.w -= __uint_as_float(vi[j + 1]);
+            // (acc 2^-ea) 2^-eb: two exact scalings, so neither product of scales can overflow
+            const float s0 = s_inv_b[h * 64 + cs * 32 + j], s1 = s_inv_b[h * 64 + cs * 32 + j + 1];
+            c4.x = fmaf(__uint_as_float(vr[j]) * sa, s0, c4.x);
+            c4.y = fmaf(__uint_as_float(vi[j]) * sa, s0, c4.y);
+            c4.z = fmaf(__uint_as_float(vr[j + 1]) * sa, s1, c4.z);
+            c4.w = fmaf(__uint_as_float(vi[j + 1]) * sa, s1, c4.w);
             *p = c4;
           }
         }
@@ -399,8 +498,13 @@ inline unsigned ucdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); 
 
 }  // namespace
 
-size_t update_split_a_bytes(int64_t M) { return size_t((M + U_TM - 1) / U_TM) * U_SLABS * U_ABYTES; }
-size_t update_split_b_bytes(int64_t N) { return size_t((N + U_TN - 1) / U_TN) * U_SLABS * U_BBYTES; }
+// the image, then one scale per padded row or column
+size_t update_split_a_bytes(int64_t M) {
+  return size_t((M + U_TM - 1) / U_TM) * (size_t(U_SLABS) * U_ABYTES + U_TM * sizeof(float));
+}
+size_t update_split_b_bytes(int64_t N) {
+  return size_t((N + U_TN - 1) / U_TN) * (size_t(U_SLABS) * U_BBYTES + U_TN * sizeof(float));
+}
 
 // C (M x N) -= A (M x K) B (K x N), complex64 row-major, K <= kLuBlock: split A and B once into
 // the workspaces (update_split_a_bytes(M), update_split_b_bytes(N) bytes, 16-byte aligned),
@@ -425,16 +529,18 @@ cudaError_t cgemm_update_tc_split(int64_t M, int64_t N, int64_t K, const void* A
   const int64_t RT = (M + U_TM - 1) / U_TM, CT = (N + U_TN - 1) / U_TN;
   const int64_t rows_pad = RT * U_TM, cols_pad = CT * U_TN;
   ProfScope prof("lu_update", s, 8.0 * double(M) * double(N) * double(K));  // the splits are part of it
-  const int nslab = int((K + 7) / 8);  // tiles packed with exactly nslab slabs each
-  split_a_kernel<<<ucdiv(rows_pad * nslab * 8, 256), 256, 0, s>>>(M, int(K), nslab, static_cast<const float2*>(A), lda,
-                                                                static_cast<float*>(ws_a), rows_pad);
-  split_b_kernel<<<ucdiv(cols_pad * nslab * 8, 256), 256, 0, s>>>(N, int(K), nslab, static_cast<const float2*>(B), ldb,
-                                                                static_cast<float*>(ws_b), cols_pad);
+  const int nslab = int((K + U_KS - 1) / U_KS);  // tiles packed with exactly nslab slabs each
+  unsigned char* img_a = static_cast<unsigned char*>(ws_a);
+  unsigned char* img_b = static_cast<unsigned char*>(ws_b);
+  float* inv_a = reinterpret_cast<float*>(img_a + RT * nslab * int64_t(U_ABYTES));
+  float* inv_b = reinterpret_cast<float*>(img_b + CT * nslab * int64_t(U_BBYTES));
+  split_a_kernel<<<ucdiv(rows_pad, 64), 256, 0, s>>>(M, int(K), nslab, static_cast<const float2*>(A), lda, img_a, inv_a,
+                                                     rows_pad);
+  split_b_kernel<<<ucdiv(cols_pad, 32), 256, 0, s>>>(N, int(K), nslab, static_cast<const float2*>(B), ldb, img_b, inv_b);
   note_launches(2);
   const unsigned grid = unsigned(std::min<int64_t>(RT * CT, std::max(nsm[dev], 1)));
   const int vec_ok = (reinterpret_cast<uintptr_t>(C) % 16 == 0) && (ldc % 2 == 0);
-  cgemm_update_split_kernel<<<grid, U_THREADS, U_SMEM, s>>>(M, N, nslab, static_cast<const unsigned char*>(ws_a),
-                                                          static_cast<const unsigned char*>(ws_b),
+  cgemm_update_split_kernel<<<grid, U_THREADS, U_SMEM, s>>>(M, N, nslab, img_a, img_b, inv_a, inv_b,
                                                           static_cast<float2*>(C), ldc, status, vec_ok);
   return launched();
 }
