@@ -5,7 +5,7 @@
 //     (<= 8 right-hand sides), which streams A once at HBM speed (IR residuals).
 //   * getrf: blocked right-looking LU.  complex64 factors: 256-column blocks, each factored
 //     as four 64-column tournament-pivoting panels (tslu.cu) with K = 64 updates between
-//     them (tc_gemm.cu), then one tcgen05 3xTF32 trailing update with K = 256 (tc_update.cu,
+//     them (tc_gemm.cu), then one tcgen05 fp16-pair trailing update with K = 256 (tc_update.cu,
 //     operands split once per block).  complex128 factors: 64-column panels by a
 //     cooperative partial-pivoting kernel whose CTAs own row chunks and meet at a software
 //     grid barrier once per column (bounded spin: on time-out the status word is set and
@@ -1461,12 +1461,14 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
   if (e != cudaSuccess) return e;
   gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, nrhs);
   if (sizeof(T) == 4 && status && dinv && nrhs <= kTrsvStreamMaxRhs) {
-    // one persistent streaming kernel per sweep
-    int* flags = nullptr;
-    e = cudaMallocAsync(reinterpret_cast<void**>(&flags), sizeof(int) * trsv_stream_scratch_ints(n, nrhs), s);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, nrhs, 0, flags, status, s);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, nrhs, 1, flags, status, s);
-    if (flags) cudaFreeAsync(flags, s);
+    // one persistent streaming kernel per sweep, tmp -> y -> tmp; the ticket lies behind y
+    char* y = nullptr;
+    const size_t ybytes = sizeof(V) * size_t(n) * size_t(nrhs);
+    e = cudaMallocAsync(reinterpret_cast<void**>(&y), ybytes + 16, s);
+    int* ticket = reinterpret_cast<int*>(y + ybytes);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, 0, ticket, status, s);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, 1, ticket, status, s);
+    if (y) cudaFreeAsync(y, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(tmp, s);
       return e;

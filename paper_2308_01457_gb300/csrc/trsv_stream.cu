@@ -5,13 +5,18 @@
 // is latency-bound (2 x n/64 dependent launches per sweep).  Here one persistent kernel
 // does a whole sweep.  The right-hand sides are cut into chunks of at most 16 columns (one
 // chunk of the exact width for 1-8); CTAs take (block, chunk) tasks in block-major order
-// from a ticket counter.  The CTA of task (i, c) accumulates L_ij y_j (U_ij x_j for the
-// backward sweep) over the blocks j that precede i in the sweep as chunk c of each one is
-// published, then solves its diagonal block (a 64 x 64 product with its precomputed
-// inverse) and publishes chunk c of y_i through flags[i * chunks + c].  A task only waits
-// for tasks that were taken earlier, by CTAs that are running or done, so the waits always
-// end; each is bounded anyway and a time-out sets the status word, which every waiter
-// polls, so the sweep ends quickly and the host reports FOSB_ERR_TIMEOUT.
+// from a ticket counter.  With D_i the inverse of the diagonal block and j the blocks that
+// precede i in the sweep, the last of them h,
+//     y_i = D_i (x_i - sum_{j != h} L_ij y_j) - E_i y_h,   E_i = D_i L_ih  (E_i formed once per factorisation),
+// so between y_h and y_i there is one 64 x 64 product and not two; everything else of a task
+// is done while y_h is still on its way.  The solution carries its own readiness: the output
+// is filled with a bit pattern that no arithmetic result has (both words all ones, a NaN
+// that the hardware never returns) and a waiting thread polls the very values it needs with
+// 8-byte loads, so a block costs one store and one load of latency instead of a fence, a flag
+// and a second read.  A task only waits for tasks that were taken earlier, by CTAs that are
+// running or done, so the waits always end; each is bounded anyway and a time-out sets the
+// status word, which every waiter polls, so the sweep ends quickly and the host reports
+// FOSB_ERR_TIMEOUT.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,7 +29,7 @@ namespace {
 
 constexpr int kTB = 64;                         // rows per block
 constexpr long long kFlagSpinLimit = 1ll << 26;
-// Poll limit of the flag waits on this device (kFlagSpinLimit unless changed by
+// Poll limit of the waits on this device (kFlagSpinLimit unless changed by
 // fosb_debug_set_wait_limit).
 __device__ long long g_flag_wait_limit = kFlagSpinLimit;
 
@@ -103,54 +108,153 @@ __global__ void __launch_bounds__(256) tri_block_inverse_kernel(const float2* __
   }
 }
 
-// Shared tiles of the streaming sweep.  A factor tile (and, after the panel product, the
-// inverse of the diagonal block) is 64 x 64 with a row pitch of 72 complex values; the
-// published block of the solution is 64 x NR with an odd pitch NRP.  Thread (g, q) of 256
-// owns rows g and g + 32 and the columns q, q + 8, ..., q + 56, so in one step of c the 16
-// threads of a half-warp read 8 consecutive complex values of two rows 72 apart (every bank
-// once) and 8 values of the solution block 2 NRP words apart (distinct banks, NRP odd).
+// E_i = D_i L_ih (which = 0: h = i - 1; which = 1, U: h = i + 1), one CTA per block; zero where
+// there is no such neighbour.
+__global__ void __launch_bounds__(256) tri_neighbour_kernel(const float2* __restrict__ LU, int64_t n, int64_t ld,
+                                                            int which, const float2* __restrict__ Dinv,
+                                                            float2* __restrict__ E) {
+  extern __shared__ float4 nb_raw[];
+  auto sD = reinterpret_cast<float2 (*)[kTB + 1]>(nb_raw);  // D, then the tile
+  auto sT = sD + kTB;
+  const int64_t ib = blockIdx.x, nblk = (n + kTB - 1) / kTB, hb = which ? ib + 1 : ib - 1;
+  const int64_t r0 = ib * kTB, c0 = hb * kTB;
+  const bool any = hb >= 0 && hb < nblk;
+  for (int e = threadIdx.x; e < kTB * kTB; e += blockDim.x) {
+    const int r = e / kTB, c = e % kTB;
+    sD[r][c] = Dinv[ib * kTB * kTB + e];
+    sT[r][c] = any && r0 + r < n && c0 + c < n ? LU[(r0 + r) * ld + c0 + c] : make_float2(0.f, 0.f);
+  }
+  __syncthreads();
+  const int r = threadIdx.x >> 2, cq = threadIdx.x & 3;  // row r, columns cq, cq + 4, ...
+  float2 acc[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) acc[c] = make_float2(0.f, 0.f);
+  for (int k = 0; k < kTB; ++k) {
+    const float2 d = sD[r][k];
+#pragma unroll
+    for (int c = 0; c < 16; ++c) cfma(acc[c], d, sT[k][cq + 4 * c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 16; ++c) E[(ib * kTB + r) * kTB + cq + 4 * c] = acc[c];
+}
+
+// Shared tiles of the streaming sweep.  A factor tile (later the inverse of the diagonal block)
+// and the neighbour product E are 64 x 64 with a row pitch of 72 complex values; the published
+// blocks of the solution are 64 x NR with a pitch that is odd for odd NR and else keeps 16-byte
+// rows in distinct banks.  Thread (g, q) of 256 owns rows g and g + 32 and the columns q, q + 8,
+// ..., q + 56, so in one step of c the 16 threads of a half-warp read 8 consecutive complex
+// values of two rows 72 apart (every bank once) and 8 rows of the solution block (distinct banks).
 constexpr int kLP = 72;
 template <int NR>
 struct StreamSmem {
-  static constexpr int NRP = NR | 1;
+  static constexpr int NRP = NR & 1 ? NR : (NR == 2 || NR == 6 ? NR : NR + 2);
   float2 L[kTB][kLP];
-  float2 Y[kTB][NRP];
+  float2 E[kTB][kLP];
+  float2 Y[2][kTB][NRP];  // the current block of the solution; minus the neighbour's
 };
 
 // acc0/acc1 (rows g, g + 32) += T[rows][cols] Y[cols][0..NR) over this thread's 8 columns
 template <int NR>
-__device__ __forceinline__ void stream_tile_product(const StreamSmem<NR>& sm, int g, int q, float2 (&acc0)[NR],
-                                                    float2 (&acc1)[NR]) {
+__device__ __forceinline__ void stream_tile_product(const float2 (*T)[kLP], const float2 (*Y)[StreamSmem<NR>::NRP],
+                                                    int g, int q, float2 (&acc0)[NR], float2 (&acc1)[NR]) {
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int cc = q + 8 * c;
-    const float2 l0 = sm.L[g][cc], l1 = sm.L[g + 32][cc];
+    const float2 l0 = T[g][cc], l1 = T[g + 32][cc];
+    if constexpr (NR % 2 == 0) {
 #pragma unroll
-    for (int k = 0; k < NR; ++k) {
-      const float2 y = sm.Y[cc][k];
-      cfma(acc0[k], l0, y);
-      cfma(acc1[k], l1, y);
+      for (int k = 0; k < NR; k += 2) {
+        const float4 y = *reinterpret_cast<const float4*>(&Y[cc][k]);
+        const float2 ya = make_float2(y.x, y.y), yb = make_float2(y.z, y.w);
+        cfma(acc0[k], l0, ya);
+        cfma(acc1[k], l1, ya);
+        cfma(acc0[k + 1], l0, yb);
+        cfma(acc1[k + 1], l1, yb);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < NR; ++k) {
+        const float2 y = Y[cc][k];
+        cfma(acc0[k], l0, y);
+        cfma(acc1[k], l1, y);
+      }
     }
   }
 }
-// sum over the 8 column owners q (lanes differing in their low three bits)
+// Sum over the 8 column owners q (lanes differing in their low three bits), scattered: lane q is
+// left with row g + 32 (q & 1) and the right-hand sides from (q >> 1) NR/4 on (NR % 4 == 0; each
+// halving step sends one half and keeps the other), or with both rows in lane q = 0.
 template <int NR>
-__device__ __forceinline__ void stream_reduce_q(float2 (&a)[NR]) {
+struct StreamOut {
+  static constexpr bool kSplit = NR % 4 == 0;
+};
+template <int NR>
+__device__ __forceinline__ void stream_reduce(float2 (&a0)[NR], float2 (&a1)[NR], int q) {
+  auto add = [](float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); };
+  auto swap2 = [](float2 v, int off) {
+    return make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off));
+  };
+  if constexpr (StreamOut<NR>::kSplit) {
 #pragma unroll
-  for (int k = 0; k < NR; ++k) {
+    for (int k = 0; k < NR; ++k) {  // rows
+      const float2 keep = q & 1 ? a1[k] : a0[k], give = q & 1 ? a0[k] : a1[k];
+      a0[k] = add(keep, swap2(give, 1));
+    }
 #pragma unroll
-    for (int off = 1; off < 8; off <<= 1) {
-      a[k].x += __shfl_xor_sync(0xffffffffu, a[k].x, off);
-      a[k].y += __shfl_xor_sync(0xffffffffu, a[k].y, off);
+    for (int k = 0; k < NR / 2; ++k) {  // halves of the right-hand sides
+      const float2 keep = q & 4 ? a0[k + NR / 2] : a0[k], give = q & 4 ? a0[k] : a0[k + NR / 2];
+      a0[k] = add(keep, swap2(give, 4));
+    }
+#pragma unroll
+    for (int k = 0; k < NR / 4; ++k) {  // quarters
+      const float2 keep = q & 2 ? a0[k + NR / 4] : a0[k], give = q & 2 ? a0[k] : a0[k + NR / 4];
+      a0[k] = add(keep, swap2(give, 2));
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < NR; ++k)
+#pragma unroll
+      for (int off = 1; off < 8; off <<= 1) {
+        a0[k] = add(a0[k], swap2(a0[k], off));
+        a1[k] = add(a1[k], swap2(a1[k], off));
+      }
+  }
+}
+// visits the (row, right-hand side, value) that this lane is left with
+template <int NR, class Fn>
+__device__ __forceinline__ void stream_each(const float2 (&a0)[NR], const float2 (&a1)[NR], int g, int q, Fn fn) {
+  if constexpr (StreamOut<NR>::kSplit) {
+#pragma unroll
+    for (int k = 0; k < NR / 4; ++k) fn(g + 32 * (q & 1), (q >> 1) * (NR / 4) + k, a0[k]);
+  } else if (q == 0) {
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      fn(g, k, a0[k]);
+      fn(g + 32, k, a1[k]);
     }
   }
 }
 
+constexpr unsigned long long kNotReady = ~0ull;
+__device__ __forceinline__ unsigned long long ld_relaxed(const float2* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(float2* p, float2 v) {
+  const unsigned long long b = (static_cast<unsigned long long>(__float_as_uint(v.y)) << 32) | __float_as_uint(v.x);
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(b) : "memory");
+}
+
+// x: the right-hand sides (n x nrhs dense), y: the solution, all ones (kNotReady) on entry.
+// Chain-bound: a block's latency is one store-to-load trip, a product and a reduction.
+// One sweep at N = 15360: 0.36 ms for 1 column, 1.4 for 16 (1.32 and 3.01 with a flag per block and
+// the diagonal solve behind the last product).
 template <int NR>
-__global__ void __launch_bounds__(256, 2) trsv_stream_kernel(const float2* __restrict__ LU, int64_t n, int64_t ld,
-                                                          const float2* __restrict__ Dinv, float2* X, int64_t ldx,
-                                                          int nrhs, int chunks, int upper, int* ticket, int* flags,
-                                                          int* status) {
+__global__ void __launch_bounds__(256, 2)
+    trsv_stream_kernel(const float2* __restrict__ LU, int64_t n, int64_t ld, const float2* __restrict__ Dinv,
+                       const float2* __restrict__ E, const float2* __restrict__ x, float2* y, int64_t nrhs, int chunks,
+                       int upper, int* ticket, int* status) {
   extern __shared__ float4 stream_raw[];
   StreamSmem<NR>& sm = *reinterpret_cast<StreamSmem<NR>*>(stream_raw);
   __shared__ long long s_task;
@@ -158,7 +262,10 @@ __global__ void __launch_bounds__(256, 2) trsv_stream_kernel(const float2* __res
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int g = t >> 3, q = t & 7;
   const int64_t nblk = (n + kTB - 1) / kTB;
+  constexpr int kPer = (kTB * NR + 255) / 256;  // values of a solution block per thread
+  const long long limit = g_flag_wait_limit;
   for (;;) {
+    __syncthreads();  // every thread is done with the last task
     if (t == 0) {
       s_task = atomicAdd(ticket, 1);
       s_abort = 0;
@@ -166,111 +273,128 @@ __global__ void __launch_bounds__(256, 2) trsv_stream_kernel(const float2* __res
     __syncthreads();
     const int64_t task = s_task;
     const int64_t b = task / chunks;
-    const int ch = int(task % chunks);
     if (b >= nblk) break;
     const int64_t ib = upper ? nblk - 1 - b : b;
     const int64_t r0 = ib * kTB;
     const int rows = int(std::min<int64_t>(kTB, n - r0));
-    const int k0 = ch * NR, nc = std::min(NR, nrhs - k0);  // this chunk's columns of X
+    const int64_t k0 = (task % chunks) * NR;
+    const int nc = int(std::min<int64_t>(NR, nrhs - k0));  // this chunk's columns
+    const int64_t far = b > 0 ? b - 1 : 0;                 // blocks before the neighbour
+    if (b > 0) {
+      const float2* e = E + ib * kTB * kTB;
+#pragma unroll
+      for (int i = 0; i < kTB * kTB / 512; ++i) {
+        const int p = t + 256 * i, r = p >> 5, c = (p & 31) * 2;  // 16-byte pieces
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                         static_cast<uint32_t>(__cvta_generic_to_shared(&sm.E[r][c]))),
+                     "l"(e + r * kTB + c)
+                     : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     float2 acc0[NR], acc1[NR];
 #pragma unroll
     for (int k = 0; k < NR; ++k) acc0[k] = acc1[k] = make_float2(0.f, 0.f);
-    const int64_t jcount = upper ? nblk - 1 - ib : ib;
-    // factor tile of block jj in registers: warp w holds rows 8w .. 8w+7, lanes the columns
-    // lane and lane + 32 (256 contiguous bytes of a row per load instruction)
+    // factor tile jj (the far blocks in publication order, then the inverse of the diagonal block)
+    // in registers: warp w holds rows 8w .. 8w+7, lanes the columns lane and lane + 32
     float2 lreg[16];
     auto fetch = [&](int64_t jj) {
-      const int64_t c0 = (upper ? nblk - 1 - jj : jj) * kTB;
-      const int cols = int(std::min<int64_t>(kTB, n - c0));
+      const bool diag = jj >= far;
+      const int64_t c0 = diag ? 0 : (upper ? nblk - 1 - jj : jj) * kTB;
+      const float2* base = diag ? Dinv + ib * kTB * kTB : LU + r0 * ld + c0;
+      const int64_t pitch = diag ? kTB : ld;
+      const int rr_n = diag ? kTB : rows, cols = diag ? kTB : int(std::min<int64_t>(kTB, n - c0));
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int rr = warp * 8 + i;
-        const float2* src = LU + (r0 + rr) * ld + c0;
-        lreg[2 * i] = (rr < rows && lane < cols) ? __ldg(src + lane) : make_float2(0.f, 0.f);
-        lreg[2 * i + 1] = (rr < rows && lane + 32 < cols) ? __ldg(src + lane + 32) : make_float2(0.f, 0.f);
+        const float2* src = base + rr * pitch;
+        lreg[2 * i] = (rr < rr_n && lane < cols) ? __ldg(src + lane) : make_float2(0.f, 0.f);
+        lreg[2 * i + 1] = (rr < rr_n && lane + 32 < cols) ? __ldg(src + lane + 32) : make_float2(0.f, 0.f);
       }
     };
-    if (jcount > 0) fetch(0);
-    for (int64_t jj = 0; jj < jcount; ++jj) {
-      const int64_t jb = upper ? nblk - 1 - jj : jj;  // in publication order
-      const int64_t c0 = jb * kTB;
-      const int cols = int(std::min<int64_t>(kTB, n - c0));
-      if (t == 0) {
-        const volatile int* f = flags + jb * chunks + ch;
-        long long spins = 0;
-        const long long limit = g_flag_wait_limit;
-        while (*f == 0) {
-          if (++spins > limit || *(volatile int*)status == FOSB_ERR_TIMEOUT) {
-            atomicExch(status, FOSB_ERR_TIMEOUT);
-            s_abort = 1;
-            break;
-          }
-          __nanosleep(32);
-        }
-        __threadfence();
-      }
-      __syncthreads();  // also: every thread is done with the tiles of the previous block
-      if (s_abort) break;
+    auto store_tile = [&]() {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         sm.L[warp * 8 + i][lane] = lreg[2 * i];
         sm.L[warp * 8 + i][lane + 32] = lreg[2 * i + 1];
       }
-      for (int e = t; e < kTB * NR; e += blockDim.x) {
-        const int rr = e / NR, k = e % NR;
-        sm.Y[rr][k] = (rr < cols && k < nc) ? __ldcg(X + (c0 + rr) * ldx + k0 + k) : make_float2(0.f, 0.f);
+    };
+    // waits for this thread's values of solution block jj (publication order)
+    float2 v[kPer];
+    auto poll = [&](int64_t jj) {
+      const int64_t c0 = (upper ? nblk - 1 - jj : jj) * kTB;
+      const int cols = int(std::min<int64_t>(kTB, n - c0));
+      long long spins = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int e = t + 256 * i, rr = e / NR, k = e % NR;
+        v[i] = make_float2(0.f, 0.f);
+        if (rr >= cols || k >= nc) continue;
+        const float2* p = y + (c0 + rr) * nrhs + k0 + k;
+        unsigned long long w = ld_relaxed(p);
+        while (w == kNotReady) {
+          if (++spins > limit || *(volatile int*)status == FOSB_ERR_TIMEOUT) {
+            atomicExch(status, FOSB_ERR_TIMEOUT);
+            s_abort = 1;
+            return;
+          }
+          w = ld_relaxed(p);
+        }
+        v[i] = make_float2(__uint_as_float(unsigned(w)), __uint_as_float(unsigned(w >> 32)));
       }
-      if (jj + 1 < jcount) fetch(jj + 1);  // in flight during the product below
+    };
+    auto store_y = [&](float2 (*Y)[StreamSmem<NR>::NRP], float sign) {
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int e = t + 256 * i;
+        if (e < kTB * NR) Y[e / NR][e % NR] = make_float2(sign * v[i].x, sign * v[i].y);
+      }
+    };
+    bool stop = false;
+    fetch(0);
+    for (int64_t jj = 0; jj < far; ++jj) {
+      poll(jj);
+      __syncthreads();  // every thread is done with the tiles of the previous block
+      stop = s_abort;   // (set before this barrier only, so all threads agree)
+      if (stop) break;
+      store_tile();
+      store_y(sm.Y[0], 1.f);
+      fetch(jj + 1);  // in flight during the product below
       __syncthreads();
-      stream_tile_product<NR>(sm, g, q, acc0, acc1);
+      stream_tile_product<NR>(sm.L, sm.Y[0], g, q, acc0, acc1);
     }
-    if (s_abort) {  // every later wait gives up at once; this task stays unpublished
-      __syncthreads();
+    if (stop) {  // every later wait gives up at once; this task stays unpublished
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
       continue;
     }
-    // right-hand side of the diagonal block: r = x - sum_j L_ij y_j
-    stream_reduce_q<NR>(acc0);
-    stream_reduce_q<NR>(acc1);
+    // right-hand side of the diagonal block: r = x - sum L_ij y_j, then D r
+    stream_reduce<NR>(acc0, acc1, q);
     __syncthreads();  // every thread is done with the last factor tile
-    if (q == 0) {
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        float2 v0 = make_float2(0.f, 0.f), v1 = v0;
-        if (k < nc) {
-          if (g < rows) {
-            const float2 x = X[(r0 + g) * ldx + k0 + k];
-            v0 = make_float2(x.x - acc0[k].x, x.y - acc0[k].y);
-          }
-          if (g + 32 < rows) {
-            const float2 x = X[(r0 + g + 32) * ldx + k0 + k];
-            v1 = make_float2(x.x - acc1[k].x, x.y - acc1[k].y);
-          }
-        }
-        sm.Y[g][k] = v0;
-        sm.Y[g + 32][k] = v1;
+    stream_each<NR>(acc0, acc1, g, q, [&](int row, int k, float2 a) {
+      float2 r = make_float2(0.f, 0.f);
+      if (row < rows && k < nc) {
+        const float2 xv = __ldg(x + (r0 + row) * nrhs + k0 + k);
+        r = make_float2(xv.x - a.x, xv.y - a.y);
       }
-    }
-    const float2* D = Dinv + ib * kTB * kTB;
-    for (int e = t; e < kTB * kTB; e += blockDim.x) sm.L[e / kTB][e % kTB] = D[e];
+      sm.Y[0][row][k] = r;
+    });
+    store_tile();
     __syncthreads();
-    // y = Dinv r, the same tile product
 #pragma unroll
     for (int k = 0; k < NR; ++k) acc0[k] = acc1[k] = make_float2(0.f, 0.f);
-    stream_tile_product<NR>(sm, g, q, acc0, acc1);
-    stream_reduce_q<NR>(acc0);
-    stream_reduce_q<NR>(acc1);
-    if (q == 0) {
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        if (k < nc) {
-          if (g < rows) X[(r0 + g) * ldx + k0 + k] = acc0[k];
-          if (g + 32 < rows) X[(r0 + g + 32) * ldx + k0 + k] = acc1[k];
-        }
-      }
+    stream_tile_product<NR>(sm.L, sm.Y[0], g, q, acc0, acc1);
+    if (b > 0) {  // - E_i y_h
+      poll(far);
+      store_y(sm.Y[1], -1.f);
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      if (s_abort) continue;
+      stream_tile_product<NR>(sm.E, sm.Y[1], g, q, acc0, acc1);
     }
-    __threadfence();
-    __syncthreads();
-    if (t == 0) atomicExch(flags + ib * chunks + ch, 1);  // publish chunk ch of block ib
+    stream_reduce<NR>(acc0, acc1, q);
+    stream_each<NR>(acc0, acc1, g, q, [&](int row, int k, float2 a) {
+      if (row < rows && k < nc) st_relaxed(y + (r0 + row) * nrhs + k0 + k, a);
+    });
   }
 }
 
@@ -279,28 +403,37 @@ __global__ void __launch_bounds__(256, 2) trsv_stream_kernel(const float2* __res
 // chunk width: the exact width for 1-8 right-hand sides, 16 above
 static int trsv_stream_width(int64_t nrhs) { return nrhs <= 8 ? int(nrhs) : 16; }
 
-size_t trsv_stream_scratch_ints(int64_t n, int64_t nrhs) {
-  const int64_t w = trsv_stream_width(std::max<int64_t>(nrhs, 1));
-  return size_t(((n + kTB - 1) / kTB) * ((nrhs + w - 1) / w) + 64);
-}
-
 cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* Dinv, cudaStream_t s) {
   const int64_t nblk = (n + kTB - 1) / kTB;
   if (nblk <= 0) return cudaSuccess;
+  constexpr size_t kSmem = size_t(2) * kTB * (kTB + 1) * sizeof(float2);
+  static bool attr[64] = {};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!attr[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(tri_neighbour_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
+    if (e != cudaSuccess) return e;
+    attr[dev] = true;
+  }
+  const float2* lu = static_cast<const float2*>(LU);
   float2* d = static_cast<float2*>(Dinv);
-  tri_block_inverse_kernel<<<unsigned(nblk), 256, 0, s>>>(static_cast<const float2*>(LU), n, ld, 0, d);
-  tri_block_inverse_kernel<<<unsigned(nblk), 256, 0, s>>>(static_cast<const float2*>(LU), n, ld, 1,
-                                                           d + nblk * kTB * kTB);
-  return launched(2);
+  const int64_t one = nblk * kTB * kTB;
+  for (int which = 0; which < 2; ++which) {
+    tri_block_inverse_kernel<<<unsigned(nblk), 256, 0, s>>>(lu, n, ld, which, d + which * one);
+    tri_neighbour_kernel<<<unsigned(nblk), 256, kSmem, s>>>(lu, n, ld, which, d + which * one, d + (2 + which) * one);
+  }
+  return launched(4);
 }
 
-size_t tri_block_inverses_bytes(int64_t n) { return size_t(2 * ((n + kTB - 1) / kTB)) * kTB * kTB * sizeof(float2); }
+size_t tri_block_inverses_bytes(int64_t n) { return size_t(4 * ((n + kTB - 1) / kTB)) * kTB * kTB * sizeof(float2); }
 
-cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* Dinv, void* X, int64_t nrhs, int upper,
-                            int* scratch, int* status, cudaStream_t s) {
+cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* Dinv, const void* X, void* Y,
+                            int64_t nrhs, int upper, int* ticket, int* status, cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
   if (nrhs > kTrsvStreamMaxRhs) return cudaErrorInvalidValue;
   static int nsm[64] = {};
+  static bool attr[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -308,31 +441,47 @@ cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* D
   const int64_t nblk = (n + kTB - 1) / kTB;
   const int w = trsv_stream_width(nrhs);
   const int chunks = int((nrhs + w - 1) / w);
-  int* ticket = scratch;
-  int* flags = scratch + 32;
-  cudaError_t e = cudaMemsetAsync(scratch, 0, sizeof(int) * (32 + nblk * chunks), s);
+  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(Y, 0xFF, sizeof(float2) * size_t(n) * size_t(nrhs), s);  // nothing ready
   if (e != cudaSuccess) return e;
   const unsigned grid = unsigned(std::min<int64_t>(nblk * chunks, int64_t(2) * std::max(nsm[dev], 1)));
   const float2* L = static_cast<const float2*>(LU);
-  const float2* D = static_cast<const float2*>(Dinv) + (upper ? nblk * kTB * kTB : 0);
-  float2* x = static_cast<float2*>(X);
-  const int nr = int(nrhs);
-#define FOSB_TS(NR)                                                                                      \
-  trsv_stream_kernel<NR><<<grid, 256, sizeof(StreamSmem<NR>), s>>>(L, n, ld, D, x, nrhs, nr, chunks, upper, ticket, \
-                                                                   flags, status)
-  switch (w) {
-    case 1: FOSB_TS(1); break;
-    case 2: FOSB_TS(2); break;
-    case 3: FOSB_TS(3); break;
-    case 4: FOSB_TS(4); break;
-    case 5: FOSB_TS(5); break;
-    case 6: FOSB_TS(6); break;
-    case 7: FOSB_TS(7); break;
-    case 8: FOSB_TS(8); break;
-    default: FOSB_TS(16); break;
+  const int64_t one = nblk * kTB * kTB;
+  const float2* D = static_cast<const float2*>(Dinv) + (upper ? one : 0);
+  const float2* E = static_cast<const float2*>(Dinv) + (upper ? 3 : 2) * one;
+  const float2* x = static_cast<const float2*>(X);
+  float2* y = static_cast<float2*>(Y);
+  auto run = [&](auto kern, size_t smem) -> cudaError_t {
+    kern<<<grid, 256, smem, s>>>(L, n, ld, D, E, x, y, nrhs, chunks, upper, ticket, status);
+    return launched();
+  };
+  if (!attr[dev]) {
+    auto opt = [&](auto kern, size_t smem) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    };
+    opt(trsv_stream_kernel<1>, sizeof(StreamSmem<1>));
+    opt(trsv_stream_kernel<2>, sizeof(StreamSmem<2>));
+    opt(trsv_stream_kernel<3>, sizeof(StreamSmem<3>));
+    opt(trsv_stream_kernel<4>, sizeof(StreamSmem<4>));
+    opt(trsv_stream_kernel<5>, sizeof(StreamSmem<5>));
+    opt(trsv_stream_kernel<6>, sizeof(StreamSmem<6>));
+    opt(trsv_stream_kernel<7>, sizeof(StreamSmem<7>));
+    opt(trsv_stream_kernel<8>, sizeof(StreamSmem<8>));
+    opt(trsv_stream_kernel<16>, sizeof(StreamSmem<16>));
+    if (e != cudaSuccess) return e;
+    attr[dev] = true;
   }
-#undef FOSB_TS
-  return launched();
+  switch (w) {
+    case 1: return run(trsv_stream_kernel<1>, sizeof(StreamSmem<1>));
+    case 2: return run(trsv_stream_kernel<2>, sizeof(StreamSmem<2>));
+    case 3: return run(trsv_stream_kernel<3>, sizeof(StreamSmem<3>));
+    case 4: return run(trsv_stream_kernel<4>, sizeof(StreamSmem<4>));
+    case 5: return run(trsv_stream_kernel<5>, sizeof(StreamSmem<5>));
+    case 6: return run(trsv_stream_kernel<6>, sizeof(StreamSmem<6>));
+    case 7: return run(trsv_stream_kernel<7>, sizeof(StreamSmem<7>));
+    case 8: return run(trsv_stream_kernel<8>, sizeof(StreamSmem<8>));
+    default: return run(trsv_stream_kernel<16>, sizeof(StreamSmem<16>));
+  }
 }
 
 // Sets the poll limit of the sweep flag waits on the current device (polls <= 0: the default).
