@@ -11,9 +11,8 @@
 //     grid barrier once per column (bounded spin: on time-out the status word is set and
 //     the kernel returns), then row swaps, the unit-lower solve of the block row and the
 //     trailing update (gemm).
-//   * getrs: complex64 factors with up to 1024 right-hand sides run one persistent
-//     streaming kernel per sweep (trsv_stream.cu); otherwise forward / backward
-//     substitution by diagonal-block solves plus gemm updates.
+//   * getrs: complex64 factors run persistent streaming kernels (trsv_stream.cu); complex128
+//     ones forward / backward substitution by diagonal-block solves plus gemm updates.
 //   * gemm_c128_ff: FP64-class complex128 products in float-float on the FP32 pipe.
 #include <cuda_runtime.h>
 
@@ -556,37 +555,6 @@ constexpr long long kSpinLimit = 1ll << 26;
 // Poll limit of the bounded grid-barrier waits on this device (kSpinLimit unless changed by
 // fosb_debug_set_wait_limit, which failure-detection tests use to make the waits give up).
 __device__ long long g_wait_limit = kSpinLimit;
-
-__device__ bool grid_barrier(unsigned* count, unsigned* gen, unsigned nblocks, int* status) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    volatile unsigned* vgen = gen;
-    unsigned my_gen = *vgen;
-    __threadfence();
-    unsigned arrived = atomicAdd(count, 1u);
-    if (arrived == nblocks - 1) {
-      *count = 0;
-      __threadfence();
-      atomicAdd(gen, 1u);
-    } else {
-      long long spins = 0;
-      const long long limit = g_wait_limit;
-      while (*vgen == my_gen) {
-        if (++spins > limit || *(volatile int*)status == FOSB_ERR_TIMEOUT) {
-          atomicExch(status, FOSB_ERR_TIMEOUT);
-          ok = 0;
-          break;
-        }
-        __nanosleep(20);
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return ok != 0;
-}
 
 // Grid barrier on a counter that only grows: every CTA adds one and waits until the count
 // reaches target (this launch's base + (column + 1) x CTAs), so no CTA has to reset it.
@@ -1457,27 +1425,31 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
   V* X = static_cast<V*>(Xv);
   V* tmp = nullptr;
   ProfScope prof("getrs", s, 8.0 * double(n) * double(n) * double(nrhs));
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(V) * n * nrhs, s);
+  // complex64 rows start on 16 bytes: the tensor-core updates then move two values at a time
+  // (163 columns at N = 7503, one sweep by superblocks 1.57 ms with rows of 163, 1.28 ms with rows of 164)
+  const int64_t ldt = sizeof(T) == 4 ? nrhs + (nrhs & 1) : nrhs;
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(V) * n * ldt, s);
   if (e != cudaSuccess) return e;
-  gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, nrhs);
-  if (sizeof(T) == 4 && status && dinv && nrhs <= kTrsvStreamMaxRhs) {
-    // one persistent streaming kernel per sweep, tmp -> y -> tmp; the ticket lies behind y
+  gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, ldt);
+  if constexpr (sizeof(T) == 4) {
+    // persistent streaming kernels, tmp -> y -> tmp; the tickets lie behind y
+    if (!status || !dinv) e = cudaErrorInvalidValue;
     char* y = nullptr;
-    const size_t ybytes = sizeof(V) * size_t(n) * size_t(nrhs);
-    e = cudaMallocAsync(reinterpret_cast<void**>(&y), ybytes + 16, s);
-    int* ticket = reinterpret_cast<int*>(y + ybytes);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, 0, ticket, status, s);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, 1, ticket, status, s);
+    const size_t ybytes = sizeof(V) * size_t(n) * size_t(ldt);
+    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&y), ybytes + 4 * trsv_stream_tickets(n) + 16, s);
+    int* tickets = reinterpret_cast<int*>(y + ybytes);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, ldt, 0, tickets, status, s);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, ldt, 1, tickets, status, s);
     if (y) cudaFreeAsync(y, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(tmp, s);
       return e;
     }
-    copy_kernel<V><<<cdiv(n * nrhs, 256), 256, 0, s>>>(tmp, n, nrhs, nrhs, X, ldx);
+    copy_kernel<V><<<cdiv(n * nrhs, 256), 256, 0, s>>>(tmp, n, nrhs, ldt, X, ldx);
     note_launches(2);  // gather + final copy
     cudaFreeAsync(tmp, s);
     return cudaGetLastError();
-  }
+  } else {
   const int nb = 64;
   enable_trsv_smem<T>();
   auto diag = [&](int64_t i0, int ib, int upper) {
@@ -1493,12 +1465,8 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
     diag(i0, ib, 0);
     int64_t rest = n - i0 - ib;
     if (rest > 0) {
-      if (sizeof(T) == 4 && status && nrhs >= 16)  // wide right-hand sides: tensor cores
-        e = cgemm_update_tc(rest, nrhs, ib, LU + (i0 + ib) * ldlu + i0, ldlu, tmp + i0 * nrhs, nrhs,
-                            tmp + (i0 + ib) * nrhs, nrhs, status, s, "trsm_update");
-      else
-        e = gemm<T>(OP_N, OP_N, rest, nrhs, ib, -1.0, 0.0, LU + (i0 + ib) * ldlu + i0, ldlu, tmp + i0 * nrhs, nrhs,
-                    1.0, tmp + (i0 + ib) * nrhs, nrhs, s);
+      e = gemm<T>(OP_N, OP_N, rest, nrhs, ib, -1.0, 0.0, LU + (i0 + ib) * ldlu + i0, ldlu, tmp + i0 * nrhs, nrhs, 1.0,
+                  tmp + (i0 + ib) * nrhs, nrhs, s);
       if (e != cudaSuccess) {
         cudaFreeAsync(tmp, s);
         return e;
@@ -1511,10 +1479,7 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
     int ib = int(i1 - i0);
     diag(i0, ib, 1);
     if (i0 > 0) {
-      if (sizeof(T) == 4 && status && nrhs >= 16)
-        e = cgemm_update_tc(i0, nrhs, ib, LU + i0, ldlu, tmp + i0 * nrhs, nrhs, tmp, nrhs, status, s, "trsm_update");
-      else
-        e = gemm<T>(OP_N, OP_N, i0, nrhs, ib, -1.0, 0.0, LU + i0, ldlu, tmp + i0 * nrhs, nrhs, 1.0, tmp, nrhs, s);
+      e = gemm<T>(OP_N, OP_N, i0, nrhs, ib, -1.0, 0.0, LU + i0, ldlu, tmp + i0 * nrhs, nrhs, 1.0, tmp, nrhs, s);
       if (e != cudaSuccess) {
         cudaFreeAsync(tmp, s);
         return e;
@@ -1524,6 +1489,7 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
   copy_kernel<V><<<cdiv(n * nrhs, 256), 256, 0, s>>>(tmp, n, nrhs, nrhs, X, ldx);
   cudaFreeAsync(tmp, s);
   return cudaGetLastError();
+  }
 }
 
 template cudaError_t getrs<double>(const void*, int64_t, int64_t, const int32_t*, void*, int64_t, int64_t, cudaStream_t,

@@ -13,7 +13,12 @@
 // is filled with a bit pattern that no arithmetic result has (both words all ones, a NaN
 // that the hardware never returns) and a waiting thread polls the very values it needs with
 // 8-byte loads, so a block costs one store and one load of latency instead of a fence, a flag
-// and a second read.  A task only waits for tasks that were taken earlier, by CTAs that are
+// and a second read.
+//
+// With many right-hand sides the tile products bound the sweep, not the chain: then the kernel
+// solves 512 rows at a time and the rows behind them are updated on the tensor cores
+// (cgemm_update_tc, K = 512) before the next 512.
+//  A task only waits for tasks that were taken earlier, by CTAs that are
 // running or done, so the waits always end; each is bounded anyway and a time-out sets the
 // status word, which every waiter polls, so the sweep ends quickly and the host reports
 // FOSB_ERR_TIMEOUT.
@@ -246,15 +251,17 @@ __device__ __forceinline__ void st_relaxed(float2* p, float2 v) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(b) : "memory");
 }
 
-// x: the right-hand sides (n x nrhs dense), y: the solution, all ones (kNotReady) on entry.
+// Blocks first .. first + count - 1 of the sweep (in its order) on their own: x are the right-hand
+// sides (n x nrhs, rows ldx apart) less everything that earlier blocks contribute, y the solution, all ones
+// (kNotReady) on entry.
 // Chain-bound: a block's latency is one store-to-load trip, a product and a reduction.
 // One sweep at N = 15360: 0.36 ms for 1 column, 1.4 for 16 (1.32 and 3.01 with a flag per block and
 // the diagonal solve behind the last product).
 template <int NR>
 __global__ void __launch_bounds__(256, 2)
     trsv_stream_kernel(const float2* __restrict__ LU, int64_t n, int64_t ld, const float2* __restrict__ Dinv,
-                       const float2* __restrict__ E, const float2* __restrict__ x, float2* y, int64_t nrhs, int chunks,
-                       int upper, int* ticket, int* status) {
+                       const float2* __restrict__ E, const float2* __restrict__ x, float2* y, int64_t nrhs, int64_t ldx, int64_t chunks,
+                       int64_t first, int64_t count, int upper, int* ticket, int* status) {
   extern __shared__ float4 stream_raw[];
   StreamSmem<NR>& sm = *reinterpret_cast<StreamSmem<NR>*>(stream_raw);
   __shared__ long long s_task;
@@ -273,8 +280,9 @@ __global__ void __launch_bounds__(256, 2)
     __syncthreads();
     const int64_t task = s_task;
     const int64_t b = task / chunks;
-    if (b >= nblk) break;
-    const int64_t ib = upper ? nblk - 1 - b : b;
+    if (b >= count) break;
+    auto block_at = [&](int64_t p) { return upper ? nblk - 1 - first - p : first + p; };
+    const int64_t ib = block_at(b);
     const int64_t r0 = ib * kTB;
     const int rows = int(std::min<int64_t>(kTB, n - r0));
     const int64_t k0 = (task % chunks) * NR;
@@ -300,7 +308,7 @@ __global__ void __launch_bounds__(256, 2)
     float2 lreg[16];
     auto fetch = [&](int64_t jj) {
       const bool diag = jj >= far;
-      const int64_t c0 = diag ? 0 : (upper ? nblk - 1 - jj : jj) * kTB;
+      const int64_t c0 = diag ? 0 : block_at(jj) * kTB;
       const float2* base = diag ? Dinv + ib * kTB * kTB : LU + r0 * ld + c0;
       const int64_t pitch = diag ? kTB : ld;
       const int rr_n = diag ? kTB : rows, cols = diag ? kTB : int(std::min<int64_t>(kTB, n - c0));
@@ -322,7 +330,7 @@ __global__ void __launch_bounds__(256, 2)
     // waits for this thread's values of solution block jj (publication order)
     float2 v[kPer];
     auto poll = [&](int64_t jj) {
-      const int64_t c0 = (upper ? nblk - 1 - jj : jj) * kTB;
+      const int64_t c0 = block_at(jj) * kTB;
       const int cols = int(std::min<int64_t>(kTB, n - c0));
       long long spins = 0;
 #pragma unroll
@@ -330,7 +338,7 @@ __global__ void __launch_bounds__(256, 2)
         const int e = t + 256 * i, rr = e / NR, k = e % NR;
         v[i] = make_float2(0.f, 0.f);
         if (rr >= cols || k >= nc) continue;
-        const float2* p = y + (c0 + rr) * nrhs + k0 + k;
+        const float2* p = y + (c0 + rr) * ldx + k0 + k;
         unsigned long long w = ld_relaxed(p);
         while (w == kNotReady) {
           if (++spins > limit || *(volatile int*)status == FOSB_ERR_TIMEOUT) {
@@ -373,7 +381,7 @@ __global__ void __launch_bounds__(256, 2)
     stream_each<NR>(acc0, acc1, g, q, [&](int row, int k, float2 a) {
       float2 r = make_float2(0.f, 0.f);
       if (row < rows && k < nc) {
-        const float2 xv = __ldg(x + (r0 + row) * nrhs + k0 + k);
+        const float2 xv = __ldg(x + (r0 + row) * ldx + k0 + k);
         r = make_float2(xv.x - a.x, xv.y - a.y);
       }
       sm.Y[0][row][k] = r;
@@ -393,15 +401,21 @@ __global__ void __launch_bounds__(256, 2)
     }
     stream_reduce<NR>(acc0, acc1, q);
     stream_each<NR>(acc0, acc1, g, q, [&](int row, int k, float2 a) {
-      if (row < rows && k < nc) st_relaxed(y + (r0 + row) * nrhs + k0 + k, a);
+      if (row < rows && k < nc) st_relaxed(y + (r0 + row) * ldx + k0 + k, a);
     });
   }
 }
 
 }  // namespace
 
-// chunk width: the exact width for 1-8 right-hand sides, 16 above
-static int trsv_stream_width(int64_t nrhs) { return nrhs <= 8 ? int(nrhs) : 16; }
+// Blocks per superblock, and when a sweep uses them: one kernel takes nblk^2/2 tile products per
+// 16-column chunk, about 3 us each over 152 SMs; a superblock takes 30 to 45 us for its own blocks
+// (8-column chunks) and 50 us per wave of update tiles, so sweeps with many right-hand sides change
+// over.  One kernel / superblocks, ms per sweep: 15360 x 80 (nblk ceil(nrhs / 16) = 1200) 3.05 / 2.53,
+// 7503 x 163 (1298) 1.57 / 1.28, 7503 x 642 4.77 / 1.95, 15360 x 642 20.0 / 5.74, 1920 x 1100 (2070)
+// 0.58 / 0.39; 7503 x 100 (826) takes 1.17 in one kernel.
+constexpr int64_t kSuper = 8;
+static bool use_superblocks(int64_t nblk, int64_t nrhs) { return nblk > kSuper && nblk * ((nrhs + 15) / 16) > 1100; }
 
 cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* Dinv, cudaStream_t s) {
   const int64_t nblk = (n + kTB - 1) / kTB;
@@ -428,33 +442,17 @@ cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* 
 
 size_t tri_block_inverses_bytes(int64_t n) { return size_t(4 * ((n + kTB - 1) / kTB)) * kTB * kTB * sizeof(float2); }
 
-cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* Dinv, const void* X, void* Y,
-                            int64_t nrhs, int upper, int* ticket, int* status, cudaStream_t s) {
+size_t trsv_stream_tickets(int64_t n) { return size_t(((n + kTB - 1) / kTB + kSuper - 1) / kSuper); }
+
+cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* Dinv, void* X, void* Y, int64_t nrhs,
+                            int64_t ldx, int upper, int* tickets, int* status, cudaStream_t s) {
   if (n <= 0 || nrhs <= 0) return cudaSuccess;
-  if (nrhs > kTrsvStreamMaxRhs) return cudaErrorInvalidValue;
   static int nsm[64] = {};
   static bool attr[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!nsm[dev]) cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
-  const int64_t nblk = (n + kTB - 1) / kTB;
-  const int w = trsv_stream_width(nrhs);
-  const int chunks = int((nrhs + w - 1) / w);
-  cudaError_t e = cudaMemsetAsync(ticket, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(Y, 0xFF, sizeof(float2) * size_t(n) * size_t(nrhs), s);  // nothing ready
-  if (e != cudaSuccess) return e;
-  const unsigned grid = unsigned(std::min<int64_t>(nblk * chunks, int64_t(2) * std::max(nsm[dev], 1)));
-  const float2* L = static_cast<const float2*>(LU);
-  const int64_t one = nblk * kTB * kTB;
-  const float2* D = static_cast<const float2*>(Dinv) + (upper ? one : 0);
-  const float2* E = static_cast<const float2*>(Dinv) + (upper ? 3 : 2) * one;
-  const float2* x = static_cast<const float2*>(X);
-  float2* y = static_cast<float2*>(Y);
-  auto run = [&](auto kern, size_t smem) -> cudaError_t {
-    kern<<<grid, 256, smem, s>>>(L, n, ld, D, E, x, y, nrhs, chunks, upper, ticket, status);
-    return launched();
-  };
+  cudaError_t e = cudaSuccess;
   if (!attr[dev]) {
     auto opt = [&](auto kern, size_t smem) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
@@ -468,20 +466,54 @@ cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* D
     opt(trsv_stream_kernel<7>, sizeof(StreamSmem<7>));
     opt(trsv_stream_kernel<8>, sizeof(StreamSmem<8>));
     opt(trsv_stream_kernel<16>, sizeof(StreamSmem<16>));
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
-  switch (w) {
-    case 1: return run(trsv_stream_kernel<1>, sizeof(StreamSmem<1>));
-    case 2: return run(trsv_stream_kernel<2>, sizeof(StreamSmem<2>));
-    case 3: return run(trsv_stream_kernel<3>, sizeof(StreamSmem<3>));
-    case 4: return run(trsv_stream_kernel<4>, sizeof(StreamSmem<4>));
-    case 5: return run(trsv_stream_kernel<5>, sizeof(StreamSmem<5>));
-    case 6: return run(trsv_stream_kernel<6>, sizeof(StreamSmem<6>));
-    case 7: return run(trsv_stream_kernel<7>, sizeof(StreamSmem<7>));
-    case 8: return run(trsv_stream_kernel<8>, sizeof(StreamSmem<8>));
-    default: return run(trsv_stream_kernel<16>, sizeof(StreamSmem<16>));
+  const int64_t nblk = (n + kTB - 1) / kTB, one = nblk * kTB * kTB;
+  const bool super = use_superblocks(nblk, nrhs);
+  // chunk width: the exact width for 1-8 right-hand sides, 16 above, 8 in superblocks (a shorter
+  // chain, and chunks enough to fill the chip)
+  const int w = nrhs <= 8 ? int(nrhs) : (super ? 8 : 16);
+  const int64_t chunks = (nrhs + w - 1) / w;
+  e = cudaMemsetAsync(tickets, 0, sizeof(int) * trsv_stream_tickets(n), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(Y, 0xFF, sizeof(float2) * size_t(n) * size_t(ldx), s);  // nothing ready
+  if (e != cudaSuccess) return e;
+  const float2* L = static_cast<const float2*>(LU);
+  const float2* D = static_cast<const float2*>(Dinv) + (upper ? one : 0);
+  const float2* E = static_cast<const float2*>(Dinv) + (upper ? 3 : 2) * one;
+  float2* x = static_cast<float2*>(X);
+  float2* y = static_cast<float2*>(Y);
+  const int64_t step = super ? kSuper : nblk;
+  for (int64_t first = 0, q = 0; first < nblk; first += step, ++q) {
+    const int64_t count = std::min(step, nblk - first);
+    const unsigned grid = unsigned(std::min<int64_t>(count * chunks, int64_t(2) * std::max(nsm[dev], 1)));
+    auto run = [&](auto kern, size_t smem) -> cudaError_t {
+      kern<<<grid, 256, smem, s>>>(L, n, ld, D, E, x, y, nrhs, ldx, chunks, first, count, upper, tickets + q, status);
+      return launched();
+    };
+    switch (w) {
+      case 1: e = run(trsv_stream_kernel<1>, sizeof(StreamSmem<1>)); break;
+      case 2: e = run(trsv_stream_kernel<2>, sizeof(StreamSmem<2>)); break;
+      case 3: e = run(trsv_stream_kernel<3>, sizeof(StreamSmem<3>)); break;
+      case 4: e = run(trsv_stream_kernel<4>, sizeof(StreamSmem<4>)); break;
+      case 5: e = run(trsv_stream_kernel<5>, sizeof(StreamSmem<5>)); break;
+      case 6: e = run(trsv_stream_kernel<6>, sizeof(StreamSmem<6>)); break;
+      case 7: e = run(trsv_stream_kernel<7>, sizeof(StreamSmem<7>)); break;
+      case 8: e = run(trsv_stream_kernel<8>, sizeof(StreamSmem<8>)); break;
+      default: e = run(trsv_stream_kernel<16>, sizeof(StreamSmem<16>)); break;
+    }
+    if (e != cudaSuccess) return e;
+    if (first + count == nblk) break;
+    // rows [lo, hi) are solved: take them out of the rows that follow in the sweep
+    const int64_t lo = upper ? (nblk - first - count) * kTB : first * kTB;
+    const int64_t hi = upper ? std::min(n, (nblk - first) * kTB) : (first + count) * kTB;
+    const int64_t r0 = upper ? 0 : hi, r1 = upper ? lo : n;
+    e = cgemm_update_tc(r1 - r0, nrhs, hi - lo, L + r0 * ld + lo, ld, y + lo * ldx, ldx, x + r0 * ldx, ldx, status, s,
+                        "trsm_update");
+    if (e != cudaSuccess) return e;
   }
+  return cudaSuccess;
 }
 
 // Sets the poll limit of the sweep flag waits on the current device (polls <= 0: the default).

@@ -54,3 +54,15 @@ def test_power_of_two_column_scaling_is_exact(F):
     F.solve(F.factor(Z), b, x)
     F.solve(F.factor(Z * d), b, y)
     assert torch.equal(x, y * d[:, None])
+
+
+@pytest.mark.parametrize("n,r", [(513, 2600), (1000, 1088), (1000, 1101), (5121, 209)])
+def test_superblocks(F, n, r):
+    """Both sides of the size where the sweeps go 512 rows at a time (1000 x 1088 is one kernel),
+    with one row in the last superblock and with odd numbers of columns."""
+    Z = _system(n, n)
+    rng = np.random.default_rng(n + 1)
+    B = torch.tensor(rng.standard_normal((n, r)) + 1j * rng.standard_normal((n, r)), dtype=torch.complex64, device="cuda")
+    X = torch.empty_like(B)
+    F.solve(F.factor(Z), B, X)
+    assert _backward_error(Z, X, B) <= (n + 4) * 2.0**-24
