@@ -223,13 +223,15 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
                          cudaStream_t s, const void* A_split = nullptr);
 // FP64-class complex GEMM on the bf16 tensor cores by exact digit splitting (oz_gemm.cu):
 // oz_prepare_a writes the digit tiles (oz_a_bytes(M, K) bytes) and row exponents (M ints)
-// of the complex128 A (M x K, lda); oz_gemm then computes C <- beta C + alpha A B for a
-// complex128 B (K x N, ldb); a bounded wait that gives up sets *status.
+// of the complex128 A (M x K, lda); oz_gemm then computes C <- beta C + alpha A B, alpha and
+// beta real, for a complex128 B (K x N, ldb) and leaves the exponents of B's columns in b_ex (N ints).  With ref_ex
+// B is a correction of a matrix with those column exponents, and digit orders below 2^-64 of that
+// matrix's are left out.  A bounded wait that gives up sets *status.
 size_t oz_a_bytes(int64_t M, int64_t K);
 cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s);
-cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha_re, double alpha_im, const void* a_digits,
-                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* status,
-                    cudaStream_t s);
+cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
+                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
+                    const int* ref_ex, int* status, cudaStream_t s);
 // dst (rows x cols float4, ldd) = (hi, lo) float split of the complex128 src
 cudaError_t split_ff(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                      cudaStream_t s);
@@ -277,7 +279,7 @@ cudaError_t convert_c64_to_c128(const void* src, int64_t rows, int64_t cols, int
 cudaError_t copy_matrix(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd, size_t elem,
                         cudaStream_t s);
 cudaError_t axpy_c64_into_c128(const void* d, int64_t rows, int64_t cols, int64_t ldd, void* x, int64_t ldx,
-                               cudaStream_t s);
+                               void* change, cudaStream_t s);
 // out = (accumulate ? out : 0) + w (M + op(M)) for a square n x n matrix M (op = OP_T or OP_C)
 cudaError_t add_mirrored(const void* M, int64_t n, int64_t ldm, int op, double w, bool accumulate, bool c64, void* out,
                          int64_t ldo, cudaStream_t s);

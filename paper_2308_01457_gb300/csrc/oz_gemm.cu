@@ -8,48 +8,56 @@
 // for every column j of X with tau_j and digits e_t.  Then
 //   (Z X)_ij = sigma_i tau_j 2^-14 sum_{s,t} 2^{-8(s+t)} sum_k d_s[i,k] e_t[k,j],
 // and a digit product is an integer of at most 2^14, so sums of the same order g = s+t over
-// 64 values of k are exact in the FP32 accumulators of the tensor cores
-// ((g+1) x 2 x 64 x 2^14 < 2^24 for g <= 6).  Orders g <= 6 (28 digit pairs) are kept:
-// the dropped terms are below 2^-56 of sigma_i tau_j per product.  After every 64 values
-// of k the seven order accumulators (Re, Im) are read out of TMEM: orders 0-3 are added
-// exactly into a 64-bit integer sum per output, orders 4-6 (below 2^-32 of them) into an
-// FP32 sum; the result is scaled by sigma_i tau_j 2^-14.
+// 128 values of k are exact in the FP32 accumulators of the tensor cores for g <= 3
+// ((g+1) x 2 x 128 x 2^14 <= 2^24).  Orders g <= 6 (28 digit pairs) are kept: the dropped
+// terms are below 2^-56 of sigma_i tau_j per product.  After every 128 values of k the seven
+// order accumulators are read out of TMEM: orders 0-3 are added exactly into a 64-bit integer
+// sum per output, orders 4-6 (below 2^-32 of them) into an FP32 sum; the result is scaled by
+// sigma_i tau_j 2^-14.
 //
-// Kernel roles (one CTA per SM, persistent over 128 x 32 output tiles): warp 0 lane 0 moves
-// the pre-tiled digit tiles of a 16-wide k step (14 A tiles of 4 KB, 14 B tiles of 1 KB)
-// into a 3-stage shared ring with bulk copies; warp 1 lane 0 issues 112 MMAs per step
-// (tcgen05.mma kind::f16, bf16, M = 128, N = 32, K = 16; the minus of Im Z Im X via the
-// negate-B bit; the MMAs that share an A tile and an instruction descriptor run back to
-// back and keep it in the A collector, so an A tile is read from shared memory once or
-// twice per step) into the 14 order
-// accumulators; warps 2-9 read the accumulators after every
-// 64 values of k and hold the sums (two warps per TMEM lane group, 16 columns each).  All
-// waits are bounded.
+// The tensor pipe: an MMA with M = 128, K = 16 takes 44 cycles for any N up to
+// 64 and 64 cycles at N = 128 (measured), so seven orders of N = 64 for one part (448 of the 512
+// TMEM columns) cost half of what Re and Im at N = 32 do: Re and Im are separate tiles that load
+// the same digits.  The collector and uniform MMA operands (oz_elect) bring them to 35 cycles.
+// Z X for N = 7503 and 163 columns: 4.63 ms with both parts at N = 32, sums after every 64 values
+// of k and the MMAs issued behind `lane == 0`, 2.24 ms so; the digits' way from L2 (86 KB per CTA
+// and step) now takes longer than the MMAs: orders up to 4 need 30 of the 56 MMAs and 5/7 of the
+// bytes and take 0.67 of the time.
+//
+// Kernel roles (one CTA per SM, persistent over 128 x 64 tiles of one part): warp 0 lane 0 moves
+// the pre-tiled digits of a 16-wide k step into two shared rings with bulk copies, one digit of Z
+// (8 KB) per slot of the first and all of X's (28 KB) per slot of the second, so that the loads
+// run two steps ahead; warp 1 lane 0 issues the 56 MMAs of a step (tcgen05.mma kind::f16, bf16,
+// M = 128, N = 64, K = 16; the minus of Im Z Im X via the negate-B bit; the MMAs of an A tile run
+// back to back and keep it in the A collector) into the order accumulators; warps 2-9 read the
+// accumulators after every 128 values of k and hold the sums (two warps per TMEM lane group, 32
+// columns each).  All waits are bounded.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "fosb_internal.h"
 
 namespace fosb {
 namespace {
 
-constexpr int OZ_TM = 128, OZ_TN = 32, OZ_KS = 16, OZ_ND = 7;  // tile rows, tile columns, k step, digits
-constexpr int OZ_KCH = 4;                                      // k steps per exact chunk (64 values)
+constexpr int OZ_TM = 128, OZ_TN = 64, OZ_KS = 16, OZ_ND = 7;  // tile rows, tile columns, k step, digits
+constexpr int OZ_KCH = 8;                                      // k steps per chunk (128 values)
 constexpr int OZ_ATILE = OZ_TM * OZ_KS * 2;                    // 4096 B
-constexpr int OZ_BTILE = OZ_TN * OZ_KS * 2;                    // 1024 B
+constexpr int OZ_BTILE = OZ_TN * OZ_KS * 2;                    // 2048 B
 constexpr int OZ_NT = OZ_ND * 2;                               // digit x part tiles per operand and step
-constexpr int OZ_STAGE = OZ_NT * (OZ_ATILE + OZ_BTILE);        // 71680 B
-constexpr int OZ_STAGES = 3;
-constexpr int OZ_SMEM = OZ_STAGES * OZ_STAGE + 1024;
+constexpr int OZ_ASLOT = 2 * OZ_ATILE, OZ_ASLOTS = 17;         // one digit of Z (Re, Im) per slot
+constexpr int OZ_BSLOT = OZ_NT * OZ_BTILE, OZ_BSLOTS = 3;      // all digits of X per slot
+constexpr int OZ_SMEM = OZ_ASLOTS * OZ_ASLOT + OZ_BSLOTS * OZ_BSLOT + 1024;
 constexpr int OZ_THREADS = 10 * 32;                            // producer, MMA, 8 flush warps
 constexpr int OZ_FLUSH = 8 * 32;
 constexpr int OZ_HN = OZ_TN / 2;                               // columns per flush thread
-constexpr int OZ_TMEM_COLS = 512;                              // 7 orders x (Re, Im) x 32 columns = 448 used
+constexpr int OZ_TMEM_COLS = 512;                              // 7 orders x 64 columns = 448 used
 constexpr long long kOzSpinLimit = 1ll << 24;
-static_assert(OZ_SMEM <= 227 * 1024, "digit stages do not fit shared memory");
+static_assert(OZ_SMEM <= 226 * 1024, "digit slots and the barriers do not fit shared memory");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -98,6 +106,13 @@ __device__ __forceinline__ void oz_mma(uint32_t tmem_d, uint64_t adesc, uint64_t
         " tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
 }
+// One lane of a converged warp.  The compiler knows that the branch on it has one thread and keeps
+// the MMA operands in uniform registers; behind `lane == 0` every MMA takes 44 cycles to issue.
+__device__ __forceinline__ bool oz_elect() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+  return p != 0;
+}
 __device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
   for (long long spins = 0; spins < kOzSpinLimit; ++spins) {
     uint32_t done;
@@ -133,6 +148,18 @@ __device__ __forceinline__ void oz_ld16(uint32_t taddr, uint32_t (&v)[16]) {
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
         "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
+}
+
+// waits for the loads above; the registers pass through, so that no use of them moves before it
+__device__ __forceinline__ void oz_wait_ld(uint32_t (&v)[16], uint32_t (&u)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+               :
+               : "memory");
+  if (&v != &u)
+    asm volatile("" : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]),
+                 "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15]));
 }
 
 // ---------------------------------------------------------------- digit splitting
@@ -264,28 +291,121 @@ __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int
 constexpr int OZ_SPLIT_WARPS = 8;  // a block covers 8 rows x 8 warps x 4 groups x 8 k = 8 x 256
 
 // ---------------------------------------------------------------- the product
+// The highest order kept in each tile of 64 columns: all of them (6) without ref.  With ref the
+// operand is a correction of a matrix whose columns have the exponents ref, and what matters is
+// the error against that matrix: dropping the orders above g leaves 2^{-8(g+1)} sigma tau per
+// product, which is at most 2^-60 sigma 2^ref (1/16 of what the product with the matrix itself
+// leaves) once 8 (g + 1) >= 60 - (ref - ex).  One warp per tile.
+__global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restrict__ ref, int64_t N,
+                                 int* __restrict__ orders) {
+  int g = ref ? 0 : OZ_ND - 1;
+  for (int q = threadIdx.x; ref && q < OZ_TN; q += 32) {
+    const int64_t c = int64_t(blockIdx.x) * OZ_TN + q;
+    if (c < N) g = max(g, min(OZ_ND - 1, (59 - min(59, max(0, ref[c] - ex[c]))) / 8));
+  }
+  g = __reduce_max_sync(0xffffffffu, g);
+  if (threadIdx.x == 0) orders[blockIdx.x] = g;
+}
+
+// The sums of one output: a = sum_g V_g 2^{24-8g} over the orders 0-3 (V_g the integer order
+// sums), exact; t the orders 4-6 (below 2^-32 of the leading terms) in FP32 in the same units, so
+// its rounding stays near 2^-50 of the result; the value is 2^-24 (a + t).
+__device__ __forceinline__ void oz_store(double* C, long long a, float t, int aex, int bex, double alpha, double beta) {
+  const double sc = ldexp(1.0, aex - 14) * ldexp(1.0, bex);
+  const double x = alpha * (ldexp(double(a) + double(t), -24) * sc);
+  *C = beta != 0.0 ? x + beta * *C : x;
+}
+// One output of a piece of a tile (below).
+struct OzPart {
+  long long a;
+  float t;
+};
+
+// A ring of shared-memory slots as its producer or consumer walks it.
+template <int SLOTS>
+struct OzRing {
+  uint32_t slot = 0, turn = 0;
+  __device__ __forceinline__ void next() {
+    if (++slot == SLOTS) {
+      slot = 0;
+      ++turn;
+    }
+  }
+};
+
+// One A tile with T digits of X (tiles 2 OZ_BTILE apart) into T consecutive orders, the A tile kept
+// in the collector; the MMAs of a group have one instruction descriptor.
+template <int T>
+__device__ __forceinline__ void oz_group(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const uint32_t dt = d + uint32_t(t) * OZ_TN;
+    const uint64_t bt = b + uint64_t(t) * (2 * OZ_BTILE >> 4);
+    if (T == 1) oz_mma_once(dt, a, bt, idesc, acc);
+    else if (t == 0) oz_mma<0>(dt, a, bt, idesc, acc);
+    else if (t == T - 1) oz_mma<2>(dt, a, bt, idesc, acc);
+    else oz_mma<1>(dt, a, bt, idesc, acc);
+  }
+}
+// The MMAs of one k step with the orders S .. G, digit by digit of Z as its slots fill; false where
+// a wait gave up.  `first`: the first product into an order's accumulator (s = 0) overwrites it.
+template <int S, int G>
+__device__ __forceinline__ bool oz_step(uint32_t tmem, uint32_t smem_a, uint64_t* a_full, uint64_t* a_empty,
+                                        OzRing<OZ_ASLOTS>& ra, uint64_t db, int im, bool first) {
+  if (!oz_wait(smem_u32(&a_full[ra.slot]), ra.turn & 1)) return false;
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint64_t da = oz_desc(smem_a + ra.slot * OZ_ASLOT);
+  const uint32_t d = tmem + uint32_t(S) * OZ_TN;
+  // Re: Re Z Re X - Im Z Im X, Im: Re Z Im X + Im Z Re X
+  oz_group<G + 1 - S>(d, da, db + uint64_t(im) * (OZ_BTILE >> 4), oz_idesc(false), first && S == 0 ? 0u : 1u);
+  oz_group<G + 1 - S>(d, da + (OZ_ATILE >> 4), db + uint64_t(1 - im) * (OZ_BTILE >> 4), im ? oz_idesc(false) : oz_idesc(true), 1u);
+  oz_commit(smem_u32(&a_empty[ra.slot]));
+  ra.next();
+  if constexpr (S < G) return oz_step<S + 1, G>(tmem, smem_a, a_full, a_empty, ra, db, im, first);
+  return true;
+}
+
+// The work: a tile is 128 rows x 64 columns of Re or of Im (tile index (row tile x CT + column
+// tile) x 2 + part); tiles 0 .. whole - 1 whole, then the last rem = tiles - whole of them, which would
+// leave most SMs without work, in `pieces` parts along k each, whose sums oz_reduce_kernel adds
+// (the integers exactly, the FP32 sums in the order of k).
+struct OzItem {
+  int64_t tile, c0, c1;  // chunks [c0, c1) of the tile
+  bool whole;
+};
+__device__ __forceinline__ OzItem oz_item(int64_t w, int64_t whole, int pieces, int64_t nch) {
+  if (w < whole) return {w, 0, nch, true};
+  const int64_t p = w - whole, q = p % pieces;
+  return {whole + p / pieces, nch * q / pieces, nch * (q + 1) / pieces, pieces == 1};
+}
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm_kernel(int64_t M, int64_t N, int64_t KC, const unsigned char* __restrict__ Ad,
                    const int* __restrict__ aex, const unsigned char* __restrict__ Bd, const int* __restrict__ bex,
-                   double alpha_re, double alpha_im, double beta, double2* __restrict__ C, int64_t ldc, int* status) {
+                   const int* __restrict__ orders, int64_t whole, int pieces, int64_t items, double alpha, double beta,
+                   double* __restrict__ C, int64_t ldc, OzPart* __restrict__ part, int* status) {
   extern __shared__ unsigned char oz_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t bar_full[OZ_STAGES], bar_empty[OZ_STAGES], bar_accf, bar_acce, bar_drain;
+  __shared__ uint64_t a_full[OZ_ASLOTS], a_empty[OZ_ASLOTS], b_full[OZ_BSLOTS], b_empty[OZ_BSLOTS];
+  __shared__ uint64_t bar_accf, bar_acce, bar_drain;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
   __shared__ volatile int fl_stop;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t RT = (M + OZ_TM - 1) / OZ_TM, CT = (N + OZ_TN - 1) / OZ_TN, tiles = RT * CT;
-  const int64_t nch = (KC + OZ_KCH - 1) / OZ_KCH;  // exact chunks per tile
+  const int64_t CT = (N + OZ_TN - 1) / OZ_TN;
+  const int64_t nch = (KC + OZ_KCH - 1) / OZ_KCH;  // chunks per tile
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
                  "r"(OZ_TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int i = 0; i < OZ_STAGES; ++i) {
-      oz_init(smem_u32(&bar_full[i]), 1);
-      oz_init(smem_u32(&bar_empty[i]), 1);
+    for (int i = 0; i < OZ_ASLOTS; ++i) {
+      oz_init(smem_u32(&a_full[i]), 1);
+      oz_init(smem_u32(&a_empty[i]), 1);
+    }
+    for (int i = 0; i < OZ_BSLOTS; ++i) {
+      oz_init(smem_u32(&b_full[i]), 1);
+      oz_init(smem_u32(&b_empty[i]), 1);
     }
     oz_init(smem_u32(&bar_accf), 1);
     oz_init(smem_u32(&bar_acce), OZ_FLUSH);
@@ -298,6 +418,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_sh;
+  const uint32_t smem_a = smem_u32(smem), smem_b = smem_a + OZ_ASLOTS * OZ_ASLOT;
   auto fail = [&]() {
     abort_sh = 1;
     atomicExch(status, FOSB_ERR_TIMEOUT);
@@ -306,37 +427,54 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   if (warp == 0) {
     // ---------------------------------------------------------- producer
     if (lane == 0) {
-      int64_t it = 0;
-      for (int64_t tile = blockIdx.x; tile < tiles && !abort_sh; tile += gridDim.x) {
-        const int64_t rt = tile / CT, ct = tile % CT;
-        for (int64_t kc = 0; kc < KC; ++kc, ++it) {
-          const int st = int(it % OZ_STAGES);
-          const int64_t use = it / OZ_STAGES;
-          if (use > 0 && !oz_wait(smem_u32(&bar_empty[st]), uint32_t((use - 1) & 1))) {
+      OzRing<OZ_ASLOTS> ra;
+      OzRing<OZ_BSLOTS> rb;
+      for (int64_t w = blockIdx.x; w < items && !abort_sh; w += gridDim.x) {
+        const OzItem item = oz_item(w, whole, pieces, nch);
+        const int64_t rt = item.tile / (2 * CT), ct = item.tile / 2 % CT;
+        const int G = orders[ct];
+        const int64_t k1 = std::min<int64_t>(KC, item.c1 * OZ_KCH);
+        for (int64_t kc = item.c0 * OZ_KCH; kc < k1 && !abort_sh; ++kc) {
+          // the digits up to the highest order are the first tiles of each operand's step
+          if (rb.turn > 0 && !oz_wait(smem_u32(&b_empty[rb.slot]), (rb.turn - 1) & 1)) {
             fail();
             break;
           }
-          unsigned char* sa = smem + st * OZ_STAGE;
-          unsigned char* sb = sa + OZ_NT * OZ_ATILE;
-          const uint32_t fb = smem_u32(&bar_full[st]);
-          oz_expect_tx(fb, OZ_STAGE);
+          const uint32_t bb = uint32_t(G + 1) * 2 * OZ_BTILE;
+          oz_expect_tx(smem_u32(&b_full[rb.slot]), bb);
+          oz_bulk_load(smem_b + rb.slot * OZ_BSLOT, Bd + (ct * KC + kc) * OZ_BSLOT, bb, smem_u32(&b_full[rb.slot]));
+          rb.next();
           const unsigned char* ga = Ad + ((rt * KC + kc) * OZ_NT) * OZ_ATILE;
-          const unsigned char* gb = Bd + ((ct * KC + kc) * OZ_NT) * OZ_BTILE;
-          for (int q = 0; q < OZ_NT; ++q) {
-            oz_bulk_load(smem_u32(sa + q * OZ_ATILE), ga + q * OZ_ATILE, OZ_ATILE, fb);
-            oz_bulk_load(smem_u32(sb + q * OZ_BTILE), gb + q * OZ_BTILE, OZ_BTILE, fb);
+          for (int s = 0; s <= G; ++s) {
+            if (ra.turn > 0 && !oz_wait(smem_u32(&a_empty[ra.slot]), (ra.turn - 1) & 1)) {
+              fail();
+              break;
+            }
+            oz_expect_tx(smem_u32(&a_full[ra.slot]), OZ_ASLOT);
+            oz_bulk_load(smem_a + ra.slot * OZ_ASLOT, ga + s * OZ_ASLOT, OZ_ASLOT, smem_u32(&a_full[ra.slot]));
+            ra.next();
           }
         }
       }
+      // no copy may land after the kernel has left (it can leave early where a wait gave up)
+      auto landed = [&](uint64_t* full, uint32_t slot, uint32_t turn, uint32_t i) {
+        const uint32_t loads = turn + (i < slot ? 1 : 0);
+        if (loads > 0) oz_wait(smem_u32(&full[i]), (loads - 1) & 1);
+      };
+      for (uint32_t i = 0; i < OZ_ASLOTS; ++i) landed(a_full, ra.slot, ra.turn, i);
+      for (uint32_t i = 0; i < OZ_BSLOTS; ++i) landed(b_full, rb.slot, rb.turn, i);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
-    if (lane == 0) {
-      const uint32_t id = oz_idesc(false), idn = oz_idesc(true);
-      int64_t it = 0, chunks = 0;
-      for (int64_t tile = blockIdx.x; tile < tiles && !abort_sh; tile += gridDim.x) {
-        for (int64_t c = 0; c < nch && !abort_sh; ++c, ++chunks) {
+    if (oz_elect()) {
+      OzRing<OZ_ASLOTS> ra;
+      OzRing<OZ_BSLOTS> rb;
+      int64_t chunks = 0;
+      for (int64_t w = blockIdx.x; w < items && !abort_sh; w += gridDim.x) {
+        const OzItem item = oz_item(w, whole, pieces, nch);
+        const int G = orders[item.tile / 2 % CT], im = int(item.tile & 1);
+        for (int64_t c = item.c0; c < item.c1 && !abort_sh; ++c, ++chunks) {
           // the order accumulators are free once the flush warps have read the last chunk
           if (chunks > 0 && !oz_wait(smem_u32(&bar_acce), uint32_t((chunks - 1) & 1))) {
             fail();
@@ -344,57 +482,31 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           }
           asm volatile("tcgen05.fence::after_thread_sync;");
           const int64_t k0 = c * OZ_KCH, k1 = std::min<int64_t>(KC, k0 + OZ_KCH);
-          for (int64_t kc = k0; kc < k1; ++kc, ++it) {
-            const int st = int(it % OZ_STAGES);
-            const int64_t use = it / OZ_STAGES;
-            if (!oz_wait(smem_u32(&bar_full[st]), uint32_t(use & 1))) {
+          for (int64_t kc = k0; kc < k1 && !abort_sh; ++kc) {
+            if (!oz_wait(smem_u32(&b_full[rb.slot]), rb.turn & 1)) {
               fail();
               break;
             }
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            // descriptors of the stage's first A and B tiles; a tile at byte offset X adds
-            // X >> 4 to the address field (shared addresses stay below 2^18, no carry)
-            const uint32_t a0 = smem_u32(smem + st * OZ_STAGE), b0 = a0 + OZ_NT * OZ_ATILE;
-            const uint64_t da = oz_desc(a0), db = oz_desc(b0);
-            // the first product into an order's accumulator in a chunk overwrites it
-            const uint32_t first = kc == k0 ? 0u : 1u;
-            // Each A tile meets its B digits t = 0 .. 6 - s in consecutive MMAs that keep it in
-            // the A collector, so it is read from shared memory once per group.  A group must
-            // keep one instruction descriptor, so digit s of Re Z is one group (Re and Im of
-            // every order), digit s of Im Z two: -Im Z Im X into Re (negate-B), Im Z Re X into Im.
-#pragma unroll
-            for (int s = 0; s < OZ_ND; ++s) {
-              const uint64_t ar = da + uint64_t((s * 2 + 0) * (OZ_ATILE >> 4));
-              const uint64_t ai = da + uint64_t((s * 2 + 1) * (OZ_ATILE >> 4));
-              const uint32_t acc = s == 0 ? first : 1u;  // s == 0 holds the first pair of each order
-              const int T = OZ_ND - s;  // B digits met by this A digit (a constant once unrolled)
-#pragma unroll
-              for (int t = 0; t < T; ++t) {
-                const int g = s + t;
-                const uint64_t br = db + uint64_t((t * 2 + 0) * (OZ_BTILE >> 4));
-                const uint64_t bi = db + uint64_t((t * 2 + 1) * (OZ_BTILE >> 4));
-                const uint32_t dre = tmem + uint32_t(g * 2 + 0) * OZ_TN, dim = tmem + uint32_t(g * 2 + 1) * OZ_TN;
-                if (t == 0) oz_mma<0>(dre, ar, br, id, acc);
-                else oz_mma<1>(dre, ar, br, id, acc);
-                if (t == T - 1) oz_mma<2>(dim, ar, bi, id, acc);
-                else oz_mma<1>(dim, ar, bi, id, acc);
-              }
-#pragma unroll
-              for (int half = 0; half < 2; ++half) {
-#pragma unroll
-                for (int t = 0; t < T; ++t) {
-                  const int g = s + t;
-                  const uint64_t b = db + uint64_t((t * 2 + (half == 0 ? 1 : 0)) * (OZ_BTILE >> 4));
-                  const uint32_t d = tmem + uint32_t(g * 2 + half) * OZ_TN;
-                  const uint32_t idd = half == 0 ? idn : id;
-                  if (T == 1) oz_mma_once(d, ai, b, idd, 1u);
-                  else if (t == 0) oz_mma<0>(d, ai, b, idd, 1u);
-                  else if (t == T - 1) oz_mma<2>(d, ai, b, idd, 1u);
-                  else oz_mma<1>(d, ai, b, idd, 1u);
-                }
-              }
+            const uint64_t db = oz_desc(smem_b + rb.slot * OZ_BSLOT);
+            auto step = [&](auto g) {
+              return oz_step<0, decltype(g)::value>(tmem, smem_a, a_full, a_empty, ra, db, im, kc == k0);
+            };
+            bool ok;
+            switch (G) {
+              case 0: ok = step(std::integral_constant<int, 0>()); break;
+              case 1: ok = step(std::integral_constant<int, 1>()); break;
+              case 2: ok = step(std::integral_constant<int, 2>()); break;
+              case 3: ok = step(std::integral_constant<int, 3>()); break;
+              case 4: ok = step(std::integral_constant<int, 4>()); break;
+              case 5: ok = step(std::integral_constant<int, 5>()); break;
+              default: ok = step(std::integral_constant<int, 6>()); break;
             }
-            oz_commit(smem_u32(&bar_empty[st]));
+            if (!ok) {
+              fail();
+              break;
+            }
+            oz_commit(smem_u32(&b_empty[rb.slot]));
+            rb.next();
           }
           if (abort_sh) break;
           oz_commit(smem_u32(&bar_accf));
@@ -410,20 +522,20 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int lane_base = (warp & 3) * 32;
     const int c0 = ((warp - 2) >> 2) * OZ_HN;
     const int r_local = lane_base + lane;
+    const uint32_t tbase = tmem + (uint32_t(lane_base) << 16) + uint32_t(c0);
     int64_t chunks = 0;
-    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-      const int64_t rt = tile / CT, ct = tile % CT;
-      // orders 0-3: exact integer sum a = sum_g V_g 2^{24-8g} (V_g the integer order sums);
-      // orders 4-6 (below 2^-32 of the leading terms): FP32 sum t in the same units, so its
-      // rounding stays near 2^-50 of the result; the value is 2^-24 (a + t)
-      long long ar_[OZ_HN], ai_[OZ_HN];
-      float tr[OZ_HN], ti[OZ_HN];
+    for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
+      const OzItem item = oz_item(w, whole, pieces, nch);
+      const int64_t rt = item.tile / (2 * CT), ct = item.tile / 2 % CT;
+      const int G = orders[ct];
+      long long a[OZ_HN];
+      float t[OZ_HN];
 #pragma unroll
       for (int j = 0; j < OZ_HN; ++j) {
-        ar_[j] = ai_[j] = 0ll;
-        tr[j] = ti[j] = 0.f;
+        a[j] = 0ll;
+        t[j] = 0.f;
       }
-      for (int64_t c = 0; c < nch; ++c, ++chunks) {
+      for (int64_t c = item.c0; c < item.c1; ++c, ++chunks) {
         if (!oz_wait(smem_u32(&bar_accf), uint32_t(chunks & 1))) {
           fail();
           fl_stop = 1;
@@ -431,27 +543,36 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         asm volatile("bar.sync 1, 256;");  // the stop decision is the same in all eight warps
         if (fl_stop) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
-#pragma unroll 1
-        for (int g = 0; g < OZ_ND; ++g) {
-          // both parts of order g in flight together, one wait
-          uint32_t v[16], w[16];
-          oz_ld16(tmem + (uint32_t(lane_base) << 16) + uint32_t(g * 2 + 0) * OZ_TN + c0, v);
-          oz_ld16(tmem + (uint32_t(lane_base) << 16) + uint32_t(g * 2 + 1) * OZ_TN + c0, w);
-          asm volatile("tcgen05.wait::ld.sync.aligned;");
-          if (g <= 3) {
-            const int sh = 24 - 8 * g;
 #pragma unroll
-            for (int j = 0; j < OZ_HN; ++j) {
-              ar_[j] += (long long)__float2int_rn(__uint_as_float(v[j])) << sh;
-              ai_[j] += (long long)__float2int_rn(__uint_as_float(w[j])) << sh;
-            }
-          } else {
-            const float sc = __int_as_float((127 + 24 - 8 * g) << 23);  // 2^{24-8g}
+        for (int h = 0; h < OZ_HN; h += 16) {
+          uint32_t v[16], u[16];
+          auto load = [&](int g) {  // orders g and g + 1
+            oz_ld16(tbase + uint32_t(g * OZ_TN + h), v);
+            if (g + 1 <= G) oz_ld16(tbase + uint32_t((g + 1) * OZ_TN + h), u);
+            oz_wait_ld(v, u);
+          };
+          auto digit = [](uint32_t x) { return __float2int_rn(__uint_as_float(x)); };
+          // orders 0 and 1: V_0 2^8 + V_1 fits 32 bits (|V_0| <= 2^22, |V_1| <= 2^23)
+          load(0);
 #pragma unroll
-            for (int j = 0; j < OZ_HN; ++j) {
-              tr[j] = fmaf(__uint_as_float(v[j]), sc, tr[j]);
-              ti[j] = fmaf(__uint_as_float(w[j]), sc, ti[j]);
+          for (int j = 0; j < 16; ++j) a[h + j] += (long long)(digit(v[j]) * 256 + (G >= 1 ? digit(u[j]) : 0)) * 65536;
+          if (G >= 2) {
+            load(2);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) a[h + j] += (long long)digit(v[j]) * 256 + (G >= 3 ? digit(u[j]) : 0);
+          }
+          if (G >= 4) {
+            load(4);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              t[h + j] = fmaf(__uint_as_float(v[j]), 0x1p-8f, t[h + j]);
+              if (G >= 5) t[h + j] = fmaf(__uint_as_float(u[j]), 0x1p-16f, t[h + j]);
             }
+          }
+          if (G >= 6) {
+            load(6);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) t[h + j] = fmaf(__uint_as_float(v[j]), 0x1p-24f, t[h + j]);
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;");
@@ -459,23 +580,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       }
       if (fl_stop) break;
       const int64_t row = rt * OZ_TM + r_local;
-      if (row < M) {
-        const double srow = ldexp(1.0, aex[row] - 14);
+      if (!item.whole) {
+        OzPart* p = part + ((w - whole) * OZ_TM + r_local) * OZ_TN + c0;
+#pragma unroll
+        for (int j = 0; j < OZ_HN; ++j) p[j] = {a[j], t[j]};
+      } else if (row < M) {
+        const int ae = aex[row];
 #pragma unroll
         for (int j = 0; j < OZ_HN; ++j) {
           const int64_t col = ct * OZ_TN + c0 + j;
-          if (col < N) {
-            const double sc = srow * ldexp(1.0, bex[col]);
-            const double xr = ldexp(double(ar_[j]) + double(tr[j]), -24) * sc;
-            const double xi = ldexp(double(ai_[j]) + double(ti[j]), -24) * sc;
-            double2 v = make_double2(alpha_re * xr - alpha_im * xi, alpha_re * xi + alpha_im * xr);
-            if (beta != 0.0) {
-              const double2 o = C[row * ldc + col];
-              v.x += beta * o.x;
-              v.y += beta * o.y;
-            }
-            C[row * ldc + col] = v;
-          }
+          if (col < N) oz_store(C + (row * ldc + col) * 2 + (item.tile & 1), a[j], t[j], ae, bex[col], alpha, beta);
         }
       }
     }
@@ -483,6 +597,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(OZ_TMEM_COLS));
+}
+
+__global__ void oz_reduce_kernel(int64_t M, int64_t N, int64_t whole, int pieces, const OzPart* __restrict__ part,
+                                 const int* __restrict__ aex, const int* __restrict__ bex, double alpha, double beta,
+                                 double* __restrict__ C, int64_t ldc) {
+  const int64_t CT = (N + OZ_TN - 1) / OZ_TN, tile = whole + blockIdx.x;
+  const int e = int(blockIdx.y) * 256 + int(threadIdx.x);  // element of the tile
+  const int64_t row = tile / (2 * CT) * OZ_TM + e / OZ_TN, col = tile / 2 % CT * OZ_TN + e % OZ_TN;
+  if (row >= M || col >= N) return;
+  OzPart s = {0, 0.f};
+  for (int q = 0; q < pieces; ++q) {
+    const OzPart p = part[(int64_t(blockIdx.x) * pieces + q) * (OZ_TM * OZ_TN) + e];
+    s.a += p.a;
+    s.t += p.t;
+  }
+  oz_store(C + (row * ldc + col) * 2 + (tile & 1), s.a, s.t, aex[row], bex[col], alpha, beta);
 }
 
 inline unsigned oz_cdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); }
@@ -504,9 +634,9 @@ cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void*
   return launched(2);
 }
 
-cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha_re, double alpha_im, const void* a_digits,
-                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* status,
-                    cudaStream_t s) {
+cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
+                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
+                    const int* ref_ex, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   static bool attr[64] = {};
   static int nsm[64] = {};
@@ -520,27 +650,36 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha_re, double alp
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
-  const int64_t KC = (K + OZ_KS - 1) / OZ_KS, CT = (N + OZ_TN - 1) / OZ_TN;
+  const int64_t KC = (K + OZ_KS - 1) / OZ_KS, CT = (N + OZ_TN - 1) / OZ_TN, nch = (KC + OZ_KCH - 1) / OZ_KCH;
   if (CT * OZ_TN / 8 > 65535) return cudaErrorInvalidValue;
-  const size_t bbytes = size_t(CT) * size_t(KC) * OZ_NT * OZ_BTILE;
+  // the tiles that would not fill the chip, in as many pieces of at least 8 chunks as there are SMs for
+  const int64_t sms = std::max(nsm[dev], 1), tiles = ((M + OZ_TM - 1) / OZ_TM) * CT * 2, rem = tiles % sms;
+  const int64_t whole = tiles - rem;
+  const int pieces = rem ? int(std::max<int64_t>(1, std::min<int64_t>(sms / rem, nch / 8))) : 1;
+  const int64_t items = whole + rem * pieces;
+  // digit tiles of B, then the pieces' sums, then the orders
+  const size_t bbytes = size_t(CT) * size_t(KC) * OZ_BSLOT;
+  const size_t pbytes = pieces > 1 ? sizeof(OzPart) * size_t(rem * pieces) * OZ_TM * OZ_TN : 0;
   unsigned char* bd = nullptr;
-  int* bex = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&bd), bbytes, s);
-  if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&bex), sizeof(int) * size_t(N), s);
-  if (e == cudaSuccess) {
-    oz_col_exp_kernel<<<unsigned(N), 256, 0, s>>>(static_cast<const double2*>(B), K, N, ldb, bex);
-    oz_split_kernel<OZ_TN><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(CT * OZ_TN / 8)), OZ_SPLIT_WARPS * 32,
-                             0, s>>>(static_cast<const double2*>(B), N, K, 1, ldb, bex, KC, bd);
-    const int64_t tiles = ((M + OZ_TM - 1) / OZ_TM) * CT;
-    const unsigned grid = unsigned(std::min<int64_t>(tiles, std::max(nsm[dev], 1)));
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&bd), bbytes + pbytes + sizeof(int) * size_t(CT), s);
+  if (e != cudaSuccess) return e;
+  OzPart* part = reinterpret_cast<OzPart*>(bd + bbytes);
+  int* orders = reinterpret_cast<int*>(bd + bbytes + pbytes);
+  oz_col_exp_kernel<<<unsigned(N), 256, 0, s>>>(static_cast<const double2*>(B), K, N, ldb, b_ex);
+  oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, N, orders);
+  oz_split_kernel<OZ_TN><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(CT * OZ_TN / 8)), OZ_SPLIT_WARPS * 32, 0,
+                           s>>>(static_cast<const double2*>(B), N, K, 1, ldb, b_ex, KC, bd);
+  {
     ProfScope prof("gemm_oz", s, 8.0 * double(M) * double(N) * double(K));
-    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, s>>>(M, N, KC, static_cast<const unsigned char*>(a_digits), a_ex, bd,
-                                                      bex, alpha_re, alpha_im, beta, static_cast<double2*>(C), ldc,
-                                                      status);
-    e = launched(3);
+    oz_gemm_kernel<<<unsigned(std::min(items, sms)), OZ_THREADS, OZ_SMEM, s>>>(
+        M, N, KC, static_cast<const unsigned char*>(a_digits), a_ex, bd, b_ex, orders, whole, pieces, items, alpha, beta,
+        static_cast<double*>(C), ldc, part, status);
+    if (pieces > 1)
+      oz_reduce_kernel<<<dim3(unsigned(rem), OZ_TM * OZ_TN / 256), 256, 0, s>>>(
+          M, N, whole, pieces, part, a_ex, b_ex, alpha, beta, static_cast<double*>(C), ldc);
   }
-  if (bd) cudaFreeAsync(bd, s);
-  if (bex) cudaFreeAsync(bex, s);
+  e = launched(pieces > 1 ? 5 : 4);
+  cudaFreeAsync(bd, s);
   return e;
 }
 
@@ -564,11 +703,12 @@ extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, con
   }
   Scratch dig(s), ex(s), st(s);
   FOSB_CUDA(dig.alloc(oz_a_bytes(M, K)));
-  FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M)));
+  FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M + N)));
   FOSB_CUDA(st.alloc(sizeof(int)));
   FOSB_CUDA(cudaMemsetAsync(st.p, 0, sizeof(int), s));
   FOSB_CUDA(oz_prepare_a(A, M, K, lda, dig.p, ex.as<int>(), s));
-  FOSB_CUDA(oz_gemm(M, N, K, 1.0, 0.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, st.as<int>(), s));
+  FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
+                    st.as<int>(), s));
   int status = 0;
   FOSB_CUDA(cudaMemcpyAsync(&status, st.p, sizeof(int), cudaMemcpyDeviceToHost, s));
   FOSB_CUDA(cudaStreamSynchronize(s));
