@@ -244,7 +244,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       xfull = xn;
     }
     if (digits)
-      FOSB_CUDA(oz_gemm(n, nrhs, n, -1.0, lu->zdig, lu->zex, full ? X : dx.p, full ? ldx : nrhs, 1.0, r.p, nrhs,
+      FOSB_CUDA(oz_gemm(OP_N, n, nrhs, n, -1.0, lu->zdig, lu->zex, full ? X : dx.p, full ? ldx : nrhs, 1.0, r.p, nrhs,
                         xex.as<int>() + (full ? 0 : nrhs), full ? nullptr : xex.as<int>(), lu->d_status, s));
     else
       FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, n, nrhs, n, -1.0, 0.0, lu->zref, lu->ldz, X, ldx, 1.0, r.p, nrhs, s,
@@ -402,7 +402,7 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
     if (n >= 256) {
       if ((e = cudaMalloc(&lu->zdig, oz_a_bytes(n, n))) != cudaSuccess ||
           (e = cudaMalloc(reinterpret_cast<void**>(&lu->zex), sizeof(int) * n)) != cudaSuccess ||
-          (e = oz_prepare_a(Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
+          (e = oz_prepare_a(OP_N, Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
         return cleanup(cuda_fail(e, "fosb_factor: digit tiles of Z"));
     }
     Scratch nrm(s);
@@ -515,7 +515,7 @@ fosb_status fosb_covariance(fosb_mesh m1, fosb_lu lu1, const void* u1, fosb_mesh
   if (c64)
     e = gemm<float>(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, 0.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
   else if (prec == FOSB_MIXED)
-    e = gemm_c128_ff(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, 0.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
+    e = gemm_c128_fp64class(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
   else
     e = gemm<double>(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, 0.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
   FOSB_CUDA(e);
@@ -550,7 +550,7 @@ namespace {
 cudaError_t gemm_prec(int prec, int opA, int opB, int64_t M, int64_t N, int64_t K, double ar, const void* A, int64_t lda,
                       const void* B, int64_t ldb, double beta, void* C, int64_t ldc, cudaStream_t s) {
   if (is_c64(prec)) return gemm<float>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
-  if (prec == FOSB_MIXED) return gemm_c128_ff(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
+  if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, s);
   return gemm<double>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
 }
 }  // namespace
@@ -626,7 +626,7 @@ fosb_status fosb_farfield_moments(fosb_mesh m1, fosb_mesh m2, double k, const do
   auto G = [&](int opA, int opB, int64_t M, int64_t N, int64_t K, double ar, const void* A, int64_t lda,
                const void* B, int64_t ldb, double beta, void* C, int64_t ldc) {
     if (c64) return gemm<float>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
-    if (prec == FOSB_MIXED) return gemm_c128_ff(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
+    if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, s);
     return gemm<double>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
   };
   if (!m2) {
@@ -685,7 +685,7 @@ fosb_status fosb_rcs_monostatic(fosb_mesh mesh, fosb_lu lu, double k, const fosb
   FOSB_CUDA(cudaMemsetAsync(A.p, 0, 16 * nd3 * N, s));
   FOSB_CUDA(launch_farfield_matrix(d, k, dxh.as<double>(), n, false, A.p, s));
   FOSB_CUDA(FA.alloc(16 * nd3 * n));
-  FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, nd3, n, N, 1.0, 0.0, A.p, N, U, ldu, 0.0, FA.p, n, s));
+  FOSB_CUDA(gemm_c128_fp64class(OP_N, OP_N, nd3, n, N, 1.0, A.p, N, U, ldu, 0.0, FA.p, n, s));
   std::vector<double> fa(2 * nd3 * n);
   FOSB_CUDA(cudaMemcpyAsync(fa.data(), FA.p, 16 * nd3 * n, cudaMemcpyDeviceToHost, s));
   FOSB_CUDA(cudaStreamSynchronize(s));
@@ -746,7 +746,7 @@ fosb_status fosb_rcs_monostatic(fosb_mesh mesh, fosb_lu lu, double k, const fosb
   FOSB_CUDA(dC.alloc(16 * nd3 * n));
   FOSB_CUDA(cudaMemcpyAsync(dC.p, Cm.data(), 16 * nd3 * n, cudaMemcpyHostToDevice, s));
   FOSB_CUDA(lam.alloc(16 * N * n));
-  FOSB_CUDA(gemm_c128_ff(OP_T, OP_N, N, n, nd3, 1.0, 0.0, A.p, N, dC.p, n, 0.0, lam.p, n, s));
+  FOSB_CUDA(gemm_c128_fp64class(OP_T, OP_N, N, n, nd3, 1.0, A.p, N, dC.p, n, 0.0, lam.p, n, s));
   FOSB_TRY(solve_internal(lu, lam.p, n, n, lam.p, n, nullptr, nullptr, s));
   FOSB_CUDA(dpw.alloc(sizeof(double) * 11 * 2 * n));
   FOSB_CUDA(cudaMemcpyAsync(dpw.p, pw.data(), sizeof(double) * 11 * 2 * n, cudaMemcpyHostToDevice, s));

@@ -223,15 +223,22 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
                          cudaStream_t s, const void* A_split = nullptr);
 // FP64-class complex GEMM on the bf16 tensor cores by exact digit splitting (oz_gemm.cu):
 // oz_prepare_a writes the digit tiles (oz_a_bytes(M, K) bytes) and row exponents (M ints)
-// of the complex128 A (M x K, lda); oz_gemm then computes C <- beta C + alpha A B, alpha and
-// beta real, for a complex128 B (K x N, ldb) and leaves the exponents of B's columns in b_ex (N ints).  With ref_ex
-// B is a correction of a matrix with those column exponents, and digit orders below 2^-64 of that
-// matrix's are left out.  A bounded wait that gives up sets *status.
+// of op(A) (M x K); oz_gemm then computes C <- beta C + alpha op(A) op(B), alpha and beta real,
+// for a complex128 op(B) (K x N) and leaves the exponents of its columns in b_ex (N ints).  With
+// ref_ex op(B) is a correction of a matrix with those column exponents, and digit orders below
+// 2^-60 of that matrix's are left out.  A bounded wait that gives up sets *status (may be null)
+// and leaves NaN.
 size_t oz_a_bytes(int64_t M, int64_t K);
-cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s);
-cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
-                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
-                    const int* ref_ex, int* status, cudaStream_t s);
+cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex,
+                         cudaStream_t s);
+cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
+                    const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
+                    int* status, cudaStream_t s);
+// C <- beta C + alpha op(A) op(B) in FP64-class arithmetic: digits where the product is large
+// enough to pay for making them, float-float (gemm_c128_ff) otherwise.
+cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,
+                                int64_t lda, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
+                                cudaStream_t s);
 // dst (rows x cols float4, ldd) = (hi, lo) float split of the complex128 src
 cudaError_t split_ff(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                      cudaStream_t s);

@@ -15,23 +15,24 @@
 // sum per output, orders 4-6 (below 2^-32 of them) into an FP32 sum; the result is scaled by
 // sigma_i tau_j 2^-14.
 //
-// The tensor pipe: an MMA with M = 128, K = 16 takes 44 cycles for any N up to
-// 64 and 64 cycles at N = 128 (measured), so seven orders of N = 64 for one part (448 of the 512
-// TMEM columns) cost half of what Re and Im at N = 32 do: Re and Im are separate tiles that load
-// the same digits.  The collector and uniform MMA operands (oz_elect) bring them to 35 cycles.
-// Z X for N = 7503 and 163 columns: 4.63 ms with both parts at N = 32, sums after every 64 values
-// of k and the MMAs issued behind `lane == 0`, 2.24 ms so; the digits' way from L2 (86 KB per CTA
-// and step) now takes longer than the MMAs: orders up to 4 need 30 of the 56 MMAs and 5/7 of the
-// bytes and take 0.67 of the time.
+// What bounds it is the issue of the MMAs and then the tensor pipe.  An MMA with M = 128, K = 16
+// takes 44 cycles for any N up to 64 behind `lane == 0`, where its operands go from vector to
+// uniform registers one by one; behind elect.sync, with every operand a compile-time offset, N = 64
+// takes 35 (32 of them the pipe) and N = 32 takes 21 (measured).  So Re and Im are separate tiles
+// of N = 64, seven orders of which fill 448 of the 512 TMEM columns, and the orders, the part and
+// the stage are compiled in.  Every wait of the issuing lane costs 80 cycles even with nothing to
+// wait for: one per step, tested ahead.  Z X at N = 7503 with 163 columns (354 half tiles over 152
+// SMs): 4.63 ms with both parts at N = 32, sums after every 64 values of k and `lane == 0`; 2.24 ms
+// with N = 64 and elect; 1.63 ms with one wait per step and a load lane per digit.  The MMAs alone
+// take 1.22 ms (1968 cycles per step of 56), the order sums 0.25 ms, the rest is waiting for L2.
 //
-// Kernel roles (one CTA per SM, persistent over 128 x 64 tiles of one part): warp 0 lane 0 moves
-// the pre-tiled digits of a 16-wide k step into two shared rings with bulk copies, one digit of Z
-// (8 KB) per slot of the first and all of X's (28 KB) per slot of the second, so that the loads
-// run two steps ahead; warp 1 lane 0 issues the 56 MMAs of a step (tcgen05.mma kind::f16, bf16,
-// M = 128, N = 64, K = 16; the minus of Im Z Im X via the negate-B bit; the MMAs of an A tile run
-// back to back and keep it in the A collector) into the order accumulators; warps 2-9 read the
-// accumulators after every 128 values of k and hold the sums (two warps per TMEM lane group, 32
-// columns each).  All waits are bounded.
+// Kernel roles (one CTA per SM, persistent over 128 x 64 tiles of one part): seven lanes of warp 0
+// move the pre-tiled digits of a 16-wide k step into one of two stages with bulk copies, lane s
+// digit s of Z (8 KB) as soon as its slot is free, lane 0 also all of X's (28 KB); one lane of warp
+// 1 issues the 56 MMAs of a step (tcgen05.mma kind::f16, bf16, M = 128, N = 64, K = 16; the minus of
+// Im Z Im X via the negate-B bit; the MMAs of an A tile run back to back and keep it in the A
+// collector) into the order accumulators; warps 2-9 read the accumulators after every 128 values of
+// k and hold the sums (two warps per TMEM lane group, 32 columns each).  All waits are bounded.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -49,15 +50,16 @@ constexpr int OZ_KCH = 8;                                      // k steps per ch
 constexpr int OZ_ATILE = OZ_TM * OZ_KS * 2;                    // 4096 B
 constexpr int OZ_BTILE = OZ_TN * OZ_KS * 2;                    // 2048 B
 constexpr int OZ_NT = OZ_ND * 2;                               // digit x part tiles per operand and step
-constexpr int OZ_ASLOT = 2 * OZ_ATILE, OZ_ASLOTS = 17;         // one digit of Z (Re, Im) per slot
-constexpr int OZ_BSLOT = OZ_NT * OZ_BTILE, OZ_BSLOTS = 3;      // all digits of X per slot
-constexpr int OZ_SMEM = OZ_ASLOTS * OZ_ASLOT + OZ_BSLOTS * OZ_BSLOT + 1024;
+constexpr int OZ_ASLOT = 2 * OZ_ATILE;                         // one digit of Z (Re, Im)
+constexpr int OZ_BSLOT = OZ_NT * OZ_BTILE;                     // all digits of X
+constexpr int OZ_STAGE = OZ_ND * OZ_ASLOT + OZ_BSLOT;          // 86016 B, one k step
+constexpr int OZ_SMEM = 2 * OZ_STAGE + 1024;
 constexpr int OZ_THREADS = 10 * 32;                            // producer, MMA, 8 flush warps
 constexpr int OZ_FLUSH = 8 * 32;
 constexpr int OZ_HN = OZ_TN / 2;                               // columns per flush thread
 constexpr int OZ_TMEM_COLS = 512;                              // 7 orders x 64 columns = 448 used
 constexpr long long kOzSpinLimit = 1ll << 24;
-static_assert(OZ_SMEM <= 226 * 1024, "digit slots and the barriers do not fit shared memory");
+static_assert(OZ_SMEM <= 226 * 1024, "digit stages and the barriers do not fit shared memory");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -113,15 +115,20 @@ __device__ __forceinline__ bool oz_elect() {
   asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
   return p != 0;
 }
+__device__ __forceinline__ uint32_t oz_test(uint32_t mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(mbar), "r"(parity)
+      : "memory");
+  return done;
+}
+template <bool SLEEP = false>
 __device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
   for (long long spins = 0; spins < kOzSpinLimit; ++spins) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(mbar), "r"(parity));
-    if (done) return true;
-    __nanosleep(32);
+    if (oz_test(mbar, parity)) return true;
+    if (SLEEP) __nanosleep(32);
   }
   return false;
 }
@@ -142,24 +149,18 @@ __device__ __forceinline__ void oz_bulk_load(uint32_t dst, const void* src, uint
 __device__ __forceinline__ void oz_commit(uint32_t mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar));
 }
-__device__ __forceinline__ void oz_ld16(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
+__device__ __forceinline__ void oz_ld8(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+               : "r"(taddr));
 }
-
 // waits for the loads above; the registers pass through, so that no use of them moves before it
-__device__ __forceinline__ void oz_wait_ld(uint32_t (&v)[16], uint32_t (&u)[16]) {
+__device__ __forceinline__ void oz_wait_ld(uint32_t (&v)[8], uint32_t (&u)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
-                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+                 "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7])
                :
                : "memory");
-  if (&v != &u)
-    asm volatile("" : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]), "+r"(u[7]),
-                 "+r"(u[8]), "+r"(u[9]), "+r"(u[10]), "+r"(u[11]), "+r"(u[12]), "+r"(u[13]), "+r"(u[14]), "+r"(u[15]));
 }
 
 // ---------------------------------------------------------------- digit splitting
@@ -170,9 +171,12 @@ __device__ __forceinline__ unsigned long long oz_abs_bits(double x) {
 }
 // the smallest e with |x| < 2^e for the largest |x| of a row or column (bit pattern mb),
 // e = 0 for zero: m = f 2^e with f in [0.5, 1)
+// Rows and columns with an infinity or NaN have the exponent OZ_BAD and give NaN.
+constexpr int OZ_BAD = 1 << 28;
 __device__ __forceinline__ int oz_exponent(unsigned long long mb) {
   int e = 0;
-  if (mb) frexp(__longlong_as_double(static_cast<long long>(mb)), &e);
+  if (mb >= 0x7FF0000000000000ull) e = OZ_BAD;
+  else if (mb) frexp(__longlong_as_double(static_cast<long long>(mb)), &e);
   return e;
 }
 __device__ __forceinline__ unsigned long long oz_umax(unsigned long long a, unsigned long long b) {
@@ -252,7 +256,7 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(uint32_t byte) {
 // each store instruction fills two whole 256-byte segments.
 template <int TR>
 __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int64_t K, int64_t rs, int64_t ks,
-                                const int* __restrict__ ex, int64_t KC, unsigned char* __restrict__ out) {
+                                bool conj, const int* __restrict__ ex, int64_t KC, unsigned char* __restrict__ out) {
   constexpr int TILE = TR * OZ_KS * 2;
   constexpr unsigned long long BIAS = 0x0080808080808080ull;
   const int lane = threadIdx.x & 31;
@@ -268,7 +272,7 @@ __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int
     if (row < rows && k < K) {
       const double2 v = A[row * rs + k * ks];
       gr[j] = static_cast<unsigned long long>(oz_fixed(v.x, e)) + BIAS;
-      gi[j] = static_cast<unsigned long long>(oz_fixed(v.y, e)) + BIAS;
+      gi[j] = static_cast<unsigned long long>(oz_fixed(conj ? -v.y : v.y, e)) + BIAS;
     }
   }
   const int64_t rt = row / TR, kc = kg >> 1;
@@ -311,7 +315,8 @@ __global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restri
 // sums), exact; t the orders 4-6 (below 2^-32 of the leading terms) in FP32 in the same units, so
 // its rounding stays near 2^-50 of the result; the value is 2^-24 (a + t).
 __device__ __forceinline__ void oz_store(double* C, long long a, float t, int aex, int bex, double alpha, double beta) {
-  const double sc = ldexp(1.0, aex - 14) * ldexp(1.0, bex);
+  double sc = ldexp(1.0, aex - 14) * ldexp(1.0, bex);
+  if (aex == OZ_BAD || bex == OZ_BAD) sc = NAN;
   const double x = alpha * (ldexp(double(a) + double(t), -24) * sc);
   *C = beta != 0.0 ? x + beta * *C : x;
 }
@@ -319,18 +324,6 @@ __device__ __forceinline__ void oz_store(double* C, long long a, float t, int ae
 struct OzPart {
   long long a;
   float t;
-};
-
-// A ring of shared-memory slots as its producer or consumer walks it.
-template <int SLOTS>
-struct OzRing {
-  uint32_t slot = 0, turn = 0;
-  __device__ __forceinline__ void next() {
-    if (++slot == SLOTS) {
-      slot = 0;
-      ++turn;
-    }
-  }
 };
 
 // One A tile with T digits of X (tiles 2 OZ_BTILE apart) into T consecutive orders, the A tile kept
@@ -347,21 +340,55 @@ __device__ __forceinline__ void oz_group(uint32_t d, uint64_t a, uint64_t b, uin
     else oz_mma<1>(dt, a, bt, idesc, acc);
   }
 }
-// The MMAs of one k step with the orders S .. G, digit by digit of Z as its slots fill; false where
-// a wait gave up.  `first`: the first product into an order's accumulator (s = 0) overwrites it.
-template <int S, int G>
-__device__ __forceinline__ bool oz_step(uint32_t tmem, uint32_t smem_a, uint64_t* a_full, uint64_t* a_empty,
-                                        OzRing<OZ_ASLOTS>& ra, uint64_t db, int im, bool first) {
-  if (!oz_wait(smem_u32(&a_full[ra.slot]), ra.turn & 1)) return false;
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint64_t da = oz_desc(smem_a + ra.slot * OZ_ASLOT);
+
+// What the MMA lane carries along.  Everything else in its inner code is a constant, so that the
+// operands of the MMAs stay in uniform registers: two stages unrolled, orders and part compiled in.
+struct OzMma {
+  uint64_t *full, *empty;  // full by stage; empty by stage and digit of Z, digit 0 also for the digits of X
+  uint32_t phase;          // phase of the full barriers, a bit per stage
+  uint32_t ready;          // the next stage was seen full
+};
+// The MMAs of one k step with the orders 0 .. G out of stage P, from digit S of Z on, part IM (0 Re,
+// 1 Im).  A wait that has nothing to wait for still takes 80 cycles, and few MMAs queue up behind
+// each other, so a stage has one barrier to wait for, tested before the last MMAs of the stage
+// before it; its slots are given back digit by digit, which costs nothing.  `acc`: 0 where the
+// step's first product into each order's accumulator (digit 0) overwrites it.
+template <int G, int IM, int P, int S>
+__device__ __forceinline__ void oz_step(OzMma& m, uint32_t tmem, uint32_t smem, uint32_t acc) {
+  if constexpr (S == (G > 0 ? G - 1 : 0)) m.ready = oz_test(smem_u32(&m.full[1 - P]), m.phase >> (1 - P) & 1);
+  const uint64_t a = oz_desc(smem + P * OZ_STAGE + S * OZ_ASLOT), b = oz_desc(smem + P * OZ_STAGE + OZ_ND * OZ_ASLOT);
   const uint32_t d = tmem + uint32_t(S) * OZ_TN;
   // Re: Re Z Re X - Im Z Im X, Im: Re Z Im X + Im Z Re X
-  oz_group<G + 1 - S>(d, da, db + uint64_t(im) * (OZ_BTILE >> 4), oz_idesc(false), first && S == 0 ? 0u : 1u);
-  oz_group<G + 1 - S>(d, da + (OZ_ATILE >> 4), db + uint64_t(1 - im) * (OZ_BTILE >> 4), im ? oz_idesc(false) : oz_idesc(true), 1u);
-  oz_commit(smem_u32(&a_empty[ra.slot]));
-  ra.next();
-  if constexpr (S < G) return oz_step<S + 1, G>(tmem, smem_a, a_full, a_empty, ra, db, im, first);
+  oz_group<G + 1 - S>(d, a, b + uint64_t(IM * (OZ_BTILE >> 4)), oz_idesc(false), S == 0 ? acc : 1u);
+  oz_group<G + 1 - S>(d, a + (OZ_ATILE >> 4), b + uint64_t((1 - IM) * (OZ_BTILE >> 4)), oz_idesc(IM == 0), 1u);
+  if constexpr (S > 0) oz_commit(smem_u32(&m.empty[P * OZ_ND + S]));
+  if constexpr (S == G) oz_commit(smem_u32(&m.empty[P * OZ_ND]));
+  if constexpr (S < G) oz_step<G, IM, P, S + 1>(m, tmem, smem, acc);
+}
+template <int G, int IM, int P>
+__device__ __forceinline__ bool oz_stage(OzMma& m, uint32_t tmem, uint32_t smem, uint32_t acc) {
+  if (!m.ready && !oz_wait(smem_u32(&m.full[P]), m.phase >> P & 1)) return false;
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  m.phase ^= 1u << P;
+  oz_step<G, IM, P, 0>(m, tmem, smem, acc);
+  return true;
+}
+// The MMAs of chunks [c0, c1) of a tile
+template <int G, int IM>
+__device__ __forceinline__ bool oz_tile(OzMma& m, uint32_t tmem, uint32_t smem, uint64_t* accf, uint64_t* acce, int64_t KC,
+                                     int64_t c0, int64_t c1, int64_t& chunks) {
+  m.ready = 0;
+  for (int64_t c = c0; c < c1; ++c, ++chunks) {
+    // the order accumulators are free once the flush warps have read the last chunk
+    if (chunks > 0 && !oz_wait(smem_u32(acce), uint32_t((chunks - 1) & 1))) return false;
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    const int steps = int(std::min<int64_t>(KC - c * OZ_KCH, OZ_KCH));
+    for (int k = 0; k < steps; k += 2) {  // a chunk starts at an even step
+      if (!oz_stage<G, IM, 0>(m, tmem, smem, k > 0)) return false;
+      if (k + 1 < steps && !oz_stage<G, IM, 1>(m, tmem, smem, 1u)) return false;
+    }
+    oz_commit(smem_u32(accf));
+  }
   return true;
 }
 
@@ -385,7 +412,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                    double* __restrict__ C, int64_t ldc, OzPart* __restrict__ part, int* status) {
   extern __shared__ unsigned char oz_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ uint64_t a_full[OZ_ASLOTS], a_empty[OZ_ASLOTS], b_full[OZ_BSLOTS], b_empty[OZ_BSLOTS];
+  __shared__ uint64_t full[2], empty[2 * OZ_ND];  // by stage; by stage and digit of Z
   __shared__ uint64_t bar_accf, bar_acce, bar_drain;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
@@ -399,14 +426,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    for (int i = 0; i < OZ_ASLOTS; ++i) {
-      oz_init(smem_u32(&a_full[i]), 1);
-      oz_init(smem_u32(&a_empty[i]), 1);
-    }
-    for (int i = 0; i < OZ_BSLOTS; ++i) {
-      oz_init(smem_u32(&b_full[i]), 1);
-      oz_init(smem_u32(&b_empty[i]), 1);
-    }
+    for (int i = 0; i < 2; ++i) oz_init(smem_u32(&full[i]), OZ_ND);
+    for (int i = 0; i < 2 * OZ_ND; ++i) oz_init(smem_u32(&empty[i]), 1);
     oz_init(smem_u32(&bar_accf), 1);
     oz_init(smem_u32(&bar_acce), OZ_FLUSH);
     oz_init(smem_u32(&bar_drain), 1);
@@ -418,98 +439,80 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = tmem_sh;
-  const uint32_t smem_a = smem_u32(smem), smem_b = smem_a + OZ_ASLOTS * OZ_ASLOT;
   auto fail = [&]() {
     abort_sh = 1;
-    atomicExch(status, FOSB_ERR_TIMEOUT);
+    if (status) atomicExch(status, FOSB_ERR_TIMEOUT);
   };
 
   if (warp == 0) {
     // ---------------------------------------------------------- producer
-    if (lane == 0) {
-      OzRing<OZ_ASLOTS> ra;
-      OzRing<OZ_BSLOTS> rb;
-      for (int64_t w = blockIdx.x; w < items && !abort_sh; w += gridDim.x) {
+    // Lane s fills digit s of Z in each stage, lane 0 also the digits of X: a wait and a copy per lane
+    // and step (one lane for all took longer over them than the MMAs of the step).  Every lane
+    // arrives at the stage's full barrier, those above the highest order with nothing to load.
+    // The lanes meet after every step, so that none runs ahead of a barrier by more than a phase.
+    const int s = lane;
+    uint32_t fills0 = 0, fills1 = 0;  // of this lane's slot in each stage
+    bool go = true;
+    if (s < OZ_ND) {
+      const uint32_t stage0 = smem_u32(smem);
+      for (int64_t w = blockIdx.x; w < items && go; w += gridDim.x) {
         const OzItem item = oz_item(w, whole, pieces, nch);
         const int64_t rt = item.tile / (2 * CT), ct = item.tile / 2 % CT;
         const int G = orders[ct];
         const int64_t k1 = std::min<int64_t>(KC, item.c1 * OZ_KCH);
-        for (int64_t kc = item.c0 * OZ_KCH; kc < k1 && !abort_sh; ++kc) {
-          // the digits up to the highest order are the first tiles of each operand's step
-          if (rb.turn > 0 && !oz_wait(smem_u32(&b_empty[rb.slot]), (rb.turn - 1) & 1)) {
+        // the digits up to the highest order are the first tiles of each operand's step
+        const uint32_t bbytes = s == 0 ? uint32_t(G + 1) * 2 * OZ_BTILE : 0u;
+        for (int64_t kc = item.c0 * OZ_KCH; kc < k1 && go; ++kc) {  // (starts even)
+          const int p = int(kc & 1);
+          const uint32_t turn = p ? fills1 : fills0;
+          bool ok = !abort_sh;
+          if (ok && s <= G && turn > 0 && !oz_wait(smem_u32(&empty[p * OZ_ND + s]), (turn - 1) & 1)) {
             fail();
-            break;
+            ok = false;
           }
-          const uint32_t bb = uint32_t(G + 1) * 2 * OZ_BTILE;
-          oz_expect_tx(smem_u32(&b_full[rb.slot]), bb);
-          oz_bulk_load(smem_b + rb.slot * OZ_BSLOT, Bd + (ct * KC + kc) * OZ_BSLOT, bb, smem_u32(&b_full[rb.slot]));
-          rb.next();
-          const unsigned char* ga = Ad + ((rt * KC + kc) * OZ_NT) * OZ_ATILE;
-          for (int s = 0; s <= G; ++s) {
-            if (ra.turn > 0 && !oz_wait(smem_u32(&a_empty[ra.slot]), (ra.turn - 1) & 1)) {
-              fail();
-              break;
-            }
-            oz_expect_tx(smem_u32(&a_full[ra.slot]), OZ_ASLOT);
-            oz_bulk_load(smem_a + ra.slot * OZ_ASLOT, ga + s * OZ_ASLOT, OZ_ASLOT, smem_u32(&a_full[ra.slot]));
-            ra.next();
+          go = __all_sync((1u << OZ_ND) - 1u, ok);
+          if (!go) break;
+          const uint32_t bar = smem_u32(&full[p]), dst = stage0 + p * OZ_STAGE;
+          oz_expect_tx(bar, s <= G ? OZ_ASLOT + bbytes : 0u);
+          if (s <= G) {
+            (p ? fills1 : fills0) = turn + 1;
+            if (s == 0) oz_bulk_load(dst + OZ_ND * OZ_ASLOT, Bd + (ct * KC + kc) * OZ_BSLOT, bbytes, bar);
+            oz_bulk_load(dst + s * OZ_ASLOT, Ad + (rt * KC + kc) * (OZ_NT * OZ_ATILE) + s * OZ_ASLOT, OZ_ASLOT, bar);
           }
         }
       }
-      // no copy may land after the kernel has left (it can leave early where a wait gave up)
-      auto landed = [&](uint64_t* full, uint32_t slot, uint32_t turn, uint32_t i) {
-        const uint32_t loads = turn + (i < slot ? 1 : 0);
-        if (loads > 0) oz_wait(smem_u32(&full[i]), (loads - 1) & 1);
-      };
-      for (uint32_t i = 0; i < OZ_ASLOTS; ++i) landed(a_full, ra.slot, ra.turn, i);
-      for (uint32_t i = 0; i < OZ_BSLOTS; ++i) landed(b_full, rb.slot, rb.turn, i);
+      // no copy may land after the kernel has left (it can leave early where a wait gave up); lane 0
+      // has filled its slot in every step
+      if (s == 0 && fills0 > 0) oz_wait(smem_u32(&full[0]), (fills0 - 1) & 1);
+      if (s == 0 && fills1 > 0) oz_wait(smem_u32(&full[1]), (fills1 - 1) & 1);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
     if (oz_elect()) {
-      OzRing<OZ_ASLOTS> ra;
-      OzRing<OZ_BSLOTS> rb;
+      OzMma m = {full, empty, 0u, 0u};
+      const uint32_t stage0 = smem_u32(smem);
       int64_t chunks = 0;
       for (int64_t w = blockIdx.x; w < items && !abort_sh; w += gridDim.x) {
         const OzItem item = oz_item(w, whole, pieces, nch);
-        const int G = orders[item.tile / 2 % CT], im = int(item.tile & 1);
-        for (int64_t c = item.c0; c < item.c1 && !abort_sh; ++c, ++chunks) {
-          // the order accumulators are free once the flush warps have read the last chunk
-          if (chunks > 0 && !oz_wait(smem_u32(&bar_acce), uint32_t((chunks - 1) & 1))) {
-            fail();
-            break;
-          }
-          asm volatile("tcgen05.fence::after_thread_sync;");
-          const int64_t k0 = c * OZ_KCH, k1 = std::min<int64_t>(KC, k0 + OZ_KCH);
-          for (int64_t kc = k0; kc < k1 && !abort_sh; ++kc) {
-            if (!oz_wait(smem_u32(&b_full[rb.slot]), rb.turn & 1)) {
-              fail();
-              break;
-            }
-            const uint64_t db = oz_desc(smem_b + rb.slot * OZ_BSLOT);
-            auto step = [&](auto g) {
-              return oz_step<0, decltype(g)::value>(tmem, smem_a, a_full, a_empty, ra, db, im, kc == k0);
-            };
-            bool ok;
-            switch (G) {
-              case 0: ok = step(std::integral_constant<int, 0>()); break;
-              case 1: ok = step(std::integral_constant<int, 1>()); break;
-              case 2: ok = step(std::integral_constant<int, 2>()); break;
-              case 3: ok = step(std::integral_constant<int, 3>()); break;
-              case 4: ok = step(std::integral_constant<int, 4>()); break;
-              case 5: ok = step(std::integral_constant<int, 5>()); break;
-              default: ok = step(std::integral_constant<int, 6>()); break;
-            }
-            if (!ok) {
-              fail();
-              break;
-            }
-            oz_commit(smem_u32(&b_empty[rb.slot]));
-            rb.next();
-          }
-          if (abort_sh) break;
-          oz_commit(smem_u32(&bar_accf));
+        auto run = [&](auto g) {
+          constexpr int G = decltype(g)::value;
+          return item.tile & 1 ? oz_tile<G, 1>(m, tmem, stage0, &bar_accf, &bar_acce, KC, item.c0, item.c1, chunks)
+                               : oz_tile<G, 0>(m, tmem, stage0, &bar_accf, &bar_acce, KC, item.c0, item.c1, chunks);
+        };
+        bool ok;
+        switch (orders[item.tile / 2 % CT]) {
+          case 0: ok = run(std::integral_constant<int, 0>()); break;
+          case 1: ok = run(std::integral_constant<int, 1>()); break;
+          case 2: ok = run(std::integral_constant<int, 2>()); break;
+          case 3: ok = run(std::integral_constant<int, 3>()); break;
+          case 4: ok = run(std::integral_constant<int, 4>()); break;
+          case 5: ok = run(std::integral_constant<int, 5>()); break;
+          default: ok = run(std::integral_constant<int, 6>()); break;
+        }
+        if (!ok) {
+          fail();
+          break;
         }
       }
       oz_commit(smem_u32(&bar_drain));  // completes once every MMA above has finished
@@ -524,6 +527,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const int r_local = lane_base + lane;
     const uint32_t tbase = tmem + (uint32_t(lane_base) << 16) + uint32_t(c0);
     int64_t chunks = 0;
+    bool stopped = false;
     for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
       const OzItem item = oz_item(w, whole, pieces, nch);
       const int64_t rt = item.tile / (2 * CT), ct = item.tile / 2 % CT;
@@ -535,50 +539,53 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         a[j] = 0ll;
         t[j] = 0.f;
       }
-      for (int64_t c = item.c0; c < item.c1; ++c, ++chunks) {
-        if (!oz_wait(smem_u32(&bar_accf), uint32_t(chunks & 1))) {
+      for (int64_t c = item.c0; c < item.c1 && !stopped; ++c, ++chunks) {
+        if (!oz_wait<true>(smem_u32(&bar_accf), uint32_t(chunks & 1))) {
           fail();
           fl_stop = 1;
         }
         asm volatile("bar.sync 1, 256;");  // the stop decision is the same in all eight warps
-        if (fl_stop) break;
+        stopped = fl_stop;
+        if (stopped) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
+        // eight columns of two orders at a time, the next ones on their way during the arithmetic
+        uint32_t v[2][8], u[2][8];
+        auto load = [&](int g, int j0, int buf) {  // orders g and g + 1
+          oz_ld8(tbase + uint32_t(g * OZ_TN + j0), v[buf]);
+          if (g + 1 <= G) oz_ld8(tbase + uint32_t((g + 1) * OZ_TN + j0), u[buf]);
+        };
+        auto digit = [](uint32_t x) { return __float2int_rn(__uint_as_float(x)); };
+        load(0, 0, 0);
 #pragma unroll
-        for (int h = 0; h < OZ_HN; h += 16) {
-          uint32_t v[16], u[16];
-          auto load = [&](int g) {  // orders g and g + 1
-            oz_ld16(tbase + uint32_t(g * OZ_TN + h), v);
-            if (g + 1 <= G) oz_ld16(tbase + uint32_t((g + 1) * OZ_TN + h), u);
-            oz_wait_ld(v, u);
-          };
-          auto digit = [](uint32_t x) { return __float2int_rn(__uint_as_float(x)); };
-          // orders 0 and 1: V_0 2^8 + V_1 fits 32 bits (|V_0| <= 2^22, |V_1| <= 2^23)
-          load(0);
+        for (int g = 0; g < OZ_ND; g += 2) {
+          if (g > G) break;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) a[h + j] += (long long)(digit(v[j]) * 256 + (G >= 1 ? digit(u[j]) : 0)) * 65536;
-          if (G >= 2) {
-            load(2);
+          for (int j0 = 0; j0 < OZ_HN; j0 += 8) {
+            const int buf = j0 >> 3 & 1;
+            oz_wait_ld(v[buf], u[buf]);
+            if (j0 + 8 < OZ_HN) load(g, j0 + 8, 1 - buf);
+            else if (g + 2 <= G) load(g + 2, 0, 0);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) a[h + j] += (long long)digit(v[j]) * 256 + (G >= 3 ? digit(u[j]) : 0);
-          }
-          if (G >= 4) {
-            load(4);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              t[h + j] = fmaf(__uint_as_float(v[j]), 0x1p-8f, t[h + j]);
-              if (G >= 5) t[h + j] = fmaf(__uint_as_float(u[j]), 0x1p-16f, t[h + j]);
+            for (int j = 0; j < 8; ++j) {
+              const float x = __uint_as_float(v[buf][j]), y = __uint_as_float(u[buf][j]);
+              if (g == 0)  // V_0 2^8 + V_1 fits 32 bits (|V_0| <= 2^22, |V_1| <= 2^23)
+                a[j0 + j] += (long long)(digit(v[buf][j]) * 256 + (G >= 1 ? digit(u[buf][j]) : 0)) * 65536;
+              else if (g == 2)
+                a[j0 + j] += (long long)digit(v[buf][j]) * 256 + (G >= 3 ? digit(u[buf][j]) : 0);
+              else if (g == 4)
+                t[j0 + j] = fmaf(x, 0x1p-8f, G >= 5 ? fmaf(y, 0x1p-16f, t[j0 + j]) : t[j0 + j]);
+              else
+                t[j0 + j] = fmaf(x, 0x1p-24f, t[j0 + j]);
             }
-          }
-          if (G >= 6) {
-            load(6);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) t[h + j] = fmaf(__uint_as_float(v[j]), 0x1p-24f, t[h + j]);
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;");
         oz_arrive(smem_u32(&bar_acce));
       }
-      if (fl_stop) break;
+      if (stopped) {  // what a wait that gave up leaves undone becomes NaN
+#pragma unroll
+        for (int j = 0; j < OZ_HN; ++j) t[j] = NAN;
+      }
       const int64_t row = rt * OZ_TM + r_local;
       if (!item.whole) {
         OzPart* p = part + ((w - whole) * OZ_TM + r_local) * OZ_TN + c0;
@@ -623,18 +630,28 @@ size_t oz_a_bytes(int64_t M, int64_t K) {
   return size_t((M + OZ_TM - 1) / OZ_TM) * size_t((K + OZ_KS - 1) / OZ_KS) * OZ_NT * OZ_ATILE;
 }
 
-cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s) {
-  if (M <= 0 || K <= 0) return cudaSuccess;
-  const int64_t KC = (K + OZ_KS - 1) / OZ_KS, MP = ((M + OZ_TM - 1) / OZ_TM) * OZ_TM;
-  if (MP / 8 > 65535) return cudaErrorInvalidValue;
-  ProfScope prof("oz_prep", s, 44.0 * double(M) * double(K));  // bytes read + written
-  oz_row_exp_kernel<<<oz_cdiv(M, 8), 256, 0, s>>>(static_cast<const double2*>(A), M, K, lda, ex);
-  oz_split_kernel<OZ_TM><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(MP / 8)), OZ_SPLIT_WARPS * 32, 0, s>>>(
-      static_cast<const double2*>(A), M, K, lda, 1, ex, KC, static_cast<unsigned char*>(digits));
+// Exponents and digit tiles of op(X) (rows x K after op, rows in tiles of TR)
+template <int TR>
+static cudaError_t oz_digits(const double2* X, int64_t rows, int64_t K, int64_t rs, int64_t ks, bool conj, int* ex,
+                             void* digits, cudaStream_t s) {
+  const int64_t KC = (K + OZ_KS - 1) / OZ_KS, RP = (rows + TR - 1) / TR * TR;
+  if (RP / 8 > 65535) return cudaErrorInvalidValue;
+  if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, ex);
+  else oz_col_exp_kernel<<<unsigned(rows), 256, 0, s>>>(X, K, rows, ks, ex);
+  oz_split_kernel<TR><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(RP / 8)), OZ_SPLIT_WARPS * 32, 0, s>>>(
+      X, rows, K, rs, ks, conj, ex, KC, static_cast<unsigned char*>(digits));
   return launched(2);
 }
 
-cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
+cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex,
+                         cudaStream_t s) {
+  if (M <= 0 || K <= 0) return cudaSuccess;
+  ProfScope prof("oz_prep", s, 44.0 * double(M) * double(K));  // bytes read + written
+  return oz_digits<OZ_TM>(static_cast<const double2*>(A), M, K, opA == OP_N ? lda : 1, opA == OP_N ? 1 : lda,
+                          opA == OP_C, ex, digits, s);
+}
+
+cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
                     const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
                     const int* ref_ex, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
@@ -665,10 +682,13 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a
   if (e != cudaSuccess) return e;
   OzPart* part = reinterpret_cast<OzPart*>(bd + bbytes);
   int* orders = reinterpret_cast<int*>(bd + bbytes + pbytes);
-  oz_col_exp_kernel<<<unsigned(N), 256, 0, s>>>(static_cast<const double2*>(B), K, N, ldb, b_ex);
+  e = oz_digits<OZ_TN>(static_cast<const double2*>(B), N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, opB == OP_C,
+                       b_ex, bd, s);
+  if (e != cudaSuccess) {
+    cudaFreeAsync(bd, s);
+    return e;
+  }
   oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, N, orders);
-  oz_split_kernel<OZ_TN><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(CT * OZ_TN / 8)), OZ_SPLIT_WARPS * 32, 0,
-                           s>>>(static_cast<const double2*>(B), N, K, 1, ldb, b_ex, KC, bd);
   {
     ProfScope prof("gemm_oz", s, 8.0 * double(M) * double(N) * double(K));
     oz_gemm_kernel<<<unsigned(std::min(items, sms)), OZ_THREADS, OZ_SMEM, s>>>(
@@ -678,9 +698,35 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a
       oz_reduce_kernel<<<dim3(unsigned(rem), OZ_TM * OZ_TN / 256), 256, 0, s>>>(
           M, N, whole, pieces, part, a_ex, b_ex, alpha, beta, static_cast<double*>(C), ldc);
   }
-  e = launched(pieces > 1 ? 5 : 4);
+  e = launched(pieces > 1 ? 3 : 2);
   cudaFreeAsync(bd, s);
   return e;
+}
+
+// FP64-class op(A) op(B) for any operands: digits of both, made here.  The digit path takes over at
+// K = 128: below, the passes over the outputs are most of either (digits / float-float, us: 1000 x
+// 1000 x 64 158 / 164, 3000 x 3000 x 32 707 / 650, 1000 x 1000 x 16 148 / 72), above it wins at any
+// M and N (100 x 16 x 100 91 / 131, 3 x 500 x 7503 630 / 653, 500 x 500 x 500 168 / 559, 7503 x 363
+// x 1089 980 / 5708, 7503 x 7503 x 642 9685 / 61614).
+cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,
+                                int64_t lda, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
+                                cudaStream_t s) {
+  if (M > 0 && N > 8 && K >= 128 && M <= 65535 * 8 - 128 &&
+      N <= 65535 * 8 - 64) {
+    char* d = nullptr;
+    const size_t ab = oz_a_bytes(M, K);
+    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), ab + sizeof(int) * size_t(M + N), s);
+    if (e == cudaSuccess) {
+      int* ex = reinterpret_cast<int*>(d + ab);
+      e = oz_prepare_a(opA, A, M, K, lda, d, ex, s);
+      if (e == cudaSuccess)
+        e = oz_gemm(opB, M, N, K, alpha, d, ex, B, ldb, beta, C, ldc, ex + M, nullptr, nullptr, s);
+      cudaFreeAsync(d, s);
+    }
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();  // no room for the digits (28 bytes per entry): float-float needs 16
+  }
+  return gemm_c128_ff(opA, opB, M, N, K, alpha, 0.0, A, lda, B, ldb, beta, C, ldc, s);
 }
 
 }  // namespace fosb
@@ -706,8 +752,8 @@ extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, con
   FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M + N)));
   FOSB_CUDA(st.alloc(sizeof(int)));
   FOSB_CUDA(cudaMemsetAsync(st.p, 0, sizeof(int), s));
-  FOSB_CUDA(oz_prepare_a(A, M, K, lda, dig.p, ex.as<int>(), s));
-  FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
+  FOSB_CUDA(oz_prepare_a(OP_N, A, M, K, lda, dig.p, ex.as<int>(), s));
+  FOSB_CUDA(oz_gemm(OP_N, M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
                     st.as<int>(), s));
   int status = 0;
   FOSB_CUDA(cudaMemcpyAsync(&status, st.p, sizeof(int), cudaMemcpyDeviceToHost, s));
