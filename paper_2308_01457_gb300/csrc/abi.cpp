@@ -377,11 +377,26 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
     fosb_lu_destroy(lu);
     return st;
   };
-  cudaError_t e = cudaMalloc(&lu->lu, elem * n * n);
+  // one allocation: cudaMalloc and cudaFree each stop the device for their mapping work
+  const bool c64 = prec != FOSB_FP64, mixed = prec == FOSB_MIXED, digits = mixed && n >= 256;
+  size_t bytes = 0;
+  auto part = [&](size_t b) {
+    const size_t at = bytes;
+    bytes += (b + 255) / 256 * 256;
+    return at;
+  };
+  const size_t o_lu = part(elem * n * n), o_ipiv = part(sizeof(int32_t) * n), o_status = part(sizeof(int) * 2);
+  const size_t o_zff = part(mixed ? sizeof(float) * 4 * n * n : 0), o_dig = part(digits ? oz_a_bytes(n, n) : 0);
+  const size_t o_ex = part(digits ? sizeof(int) * n : 0), o_dinv = part(c64 ? tri_block_inverses_bytes(n) : 0);
+  lu->pooled = tl_pool != nullptr;
+  lu->stream = s;
+  cudaError_t e = lu->pooled ? device_alloc(&lu->block, bytes, s) : cudaMalloc(&lu->block, bytes);
   if (e != cudaSuccess) return cleanup(cuda_fail(e, "fosb_factor: factor storage"));
-  if ((e = cudaMalloc(&lu->ipiv, sizeof(int32_t) * n)) != cudaSuccess ||
-      (e = cudaMalloc(&lu->d_status, sizeof(int) * 2)) != cudaSuccess)
-    return cleanup(cuda_fail(e, "fosb_factor: pivots"));
+  char* base = static_cast<char*>(lu->block);
+  lu->lu = base + o_lu;
+  lu->ipiv = reinterpret_cast<int32_t*>(base + o_ipiv);
+  lu->d_status = reinterpret_cast<int*>(base + o_status);
+  if (c64) lu->dinv = base + o_dinv;
   if ((e = cudaMemsetAsync(lu->d_status, 0, sizeof(int) * 2, s)) != cudaSuccess)
     return cleanup(cuda_fail(e, "fosb_factor"));
   if (prec == FOSB_FP64)
@@ -395,14 +410,14 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
     lu->zref = Z;
     lu->ldz = ldz;
     // the residual GEMMs read Z as (hi, lo) float pairs: split it once here (n x n float4)
-    if ((e = cudaMalloc(&lu->zff, sizeof(float) * 4 * n * n)) != cudaSuccess ||
-        (e = split_ff(Z, n, n, ldz, lu->zff, n, s)) != cudaSuccess)
+    lu->zff = base + o_zff;
+    if ((e = split_ff(Z, n, n, ldz, lu->zff, n, s)) != cudaSuccess)
       return cleanup(cuda_fail(e, "fosb_factor: split copy of Z"));
     // and as exact bf16 digits for residuals with many right-hand sides (about 28 n^2 bytes)
-    if (n >= 256) {
-      if ((e = cudaMalloc(&lu->zdig, oz_a_bytes(n, n))) != cudaSuccess ||
-          (e = cudaMalloc(reinterpret_cast<void**>(&lu->zex), sizeof(int) * n)) != cudaSuccess ||
-          (e = oz_prepare_a(OP_N, Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
+    if (digits) {
+      lu->zdig = base + o_dig;
+      lu->zex = reinterpret_cast<int*>(base + o_ex);
+      if ((e = oz_prepare_a(OP_N, Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
         return cleanup(cuda_fail(e, "fosb_factor: digit tiles of Z"));
     }
     Scratch nrm(s);
@@ -438,8 +453,7 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
       return cleanup(cuda_fail(e, "fosb_factor: permutation"));
   }
   if (prec != FOSB_FP64) {  // inverted diagonal blocks for the streaming triangular sweeps
-    if ((e = cudaMalloc(&lu->dinv, tri_block_inverses_bytes(n))) != cudaSuccess ||
-        (e = tri_block_inverses_c64(lu->lu, n, n, lu->dinv, s)) != cudaSuccess)
+    if ((e = tri_block_inverses_c64(lu->lu, n, n, lu->dinv, s)) != cudaSuccess)
       return cleanup(cuda_fail(e, "fosb_factor: diagonal-block inverses"));
   }
   *out = lu;
@@ -464,13 +478,10 @@ fosb_status fosb_lu_info(fosb_lu lu, int64_t* n, int* prec, double* znorm_inf) {
 
 fosb_status fosb_lu_destroy(fosb_lu lu) {
   if (!lu) return FOSB_OK;
-  if (lu->lu) cudaFree(lu->lu);
-  if (lu->ipiv) cudaFree(lu->ipiv);
-  if (lu->d_status) cudaFree(lu->d_status);
-  if (lu->zff) cudaFree(lu->zff);
-  if (lu->dinv) cudaFree(lu->dinv);
-  if (lu->zdig) cudaFree(lu->zdig);
-  if (lu->zex) cudaFree(lu->zex);
+  if (lu->block) {
+    if (lu->pooled) cudaFreeAsync(lu->block, lu->stream);
+    else cudaFree(lu->block);
+  }
   delete lu;
   return FOSB_OK;
 }

@@ -47,11 +47,18 @@ class ProfScope {
 };
 
 // Stream-ordered scratch buffer released at scope exit.
+// Stream-ordered device memory of the calling thread: from the device's default pool, or from the
+// pool that a call has given its worker threads (fosb_solve_batched).
+extern thread_local cudaMemPool_t tl_pool;
+inline cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s) {
+  return tl_pool ? cudaMallocFromPoolAsync(p, bytes, tl_pool, s) : cudaMallocAsync(p, bytes, s);
+}
+
 struct Scratch {
   void* p = nullptr;
   cudaStream_t s = nullptr;
   explicit Scratch(cudaStream_t st) : s(st) {}
-  cudaError_t alloc(size_t bytes) { return cudaMallocAsync(&p, bytes > 16 ? bytes : size_t(16), s); }
+  cudaError_t alloc(size_t bytes) { return device_alloc(&p, bytes > 16 ? bytes : size_t(16), s); }
   ~Scratch() {
     if (p) cudaFreeAsync(p, s);
   }
@@ -118,12 +125,16 @@ struct fosb_lu_s {
   int device = 0;
   int prec = 0;
   int64_t n = 0;
+  void* block = nullptr;       // the one allocation that the arrays below share
+  bool pooled = false;         // block is stream-ordered memory of `stream`, else from cudaMalloc
+  cudaStream_t stream = nullptr;
   void* lu = nullptr;          // n x n factors (complex128 for FP64, complex64 otherwise), row-major ld = n
   int32_t* ipiv = nullptr;     // composed row permutation, device
   const void* zref = nullptr;  // MIXED: non-owning complex128 Z for residuals
   int64_t ldz = 0;
   void* zff = nullptr;         // MIXED: (hi, lo) float split of Z (n x n float4) for the residual GEMMs
-  void* dinv = nullptr;        // complex64 factors: inverses of the 64 x 64 diagonal blocks of L, then of U
+  void* dinv = nullptr;        // complex64 factors: inverses of the 64 x 64 diagonal blocks of L, then of U, then
+                               // their products with the neighbouring tiles
   void* zdig = nullptr;        // MIXED: bf16 digit tiles of Z for the tensor-core residual GEMMs (oz_gemm)
   int* zex = nullptr;          // MIXED: their row exponents
   double znorm_inf = 0.0;      // ||Z||_inf (FP64)

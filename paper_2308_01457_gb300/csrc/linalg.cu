@@ -1144,7 +1144,7 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
   // cached split of A when there is one, else FP64 (a 64-wide tile would be mostly padding)
   if (K > 0 && opA == OP_N && opB == OP_N && N <= 8 && A_split) {
     float4* bs = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&bs), size_t(K * N) * sizeof(float4), s);
+    cudaError_t e = device_alloc(reinterpret_cast<void**>(&bs), size_t(K * N) * sizeof(float4), s);
     if (e == cudaSuccess) e = split_ff(B, K, N, ldb, bs, N, s);
     if (e == cudaSuccess) {
       ProfScope prof("gemm_ff", s, 8.0 * double(M) * double(N) * double(K));
@@ -1176,10 +1176,10 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
   const int64_t ar = opA == OP_N ? M : K, ac = opA == OP_N ? K : M;
   const int64_t br = opB == OP_N ? K : N, bc = opB == OP_N ? N : K;
   float4 *as = nullptr, *bs = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&bs), size_t(br * bc) * sizeof(float4), s);
+  cudaError_t e = device_alloc(reinterpret_cast<void**>(&bs), size_t(br * bc) * sizeof(float4), s);
   if (e == cudaSuccess) e = split_ff(B, br, bc, ldb, bs, bc, s);
   if (e == cudaSuccess && !A_split) {
-    e = cudaMallocAsync(reinterpret_cast<void**>(&as), size_t(ar * ac) * sizeof(float4), s);
+    e = device_alloc(reinterpret_cast<void**>(&as), size_t(ar * ac) * sizeof(float4), s);
     if (e == cudaSuccess) e = split_ff(A, ar, ac, lda, as, ac, s);
   }
   const float4* a4 = A_split ? static_cast<const float4*>(A_split) : as;
@@ -1232,7 +1232,7 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
   size_t G_cap = size_t(std::min<int64_t>(gmax, std::max<int64_t>(1, (n + 63) / 64)));
   size_t bytes = 256 + 2 * G_cap * nb * sizeof(V) + 2 * nb * sizeof(V);
   char* scratch = nullptr;
-  FOSB_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&scratch), bytes, s));
+  FOSB_CUDA(device_alloc(reinterpret_cast<void**>(&scratch), bytes, s));
   FOSB_CUDA(cudaMemsetAsync(scratch, 0, 256, s));
   PanelScratch* scr = reinterpret_cast<PanelScratch*>(scratch);
   V* cand_data = reinterpret_cast<V*>(scratch + 256);
@@ -1245,9 +1245,9 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
   void* ws_a = nullptr;  // complex64: the trailing update's operands, split once per block
   void* ws_b = nullptr;
   if constexpr (sizeof(T) == 4) {
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tslu_scr), tslu_scratch_bytes(n), s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&ws_a, update_split_a_bytes(n), s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&ws_b, update_split_b_bytes(n), s);
+    cudaError_t e = device_alloc(reinterpret_cast<void**>(&tslu_scr), tslu_scratch_bytes(n), s);
+    if (e == cudaSuccess) e = device_alloc(&ws_a, update_split_a_bytes(n), s);
+    if (e == cudaSuccess) e = device_alloc(&ws_b, update_split_b_bytes(n), s);
     if (e == cudaSuccess) e = tslu_identity(ipiv, n, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(scratch, s);
@@ -1430,7 +1430,7 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
   // complex64 rows start on 16 bytes: the tensor-core updates then move two values at a time
   // (163 columns at N = 7503, one sweep by superblocks 1.57 ms with rows of 163, 1.28 ms with rows of 164)
   const int64_t ldt = sizeof(T) == 4 ? nrhs + (nrhs & 1) : nrhs;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(V) * n * ldt, s);
+  cudaError_t e = device_alloc(reinterpret_cast<void**>(&tmp), sizeof(V) * n * ldt, s);
   if (e != cudaSuccess) return e;
   gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, ldt);
   if constexpr (sizeof(T) == 4) {
@@ -1438,7 +1438,7 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
     if (!status || !dinv) e = cudaErrorInvalidValue;
     char* y = nullptr;
     const size_t ybytes = sizeof(V) * size_t(n) * size_t(ldt);
-    if (e == cudaSuccess) e = cudaMallocAsync(reinterpret_cast<void**>(&y), ybytes + 4 * trsv_stream_tickets(n) + 16, s);
+    if (e == cudaSuccess) e = device_alloc(reinterpret_cast<void**>(&y), ybytes + 4 * trsv_stream_tickets(n) + 16, s);
     int* tickets = reinterpret_cast<int*>(y + ybytes);
     if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, ldt, 0, tickets, status, s);
     if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, ldt, 1, tickets, status, s);

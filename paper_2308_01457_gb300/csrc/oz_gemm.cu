@@ -678,7 +678,7 @@ cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, cons
   const size_t bbytes = size_t(CT) * size_t(KC) * OZ_BSLOT;
   const size_t pbytes = pieces > 1 ? sizeof(OzPart) * size_t(rem * pieces) * OZ_TM * OZ_TN : 0;
   unsigned char* bd = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&bd), bbytes + pbytes + sizeof(int) * size_t(CT), s);
+  cudaError_t e = device_alloc(reinterpret_cast<void**>(&bd), bbytes + pbytes + sizeof(int) * size_t(CT), s);
   if (e != cudaSuccess) return e;
   OzPart* part = reinterpret_cast<OzPart*>(bd + bbytes);
   int* orders = reinterpret_cast<int*>(bd + bbytes + pbytes);
@@ -715,7 +715,7 @@ cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t 
       N <= 65535 * 8 - 64) {
     char* d = nullptr;
     const size_t ab = oz_a_bytes(M, K);
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), ab + sizeof(int) * size_t(M + N), s);
+    cudaError_t e = device_alloc(reinterpret_cast<void**>(&d), ab + sizeof(int) * size_t(M + N), s);
     if (e == cudaSuccess) {
       int* ex = reinterpret_cast<int*>(d + ab);
       e = oz_prepare_a(opA, A, M, K, lda, d, ex, s);
