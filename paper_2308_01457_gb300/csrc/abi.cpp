@@ -257,8 +257,8 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       res = std::max(res, bn[c] > 0 ? rn[c] / bn[c] : rn[c]);
     }
     if (it == 0) res0 = res;
-    if (berr <= tol && own_tol && berr > 0.25 * tol && it < max_iters) {
-      // just below the default tolerance, whose last factor of 4 is above the rounding floor: the
+    if (berr <= tol && own_tol && berr > 0.0625 * tol && it < max_iters) {
+      // just below the default tolerance, whose last factor of 16 is above the rounding floor: the
       // correction that this residual gives is worth its sweep (a better factorisation may stop a
       // step earlier and must not end further off)
       FOSB_CUDA(convert_c128_to_c64(r.p, n, nrhs, nrhs, d.p, nrhs, s));
