@@ -8,10 +8,12 @@
 // Per point pair (x_p on the test triangle, y_q on the trial triangle):
 //   d = (o1 - o2) + (x_p - o1) - (y_q - o2);  r = |d| (rsqrt seed + one Newton step);
 //   1/r (Newton step on the seed); theta = k r;
-//   exp(i theta): theta = j pi/64 + delta (Cody-Waite with a 3-part pi/64, j < 1024),
-//   sin/cos(delta) by Taylor series to delta^7 (|delta| <= pi/128) in float-float for
-//   the leading terms, combined with a 128-entry table of sin/cos(j pi/64);
+//   exp(i theta): theta = j pi/512 + delta (Cody-Waite, j < 8192), combined with a 1024-entry table of
+//   sin/cos(j pi/512); |delta| <= pi/1024, so sin(delta) - delta and cos(delta) - 1 are a few FP32
+//   terms and only two products and their sum need error-free transformations;
 //   G0 = exp(i theta)/r.
+// What bounds it is FP32 issue (about 430 instructions per point pair).  N = 30720, 7.5 G point pairs: 96
+// ms (106 with a 128-entry phase table and FP32 rounding and conversion on the slow pipe).
 // The pair's 3 x 3 barycentric moment matrix
 //   mu_ab = sum_pq w_p w_q lambda_pa beta_qb G0(x_p, y_q)
 // determines the RWG block exactly (with P_a, Q_b the vertices):
@@ -75,6 +77,15 @@ __device__ __forceinline__ ff ff_sqr(ff a) {
   e = fmaf(2.0f * a.h, a.l, e);
   return fast_two_sum(p, e);
 }
+// a b as p + e with |e| up to a few ulp of p: for operands of further products and sums
+__device__ __forceinline__ ff mul_raw(ff a, ff b) {
+  const float p = a.h * b.h;
+  return {p, fmaf(a.h, b.l, fmaf(a.l, b.h, fmaf(a.h, b.h, -p)))};
+}
+__device__ __forceinline__ ff sqr_raw(ff a) {
+  const float p = a.h * a.h;
+  return {p, fmaf(a.h + a.h, a.l, fmaf(a.h, a.h, -p))};
+}
 // acc += a * c (compensated; acc is renormalised by the caller when read)
 __device__ __forceinline__ void acc_mul(ff& acc, ff a, ff c) {
   float p = a.h * c.h;
@@ -93,13 +104,14 @@ struct CFF {
   ff r, i;
 };
 
-// constants: sin / cos (j pi / 64), j = 0..127, as (S.h, S.l, C.h, C.l); w_q beta_qb as ff
-__constant__ float c_sctab[128][4];
+// sin / cos (j pi / 512), j = 0..1023, as (S.h, S.l, C.h, C.l); w_q beta_qb as ff
+constexpr int kSinCos = 1024;
+__device__ float4 g_sctab[kSinCos];
 __constant__ float c_wb[6][3][2];
 
 struct FFConst {
-  ff k, k4, kinv, inv4pi, sixth;
-  float c1, c2, c3, inv_c;  // pi/64 = c1 + c2 + c3 (c1, c2 with <= 14 significant bits); 64/pi
+  ff k, k4, kinv, inv4pi;
+  float c1, c2, c3, inv_c;  // pi/512 = c1 + c2 + c3; 512/pi
 };
 
 // (32-bit indices: a dense Z on this card has fewer than 2^17 triangles, 60 nt < 2^31)
@@ -107,30 +119,31 @@ __device__ __forceinline__ ff ldff(const float* base, int nt, int f, int t) {
   return {base[f * nt + t], base[(f + 1) * nt + t]};
 }
 
-// exp(i theta) for theta = th + tl >= 0, |j| < 1024, table in shared memory
-__device__ __forceinline__ void expi_ff(ff theta, const FFConst& C, const float (*tab)[4], ff& cs, ff& sn) {
-  const float jf = rintf(theta.h * C.inv_c);
-  const int j = int(jf);
-  float a = fmaf(-jf, C.c1, theta.h);  // exact
-  ff dl = two_sum(a, -jf * C.c2);      // jf * c2 exact
-  dl.l += theta.l - jf * C.c3;
-  dl = fast_two_sum(dl.h, dl.l);
-  const ff d2 = ff_sqr(dl);
-  const float d2h = d2.h;
-  // sin(delta) = delta (1 - d2/6 + d2^2/120 - d2^3/5040)
-  ff t = ff_mul(d2, C.sixth);
-  ff ps = fast_two_sum(1.0f, -t.h);
-  ps.l += -t.l + d2h * d2h * (1.0f / 120.0f - d2h * (1.0f / 5040.0f));
-  ps = norm(ps);
-  const ff sd = ff_mul(dl, ps);
-  // cos(delta) = 1 - d2/2 + d2^2/24 - d2^3/720
-  ff cd = fast_two_sum(1.0f, -0.5f * d2.h);
-  cd.l += -0.5f * d2.l + d2h * d2h * (1.0f / 24.0f - d2h * (1.0f / 720.0f));
-  cd = norm(cd);
-  const int idx = j & 127;
-  const ff S = {tab[idx][0], tab[idx][1]}, Cc = {tab[idx][2], tab[idx][3]};
-  sn = ff_add_fast(ff_mul(S, cd), ff_mul(Cc, sd));
-  cs = ff_add(ff_mul(Cc, cd), ff_neg(ff_mul(S, sd)));
+// B (1 + c) + A d for small c and d: two products and two sums with their errors
+__device__ __forceinline__ ff rotate_part(float Bh, float Bl, float Ah, float Al, ff d, ff c) {
+  const ff u = mul_raw({Ah, Al}, d), v = mul_raw({Bh, Bl}, c);
+  const ff t = two_sum(u.h, v.h), s = two_sum(Bh, t.h);
+  return {s.h, s.l + ((t.l + u.l) + (v.l + Bl))};
+}
+// exp(i theta) for theta = th + tl in [0, kFFMaxPhase), table in shared memory.  jf c1 - th is exact (c1 has
+// 24 bits and the difference fewer), jf c2 is split by an FMA.  Absolute error, CPU model of this code on
+// 400,000 phases: rms 2^-50.1, largest 2^-47.2 over [0, 48) (with a 128-entry table, sin(delta) and
+// cos(delta) to delta^7 in float-float and pi/64 in 14-bit parts: 2^-46.3, 2^-43.1).
+__device__ __forceinline__ void expi_ff(ff theta, const FFConst& C, const float4* tab, ff& cs, ff& sn) {
+  const float shifted = fmaf(theta.h, C.inv_c, 12582912.0f);  // j in the low bits
+  const float jf = shifted - 12582912.0f;
+  const float4 T = tab[__float_as_uint(shifted) & (kSinCos - 1)];
+  const float a = fmaf(-jf, C.c1, theta.h);
+  const float b = -jf * C.c2, be = fmaf(-jf, C.c2, -b);
+  const ff w = two_sum(b, theta.l);
+  ff dl = two_sum(a, w.h);
+  dl.l = fmaf(-jf, C.c3, dl.l + (w.l + be));
+  const ff d2 = sqr_raw(dl);
+  // sin(delta) = delta (1 - d2/6 + d2^2/120), cos(delta) - 1 = -d2/2 + d2^2/24
+  const ff sd = {dl.h, fmaf(dl.h, d2.h * fmaf(d2.h, 1.0f / 120.0f, -1.0f / 6.0f), dl.l)};
+  const ff c1 = {-0.5f * d2.h, fmaf(d2.h * d2.h, 1.0f / 24.0f, -0.5f * d2.l)};
+  sn = rotate_part(T.x, T.y, T.z, T.w, sd, c1);
+  cs = rotate_part(T.z, T.w, -T.x, -T.y, sd, c1);
 }
 
 // One regular point pair block: test triangle t1, trial triangle t2 (t1 < t2 < m.nt); adds the
@@ -143,7 +156,7 @@ __device__ __forceinline__ void expi_ff(ff theta, const FFConst& C, const float 
 // gives K_ij = -(s_i l_i s'_j l'_j / (16 pi)) sum_ab nu_ab (p_i - q_j).((Q_b - q_j) x (P_a - p_i)).
 template <bool MFIO>
 __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst& C, double* Z, double* ZK,
-                                                int64_t ldz, int t1, int t2, const float (*tab)[4]) {
+                                                int64_t ldz, int t1, int t2, const float4* tab) {
   const int nt = int(m.nt);
   int v1[3], v2[3];
 #pragma unroll
@@ -177,78 +190,74 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
     ff E[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) E[c] = ff_add(D[c], ldff(F, nt, (p * 3 + c) * 2, t1));
-    CFF A[3], B[MFIO ? 3 : 1];
+    CFF A[MFIO ? 2 : 1][3];
 #pragma unroll
-    for (int b = 0; b < 3; ++b) A[b] = CFF{{0.f, 0.f}, {0.f, 0.f}};
-    if constexpr (MFIO) {
+    for (int f = 0; f < (MFIO ? 2 : 1); ++f)
 #pragma unroll
-      for (int b = 0; b < 3; ++b) B[b] = CFF{{0.f, 0.f}, {0.f, 0.f}};
-    }
+      for (int b = 0; b < 3; ++b) A[f][b] = CFF{{0.f, 0.f}, {0.f, 0.f}};
     // two point pairs per iteration: enough independent work per warp, a third of the code
-    // of a full unroll (instruction fetch bounded the fully unrolled loop)
-#pragma unroll 2
+    // of a full unroll (instruction fetch bounded the fully unrolled loop); with the MFIO one, whose
+    // registers then let four CTAs share an SM instead of three (PMCHWT, N = 7680: 37.0 -> 33.2 ms)
+    constexpr int kUnroll = MFIO ? 1 : 2;
+#pragma unroll kUnroll
     for (int q = 0; q < 6; ++q) {
-      ff dx = ff_add_fast(E[0], ff_neg(ldff(F, nt, (q * 3 + 0) * 2, t2)));
-      ff dy = ff_add_fast(E[1], ff_neg(ldff(F, nt, (q * 3 + 1) * 2, t2)));
-      ff dz = ff_add_fast(E[2], ff_neg(ldff(F, nt, (q * 3 + 2) * 2, t2)));
-      ff r2 = ff_add_fast(ff_add_fast(ff_sqr(dx), ff_sqr(dy)), ff_sqr(dz));
+      const ff dx = ff_add_fast(E[0], ff_neg(ldff(F, nt, (q * 3 + 0) * 2, t2)));
+      const ff dy = ff_add_fast(E[1], ff_neg(ldff(F, nt, (q * 3 + 1) * 2, t2)));
+      const ff dz = ff_add_fast(E[2], ff_neg(ldff(F, nt, (q * 3 + 2) * 2, t2)));
+      const ff xx = ff_sqr(dx), yy = ff_sqr(dy), zz = ff_sqr(dz);
+      const ff r2 = ff_add_fast(ff_add_fast(xx, yy), zz);
       const float y0 = rsqrtf(r2.h);
       const float s0 = r2.h * y0;
       const float er = fmaf(-s0, s0, r2.h) + r2.l;
       const ff r = fast_two_sum(s0, er * (0.5f * y0));
-      const ff rq = ff_mul_f(r, y0);                     // r * y0 ~ 1
-      const float corr = ((1.0f - rq.h) - rq.l) * y0;    // 1 - rq.h exact (rq.h ~ 1)
+      const ff rq = ff_mul_f(r, y0);                   // r * y0 ~ 1
+      const float corr = ((1.0f - rq.h) - rq.l) * y0;  // 1 - rq.h exact (rq.h ~ 1)
       const ff rinv = fast_two_sum(y0, corr);
       ff cs, sn;
       const ff kr = ff_mul(C.k, r);
       expi_ff(kr, C, tab, cs, sn);
-      const CFF G = {ff_mul(cs, rinv), ff_mul(sn, rinv)};
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const ff wb = {c_wb[q][b][0], c_wb[q][b][1]};
-        acc_mul(A[b].r, G.r, wb);
-        acc_mul(A[b].i, G.i, wb);
-      }
+      CFF G[MFIO ? 2 : 1];
+      G[0] = {mul_raw(cs, rinv), mul_raw(sn, rinv)};
       if constexpr (MFIO) {
         // g = G (ikr - 1) / r^2: Re = -(G.r + G.i kr) / r^2, Im = (G.r kr - G.i) / r^2
         const ff rinv2 = ff_sqr(rinv);
-        const CFF g = {ff_neg(ff_mul(ff_add(G.r, ff_mul(G.i, kr)), rinv2)),
-                       ff_mul(ff_add(ff_mul(G.r, kr), ff_neg(G.i)), rinv2)};
+        G[1] = {ff_neg(mul_raw(ff_add_fast(G[0].r, mul_raw(G[0].i, kr)), rinv2)),
+                mul_raw(ff_add_fast(mul_raw(G[0].r, kr), ff_neg(G[0].i)), rinv2)};
+      }
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-          const ff wb = {c_wb[q][b][0], c_wb[q][b][1]};
-          acc_mul(B[b].r, g.r, wb);
-          acc_mul(B[b].i, g.i, wb);
+      for (int b = 0; b < 3; ++b) {
+        const ff wb = {c_wb[q][b][0], c_wb[q][b][1]};
+#pragma unroll
+        for (int f = 0; f < (MFIO ? 2 : 1); ++f) {
+          acc_mul(A[f][b].r, G[f].r, wb);
+          acc_mul(A[f][b].i, G[f].i, wb);
         }
       }
     }
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      A[b].r = norm(A[b].r);
-      A[b].i = norm(A[b].i);
-    }
+    for (int f = 0; f < (MFIO ? 2 : 1); ++f)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        A[f][b].r = norm(A[f][b].r);
+        A[f][b].i = norm(A[f][b].i);
+      }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const ff wa = {c_wb[p][a][0], c_wb[p][a][1]};
 #pragma unroll
       for (int b = 0; b < 3; ++b) {
-        acc_mul(mu[a][b].r, A[b].r, wa);
-        acc_mul(mu[a][b].i, A[b].i, wa);
+        acc_mul(mu[a][b].r, A[0][b].r, wa);
+        acc_mul(mu[a][b].i, A[0][b].i, wa);
       }
     }
     if constexpr (MFIO) {
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        B[b].r = norm(B[b].r);
-        B[b].i = norm(B[b].i);
-      }
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const ff wa = {c_wb[p][a][0], c_wb[p][a][1]};
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-          acc_mul(nu[a][b].r, B[b].r, wa);
-          acc_mul(nu[a][b].i, B[b].i, wa);
+          acc_mul(nu[a][b].r, A[1][b].r, wa);
+          acc_mul(nu[a][b].i, A[1][b].i, wa);
         }
       }
     }
@@ -396,8 +405,8 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
 __global__ void __launch_bounds__(128) efie_regular_ff_kernel(DevMesh m, FFConst C, double* Z, int64_t ldz) {
   int64_t rg, cb;
   if (!pair_tile(m.nt, 4, blockIdx.y, blockIdx.x, rg, cb)) return;
-  __shared__ float tab[128][4];
-  for (int e = threadIdx.x; e < 128 * 4; e += blockDim.x) tab[e >> 2][e & 3] = c_sctab[e >> 2][e & 3];
+  __shared__ float4 tab[kSinCos];
+  for (int e = threadIdx.x; e < kSinCos; e += blockDim.x) tab[e] = g_sctab[e];
   __syncthreads();
   const int t1 = int(rg) * 4 + (threadIdx.x >> 5), t2 = int(cb) * 32 + (threadIdx.x & 31);
   if (t2 >= int(m.nt) || t1 >= t2) return;
@@ -405,12 +414,12 @@ __global__ void __launch_bounds__(128) efie_regular_ff_kernel(DevMesh m, FFConst
 }
 
 // Dielectric (PMCHWT) system: the EFIO block into ZT and the MFIO block into ZK.
-__global__ void __launch_bounds__(128, 3) pmchwt_regular_ff_kernel(DevMesh m, FFConst C, double* ZT, double* ZK,
+__global__ void __launch_bounds__(128, 4) pmchwt_regular_ff_kernel(DevMesh m, FFConst C, double* ZT, double* ZK,
                                                                 int64_t ldz) {
   int64_t rg, cb;
   if (!pair_tile(m.nt, 4, blockIdx.y, blockIdx.x, rg, cb)) return;
-  __shared__ float tab[128][4];
-  for (int e = threadIdx.x; e < 128 * 4; e += blockDim.x) tab[e >> 2][e & 3] = c_sctab[e >> 2][e & 3];
+  __shared__ float4 tab[kSinCos];
+  for (int e = threadIdx.x; e < kSinCos; e += blockDim.x) tab[e] = g_sctab[e];
   __syncthreads();
   const int t1 = int(rg) * 4 + (threadIdx.x >> 5), t2 = int(cb) * 32 + (threadIdx.x & 31);
   if (t2 >= int(m.nt) || t1 >= t2) return;
@@ -434,11 +443,11 @@ template <int WARPS, int MINB>
 __global__ void __launch_bounds__(WARPS * 32, MINB) efie_regular_ff_batched_kernel(const FFBatchItem* __restrict__ items,
                                                                              int nitems, int64_t total_tiles,
                                                                              unsigned long long* ticket) {
-  __shared__ float tab[128][4];
+  __shared__ float4 tab[kSinCos];
   __shared__ FFBatchItem s_item;
   __shared__ long long s_tile;
   __shared__ int s_idx;
-  for (int e = threadIdx.x; e < 128 * 4; e += blockDim.x) tab[e >> 2][e & 3] = c_sctab[e >> 2][e & 3];
+  for (int e = threadIdx.x; e < kSinCos; e += blockDim.x) tab[e] = g_sctab[e];
   int cur = -1;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -487,32 +496,29 @@ ff split_ff(double x) {
   split(x, r.h, r.l);
   return r;
 }
-// round a double to a float with at most `bits` significant bits
-float truncate_bits(double x, int bits) {
-  int e;
-  double m = std::frexp(x, &e);  // x = m 2^e, 0.5 <= |m| < 1
-  double scale = std::ldexp(1.0, bits);
-  return float(std::ldexp(std::nearbyint(m * scale) / scale, e));
-}
-
 }  // namespace
 
 void upload_rules_ff(const Rules& r) {
-  float tab[128][4];
-  for (int j = 0; j < 128; ++j) {
-    double th = j * M_PI / 64.0;
-    split(std::sin(th), tab[j][0], tab[j][1]);
-    split(std::cos(th), tab[j][2], tab[j][3]);
+  std::vector<float4> tab(kSinCos);
+  for (int j = 0; j < kSinCos; ++j) {
+    // from the first octant, where the angle's own rounding is below 2^-54
+    const int quarter = j / (kSinCos / 4), m = j % (kSinCos / 4), n = kSinCos / 4 - m;
+    const bool low = m <= kSinCos / 8;
+    const double th = 2.0 * M_PI / kSinCos * (low ? m : n);
+    const double s0 = low ? std::sin(th) : std::cos(th), c0 = low ? std::cos(th) : std::sin(th);
+    const double sn[4] = {s0, c0, -s0, -c0};
+    split(sn[quarter], tab[j].x, tab[j].y);
+    split(sn[(quarter + 1) % 4], tab[j].z, tab[j].w);
   }
-  cudaMemcpyToSymbol(c_sctab, tab, sizeof(tab));
+  cudaMemcpyToSymbol(g_sctab, tab.data(), sizeof(float4) * kSinCos);
   float wb[6][3][2];
   for (int q = 0; q < 6; ++q)
     for (int b = 0; b < 3; ++b) split(r.w[q] * r.bary[q][b], wb[q][b][0], wb[q][b][1]);
   cudaMemcpyToSymbol(c_wb, wb, sizeof(wb));
 }
 
-// k * diameter must stay below kFFMaxPhase: the phase index j = rint(k r 64/pi) then
-// stays below 1024, which keeps j * c1 and j * c2 exact in FP32.
+// k * diameter must stay below kFFMaxPhase: the phase index j = rint(k r 512/pi) then
+// stays below 8192, which keeps theta - j c1 exact in FP32.
 double ff_max_phase() { return 48.0; }
 
 namespace {
@@ -522,12 +528,12 @@ FFConst make_ff_const(double k) {
   C.k4 = split_ff(k / 4.0);
   C.kinv = split_ff(1.0 / k);
   C.inv4pi = split_ff(1.0 / (4.0 * M_PI));
-  C.sixth = split_ff(1.0 / 6.0);
-  const double pi64 = M_PI / 64.0;
-  C.c1 = truncate_bits(pi64, 14);
-  C.c2 = truncate_bits(pi64 - double(C.c1), 14);
-  C.c3 = float(pi64 - double(C.c1) - double(C.c2));
-  C.inv_c = float(64.0 / M_PI);
+  // pi = M_PI + 1.2246467991473532e-16 (Cody-Waite constants from 107 bits)
+  const double hi = M_PI / 512.0, lo = 1.2246467991473532e-16 / 512.0;
+  C.c1 = float(hi);
+  C.c2 = float(hi - double(C.c1));
+  C.c3 = float((hi - double(C.c1) - double(C.c2)) + lo);
+  C.inv_c = float(512.0 / M_PI);
   return C;
 }
 }  // namespace
