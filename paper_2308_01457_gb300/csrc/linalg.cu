@@ -725,6 +725,7 @@ __global__ void __launch_bounds__(kPanelThreads) panel_smem_kernel(typename C2<T
   const int nr = hi > lo ? int(hi - lo) : 0;
   __shared__ unsigned long long s_key[kPanelThreads / 32];
   __shared__ V s_piv[64];
+  __shared__ V s_inv;
   __shared__ int64_t s_p;
   // identity pivots first: if a barrier wait gives up, the columns not reached keep valid rows
   if (blockIdx.x == 0)
@@ -774,6 +775,11 @@ __global__ void __launch_bounds__(kPanelThreads) panel_smem_kernel(typename C2<T
     const int64_t p = s_p;
     const V* pdata = cand_data + (int64_t(par) * G + p / chunk) * jb;
     for (int c = threadIdx.x; c < jb; c += blockDim.x) s_piv[c] = __ldcg(pdata + c);
+    if (threadIdx.x == j) {  // the thread that has just stored it; the FP64 divisions by one thread, not by all
+      const V pv = s_piv[j];
+      const T den = pv.x * pv.x + pv.y * pv.y;
+      s_inv = den > T(0) ? V{pv.x / den, -pv.y / den} : V{T(0), T(0)};
+    }
     __syncthreads();
     if (p != j) {
       if (j >= lo && j < hi)
@@ -782,9 +788,7 @@ __global__ void __launch_bounds__(kPanelThreads) panel_smem_kernel(typename C2<T
         for (int c = threadIdx.x; c < jb; c += blockDim.x) sP[(p - lo) * jb + c] = __ldcg(rowj + par * jb + c);
     }
     __syncthreads();
-    const V pv = s_piv[j];
-    const T den = pv.x * pv.x + pv.y * pv.y;
-    const V inv = den > T(0) ? V{pv.x / den, -pv.y / den} : V{T(0), T(0)};
+    const V inv = s_inv;
     const int r0 = (int64_t(j) + 1 > lo) ? int(int64_t(j) + 1 - lo) : 0;
     for (int r = r0 + threadIdx.x; r < nr; r += blockDim.x) sP[r * jb + j] = cmul<T>(sP[r * jb + j], inv);
     __syncthreads();
@@ -1029,8 +1033,13 @@ cudaError_t launch_panel(typename C2<T>::type* Ap, int64_t m, int jb, int64_t ld
     attr[dev] = true;
   }
   const int64_t rows_cap = kPanelSmemBudget / (int64_t(jb) * int64_t(sizeof(V)));
+  // rows per CTA: the FP64 update of a column takes 64 clocks per row on an SM's FP64 pipe, against
+  // 2 us for the barrier of any number of CTAs.  Panels of an N = 1920 (7680) factorisation: 27.7 (118)
+  // ms with 192 rows per CTA and the division by every thread, 15.2 (61) with 64, 12.0 (50) with
+  // 32, 10.4 (47) with 16.
+  const int64_t rows = sizeof(T) == 8 ? 16 : 256;
   int64_t G = std::min<int64_t>(std::min<int64_t>(G_cap, nsm),
-                                std::max<int64_t>((m + rows_cap - 1) / rows_cap, (m + 255) / 256));
+                                std::max<int64_t>((m + rows_cap - 1) / rows_cap, (m + rows - 1) / rows));
   G = std::max<int64_t>(G, 1);
   const int64_t chunk = (m + G - 1) / G;
   const size_t smem = size_t(chunk) * jb * sizeof(V);
@@ -1229,7 +1238,7 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
   if (per_sm < 1) return fail(FOSB_ERR_CUDA, "getrf: panel kernel cannot be resident");
   const int gmax = nsm * per_sm;
   // scratch: barrier/key header + candidate rows + row j (double-buffered)
-  size_t G_cap = size_t(std::min<int64_t>(gmax, std::max<int64_t>(1, (n + 63) / 64)));
+  size_t G_cap = size_t(std::min<int64_t>(std::min(gmax, nsm), std::max<int64_t>(1, (n + 15) / 16)));
   size_t bytes = 256 + 2 * G_cap * nb * sizeof(V) + 2 * nb * sizeof(V);
   char* scratch = nullptr;
   FOSB_CUDA(device_alloc(reinterpret_cast<void**>(&scratch), bytes, s));
