@@ -245,6 +245,11 @@ cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t l
 cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
                     const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
                     int* status, cudaStream_t s);
+// C <- C - L U (M x K, K x N) of an FP64 factorisation in digits, rows and columns of the operands
+// balanced first; scratch: oz_update_bytes(max(M, N), K).
+size_t oz_update_bytes(int64_t n, int64_t K);
+cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
+                      int64_t ldc, void* scratch, int* status, cudaStream_t s);
 // C <- beta C + alpha op(A) op(B) in FP64-class arithmetic: digits where the product is large
 // enough to pay for making them, float-float (gemm_c128_ff) otherwise.
 cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,

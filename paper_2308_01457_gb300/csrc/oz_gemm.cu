@@ -10,9 +10,10 @@
 // and a digit product is an integer of at most 2^14, so sums of the same order g = s+t over
 // 128 values of k are exact in the FP32 accumulators of the tensor cores for g <= 3
 // ((g+1) x 2 x 128 x 2^14 <= 2^24).  Orders g <= 6 (28 digit pairs) are kept: the dropped
-// terms are below 2^-56 of sigma_i tau_j per product.  After every 128 values of k the seven
-// order accumulators are read out of TMEM: orders 0-3 are added exactly into a 64-bit integer
-// sum per output, orders 4-6 (below 2^-32 of them) into an FP32 sum; the result is scaled by
+// terms are below 2^-56 of sigma_i tau_j per product (the trailing updates of FP64 factorisations keep
+// order 7 too, 34 pairs, and leave nothing of that size but the rounding of the operands).  After every 128 values of k the seven
+// order accumulators are read out of TMEM: orders 0-4 are added into a 64-bit integer
+// sum per output, orders 5-6 (below 2^-40 of them) into an FP32 sum; the result is scaled by
 // sigma_i tau_j 2^-14.
 //
 // What bounds it is the issue of the MMAs and then the tensor pipe.  An MMA with M = 128, K = 16
@@ -37,6 +38,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <type_traits>
 
@@ -57,7 +59,7 @@ constexpr int OZ_SMEM = 2 * OZ_STAGE + 1024;
 constexpr int OZ_THREADS = 10 * 32;                            // producer, MMA, 8 flush warps
 constexpr int OZ_FLUSH = 8 * 32;
 constexpr int OZ_HN = OZ_TN / 2;                               // columns per flush thread
-constexpr int OZ_TMEM_COLS = 512;                              // 7 orders x 64 columns = 448 used
+constexpr int OZ_TMEM_COLS = 512;                              // 7 or 8 orders x 64 columns
 constexpr long long kOzSpinLimit = 1ll << 24;
 static_assert(OZ_SMEM <= 226 * 1024, "digit stages and the barriers do not fit shared memory");
 
@@ -219,6 +221,59 @@ __global__ void oz_col_exp_kernel(const double2* __restrict__ A, int64_t rows, i
     ex[col] = oz_exponent(m);
   }
 }
+// The exponents of a trailing update's operands L (M x K) and U (K x N), which are first balanced: column
+// k of L times, row k of U over 2^{d_k}, d_k the exponent of the largest finite entry of U's row k
+// relative to its column's largest (exponents cj).  A row of L then has its largest entry where
+// its largest products are, and the digits lose no more than FP64 does when rows or columns of the
+// matrix differ in scale (rows scaled by 10^-6 .. 10^6, n = 130: componentwise backward error
+// 2.6e-15 with FP64 products, 4.6e-11 without the balance, 2.4e-15 so).
+__global__ void oz_balance_kernel(const double2* __restrict__ U, int64_t N, int64_t ld, const int* __restrict__ cj,
+                                  int* __restrict__ dk) {
+  __shared__ int red[8];
+  const double2* u = U + int64_t(blockIdx.x) * ld;
+  int e = INT_MIN;
+#pragma unroll 4
+  for (int64_t j = threadIdx.x; j < N; j += blockDim.x) {
+    const unsigned long long b = oz_umax(oz_abs_bits(u[j].x), oz_abs_bits(u[j].y));
+    if (b && b < 0x7FF0000000000000ull && cj[j] != OZ_BAD) e = max(e, oz_exponent(b) - cj[j]);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < int(blockDim.x >> 5); ++w) e = max(e, red[w]);
+    dk[blockIdx.x] = e == INT_MIN ? 0 : e;
+  }
+}
+// Exponents of the balanced rows of L (rs = ld, ks = 1, sign +1: a warp per row) ...
+__global__ void oz_balanced_row_exp_kernel(const double2* __restrict__ A, int64_t rows, int64_t K, int64_t ld,
+                                           const int* __restrict__ dk, int* __restrict__ ex) {
+  const int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (row >= rows) return;
+  int e = INT_MIN;
+  for (int64_t k = lane; k < K; k += 32) {
+    const double2 v = A[row * ld + k];
+    const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
+    if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) + dk[k]);
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if (lane == 0) ex[row] = e == INT_MIN ? 0 : e;
+}
+// ... and of the columns of U, balanced or (no dk) as they are (a thread per column)
+__global__ void oz_balanced_col_exp_kernel(const double2* __restrict__ A, int64_t cols, int64_t K, int64_t ld,
+                                           const int* __restrict__ dk, int* __restrict__ ex) {
+  const int64_t col = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (col >= cols) return;
+  int e = INT_MIN;
+#pragma unroll 8
+  for (int64_t k = 0; k < K; ++k) {
+    const double2 v = A[k * ld + col];
+    const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
+    if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) - (dk ? dk[k] : 0));
+  }
+  ex[col] = e == INT_MIN ? 0 : e;
+}
 // x 2^(55 - e) rounded to an integer (|x| < 2^e, so |F| <= 2^55), from the bit pattern:
 // x = M 2^(b - 1075) with the 53-bit significand M (b the biased exponent; subnormals have
 // b = 1 and no hidden bit), so F = M 2^(b - 1020 - e), a left shift of at most 2 or a right
@@ -244,7 +299,7 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(uint32_t byte) {
   return __float_as_uint(__uint_as_float(0x4B000000u | byte) - 8388736.0f) >> 16;
 }
 // Digit tiles of a matrix read as rows x K elements (element (r, k) at A[r * rs + k * ks]),
-// one power-of-two exponent per row, zero-padded to whole tiles of TR rows x 16 k:
+// one power-of-two exponent per row (and with dk a factor 2^{sign dk[k]} per k), zero-padded to whole tiles of TR rows x 16 k:
 // tile (rt, kc, s, p) of TR x 16 bf16 at byte offset (((rt * KC + kc) * 7 + s) * 2 + p) * TR * 32.
 // Z (rs = ld, ks = 1, TR = 128) and X read by columns (rs = 1, ks = ld, TR = 32) both land here.
 // Digits: F = x 2^(55 - e) rounded (above) is written in balanced base 256,
@@ -256,7 +311,8 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(uint32_t byte) {
 // each store instruction fills two whole 256-byte segments.
 template <int TR>
 __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int64_t K, int64_t rs, int64_t ks,
-                                bool conj, const int* __restrict__ ex, int64_t KC, unsigned char* __restrict__ out) {
+                                bool conj, const int* __restrict__ ex, const int* __restrict__ dk, int sign, int64_t KC,
+                                unsigned char* __restrict__ out) {
   constexpr int TILE = TR * OZ_KS * 2;
   constexpr unsigned long long BIAS = 0x0080808080808080ull;
   const int lane = threadIdx.x & 31;
@@ -271,8 +327,9 @@ __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int
     gr[j] = gi[j] = BIAS;
     if (row < rows && k < K) {
       const double2 v = A[row * rs + k * ks];
-      gr[j] = static_cast<unsigned long long>(oz_fixed(v.x, e)) + BIAS;
-      gi[j] = static_cast<unsigned long long>(oz_fixed(conj ? -v.y : v.y, e)) + BIAS;
+      const int ek = dk ? e - sign * dk[k] : e;
+      gr[j] = static_cast<unsigned long long>(oz_fixed(v.x, ek)) + BIAS;
+      gi[j] = static_cast<unsigned long long>(oz_fixed(conj ? -v.y : v.y, ek)) + BIAS;
     }
   }
   const int64_t rt = row / TR, kc = kg >> 1;
@@ -295,14 +352,14 @@ __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int
 constexpr int OZ_SPLIT_WARPS = 8;  // a block covers 8 rows x 8 warps x 4 groups x 8 k = 8 x 256
 
 // ---------------------------------------------------------------- the product
-// The highest order kept in each tile of 64 columns: all of them (6) without ref.  With ref the
+// The highest order kept in each tile of 64 columns: gmax without ref.  With ref the
 // operand is a correction of a matrix whose columns have the exponents ref, and what matters is
 // the error against that matrix: dropping the orders above g leaves 2^{-8(g+1)} sigma tau per
 // product, which is at most 2^-60 sigma 2^ref (1/16 of what the product with the matrix itself
 // leaves) once 8 (g + 1) >= 60 - (ref - ex).  One warp per tile.
-__global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restrict__ ref, int64_t N,
+__global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restrict__ ref, int64_t N, int gmax,
                                  int* __restrict__ orders) {
-  int g = ref ? 0 : OZ_ND - 1;
+  int g = ref ? 0 : gmax;
   for (int q = threadIdx.x; ref && q < OZ_TN; q += 32) {
     const int64_t c = int64_t(blockIdx.x) * OZ_TN + q;
     if (c < N) g = max(g, min(OZ_ND - 1, (59 - min(59, max(0, ref[c] - ex[c]))) / 8));
@@ -311,13 +368,14 @@ __global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restri
   if (threadIdx.x == 0) orders[blockIdx.x] = g;
 }
 
-// The sums of one output: a = sum_g V_g 2^{24-8g} over the orders 0-3 (V_g the integer order
-// sums), exact; t the orders 4-6 (below 2^-32 of the leading terms) in FP32 in the same units, so
-// its rounding stays near 2^-50 of the result; the value is 2^-24 (a + t).
-__device__ __forceinline__ void oz_store(double* C, long long a, float t, int aex, int bex, double alpha, double beta) {
-  double sc = ldexp(1.0, aex - 14) * ldexp(1.0, bex);
-  if (aex == OZ_BAD || bex == OZ_BAD) sc = NAN;
-  const double x = alpha * (ldexp(double(a) + double(t), -24) * sc);
+// The sums of one output: a = sum_g V_g 2^{unit-8g} over the orders that this leaves whole (V_g the
+// integer order sums), exact; t the others in FP32 in the same units; the value is 2^-unit (a + t).
+// unit 32 (orders 0-4 exact, the rounding of t near 2^-58 of the result) as long as K <= 2^15 keeps a
+// below 2^62, 24 (orders 0-3, 2^-53) above.
+__device__ __forceinline__ void oz_store(double* C, long long a, float t, int aex, int bex, int unit, double alpha,
+                                         double beta) {
+  const double v = double(a) + double(t);
+  const double x = alpha * (aex == OZ_BAD || bex == OZ_BAD ? NAN : ldexp(v, aex + bex - 14 - unit));
   *C = beta != 0.0 ? x + beta * *C : x;
 }
 // One output of a piece of a tile (below).
@@ -329,9 +387,11 @@ struct OzPart {
 // One A tile with T digits of X (tiles 2 OZ_BTILE apart) into T consecutive orders, the A tile kept
 // in the collector; the MMAs of a group have one instruction descriptor.
 template <int T>
-__device__ __forceinline__ void oz_group(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void oz_group(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc_first,
+                                         uint32_t acc_last) {
 #pragma unroll
   for (int t = 0; t < T; ++t) {
+    const uint32_t acc = t == T - 1 ? acc_last : acc_first;
     const uint32_t dt = d + uint32_t(t) * OZ_TN;
     const uint64_t bt = b + uint64_t(t) * (2 * OZ_BTILE >> 4);
     if (T == 1) oz_mma_once(dt, a, bt, idesc, acc);
@@ -355,15 +415,19 @@ struct OzMma {
 // step's first product into each order's accumulator (digit 0) overwrites it.
 template <int G, int IM, int P, int S>
 __device__ __forceinline__ void oz_step(OzMma& m, uint32_t tmem, uint32_t smem, uint32_t acc) {
-  if constexpr (S == (G > 0 ? G - 1 : 0)) m.ready = oz_test(smem_u32(&m.full[1 - P]), m.phase >> (1 - P) & 1);
+  constexpr int SL = G < OZ_ND ? G : OZ_ND - 1;                    // the last digit of Z
+  constexpr int T = G + 1 - S < OZ_ND ? G + 1 - S : int(OZ_ND);  // digits of X that this one meets
+  if constexpr (S == (SL > 0 ? SL - 1 : 0)) m.ready = oz_test(smem_u32(&m.full[1 - P]), m.phase >> (1 - P) & 1);
   const uint64_t a = oz_desc(smem + P * OZ_STAGE + S * OZ_ASLOT), b = oz_desc(smem + P * OZ_STAGE + OZ_ND * OZ_ASLOT);
   const uint32_t d = tmem + uint32_t(S) * OZ_TN;
   // Re: Re Z Re X - Im Z Im X, Im: Re Z Im X + Im Z Re X
-  oz_group<G + 1 - S>(d, a, b + uint64_t(IM * (OZ_BTILE >> 4)), oz_idesc(false), S == 0 ? acc : 1u);
-  oz_group<G + 1 - S>(d, a + (OZ_ATILE >> 4), b + uint64_t((1 - IM) * (OZ_BTILE >> 4)), oz_idesc(IM == 0), 1u);
+  // (the first product of order 7 is digit 1 of Z with digit 6 of X)
+  oz_group<T>(d, a, b + uint64_t(IM * (OZ_BTILE >> 4)), oz_idesc(false), S == 0 ? acc : 1u,
+              S == 0 || S + T - 1 == OZ_ND && S == 1 ? acc : 1u);
+  oz_group<T>(d, a + (OZ_ATILE >> 4), b + uint64_t((1 - IM) * (OZ_BTILE >> 4)), oz_idesc(IM == 0), 1u, 1u);
   if constexpr (S > 0) oz_commit(smem_u32(&m.empty[P * OZ_ND + S]));
-  if constexpr (S == G) oz_commit(smem_u32(&m.empty[P * OZ_ND]));
-  if constexpr (S < G) oz_step<G, IM, P, S + 1>(m, tmem, smem, acc);
+  if constexpr (S == SL) oz_commit(smem_u32(&m.empty[P * OZ_ND]));
+  if constexpr (S < SL) oz_step<G, IM, P, S + 1>(m, tmem, smem, acc);
 }
 template <int G, int IM, int P>
 __device__ __forceinline__ bool oz_stage(OzMma& m, uint32_t tmem, uint32_t smem, uint32_t acc) {
@@ -408,7 +472,7 @@ __device__ __forceinline__ OzItem oz_item(int64_t w, int64_t whole, int pieces, 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm_kernel(int64_t M, int64_t N, int64_t KC, const unsigned char* __restrict__ Ad,
                    const int* __restrict__ aex, const unsigned char* __restrict__ Bd, const int* __restrict__ bex,
-                   const int* __restrict__ orders, int64_t whole, int pieces, int64_t items, double alpha, double beta,
+                   const int* __restrict__ orders, int64_t whole, int pieces, int64_t items, int unit, double alpha, double beta,
                    double* __restrict__ C, int64_t ldc, OzPart* __restrict__ part, int* status) {
   extern __shared__ unsigned char oz_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(oz_raw) + 1023) & ~uintptr_t(1023));
@@ -461,7 +525,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const int G = orders[ct];
         const int64_t k1 = std::min<int64_t>(KC, item.c1 * OZ_KCH);
         // the digits up to the highest order are the first tiles of each operand's step
-        const uint32_t bbytes = s == 0 ? uint32_t(G + 1) * 2 * OZ_BTILE : 0u;
+        const uint32_t bbytes = s == 0 ? uint32_t(min(G + 1, int(OZ_ND))) * 2 * OZ_BTILE : 0u;
         for (int64_t kc = item.c0 * OZ_KCH; kc < k1 && go; ++kc) {  // (starts even)
           const int p = int(kc & 1);
           const uint32_t turn = p ? fills1 : fills0;
@@ -508,7 +572,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           case 3: ok = run(std::integral_constant<int, 3>()); break;
           case 4: ok = run(std::integral_constant<int, 4>()); break;
           case 5: ok = run(std::integral_constant<int, 5>()); break;
-          default: ok = run(std::integral_constant<int, 6>()); break;
+          case 6: ok = run(std::integral_constant<int, 6>()); break;
+          default: ok = run(std::integral_constant<int, 7>()); break;
         }
         if (!ok) {
           fail();
@@ -555,9 +620,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           if (g + 1 <= G) oz_ld8(tbase + uint32_t((g + 1) * OZ_TN + j0), u[buf]);
         };
         auto digit = [](uint32_t x) { return __float2int_rn(__uint_as_float(x)); };
+        const float w5 = unit == 32 ? 0x1p-8f : 0x1p-16f;  // 2^{unit-40}
         load(0, 0, 0);
 #pragma unroll
-        for (int g = 0; g < OZ_ND; g += 2) {
+        for (int g = 0; g <= OZ_ND; g += 2) {
           if (g > G) break;
 #pragma unroll
           for (int j0 = 0; j0 < OZ_HN; j0 += 8) {
@@ -569,13 +635,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             for (int j = 0; j < 8; ++j) {
               const float x = __uint_as_float(v[buf][j]), y = __uint_as_float(u[buf][j]);
               if (g == 0)  // V_0 2^8 + V_1 fits 32 bits (|V_0| <= 2^22, |V_1| <= 2^23)
-                a[j0 + j] += (long long)(digit(v[buf][j]) * 256 + (G >= 1 ? digit(u[buf][j]) : 0)) * 65536;
+                a[j0 + j] += (long long)(digit(v[buf][j]) * 256 + (G >= 1 ? digit(u[buf][j]) : 0)) * (1 << (unit - 8));
               else if (g == 2)
-                a[j0 + j] += (long long)digit(v[buf][j]) * 256 + (G >= 3 ? digit(u[buf][j]) : 0);
-              else if (g == 4)
-                t[j0 + j] = fmaf(x, 0x1p-8f, G >= 5 ? fmaf(y, 0x1p-16f, t[j0 + j]) : t[j0 + j]);
-              else
-                t[j0 + j] = fmaf(x, 0x1p-24f, t[j0 + j]);
+                a[j0 + j] += (long long)digit(v[buf][j]) * (1 << (unit - 16)) +
+                             (G >= 3 ? (long long)digit(u[buf][j]) * (1 << (unit - 24)) : 0ll);
+              else if (g == 4) {
+                if (unit == 32) a[j0 + j] += digit(v[buf][j]);
+                else t[j0 + j] = fmaf(x, 0x1p-8f, t[j0 + j]);
+                if (G >= 5) t[j0 + j] = fmaf(y, w5, t[j0 + j]);
+              } else {
+                if (G >= 7) t[j0 + j] = fmaf(y, w5 * 0x1p-16f, t[j0 + j]);
+                t[j0 + j] = fmaf(x, w5 * 0x1p-8f, t[j0 + j]);
+              }
             }
           }
         }
@@ -596,7 +667,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 #pragma unroll
         for (int j = 0; j < OZ_HN; ++j) {
           const int64_t col = ct * OZ_TN + c0 + j;
-          if (col < N) oz_store(C + (row * ldc + col) * 2 + (item.tile & 1), a[j], t[j], ae, bex[col], alpha, beta);
+          if (col < N) oz_store(C + (row * ldc + col) * 2 + (item.tile & 1), a[j], t[j], ae, bex[col], unit, alpha, beta);
         }
       }
     }
@@ -607,8 +678,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
 }
 
 __global__ void oz_reduce_kernel(int64_t M, int64_t N, int64_t whole, int pieces, const OzPart* __restrict__ part,
-                                 const int* __restrict__ aex, const int* __restrict__ bex, double alpha, double beta,
-                                 double* __restrict__ C, int64_t ldc) {
+                                 const int* __restrict__ aex, const int* __restrict__ bex, int unit, double alpha,
+                                 double beta, double* __restrict__ C, int64_t ldc) {
   const int64_t CT = (N + OZ_TN - 1) / OZ_TN, tile = whole + blockIdx.x;
   const int e = int(blockIdx.y) * 256 + int(threadIdx.x);  // element of the tile
   const int64_t row = tile / (2 * CT) * OZ_TM + e / OZ_TN, col = tile / 2 % CT * OZ_TN + e % OZ_TN;
@@ -619,7 +690,7 @@ __global__ void oz_reduce_kernel(int64_t M, int64_t N, int64_t whole, int pieces
     s.a += p.a;
     s.t += p.t;
   }
-  oz_store(C + (row * ldc + col) * 2 + (tile & 1), s.a, s.t, aex[row], bex[col], alpha, beta);
+  oz_store(C + (row * ldc + col) * 2 + (tile & 1), s.a, s.t, aex[row], bex[col], unit, alpha, beta);
 }
 
 inline unsigned oz_cdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); }
@@ -630,16 +701,19 @@ size_t oz_a_bytes(int64_t M, int64_t K) {
   return size_t((M + OZ_TM - 1) / OZ_TM) * size_t((K + OZ_KS - 1) / OZ_KS) * OZ_NT * OZ_ATILE;
 }
 
-// Exponents and digit tiles of op(X) (rows x K after op, rows in tiles of TR)
+// Exponents and digit tiles of op(X) (rows x K after op, rows in tiles of TR); with dk balanced: op(X)
+// is L (sign +1) or U by its columns (sign -1)
 template <int TR>
-static cudaError_t oz_digits(const double2* X, int64_t rows, int64_t K, int64_t rs, int64_t ks, bool conj, int* ex,
-                             void* digits, cudaStream_t s) {
+static cudaError_t oz_digits(const double2* X, int64_t rows, int64_t K, int64_t rs, int64_t ks, bool conj,
+                             const int* dk, int sign, int* ex, void* digits, cudaStream_t s) {
   const int64_t KC = (K + OZ_KS - 1) / OZ_KS, RP = (rows + TR - 1) / TR * TR;
   if (RP / 8 > 65535) return cudaErrorInvalidValue;
-  if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, ex);
+  if (dk && sign > 0) oz_balanced_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, dk, ex);
+  else if (dk) oz_balanced_col_exp_kernel<<<oz_cdiv(rows, 64), 64, 0, s>>>(X, rows, K, ks, dk, ex);
+  else if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, ex);
   else oz_col_exp_kernel<<<unsigned(rows), 256, 0, s>>>(X, K, rows, ks, ex);
   oz_split_kernel<TR><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(RP / 8)), OZ_SPLIT_WARPS * 32, 0, s>>>(
-      X, rows, K, rs, ks, conj, ex, KC, static_cast<unsigned char*>(digits));
+      X, rows, K, rs, ks, conj, ex, dk, sign, KC, static_cast<unsigned char*>(digits));
   return launched(2);
 }
 
@@ -648,12 +722,12 @@ cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t l
   if (M <= 0 || K <= 0) return cudaSuccess;
   ProfScope prof("oz_prep", s, 44.0 * double(M) * double(K));  // bytes read + written
   return oz_digits<OZ_TM>(static_cast<const double2*>(A), M, K, opA == OP_N ? lda : 1, opA == OP_N ? 1 : lda,
-                          opA == OP_C, ex, digits, s);
+                          opA == OP_C, nullptr, 0, ex, digits, s);
 }
 
-cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
-                    const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
-                    const int* ref_ex, int* status, cudaStream_t s) {
+static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
+                              const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
+                              const int* ref_ex, const int* dk, int gmax, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   static bool attr[64] = {};
   static int nsm[64] = {};
@@ -674,6 +748,7 @@ cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, cons
   const int64_t whole = tiles - rem;
   const int pieces = rem ? int(std::max<int64_t>(1, std::min<int64_t>(sms / rem, nch / 8))) : 1;
   const int64_t items = whole + rem * pieces;
+  const int unit = K <= (1 << 15) ? 32 : 24;  // of the integer sums (oz_store)
   // digit tiles of B, then the pieces' sums, then the orders
   const size_t bbytes = size_t(CT) * size_t(KC) * OZ_BSLOT;
   const size_t pbytes = pieces > 1 ? sizeof(OzPart) * size_t(rem * pieces) * OZ_TM * OZ_TN : 0;
@@ -683,23 +758,48 @@ cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, cons
   OzPart* part = reinterpret_cast<OzPart*>(bd + bbytes);
   int* orders = reinterpret_cast<int*>(bd + bbytes + pbytes);
   e = oz_digits<OZ_TN>(static_cast<const double2*>(B), N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, opB == OP_C,
-                       b_ex, bd, s);
+                       dk, -1, b_ex, bd, s);
   if (e != cudaSuccess) {
     cudaFreeAsync(bd, s);
     return e;
   }
-  oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, N, orders);
+  oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, N, gmax, orders);
   {
     ProfScope prof("gemm_oz", s, 8.0 * double(M) * double(N) * double(K));
     oz_gemm_kernel<<<unsigned(std::min(items, sms)), OZ_THREADS, OZ_SMEM, s>>>(
-        M, N, KC, static_cast<const unsigned char*>(a_digits), a_ex, bd, b_ex, orders, whole, pieces, items, alpha, beta,
+        M, N, KC, static_cast<const unsigned char*>(a_digits), a_ex, bd, b_ex, orders, whole, pieces, items, unit, alpha, beta,
         static_cast<double*>(C), ldc, part, status);
     if (pieces > 1)
       oz_reduce_kernel<<<dim3(unsigned(rem), OZ_TM * OZ_TN / 256), 256, 0, s>>>(
-          M, N, whole, pieces, part, a_ex, b_ex, alpha, beta, static_cast<double*>(C), ldc);
+          M, N, whole, pieces, part, a_ex, b_ex, unit, alpha, beta, static_cast<double*>(C), ldc);
   }
   e = launched(pieces > 1 ? 3 : 2);
   cudaFreeAsync(bd, s);
+  return e;
+}
+
+cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
+                    const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
+                    int* status, cudaStream_t s) {
+  return oz_product(opB, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, nullptr, OZ_ND - 1, status, s);
+}
+
+size_t oz_update_bytes(int64_t n, int64_t K) { return oz_a_bytes(n, K) + sizeof(int) * size_t(2 * n + K); }
+
+cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
+                      int64_t ldc, void* scratch, int* status, cudaStream_t s) {
+  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  char* dig = static_cast<char*>(scratch);
+  int* dk = reinterpret_cast<int*>(dig + oz_a_bytes(M, K));
+  int *lex = dk + K, *uex = lex + M;
+  const double2* u = static_cast<const double2*>(U);
+  oz_balanced_col_exp_kernel<<<oz_cdiv(N, 64), 64, 0, s>>>(u, N, K, ldu, nullptr, uex);
+  oz_balance_kernel<<<unsigned(K), 256, 0, s>>>(u, N, ldu, uex, dk);
+  cudaError_t e = launched(2);
+  if (e == cudaSuccess)
+    e = oz_digits<OZ_TM>(static_cast<const double2*>(L), M, K, ldl, 1, false, dk, 1, lex, dig, s);
+  if (e == cudaSuccess)
+    e = oz_product(OP_N, M, N, K, -1.0, dig, lex, U, ldu, 1.0, C, ldc, uex, nullptr, dk, OZ_ND, status, s);
   return e;
 }
 
