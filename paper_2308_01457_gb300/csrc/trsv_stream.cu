@@ -3,7 +3,7 @@
 //
 // A blocked sweep that launches one diagonal solve and one panel update per 64-row block
 // is latency-bound (2 x n/64 dependent launches per sweep).  Here one persistent kernel
-// does a whole sweep.  The right-hand sides are cut into chunks of at most 16 columns (one
+// does a whole sweep.  The right-hand sides are cut into chunks of at most 8 columns (one
 // chunk of the exact width for 1-8); CTAs take (block, chunk) tasks in block-major order
 // from a ticket counter.  With D_i the inverse of the diagonal block and j the blocks that
 // precede i in the sweep, the last of them h,
@@ -255,8 +255,8 @@ __device__ __forceinline__ void st_relaxed(float2* p, float2 v) {
 // sides (n x nrhs, rows ldx apart) less everything that earlier blocks contribute, y the solution, all ones
 // (kNotReady) on entry.
 // Chain-bound: a block's latency is one store-to-load trip, a product and a reduction.
-// One sweep at N = 15360: 0.36 ms for 1 column, 1.4 for 16 (1.32 and 3.01 with a flag per block and
-// the diagonal solve behind the last product).
+// One sweep at N = 15360: 0.36 ms for 1 column, 0.82 for 16 (1.32 and 3.01 with a flag per block, the
+// diagonal solve behind the last product and chunks of 16 columns).
 template <int NR>
 __global__ void __launch_bounds__(256, 2)
     trsv_stream_kernel(const float2* __restrict__ LU, int64_t n, int64_t ld, const float2* __restrict__ Dinv,
@@ -409,13 +409,22 @@ __global__ void __launch_bounds__(256, 2)
 }  // namespace
 
 // Blocks per superblock, and when a sweep uses them: one kernel takes nblk^2/2 tile products per
-// 16-column chunk, about 3 us each over 152 SMs; a superblock takes 30 to 45 us for its own blocks
-// (8-column chunks) and 50 us per wave of update tiles, so sweeps with many right-hand sides change
-// over.  One kernel / superblocks, ms per sweep: 15360 x 80 (nblk ceil(nrhs / 16) = 1200) 3.05 / 2.53,
-// 7503 x 163 (1298) 1.57 / 1.28, 7503 x 642 4.77 / 1.95, 15360 x 642 20.0 / 5.74, 1920 x 1100 (2070)
-// 0.58 / 0.39; 7503 x 100 (826) takes 1.17 in one kernel.
+// chunk of columns, so with many right-hand sides sweeps change over to superblocks of 25 to 45 us
+// (their own blocks) and 50 us per wave of update tiles.  One kernel / superblocks, ms per sweep:
+// 15360 x 64 (nblk ceil(nrhs / 16) = 960) 2.26 / 2.40, 1920 x 642 (1230) 0.39 / 0.36, 7503 x 163 (1298)
+// 1.43 / 1.25, 15360 x 163 (2640) 5.35 / 3.12, 7503 x 642 4.77 / 2.07, 15360 x 642 20.0 / 5.98.
 constexpr int64_t kSuper = 8;
 static bool use_superblocks(int64_t nblk, int64_t nrhs) { return nblk > kSuper && nblk * ((nrhs + 15) / 16) > 1100; }
+
+// Columns per chunk.  The chain of a chunk takes 2.2 us per block with 4 columns, 3.2 with 8, 5.5 with
+// 16, and the chunks run side by side until the tile products of all of them fill the SMs, about where
+// 4 columns need 1200 block-chunks (ms per sweep with 4 / 8 / 16 columns: 1920 x 16 0.074 / 0.102 /
+// 0.170, 1920 x 163 (1230) 0.157 / 0.164 / 0.235, 7503 x 16 0.278 / 0.404 / 0.663, 7503 x 64 (1888) 0.734 /
+// 0.644 / 0.895, 15360 x 16 (960) 0.82 / 0.88 / 1.41, 15360 x 32 (1920) 1.48 / 1.29 / 1.84).
+static int chunk_width(int64_t blocks, int64_t nrhs) {
+  if (nrhs <= 2) return int(nrhs);
+  return blocks * ((nrhs + 3) / 4) <= 1200 ? 4 : 8;
+}
 
 cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* Dinv, cudaStream_t s) {
   const int64_t nblk = (n + kTB - 1) / kTB;
@@ -459,22 +468,16 @@ cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* D
     };
     opt(trsv_stream_kernel<1>, sizeof(StreamSmem<1>));
     opt(trsv_stream_kernel<2>, sizeof(StreamSmem<2>));
-    opt(trsv_stream_kernel<3>, sizeof(StreamSmem<3>));
     opt(trsv_stream_kernel<4>, sizeof(StreamSmem<4>));
-    opt(trsv_stream_kernel<5>, sizeof(StreamSmem<5>));
-    opt(trsv_stream_kernel<6>, sizeof(StreamSmem<6>));
-    opt(trsv_stream_kernel<7>, sizeof(StreamSmem<7>));
     opt(trsv_stream_kernel<8>, sizeof(StreamSmem<8>));
-    opt(trsv_stream_kernel<16>, sizeof(StreamSmem<16>));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     attr[dev] = true;
   }
   const int64_t nblk = (n + kTB - 1) / kTB, one = nblk * kTB * kTB;
   const bool super = use_superblocks(nblk, nrhs);
-  // chunk width: the exact width for 1-8 right-hand sides, 16 above, 8 in superblocks (a shorter
-  // chain, and chunks enough to fill the chip)
-  const int w = nrhs <= 8 ? int(nrhs) : (super ? 8 : 16);
+  const int64_t step = super ? kSuper : nblk;
+  const int w = chunk_width(step, nrhs);
   const int64_t chunks = (nrhs + w - 1) / w;
   e = cudaMemsetAsync(tickets, 0, sizeof(int) * trsv_stream_tickets(n), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(Y, 0xFF, sizeof(float2) * size_t(n) * size_t(ldx), s);  // nothing ready
@@ -484,7 +487,6 @@ cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* D
   const float2* E = static_cast<const float2*>(Dinv) + (upper ? 3 : 2) * one;
   float2* x = static_cast<float2*>(X);
   float2* y = static_cast<float2*>(Y);
-  const int64_t step = super ? kSuper : nblk;
   for (int64_t first = 0, q = 0; first < nblk; first += step, ++q) {
     const int64_t count = std::min(step, nblk - first);
     const unsigned grid = unsigned(std::min<int64_t>(count * chunks, int64_t(2) * std::max(nsm[dev], 1)));
@@ -495,13 +497,8 @@ cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* D
     switch (w) {
       case 1: e = run(trsv_stream_kernel<1>, sizeof(StreamSmem<1>)); break;
       case 2: e = run(trsv_stream_kernel<2>, sizeof(StreamSmem<2>)); break;
-      case 3: e = run(trsv_stream_kernel<3>, sizeof(StreamSmem<3>)); break;
       case 4: e = run(trsv_stream_kernel<4>, sizeof(StreamSmem<4>)); break;
-      case 5: e = run(trsv_stream_kernel<5>, sizeof(StreamSmem<5>)); break;
-      case 6: e = run(trsv_stream_kernel<6>, sizeof(StreamSmem<6>)); break;
-      case 7: e = run(trsv_stream_kernel<7>, sizeof(StreamSmem<7>)); break;
-      case 8: e = run(trsv_stream_kernel<8>, sizeof(StreamSmem<8>)); break;
-      default: e = run(trsv_stream_kernel<16>, sizeof(StreamSmem<16>)); break;
+      default: e = run(trsv_stream_kernel<8>, sizeof(StreamSmem<8>)); break;
     }
     if (e != cudaSuccess) return e;
     if (first + count == nblk) break;
