@@ -187,7 +187,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   }
   if (lu->prec == FOSB_FP32) {
     if (X != B) FOSB_CUDA(copy_matrix(B, n, nrhs, ldb, X, ldx, 8, s));
-    FOSB_CUDA(getrs<float>(lu->lu, n, n, lu->ipiv, X, nrhs, ldx, s, lu->d_status, lu->dinv));
+    FOSB_CUDA(getrs<float>(lu->lu, n, n, lu->ipiv, X, nrhs, ldx, s, lu->d_status, lu->dinv, true));
     return FOSB_OK;
   }
   // MIXED: complex64 factors, FP64 residuals.
@@ -453,7 +453,7 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
       return cleanup(cuda_fail(e, "fosb_factor: permutation"));
   }
   if (prec != FOSB_FP64) {  // inverted diagonal blocks for the streaming triangular sweeps
-    if ((e = tri_block_inverses_c64(lu->lu, n, n, lu->dinv, s)) != cudaSuccess)
+    if ((e = tri_block_inverses_c64(lu->lu, n, n, lu->dinv, prec == FOSB_FP32, s)) != cudaSuccess)
       return cleanup(cuda_fail(e, "fosb_factor: diagonal-block inverses"));
   }
   *out = lu;

@@ -284,17 +284,18 @@ fosb_status getrf_external_scratch(void* A, int64_t n, int64_t lda, int32_t* ipi
                                    int64_t max_ctas, cudaStream_t s);
 template <typename T>
 cudaError_t getrs(const void* LU, int64_t n, int64_t ldlu, const int32_t* ipiv, void* X, int64_t nrhs, int64_t ldx,
-                  cudaStream_t s, int* status = nullptr, const void* dinv = nullptr);
+                  cudaStream_t s, int* status = nullptr, const void* dinv = nullptr, bool direct = false);
 // One whole triangular sweep with complex64 factors (unit lower if upper == 0, else upper
 // with its diagonal) for right-hand sides X -> Y, both n x nrhs with rows ldx apart (even, so that the
 // updates between superblocks move 16 bytes at a time) and distinct, X used up, given the inverses of the diagonal blocks and their products with the neighbouring tiles
 // (tri_block_inverses_c64); tickets: trsv_stream_tickets(n) ints of scratch; a bounded wait that
-// gives up sets *status.
+// gives up sets *status.  direct (in both calls): nothing refines the solution afterwards, so the
+// inverses are refined and the products with the neighbouring tiles not used.
 size_t trsv_stream_tickets(int64_t n);
 size_t tri_block_inverses_bytes(int64_t n);
-cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* Dinv, cudaStream_t s);
+cudaError_t tri_block_inverses_c64(const void* LU, int64_t n, int64_t ld, void* Dinv, bool direct, cudaStream_t s);
 cudaError_t trsv_stream_c64(const void* LU, int64_t n, int64_t ld, const void* Dinv, void* X, void* Y, int64_t nrhs,
-                            int64_t ldx, int upper, int* tickets, int* status, cudaStream_t s);
+                            int64_t ldx, int upper, bool direct, int* tickets, int* status, cudaStream_t s);
 cudaError_t convert_c128_to_c64(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                                 cudaStream_t s);
 cudaError_t convert_c64_to_c128(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,

@@ -301,14 +301,33 @@ __device__ __forceinline__ void ff_acc(float& h, float& l, float xh, float xl, f
   h = s;
 }
 
+// hi = float(x), lo = float(x - hi), both rounded to nearest, from the bits of x: the four FP64
+// instructions of that (conversions included) bounded the split of a large Z (N = 15360: 3.1 ms).
+__device__ __forceinline__ void split_bits(double x, float& hi, float& lo) {
+  const unsigned h = unsigned(__double2hiint(x)), l = unsigned(__double2loint(x));
+  const int e = int(h >> 20) & 0x7FF;
+  if (e < 960 || e > 1140) {  // zero, far from 1, infinite or NaN
+    hi = float(x);
+    lo = float(x - double(hi));
+    return;
+  }
+  // the significand is q 2^29 + rem; q rounded to nearest even leaves r = rem or rem - 2^29
+  const unsigned q = 0x800000u | ((h & 0xFFFFFu) << 3) | (l >> 29), rem = l & 0x1FFFFFFFu;
+  const unsigned up = rem + (q & 1u) > 0x10000000u ? 1u : 0u;
+  const int r = int(rem) - int(up << 29);
+  hi = __uint_as_float((h & 0x80000000u) | ((unsigned(e - 1023 + 127) << 23) + (q + up - 0x800000u)));
+  lo = __int2float_rn(int(h) < 0 ? -r : r) * __uint_as_float(unsigned(e - 1075 + 127) << 23);
+}
 __global__ void split_ff_kernel(const double2* __restrict__ src, int64_t rows, int64_t cols, int64_t lds,
                                 float4* __restrict__ dst, int64_t ldd) {
   const int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= rows * cols) return;
   const int64_t i = e / cols, j = e % cols;
   const double2 v = src[i * lds + j];
-  const float rh = float(v.x), ih = float(v.y);
-  dst[i * ldd + j] = make_float4(rh, float(v.x - double(rh)), ih, float(v.y - double(ih)));
+  float4 o;
+  split_bits(v.x, o.x, o.y);
+  split_bits(v.y, o.z, o.w);
+  dst[i * ldd + j] = o;
 }
 
 // Few right-hand sides (NC <= 8) on a pre-split A (op N): one warp per row, lanes stride
@@ -860,73 +879,100 @@ __global__ void trsm_diag_kernel(const typename C2<T>::type* D, int64_t ldd, int
   }
 }
 
+template <typename T>
+__device__ __forceinline__ typename C2<T>::type cmul_add(typename C2<T>::type a, typename C2<T>::type b,
+                                                         typename C2<T>::type c) {  // a b + c
+  return {fma(-a.y, b.y, fma(a.x, b.x, c.x)), fma(a.y, b.x, fma(a.x, b.y, c.y))};
+}
+
 // Few right-hand sides: one warp per column, lanes own rows (lane, lane + 32) of the
 // nb x nb diagonal block, which is staged transposed in shared memory (conflict-free
 // column reads).  Forward (unit lower) or backward (upper, with the diagonal) sweep.
 template <typename T>
 __global__ void __launch_bounds__(256) trsv_warp_kernel(const typename C2<T>::type* D, int64_t ldd, int nb, int upper,
-                                                        typename C2<T>::type* X, int64_t ldx, int64_t ncols) {
+                                                        typename C2<T>::type* X, int64_t ldx, int64_t ncols, int per_cta) {
   using V = typename C2<T>::type;
   extern __shared__ unsigned char smem_raw[];
-  V* Dt = reinterpret_cast<V*>(smem_raw);  // Dt[k * nb + r] = D[r, k]
+  V* Dt = reinterpret_cast<V*>(smem_raw);  // Dt[k * (nb + 1) + r] = D[r, k]
+  const int pitch = nb + 1;
   for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
     int r = e / nb, k = e % nb;
-    Dt[k * nb + r] = D[int64_t(r) * ldd + k];
+    Dt[k * pitch + r] = D[int64_t(r) * ldd + k];
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t c = int64_t(blockIdx.x) * 8 + warp;
-  if (c >= ncols) return;
+  const int64_t c = int64_t(blockIdx.x) * per_cta + warp;
+  if (warp >= per_cta || c >= ncols) return;
   const V zero = {T(0), T(0)};
   V x0 = lane < nb ? X[int64_t(lane) * ldx + c] : zero;
   V x1 = lane + 32 < nb ? X[int64_t(lane + 32) * ldx + c] : zero;
-  auto bcast = [&](int i) {
-    V v = i < 32 ? x0 : x1;
+  auto bcast = [&](V v, int i) {
     v.x = __shfl_sync(0xffffffffu, v.x, i & 31);
     v.y = __shfl_sync(0xffffffffu, v.y, i & 31);
     return v;
   };
-  auto fms = [](V a, V d, V x) {  // a - d x
+  auto fms = [](V a, V d, V x) {  // a - d x; one rounding at the size of a (two with FMAs into a)
     a.x -= d.x * x.x - d.y * x.y;
     a.y -= d.x * x.y + d.y * x.x;
     return a;
   };
   if (!upper) {
-    for (int i = 0; i < nb - 1; ++i) {
-      V xi = bcast(i);
-      if (lane > i && lane < nb) x0 = fms(x0, Dt[i * nb + lane], xi);
-      if (lane + 32 > i && lane + 32 < nb) x1 = fms(x1, Dt[i * nb + lane + 32], xi);
+    for (int i = 0; i < nb - 1 && i < 32; ++i) {
+      const V xi = bcast(x0, i);
+      if (lane > i && lane < nb) x0 = fms(x0, Dt[i * pitch + lane], xi);
+      if (lane + 32 < nb) x1 = fms(x1, Dt[i * pitch + lane + 32], xi);
+    }
+    for (int i = 32; i < nb - 1; ++i) {
+      const V xi = bcast(x1, i);
+      if (lane + 32 > i && lane + 32 < nb) x1 = fms(x1, Dt[i * pitch + lane + 32], xi);
     }
   } else {
-    for (int i = nb - 1; i >= 0; --i) {
-      V d = Dt[i * nb + i];
-      T den = d.x * d.x + d.y * d.y;
-      bool mine0 = i < 32 && lane == i, mine1 = i >= 32 && lane == i - 32;
-      if (mine0 || mine1) {
-        V v = mine0 ? x0 : x1;
-        V q = den > T(0) ? V{(v.x * d.x + v.y * d.y) / den, (v.y * d.x - v.x * d.y) / den} : zero;
-        if (mine0) x0 = q; else x1 = q;
-      }
-      V xi = bcast(i);
-      if (lane < i) x0 = fms(x0, Dt[i * nb + lane], xi);
-      if (lane + 32 < i) x1 = fms(x1, Dt[i * nb + lane + 32], xi);
+    // the reciprocals of the diagonal first, all lanes at once (a division per step is 30 FP64
+    // instructions for one lane); a quotient is x times the reciprocal plus one correction
+    auto recip = [&](int i) {
+      const V d = i < nb ? Dt[i * pitch + i] : zero;
+      const T den = d.x * d.x + d.y * d.y;
+      return den > T(0) ? V{d.x / den, -d.y / den} : zero;
+    };
+    const V r0 = recip(lane), r1 = recip(lane + 32);
+    const V d0 = lane < nb ? Dt[lane * pitch + lane] : zero, d1 = lane + 32 < nb ? Dt[(lane + 32) * pitch + lane + 32] : zero;
+    for (int i = nb - 1; i >= 32; --i) {
+      V q = cmul<T>(x1, r1);
+      q = cmul_add<T>(fms(x1, d1, q), r1, q);
+      if (lane == i - 32) x1 = q;
+      const V xi = bcast(x1, i);
+      x0 = fms(x0, Dt[i * pitch + lane], xi);
+      if (lane + 32 < i) x1 = fms(x1, Dt[i * pitch + lane + 32], xi);
+    }
+    for (int i = min(nb, 32) - 1; i >= 0; --i) {
+      V q = cmul<T>(x0, r0);
+      q = cmul_add<T>(fms(x0, d0, q), r0, q);
+      if (lane == i) x0 = q;
+      const V xi = bcast(x0, i);
+      if (lane < i) x0 = fms(x0, Dt[i * pitch + lane], xi);
     }
   }
   if (lane < nb) X[int64_t(lane) * ldx + c] = x0;
   if (lane + 32 < nb) X[int64_t(lane + 32) * ldx + c] = x1;
 }
 
-// Opt the warp-per-column solve into 64 KB of dynamic shared memory (a 64 x 64 complex128 block).
+// Solves on the diagonal block D (nb <= 64), a warp per column.  FP64-bound for wide right-hand sides, so
+// the columns are spread over all SMs before a CTA takes more than one of them.
 template <typename T>
-void enable_trsv_smem() {
-  static bool done[64] = {};
+void trsv_block(const typename C2<T>::type* D, int64_t ldd, int nb, int upper, typename C2<T>::type* X, int64_t ldx,
+                int64_t ncols, cudaStream_t s) {
+  using V = typename C2<T>::type;
+  static int nsm[64] = {};
   int dev = 0;
   cudaGetDevice(&dev);
-  if (dev >= 0 && dev < 64 && !done[dev]) {
-    cudaFuncSetAttribute(trsv_warp_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         int(64 * 64 * sizeof(typename C2<T>::type)));
-    done[dev] = true;
+  dev = std::min(std::max(dev, 0), 63);
+  if (!nsm[dev]) {
+    cudaFuncSetAttribute(trsv_warp_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(64 * 65 * sizeof(V)));
+    cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev);
   }
+  const int per_cta = int(std::min<int64_t>(8, (ncols + nsm[dev] - 1) / std::max(nsm[dev], 1)));
+  trsv_warp_kernel<T><<<cdiv(ncols, per_cta), 256, size_t(nb) * (nb + 1) * sizeof(V), s>>>(D, ldd, nb, upper, X, ldx,
+                                                                                          ncols, per_cta);
 }
 
 template <typename T>
@@ -983,12 +1029,32 @@ __global__ void row_norm_kernel(const double2* A, int64_t rows, int64_t cols, in
 }
 
 // per-column max |Re| + |Im| (out has cols entries)
-__global__ void col_absmax_kernel(const double2* A, int64_t rows, int64_t cols, int64_t lda, double* out) {
-  int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (e >= rows * cols) return;
-  int64_t i = e / cols, j = e % cols;
-  double2 v = A[i * lda + j];
-  atomic_max_pos(out + j, fabs(v.x) + fabs(v.y));
+// Largest |Re| + |Im| per column: a block takes cw columns x 256 / cw row lanes of 32 rows each and sends
+// one atomic per column (one per element took 73 us for 7503 x 163, 12 us so).
+__global__ void __launch_bounds__(256) col_absmax_kernel(const double2* __restrict__ A, int64_t rows, int64_t cols,
+                                                         int64_t lda, int cw, double* out) {
+  __shared__ unsigned long long red[256];
+  const int lanes = 256 / cw, cl = int(threadIdx.x) % cw, rl = int(threadIdx.x) / cw;
+  const int64_t col = int64_t(blockIdx.y) * cw + cl, r0 = int64_t(blockIdx.x) * 32 * lanes;
+  unsigned long long m = 0ull;
+  if (col < cols) {
+#pragma unroll 8
+    for (int i = 0; i < 32; ++i) {
+      const int64_t row = r0 + int64_t(i) * lanes + rl;
+      if (row < rows) {
+        const double2 v = A[row * lda + col];
+        // non-negative doubles (and NaN, above them) order like their bit patterns
+        const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(fabs(v.x) + fabs(v.y)));
+        m = b > m ? b : m;
+      }
+    }
+  }
+  red[threadIdx.x] = m;
+  __syncthreads();
+  if (rl == 0 && col < cols) {
+    for (int q = 1; q < lanes; ++q) m = red[q * cw + cl] > m ? red[q * cw + cl] : m;
+    atomicMax(reinterpret_cast<unsigned long long*>(out + col), m);
+  }
 }
 
 template <typename T>
@@ -1293,8 +1359,7 @@ fosb_status getrf(void* Av, int64_t n, int64_t lda, int32_t* ipiv, int* d_status
     if constexpr (sizeof(T) == 4) {
       return tri_lower_unit_cols(D, lda, jb, X, lda, ncols, s);  // four threads per column
     } else {
-      enable_trsv_smem<T>();
-      trsv_warp_kernel<T><<<cdiv(ncols, 8), 256, size_t(jb) * jb * sizeof(V), s>>>(D, lda, jb, 0, X, lda, ncols);
+      trsv_block<T>(D, lda, jb, 0, X, lda, ncols, s);
       return launched();
     }
   };
@@ -1415,8 +1480,7 @@ fosb_status getrf_external_scratch(void* Av, int64_t n, int64_t lda, int32_t* ip
     note_launches(2);
     int64_t rest = n - j0 - jb;
     if (rest > 0) {
-      enable_trsv_smem<T>();
-      trsv_warp_kernel<T><<<cdiv(rest, 8), 256, size_t(jb) * jb * sizeof(V), s>>>(Ap, lda, jb, 0, Ap + jb, lda, rest);
+      trsv_block<T>(Ap, lda, jb, 0, Ap + jb, lda, rest, s);
       note_launches(1);
       if constexpr (sizeof(T) == 4)
         FOSB_CUDA(cgemm_update_tc(rest, rest, jb, Ap + jb * lda, lda, Ap + jb, lda, Ap + jb * lda + jb, lda, d_status, s,
@@ -1447,7 +1511,7 @@ template fosb_status getrf_external_scratch<float>(void*, int64_t, int64_t, int3
 // X <- Z^{-1} X given the factors (perm = composed row permutation, device).
 template <typename T>
 cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm, void* Xv, int64_t nrhs, int64_t ldx,
-                  cudaStream_t s, int* status, const void* dinv) {
+                  cudaStream_t s, int* status, const void* dinv, bool direct) {
   using V = typename C2<T>::type;
   const V* LU = static_cast<const V*>(LUv);
   V* X = static_cast<V*>(Xv);
@@ -1466,8 +1530,8 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
     const size_t ybytes = sizeof(V) * size_t(n) * size_t(ldt);
     if (e == cudaSuccess) e = device_alloc(reinterpret_cast<void**>(&y), ybytes + 4 * trsv_stream_tickets(n) + 16, s);
     int* tickets = reinterpret_cast<int*>(y + ybytes);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, ldt, 0, tickets, status, s);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, ldt, 1, tickets, status, s);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, ldt, 0, direct, tickets, status, s);
+    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, ldt, 1, direct, tickets, status, s);
     if (y) cudaFreeAsync(y, s);
     if (e != cudaSuccess) {
       cudaFreeAsync(tmp, s);
@@ -1479,11 +1543,8 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
     return cudaGetLastError();
   } else {
   const int nb = 64;
-  enable_trsv_smem<T>();
   auto diag = [&](int64_t i0, int ib, int upper) {
-    const V* D = LU + i0 * ldlu + i0;
-    trsv_warp_kernel<T><<<cdiv(nrhs, 8), 256, size_t(ib) * ib * sizeof(V), s>>>(D, ldlu, ib, upper, tmp + i0 * nrhs,
-                                                                               nrhs, nrhs);
+    trsv_block<T>(LU + i0 * ldlu + i0, ldlu, ib, upper, tmp + i0 * nrhs, nrhs, nrhs, s);
     note_launches(1);
   };
   note_launches(2);  // gather + final copy
@@ -1521,9 +1582,9 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
 }
 
 template cudaError_t getrs<double>(const void*, int64_t, int64_t, const int32_t*, void*, int64_t, int64_t, cudaStream_t,
-                                   int*, const void*);
+                                   int*, const void*, bool);
 template cudaError_t getrs<float>(const void*, int64_t, int64_t, const int32_t*, void*, int64_t, int64_t, cudaStream_t,
-                                  int*, const void*);
+                                  int*, const void*, bool);
 
 cudaError_t convert_c128_to_c64(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                                 cudaStream_t s) {
@@ -1572,7 +1633,11 @@ cudaError_t absmax_c128(const void* A, int64_t rows, int64_t cols, int64_t lda, 
   cudaError_t e = cudaMemsetAsync(d_out, 0, sizeof(double) * cols, s);
   if (e != cudaSuccess) return e;
   if (rows * cols == 0) return cudaSuccess;
-  col_absmax_kernel<<<cdiv(rows * cols, 256), 256, 0, s>>>(static_cast<const double2*>(A), rows, cols, lda, d_out);
+  int cw = 1;
+  while (cw < 32 && cw < cols) cw *= 2;
+  if (cdiv(cols, cw) > 65535u) return cudaErrorInvalidValue;
+  col_absmax_kernel<<<dim3(cdiv(rows, 32 * (256 / cw)), cdiv(cols, cw)), 256, 0, s>>>(static_cast<const double2*>(A), rows,
+                                                                                  cols, lda, cw, d_out);
   return launched();
 }
 

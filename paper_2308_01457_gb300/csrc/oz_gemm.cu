@@ -260,19 +260,28 @@ __global__ void oz_balanced_row_exp_kernel(const double2* __restrict__ A, int64_
   e = __reduce_max_sync(0xffffffffu, e);
   if (lane == 0) ex[row] = e == INT_MIN ? 0 : e;
 }
-// ... and of the columns of U, balanced or (no dk) as they are (a thread per column)
-__global__ void oz_balanced_col_exp_kernel(const double2* __restrict__ A, int64_t cols, int64_t K, int64_t ld,
-                                           const int* __restrict__ dk, int* __restrict__ ex) {
-  const int64_t col = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (col >= cols) return;
+// ... and of the columns of U, balanced or (no dk) as they are (32 columns x 8 lanes along k)
+__global__ void __launch_bounds__(256) oz_balanced_col_exp_kernel(const double2* __restrict__ A, int64_t cols, int64_t K,
+                                                                  int64_t ld, const int* __restrict__ dk,
+                                                                  int* __restrict__ ex) {
+  __shared__ int red[256];
+  const int cl = threadIdx.x & 31, kl = threadIdx.x >> 5;
+  const int64_t col = int64_t(blockIdx.x) * 32 + cl;
   int e = INT_MIN;
+  if (col < cols) {
 #pragma unroll 8
-  for (int64_t k = 0; k < K; ++k) {
-    const double2 v = A[k * ld + col];
-    const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
-    if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) - (dk ? dk[k] : 0));
+    for (int64_t k = kl; k < K; k += 8) {
+      const double2 v = A[k * ld + col];
+      const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
+      if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) - (dk ? dk[k] : 0));
+    }
   }
-  ex[col] = e == INT_MIN ? 0 : e;
+  red[threadIdx.x] = e;
+  __syncthreads();
+  if (kl == 0 && col < cols) {
+    for (int w = 1; w < 8; ++w) e = max(e, red[w * 32 + cl]);
+    ex[col] = e == INT_MIN ? 0 : e;
+  }
 }
 // x 2^(55 - e) rounded to an integer (|x| < 2^e, so |F| <= 2^55), from the bit pattern:
 // x = M 2^(b - 1075) with the 53-bit significand M (b the biased exponent; subnormals have
@@ -709,7 +718,7 @@ static cudaError_t oz_digits(const double2* X, int64_t rows, int64_t K, int64_t 
   const int64_t KC = (K + OZ_KS - 1) / OZ_KS, RP = (rows + TR - 1) / TR * TR;
   if (RP / 8 > 65535) return cudaErrorInvalidValue;
   if (dk && sign > 0) oz_balanced_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, dk, ex);
-  else if (dk) oz_balanced_col_exp_kernel<<<oz_cdiv(rows, 64), 64, 0, s>>>(X, rows, K, ks, dk, ex);
+  else if (dk) oz_balanced_col_exp_kernel<<<oz_cdiv(rows, 32), 256, 0, s>>>(X, rows, K, ks, dk, ex);
   else if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, ex);
   else oz_col_exp_kernel<<<unsigned(rows), 256, 0, s>>>(X, K, rows, ks, ex);
   oz_split_kernel<TR><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(RP / 8)), OZ_SPLIT_WARPS * 32, 0, s>>>(
@@ -793,7 +802,7 @@ cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ld
   int* dk = reinterpret_cast<int*>(dig + oz_a_bytes(M, K));
   int *lex = dk + K, *uex = lex + M;
   const double2* u = static_cast<const double2*>(U);
-  oz_balanced_col_exp_kernel<<<oz_cdiv(N, 64), 64, 0, s>>>(u, N, K, ldu, nullptr, uex);
+  oz_balanced_col_exp_kernel<<<oz_cdiv(N, 32), 256, 0, s>>>(u, N, K, ldu, nullptr, uex);
   oz_balance_kernel<<<unsigned(K), 256, 0, s>>>(u, N, ldu, uex, dk);
   cudaError_t e = launched(2);
   if (e == cudaSuccess)
