@@ -130,7 +130,7 @@ uint64_t fosb_kernel_launches(void);
  * (then clears) the family's total device time in ms, launch count and work:
  *   "lu_update"      tcgen05 complex64 trailing update, work = 8 M N K flops
  *   "lu_panel"       cooperative panel factorisation, work = 8 m jb^2 / 2 flops
- *   "asm_regular"    regular-pair assembly, work = point pairs (36 per triangle pair)
+ *   "asm_regular"    regular-pair assembly, work = point pairs (36 per unordered triangle pair)
  *   "asm_singular"   Sauter-Schwab pairs, work = point pairs
  *   "gemm_ff"        float-float complex128 GEMM, work = 8 M N K flops
  * Any pointer may be NULL. */
@@ -192,7 +192,8 @@ fosb_status fosb_assemble_efie(fosb_mesh mesh, double k, const fosb_quad_opts* o
  *          handle also owns two residual copies of Z: a float-float split (16 n^2 bytes)
  *          and, for n >= 256, exact bf16 digit tiles (28 n^2 bytes) for the FP64-class
  *          tensor-core residuals of solves with 5 or more right-hand sides; and the
- *          inverses of its 64 x 64 diagonal blocks for the streaming triangular sweeps.
+ *          inverses of its 64 x 64 diagonal blocks (with their products with the
+ *          neighbouring tiles) for the streaming triangular sweeps.
  * Synchronises `stream` at the end (the pivot search reports FOSB_ERR_SINGULAR).
  * Errors: FOSB_ERR_OOM when device memory runs out (nothing is leaked). */
 fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu* out, void* stream);
@@ -491,9 +492,9 @@ fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, const void* A,
  * Every spin-wait of the library's kernels gives up after a number of polls, sets the
  * status word of the call to FOSB_ERR_TIMEOUT and returns, so the call reports
  * FOSB_ERR_TIMEOUT and the context stays usable.  This sets that number for the LU panel
- * grid barriers and the streaming triangular-sweep flags on the current device (polls <= 0
+ * grid barriers and the streaming triangular sweeps' waits on the current device (polls <= 0
  * restores the default 2^26, about 2 s); failure-detection tests use a tiny limit to make
- * the waits run out.  The tensor-core kernels keep their own limits.  A factorisation whose
+ * the waits run out.  The tensor-core and cluster-panel kernels keep their own limits.  A factorisation whose
  * wait ran out leaves its outputs unspecified; destroy and recreate its handle. */
 fosb_status fosb_debug_set_wait_limit(int64_t polls);
 

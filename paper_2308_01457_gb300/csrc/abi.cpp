@@ -218,8 +218,11 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   const bool digits = lu->zdig && nrhs > 4;
   Scratch dx(s), xex(s);
   if (digits) {
-    FOSB_CUDA(dx.alloc(sizeof(double) * 2 * n * nrhs));
     FOSB_CUDA(xex.alloc(sizeof(int) * 2 * nrhs));
+    if (dx.alloc(sizeof(double) * 2 * n * nrhs) != cudaSuccess) {  // no room: full residuals
+      dx.p = nullptr;
+      cudaGetLastError();
+    }
   }
   std::vector<double> bn, xn, rn, xfull;
   FOSB_TRY(col_norms(Bsrc, n, nrhs, ldbs, nb.as<double>(), bn, s));
@@ -237,7 +240,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   int it = 0;
   for (; solver != FOSB_REFINE_GMRES;) {
     FOSB_TRY(col_norms(X, n, nrhs, ldx, nb.as<double>(), xn, s));
-    bool full = !digits || it == 0;
+    bool full = !dx.p || it == 0;
     for (int64_t c = 0; c < nrhs && !full; ++c) full = !(xn[c] >= 0.5 * xfull[c]);
     if (full) {
       FOSB_CUDA(copy_matrix(Bsrc, n, nrhs, ldbs, r.p, nrhs, 16, s));
