@@ -85,7 +85,7 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 tensor ratio of the part
 LU_BLOCK = 256  # column block of the complex64 LU: every trailing update has K = 256
 # DRAM bytes (read + write) per complex64 output element of one tcgen05 LU-update launch,
 # from the ncu capture summarised in profiles/ (C is read and written once: 16 B algorithmic)
-LU_UPDATE_DRAM_BYTES_PER_OUTPUT = (653.6512e6 + 390.073344e6) / 7424.0**2  # 18.94 B
+LU_UPDATE_DRAM_BYTES_PER_OUTPUT = (543.779072e6 + 382.323712e6) / 7424.0**2  # 16.80 B
 
 
 def _peaks():
@@ -272,30 +272,30 @@ def run_fosb(args):
     fp_peak = upeaks["fp32"] if arith == F.ASM_FF else upeaks["fp64"]
     # algorithmic work -> (bound, flops, peak, kernel, note) per family
     fam_model = {
-        "lu_update": ("tensor", 1.0, tf32_peak,
-                      "cgemm_update_split_kernel (persistent tcgen05 kind::tf32 N = 256, 3xTF32 complex, operands "
+        "lu_update": ("tensor", 1.0, bf16,
+                      "cgemm_update_split_kernel (persistent tcgen05 kind::f16 N = 256, fp16-pair complex, operands "
                       "split once per block and bulk-copied; the split kernels are timed with it)",
-                      f"TF32 dense = bf16 sustained {bf16} ({bf16_src}) x 1.1/2.25; work = useful complex flops "
-                      "8MNK; 3xTF32 executes 3x that on the tensor pipe (tensor_pipe_frac: executed TF32 rate / "
-                      "the TF32 MMA rate fosb_peak_microbench measures, which is above the nominal-ratio peak)"),
+                      f"fp16 dense = bf16 sustained {bf16} ({bf16_src}); work = useful complex flops 8MNK; fp16 pairs "
+                      "execute 3x that on the tensor pipe (tensor_pipe_frac: executed rate / the 16-bit MMA rate "
+                      "fosb_peak_microbench measures)"),
         "lu_update64": ("tensor", 1.0, tf32_peak,
                         "cgemm_update_tc_ws_kernel (the K = 64 updates inside each 256-column block of the LU)",
                         "work = useful complex flops 8MNK"),
         "asm_regular": ("alu", 27.0, fp_peak,
-                        "efie_regular_ff_kernel" if arith == F.ASM_FF else "efie_regular_kernel<double>",
-                        "27 algorithmic FP ops per point pair; peak = the FP32 (float-float) or FP64 FMA pipe "
+                        "efie_regular_ff_kernel" if arith == F.ASM_FF else "efie_regular_fp64_kernel",
+                        "27 algorithmic FP ops per unordered point pair; peak = the FP32 (float-float) or FP64 FMA pipe "
                         "measured by fosb_peak_microbench"),
         "gemm_ff": ("alu", 1.0, upeaks["fp32"], "zgemm_ff_kernel (float-float complex128 GEMM)",
                     "work = complex128 flops 8MNK executed as ~48 FP32 instructions per complex MAC; "
                     "peak = measured FP32 FMA pipe"),
-        "lu_panel": ("latency", 1.0, None, "tslu_gepp_kernel (tournament-pivoting panel)",
+        "lu_panel": ("latency", 1.0, None, "panel_cluster_kernel (tournament-pivoting panel)",
                      "latency-bound: 64 sequential pivot steps per tree level"),
         "gemm_oz": ("tensor", 1.0, bf16, "oz_gemm_kernel (bf16 digit-split tcgen05, FP64-class complex)",
-                    "work = complex128 flops 8MNK; executes 112 bf16 MMAs (28 digit pairs x 4) per complex product, "
-                    "so frac <= 8/(112 x 2)"),
-        "trsm_update": ("tensor", 1.0, tf32_peak, "cgemm_update_tc_ws_kernel in the blocked triangular sweeps (K = 64)",
-                        "sweep updates of solves with 16 or more right-hand sides; work = useful complex flops 8MNK"),
-        "oz_prep": ("hbm", 1.0, peaks.get("hbm_gbs", 6800.0), "oz_row_exp_kernel + oz_split_a_kernel (digit tiles of Z)",
+                    "work = complex128 flops 8MNK; executes up to 28 digit pairs x 4 real products per complex "
+                    "product, so frac is about 8/(112 x 2) at most"),
+        "trsm_update": ("tensor", 1.0, tf32_peak, "cgemm_update_tc_ws_kernel between superblocks of the triangular sweeps (K = 512)",
+                        "sweep updates of solves with many right-hand sides; work = useful complex flops 8MNK"),
+        "oz_prep": ("hbm", 1.0, peaks.get("hbm_gbs", 6800.0), "oz_row_exp_kernel + oz_split_kernel (digit tiles of Z)",
                     "work = bytes: 16 B read + 28 B of digits written per element of Z"),
         # the whole triangular solve; it contains the trsm_update launches, so it is not a
         # candidate for the dominant family
@@ -320,8 +320,8 @@ def run_fosb(args):
         if LU_UPDATE_DRAM_BYTES_PER_OUTPUT is not None:
             roofline["traffic"] = round(LU_UPDATE_DRAM_BYTES_PER_OUTPUT * avg_outputs)
         roofline["algorithmic_bytes"] = round(16.0 * avg_outputs)
-        if upeaks.get("tf32"):
-            roofline["tensor_pipe_frac"] = round(3.0 * achieved / upeaks["tf32"], 4)
+        if upeaks.get("bf16"):
+            roofline["tensor_pipe_frac"] = round(3.0 * achieved / upeaks["bf16"], 4)
     secondary = {}
     for f, (b, wsc, pk, kn, _) in fam_model.items():
         s_ = fam_stats[f]
@@ -339,7 +339,7 @@ def run_fosb(args):
         "metric": METRIC, "value": round(ms / 1e3, 4), "unit": "s per FOSB step", "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "mixed: 3xTF32 tensor-core LU (c64 factors), float-float (f32x2) assembly and FP64-class "
+        "dtype": "mixed: fp16-pair tensor-core LU (c64 factors), float-float (f32x2) assembly and FP64-class "
                  "refinement residuals, f64 singular quadrature", "data": "synthetic",
         "config": {"workload": args.workload, "levels": W["levels"], "N_levels": [N[l] for l in sorted(N)],
                    "triangles_finest": T, "k": W["k"], "n_dir": W["n_dir"], "ct": [W["L0"], W["L"]],
@@ -448,10 +448,10 @@ def run_batched(args):
         fam[f] = (ms_c.value / 2, n_c.value / 2, w_c.value / 2)
     peaks = _peaks()
     bf16 = peaks.get("bf16_tflops_sustained", 1700.0)
-    model = {"lu_update": ("tensor", 1.0, bf16 * TF32_PER_BF16, "cgemm_update_split_kernel"),
+    model = {"lu_update": ("tensor", 1.0, bf16, "cgemm_update_split_kernel"),
              "lu_update64": ("tensor", 1.0, bf16 * TF32_PER_BF16, "cgemm_update_tc_ws_kernel"),
              "asm_regular": ("alu", 27.0, upeaks["fp32"], "efie_regular_ff_batched_kernel (persistent, ticketed tiles)"),
-             "lu_panel": ("latency", 1.0, None, "tslu_gepp_kernel"),
+             "lu_panel": ("latency", 1.0, None, "panel_cluster_kernel"),
              "asm_singular": ("alu", 1.0, None, "efie_singular_batched_kernel"),
              "gemm_oz": ("tensor", 1.0, bf16, "oz_gemm_kernel"), "gemm_ff": ("alu", 1.0, upeaks["fp32"], "zgemm_ff_kernel"),
              "oz_prep": ("hbm", 1.0, peaks.get("hbm_gbs", 6800.0), "oz digit prep")}
@@ -462,7 +462,7 @@ def run_batched(args):
     roofline = {"bound": bound, "achieved": round(ach, 3), "peak": round(pk, 2) if pk else None, "unit": unit,
                 "frac": round(ach / pk, 4) if pk else None, "traffic": None, "kernel": kname, "family": dom,
                 "ms_per_step": round(fam[dom][0], 2), "launches_per_step": fam[dom][1],
-                "peak_source": "measured (MEASURED_PEAKS.json bf16 sustained x 1.1/2.25 for TF32; FP32 FMA pipe by "
+                "peak_source": "measured (MEASURED_PEAKS.json bf16 sustained, x 1.1/2.25 for TF32; FP32 FMA pipe by "
                                "fosb_peak_microbench); family times overlap across the worker streams"}
     calls = {f: {"ms_per_step": round(v[0], 2), "launches_per_step": v[1]} for f, v in fam.items()}
     N = [h.n_edges for h in prob.handles]
@@ -473,7 +473,7 @@ def run_batched(args):
     line = {"metric": METRIC, "value": round(ms / 1e3, 4), "unit": "s per batch step", "n_gpus": ws,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "mixed: float-float (f32x2) regular pairs, f64 singular pairs, 3xTF32 tensor-core LU "
+            "dtype": "mixed: float-float (f32x2) regular pairs, f64 singular pairs, fp16-pair tensor-core LU "
                      "(c64 factors) with FP64-class refinement", "data": "synthetic",
             "config": {"workload": args.workload, "scatterers": len(N),
                        "N_counts": {str(n): N.count(n) for n in sorted(set(N))}, "n_dir": W["n_dir"],
@@ -566,7 +566,7 @@ def run_mc(args):
     line = {"metric": METRIC, "value": round(ms / 1e3, 4), "unit": "s per Monte Carlo run", "n_gpus": ws,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "mixed: float-float regular pairs, f64 singular pairs, 3xTF32 LU with FP64-class refinement",
+            "dtype": "mixed: float-float regular pairs, f64 singular pairs, fp16-pair LU with FP64-class refinement",
             "data": "synthetic",
             "config": {"workload": args.workload, "N": N, "samples": W["nsamp"], "k": W["k"], "n_dir": W["n_dir"],
                        "sigma": W["sigma"], "ell": W["ell"], "scatterer": "PEC" if W.get("eps_r") is None else
@@ -664,7 +664,7 @@ def run_lowrank(args):
     line = {"metric": METRIC, "value": round(ms / 1e3, 4), "unit": "s per FOSB step", "n_gpus": ws,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "mixed: float-float regular pairs, f64 singular pairs, 3xTF32 LU with FP64-class refinement, "
+            "dtype": "mixed: float-float regular pairs, f64 singular pairs, fp16-pair LU with FP64-class refinement, "
                      "f64 pivoted Cholesky", "data": "synthetic",
             "config": {"workload": args.workload, "N": prob.levels[L].mesh.n_edges, "V": V, "k": W["k"],
                        "n_dir": W["n_dir"], "sigma": W["sigma"], "ell": W["ell"], "tol": W["tol"],
@@ -791,7 +791,6 @@ def run_pmchwt(args):
     phase = {k: round(statistics.mean(v), 2) for k, v in timers.items()}
     peaks = _peaks()
     bf16 = peaks.get("bf16_tflops_sustained", 1700.0)
-    tf32_peak = bf16 * TF32_PER_BF16
     model = {
         "pmchwt_regular": ("alu", PMCHWT_OPS_PER_POINT_PAIR, upeaks["fp32" if arith == F.ASM_FF else "fp64"],
                            "pmchwt_regular_ff_kernel (float-float)" if arith == F.ASM_FF
@@ -799,9 +798,9 @@ def run_pmchwt(args):
                            f"{PMCHWT_OPS_PER_POINT_PAIR:.0f} algorithmic FP64-class ops per point pair and "
                            "wavenumber (work = point pairs of both launches); peak = the FP32 (float-float) or FP64 "
                            "FMA pipe measured by fosb_peak_microbench"),
-        "lu_update": ("tensor", 1.0, tf32_peak, "cgemm_update_split_kernel (tcgen05 kind::tf32, 3xTF32 complex)",
-                      "TF32 dense = measured bf16 sustained x 1.1/2.25; work = useful complex flops 8MNK"),
-        "lu_panel": ("latency", 1.0, None, "tslu_gepp_kernel (tournament-pivoting panel)", "latency-bound"),
+        "lu_update": ("tensor", 1.0, bf16, "cgemm_update_split_kernel (tcgen05 kind::f16, fp16-pair complex)",
+                      "fp16 dense = measured bf16 sustained; work = useful complex flops 8MNK"),
+        "lu_panel": ("latency", 1.0, None, "panel_cluster_kernel (tournament-pivoting panel)", "latency-bound"),
         "pmchwt_singular": ("alu", 1.0, None, "pmchwt_singular_kernel (FP64 Sauter-Schwab)",
                             "work = touching pairs per launch"),
     }
@@ -853,7 +852,7 @@ def run_pmchwt(args):
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
             "dtype": ("mixed: float-float (f32x2) regular pairs, f64 singular pairs" if arith == F.ASM_FF
-                      else "mixed: f64 assembly") + ", 3xTF32 tensor-core LU (c64 factors) with FP64-class refinement",
+                      else "mixed: f64 assembly") + ", fp16-pair tensor-core LU (c64 factors) with FP64-class refinement",
             "data": "synthetic",
             "config": {"workload": args.workload, "triangles": sm.nt, "N": N, "unknowns": 2 * N, "k0": W["k"],
                        "eps_r": W["eps_r"], "mu_r": W["mu_r"], "n_dir": W["n_dir"], "assembly": args.arith,
@@ -961,7 +960,7 @@ def run_dect(args):
     line = {"metric": METRIC, "value": round(ms / 1e3, 4), "unit": "s per CT step", "n_gpus": ws,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 2), "higher_is_better": False,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": "mixed: float-float (f32x2) regular pairs, f64 singular pairs, 3xTF32 tensor-core LU with "
+            "dtype": "mixed: float-float (f32x2) regular pairs, f64 singular pairs, fp16-pair tensor-core LU with "
                      "FP64-class refinement", "data": "synthetic",
             "config": {"workload": args.workload, "levels": W["levels"],
                        "unknowns": [2 * prob.meshes[l].n_edges for l in W["levels"]], "k0": W["k"],
@@ -1063,7 +1062,7 @@ def run_fp64_compare(W, meshes, dirs, out_mixed, ms_mixed):
                         "factor_finest": round(sum(x.elapsed_time(y) for x, y in timers[f"factor_l{L}"]), 2),
                         "covariance_ct": round(sum(x.elapsed_time(y) for x, y in timers["covariance_ct"]), 2)},
            "rel_diff_mean_farfield": rel(out_mixed[0], Fm), "rel_diff_ct_covariance": rel(out_mixed[1], cov),
-           "note": "one step, same workload, FP64 assembly and complex128 LU (DMMA), timed with CUDA events"}
+           "note": "one step, same workload, FP64 assembly and complex128 LU (trailing updates in digits), timed with CUDA events"}
     prob.release()
     del prob
     torch.cuda.empty_cache()

@@ -12,7 +12,7 @@
 //   sin/cos(j pi/512); |delta| <= pi/1024, so sin(delta) - delta and cos(delta) - 1 are a few FP32
 //   terms and only two products and their sum need error-free transformations;
 //   G0 = exp(i theta)/r.
-// What bounds it is FP32 issue (about 430 instructions per point pair).  N = 30720, 7.5 G point pairs: 96
+// What bounds it is FP32 issue (about 430 instructions per point pair).  N = 30720, 7.5 G point pairs: 98
 // ms (106 with a 128-entry phase table and FP32 rounding and conversion on the slow pipe).
 // The pair's 3 x 3 barycentric moment matrix
 //   mu_ab = sum_pq w_p w_q lambda_pa beta_qb G0(x_p, y_q)
@@ -217,7 +217,7 @@ __device__ __forceinline__ void regular_ff_pair(const DevMesh& m, const FFConst&
       const ff kr = ff_mul(C.k, r);
       expi_ff(kr, C, tab, cs, sn);
       CFF G[MFIO ? 2 : 1];
-      G[0] = {mul_raw(cs, rinv), mul_raw(sn, rinv)};
+      G[0] = {ff_mul(cs, rinv), ff_mul(sn, rinv)};
       if constexpr (MFIO) {
         // g = G (ikr - 1) / r^2: Re = -(G.r + G.i kr) / r^2, Im = (G.r kr - G.i) / r^2
         const ff rinv2 = ff_sqr(rinv);
