@@ -31,9 +31,13 @@
 //   warp 0  producer: per slab waits empty[s], expect_tx 40 KB, two bulk copies;
 //   warp 1  MMA issuer: waits full[s], 6 MMAs into accumulator buffer b, commits empty[s];
 //           after a tile's last slab commits tfull[b];
-//   warps 2-5 epilogue (TMEM lane quarters 2, 3, 0, 1): per 64-column half, C is prefetched
-//           by cp.async into a padded shared tile, the accumulator row of each thread is
-//           subtracted in place, and the half is stored with coalesced 16-byte writes.
+//   warps 2-9 epilogue, two groups of four (TMEM lane quarters 2, 3, 0, 1): per 32-column quarter,
+//           C is prefetched by cp.async into a padded shared tile, the accumulator row of each thread
+//           is subtracted in place, and the quarter is stored with coalesced 16-byte writes.
+// The 59 updates of an N = 15360 factorisation: 26.4 ms with one group on 64-column halves, 22.4 ms so.
+// What bounds it: operands and C reach the SMs at 11 TB/s, and the MMAs' operand reads with the copies'
+// writes want 146 of the 128 B a clock that shared memory gives at the full MMA rate (an elected MMA
+// lane and waits tested ahead changed nothing).
 // Every wait is bounded; a time-out sets the status word and an abort flag, the MMA thread
 // drains its MMAs and the producer waits for its copies in flight before TMEM is freed.
 #include <cuda_fp16.h>
@@ -56,11 +60,12 @@ constexpr int U_ABYTES = 4 * U_PART;           // A parts of one slab
 constexpr int U_BBYTES = 6 * U_PART;           // B parts of one slab
 constexpr int U_STAGE = U_ABYTES + U_BBYTES;   // 40 KB
 constexpr int U_STAGES = 3;
-constexpr int U_EPI_LD = 66;                   // padded float2 row of the 64-column tile (16-byte rows)
-constexpr int U_EPI_BYTES = U_TM * U_EPI_LD * 8;
+constexpr int U_EPI_N = 32;                    // columns of C that an epilogue group holds at a time
+constexpr int U_EPI_LD = U_EPI_N + 2;          // padded float2 row of them (16-byte rows)
+constexpr int U_EPI_BYTES = 2 * U_TM * U_EPI_LD * 8;
 constexpr int U_EPI_OFF = U_STAGES * U_STAGE;
 constexpr int U_SMEM = U_EPI_OFF + U_EPI_BYTES + 1024;  // + alignment slack
-constexpr int U_THREADS = 6 * 32;
+constexpr int U_THREADS = 10 * 32;              // producer, MMA, two epilogue groups of four warps
 constexpr int U_GROUP = 16;                    // row tiles per super-row
 constexpr long long U_SPIN = 1ll << 24;
 static_assert(U_SMEM <= 227 * 1024, "stages and drain tile exceed shared memory");
@@ -129,9 +134,9 @@ __device__ __forceinline__ void u_bar(int id, int n) { asm volatile("bar.sync %0
 __device__ __forceinline__ void u_cp16(uint32_t dst, const void* src, int bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-// float2 index of the 16-byte piece holding columns (2 j, 2 j + 1) of row r in the 64-column
-// drain tile; the 528-byte row pitch keeps 8 consecutive rows reading piece j in 8 different
-// bank groups (row-per-thread phase) and a row's 32 pieces contiguous (coalesced phases)
+// float2 index of the 16-byte piece holding columns (2 j, 2 j + 1) of row r in a 32-column
+// buffer; the 272-byte row pitch keeps 8 consecutive rows reading piece j in 8 different
+// bank groups (row-per-thread phase) and a row's 16 pieces contiguous (coalesced phases)
 __device__ __forceinline__ int u_piece(int r, int j) { return r * U_EPI_LD + (j << 1); }
 __device__ __forceinline__ void u_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void u_cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
@@ -279,12 +284,11 @@ __global__ void __launch_bounds__(U_THREADS, 1)
                               int vec_ok) {
   extern __shared__ unsigned char u_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(u_raw) + 1023) & ~uintptr_t(1023));
-  float2* sE = reinterpret_cast<float2*>(smem + U_EPI_OFF);
   __shared__ uint64_t bar_full[U_STAGES], bar_empty[U_STAGES], bar_tfull[2], bar_tempty[2], bar_drain;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
-  __shared__ volatile int epi_stop;
-  __shared__ float s_inv_b[U_TN];  // the tile's column scales
+  __shared__ volatile int epi_stop[2];
+  __shared__ float s_inv_b[2][U_TN];  // the column scales of each epilogue group's tile
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t RT = (M + U_TM - 1) / U_TM, CT = (N + U_TN - 1) / U_TN, tiles = RT * CT;
   if (warp == 0) {
@@ -298,12 +302,12 @@ __global__ void __launch_bounds__(U_THREADS, 1)
     }
     for (int i = 0; i < 2; ++i) {
       u_init(su32(&bar_tfull[i]), 1);
-      u_init(su32(&bar_tempty[i]), 128);
+      u_init(su32(&bar_tempty[i]), 256);
     }
     u_init(su32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
     abort_sh = 0;
-    epi_stop = 0;
+    epi_stop[0] = epi_stop[1] = 0;
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
@@ -385,15 +389,20 @@ __global__ void __launch_bounds__(U_THREADS, 1)
     }
     __syncwarp();
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2-5)
-    // Per 64-column half of a tile: the C half-tile is copied into the padded shared tile by
-    // cp.async (4096 16-byte pieces in flight; for the first half issued before the
-    // accumulator wait), thread r subtracts its TMEM row (lane r) in place, and the half is
-    // stored with coalesced 16-byte writes.  Without 16-byte alignment of C the tile takes
-    // the negated accumulator and C is updated element by element.
-    const int et = tid - 2 * 32;             // 0..127
-    const int lane_base = (warp & 3) * 32;   // TMEM lane quarter of this warp
+    // ------------------------------------------------------------ epilogue (warps 2-9)
+    // Two groups of four warps, each with its own buffer and barrier, take the 32-column quarters
+    // g and g + 2 of a tile: the quarter of C is copied into the padded shared tile by cp.async (for
+    // the first quarter issued before the accumulator wait), thread r subtracts its TMEM row (lane
+    // r) in place, and the quarter is stored with coalesced 16-byte writes.  One group on 64-column
+    // halves left the tensor pipe 44 % active: a half's way from and to memory took longer than its
+    // MMAs.  Without 16-byte alignment of C the tile takes the negated accumulator and C is updated
+    // element by element.
+    const int grp = (warp - 2) >> 2;
+    const int et = tid - 2 * 32 - grp * 128;  // 0..127
+    const int lane_base = (warp & 3) * 32;    // TMEM lane quarter of this warp
     const int r_local = lane_base + lane;
+    float2* sE = reinterpret_cast<float2*>(smem + U_EPI_OFF) + grp * (U_TM * U_EPI_LD);
+    float* s_scale = s_inv_b[grp];
     int64_t tcount = 0;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++tcount) {
       const int b = int(tcount & 1);
@@ -403,28 +412,29 @@ __global__ void __launch_bounds__(U_THREADS, 1)
       const int64_t row0 = rt * U_TM, col0 = ct * U_TN;
       const uint32_t d = tmem + uint32_t(b) * 256 + (uint32_t(lane_base) << 16);
       const float sa = -inv_a[row0 + r_local];
-      s_inv_b[et] = inv_b[col0 + et];  // read after the barrier below; the last tile's reads are behind one
+      s_scale[et] = inv_b[col0 + et];  // read after the barrier below; the last tile's reads are behind one
 #pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
+      for (int h = grp; h < 4; h += 2) {
+        const int64_t gc0 = col0 + h * U_EPI_N;
         if (vec_ok) {
 #pragma unroll 8
-          for (int q = 0; q < 32; ++q) {
-            const int e = et + 128 * q;  // 0 .. 4095 pairs of complex
-            const int r = e >> 5, c = (e & 31) * 2;
-            const int64_t gr = row0 + r, gc = col0 + h * 64 + c;
+          for (int q = 0; q < U_EPI_N / 2; ++q) {
+            const int e = et + 128 * q;  // 0 .. 2047 pairs of complex
+            const int r = e / (U_EPI_N / 2), c = (e % (U_EPI_N / 2)) * 2;
+            const int64_t gr = row0 + r, gc = gc0 + c;
             const int bytes = gr < M ? (gc + 1 < N ? 16 : (gc < N ? 8 : 0)) : 0;
             u_cp16(su32(&sE[u_piece(r, c >> 1)]), bytes ? static_cast<const void*>(C + gr * ldc + gc) : C, bytes);
           }
           u_cp_commit();
         }
-        if (h == 0) {
+        if (h == grp) {
           // the stop decision must be the same in all four warps (they share named barriers)
           if (!u_wait(su32(&bar_tfull[b]), uint32_t(ub & 1))) {
             fail();
-            epi_stop = 1;
+            epi_stop[grp] = 1;
           }
-          u_bar(1, 128);
-          if (epi_stop) {
+          u_bar(1 + grp, 128);
+          if (epi_stop[grp]) {
             u_cp_wait_all();  // no copy may land after the kernel has left
             break;
           }
@@ -432,20 +442,19 @@ __global__ void __launch_bounds__(U_THREADS, 1)
         }
         if (vec_ok) {
           u_cp_wait_all();
-          u_bar(1, 128);  // every thread's pieces of C are in the tile
+          u_bar(1 + grp, 128);  // every thread's pieces of C are in the tile
         }
-#pragma unroll 1
-        for (int cs = 0; cs < 2; ++cs) {
+        {
           uint32_t vr[32], vi[32];
-          u_ld32(d + h * 64 + cs * 32, vr);
-          u_ld32(d + 128 + h * 64 + cs * 32, vi);
+          u_ld32(d + h * U_EPI_N, vr);
+          u_ld32(d + 128 + h * U_EPI_N, vi);
           asm volatile("tcgen05.wait::ld.sync.aligned;");
 #pragma unroll
-          for (int j = 0; j < 32; j += 2) {
-            float4* p = reinterpret_cast<float4*>(&sE[u_piece(r_local, cs * 16 + (j >> 1))]);
+          for (int j = 0; j < U_EPI_N; j += 2) {
+            float4* p = reinterpret_cast<float4*>(&sE[u_piece(r_local, j >> 1)]);
             float4 c4 = vec_ok ? *p : make_float4(0.f, 0.f, 0.f, 0.f);
             // (acc 2^-ea) 2^-eb: two exact scalings, so neither product of scales can overflow
-            const float s0 = s_inv_b[h * 64 + cs * 32 + j], s1 = s_inv_b[h * 64 + cs * 32 + j + 1];
+            const float s0 = s_scale[h * U_EPI_N + j], s1 = s_scale[h * U_EPI_N + j + 1];
             c4.x = fmaf(__uint_as_float(vr[j]) * sa, s0, c4.x);
             c4.y = fmaf(__uint_as_float(vi[j]) * sa, s0, c4.y);
             c4.z = fmaf(__uint_as_float(vr[j + 1]) * sa, s1, c4.z);
@@ -453,17 +462,17 @@ __global__ void __launch_bounds__(U_THREADS, 1)
             *p = c4;
           }
         }
-        if (h == 1) {  // every accumulator value of this buffer has been read
+        if (h >= 2) {  // every accumulator value of this group's quarters has been read
           asm volatile("tcgen05.fence::before_thread_sync;");
           u_arrive(su32(&bar_tempty[b]));
         }
-        u_bar(1, 128);
+        u_bar(1 + grp, 128);
         if (vec_ok) {
 #pragma unroll 8
-          for (int q = 0; q < 32; ++q) {
+          for (int q = 0; q < U_EPI_N / 2; ++q) {
             const int e = et + 128 * q;
-            const int r = e >> 5, c = (e & 31) * 2;
-            const int64_t gr = row0 + r, gc = col0 + h * 64 + c;
+            const int r = e / (U_EPI_N / 2), c = (e % (U_EPI_N / 2)) * 2;
+            const int64_t gr = row0 + r, gc = gc0 + c;
             if (gr < M && gc + 1 < N) {
               *reinterpret_cast<float4*>(C + gr * ldc + gc) = *reinterpret_cast<const float4*>(&sE[u_piece(r, c >> 1)]);
             } else if (gr < M && gc < N) {
@@ -472,10 +481,10 @@ __global__ void __launch_bounds__(U_THREADS, 1)
           }
         } else {
 #pragma unroll 4
-          for (int q = 0; q < 64; ++q) {
-            const int e = et + 128 * q;  // 0 .. 8191
-            const int r = e >> 6, c = e & 63;
-            const int64_t gr = row0 + r, gc = col0 + h * 64 + c;
+          for (int q = 0; q < U_EPI_N; ++q) {
+            const int e = et + 128 * q;  // 0 .. 4095
+            const int r = e / U_EPI_N, c = e % U_EPI_N;
+            const int64_t gr = row0 + r, gc = gc0 + c;
             if (gr < M && gc < N) {  // the tile holds -D here: C += it
               const float2 dd = sE[u_piece(r, c >> 1) + (c & 1)];
               float2 o = C[gr * ldc + gc];
@@ -485,8 +494,9 @@ __global__ void __launch_bounds__(U_THREADS, 1)
             }
           }
         }
-        u_bar(1, 128);  // the tile is free for the next half's copies
+        u_bar(1 + grp, 128);  // the buffer is free for the next quarter's copies
       }
+      if (epi_stop[grp]) break;
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
