@@ -12,7 +12,7 @@
 //   sin/cos(j pi/512); |delta| <= pi/1024, so sin(delta) - delta and cos(delta) - 1 are a few FP32
 //   terms and only two products and their sum need error-free transformations;
 //   G0 = exp(i theta)/r.
-// What bounds it is FP32 issue (about 430 instructions per point pair).  N = 30720, 7.5 G point pairs: 98
+// What bounds it is FP32 issue (456 instructions per point pair).  N = 30720, 7.5 G point pairs: 98
 // ms (106 with a 128-entry phase table and FP32 rounding and conversion on the slow pipe).
 // The pair's 3 x 3 barycentric moment matrix
 //   mu_ab = sum_pq w_p w_q lambda_pa beta_qb G0(x_p, y_q)
