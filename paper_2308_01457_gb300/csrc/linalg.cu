@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(256) col_absmax_kernel(const double2* __restri
                                                          int64_t lda, int cw, double* out) {
   __shared__ unsigned long long red[256];
   const int lanes = 256 / cw, cl = int(threadIdx.x) % cw, rl = int(threadIdx.x) / cw;
-  const int64_t col = int64_t(blockIdx.y) * cw + cl, r0 = int64_t(blockIdx.x) * 32 * lanes;
+  const int64_t col = int64_t(blockIdx.x) * cw + cl, r0 = int64_t(blockIdx.y) * 32 * lanes;
   unsigned long long m = 0ull;
   if (col < cols) {
 #pragma unroll 8
@@ -1635,8 +1635,8 @@ cudaError_t absmax_c128(const void* A, int64_t rows, int64_t cols, int64_t lda, 
   if (rows * cols == 0) return cudaSuccess;
   int cw = 1;
   while (cw < 32 && cw < cols) cw *= 2;
-  if (cdiv(cols, cw) > 65535u) return cudaErrorInvalidValue;
-  col_absmax_kernel<<<dim3(cdiv(rows, 32 * (256 / cw)), cdiv(cols, cw)), 256, 0, s>>>(static_cast<const double2*>(A), rows,
+  if (cdiv(rows, 32 * (256 / cw)) > 65535u) return cudaErrorInvalidValue;  // 16.7 M rows
+  col_absmax_kernel<<<dim3(cdiv(cols, cw), cdiv(rows, 32 * (256 / cw))), 256, 0, s>>>(static_cast<const double2*>(A), rows,
                                                                                   cols, lda, cw, d_out);
   return launched();
 }
