@@ -1,8 +1,10 @@
 // Trailing update C -= A B of the blocked complex64 LU on the tcgen05 tensor cores, fed by
 // bulk copies of operands split once per block into two fp16 values per real number.
 //
-// The split.  Every row i of A and column j of B is scaled by a power of two that brings its
-// largest |Re|, |Im| into [2^14, 2^15), and x s = x_h + x_l with x_h = fp16(x s), x_l = fp16(x s - x_h):
+// The split.  A and B are first balanced along k: row k of B over 2^{d_k}, column k of A times 2^{d_k},
+// d_k the exponent of the largest entry of B's row k relative to its column's largest.  Then every row
+// i of A and column j of B is scaled by a power of two that brings its largest |Re|, |Im| into
+// [2^14, 2^15), and x s = x_h + x_l with x_h = fp16(x s), x_l = fp16(x s - x_h):
 //   x y ~ x_h y_h + x_h y_l + x_l y_h,
 // accumulated in FP32 and scaled back exactly.  fp16 carries 11 significand bits as TF32 does, so
 // the pair holds 22 bits like the 3xTF32 split (down to 2^-18 of the row's largest value, below
@@ -10,6 +12,9 @@
 // Error against 64 bits at K = 256, normwise: 1.9e-6 (3xTF32 3.6e-6) on uniform operands, on operands graded
 // over six decades inside their rows and on ones scaled by row and column over as many: half as
 // many accumulations in the tensor core.
+// The balance is for matrices whose rows differ in scale: U12's rows then carry the scales and L21's
+// columns their inverses, so the products are of one size but lie far below a row's times a column's
+// largest value.
 //
 // Split once, copied many times.  A (L21, M x K) and B (U12, K x N) are each split by one
 // pass per column block (K <= 256) into the exact shared-memory image the MMAs read: for every
@@ -142,21 +147,28 @@ __device__ __forceinline__ void u_cp_commit() { asm volatile("cp.async.commit_gr
 __device__ __forceinline__ void u_cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // ---------------------------------------------------------------- splits
-// Power of two that brings a row's or column's largest |Re|, |Im| (as a float bit pattern) into
-// [2^14, 2^15), and its inverse: exponents kept inside the normal range (both exact), one for
-// zero and for what is not finite.
-__device__ __forceinline__ float split_scale(unsigned mb, float& inv) {
-  const int e = int(mb >> 23);  // biased; 0 for zero and subnormals
-  const int sh = (e == 0 || e == 255) ? 0 : max(-110, min(110, 14 + 127 - e));
-  inv = __uint_as_float(unsigned(127 - sh) << 23);
-  return __uint_as_float(unsigned(127 + sh) << 23);
+// 2^e for a normal result, and x 2^e for |e| <= 252 as two exact factors
+__device__ __forceinline__ float pow2(int e) { return __uint_as_float(unsigned(127 + e) << 23); }
+__device__ __forceinline__ float scale2(float x, int e) { return x * pow2(e >> 1) * pow2(e - (e >> 1)); }
+// Biased exponent of the larger of |Re|, |Im|: kNone for zero, kBad for infinities and NaN.
+constexpr int kNone = -(1 << 20), kBad = 1 << 20;
+__device__ __forceinline__ int value_exp(float2 v) {
+  const unsigned b = max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu);
+  return b == 0u ? kNone : (b >= 0x7F800000u ? kBad : int(b >> 23));
 }
+// Exponent of the power of two that brings a row's or column's largest |Re|, |Im| (biased exponent e)
+// into [2^14, 2^15), as far as it and its inverse are normal floats; 0 for zero and for what is not finite.
+__device__ __forceinline__ int scale_exp(int e) {
+  return e <= kNone / 2 || e >= kBad / 2 ? 0 : max(-126, min(126, 14 + 127 - e));
+}
+// Balance exponent of a value of k: at least -100, so that the scales stay normal floats; 0 for a zero row
+__device__ __forceinline__ int balance(int d) { return d <= kNone / 2 ? 0 : max(d, -100); }
 // fp16 pair of 8 scaled values, packed for two 16-byte stores
-__device__ __forceinline__ void split8(const float (&x)[8], float s, uint4& hi, uint4& lo) {
+__device__ __forceinline__ void split8(const float (&x)[8], uint4& hi, uint4& lo) {
   uint32_t h[4], l[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const float a = x[2 * i] * s, b = x[2 * i + 1] * s;
+    const float a = x[2 * i], b = x[2 * i + 1];
     const __half2 hh = __floats2half2_rn(a, b);
     const float2 back = __half22float2(hh);
     const __half2 ll = __floats2half2_rn(a - back.x, b - back.y);
@@ -166,50 +178,115 @@ __device__ __forceinline__ void split8(const float (&x)[8], float s, uint4& hi, 
   hi = make_uint4(h[0], h[1], h[2], h[3]);
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
-__device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
 __device__ __forceinline__ uint4 neg8(uint4 v) {
   return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
+}
+
+// The balance exponents of 8 values of k from k0 on (a multiple of 8; dk has U_KB entries)
+__device__ __forceinline__ void balance8(const int* __restrict__ dk, int k0, int (&d)[8]) {
+  const int4 p = *reinterpret_cast<const int4*>(dk + k0), q = *reinterpret_cast<const int4*>(dk + k0 + 4);
+  const int v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) d[i] = balance(v[i]);
+}
+
+// Exponents of B's columns (value_exp of the largest entry; a CTA per 32 columns, the warps sharing
+// the values of k), and dk = "none yet" for the kernel below.
+__global__ void __launch_bounds__(1024) col_exp_kernel(int64_t N, int K, const float2* __restrict__ B, int64_t ldb,
+                                                      int* __restrict__ ex, int* __restrict__ dk) {
+  __shared__ int s_e[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t col = int64_t(blockIdx.x) * 32 + lane;
+  if (blockIdx.x == 0 && threadIdx.x < U_KB) dk[threadIdx.x] = kNone;
+  int e = kNone;
+#pragma unroll
+  for (int i = 0; i < U_KB / 32; ++i) {
+    const int k = warp + 32 * i;
+    if (col < N && k < K) e = max(e, value_exp(B[int64_t(k) * ldb + col]));
+  }
+  s_e[warp][lane] = e;
+  __syncthreads();
+  e = __reduce_max_sync(0xffffffffu, s_e[lane][warp]);
+  if (lane == 0) ex[int64_t(blockIdx.x) * 32 + warp] = e;
+}
+// dk[k] = the exponent of the largest finite entry of B's row k relative to its column's largest (<= 0; a
+// column's own largest entry has 0, so the column exponents are those of the balanced B too).  A CTA per
+// 128 columns and 32 values of k, all its loads in flight, one atomic per k.  Bound by latency: an
+// update of an N = 15360 factorisation takes 4 us longer for the column exponents and 6 us for this;
+// all 59 updates with their splits 25.0 ms, 24.1 ms without the balance.
+constexpr int kBalCols = 128, kBalRows = 32;
+__global__ void __launch_bounds__(256) row_balance_kernel(int64_t N, int K, const float2* __restrict__ B, int64_t ldb,
+                                                          const int* __restrict__ ex, int* __restrict__ dk) {
+  constexpr int Q = kBalCols / 32, P = kBalRows / 8;
+  const int lane = threadIdx.x & 31, k0 = int(blockIdx.y) * kBalRows + int(threadIdx.x >> 5);
+  const int64_t c0 = int64_t(blockIdx.x) * kBalCols + lane;
+  float2 v[P][Q];
+  int cj[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) cj[q] = c0 + 32 * q < N ? ex[c0 + 32 * q] : kBad;
+#pragma unroll
+  for (int p = 0; p < P; ++p)
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const int k = k0 + 8 * p;
+      v[p][q] = k < K && c0 + 32 * q < N ? B[int64_t(k) * ldb + c0 + 32 * q] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+  for (int p = 0; p < P; ++p) {
+    int d = kNone;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {  // (the products of a column that is not finite are not finite anyway)
+      const int e = value_exp(v[p][q]);
+      if (e != kNone && cj[q] != kBad) d = max(d, e - cj[q]);
+    }
+    d = __reduce_max_sync(0xffffffffu, d);
+    if (lane == 0 && d != kNone) atomicMax(dk + k0 + 8 * p, d);
+  }
 }
 
 // A (M x K, lda), K <= 256 in nslab = ceil(K / 16) slabs: out[(rt * nslab + s) * 16 KB + p * 4 KB +
 // part_off(r, k)], parts Re_h, Re_l, Im_h, Im_l; zero outside M x K; inv[row] the inverse scales.  A warp per
 // 8 rows: lane (row, group) takes every fourth group of 8 values of k, first for the row's largest
-// value, then (from the cache) for the split; 8 rows' 16-byte stores are 128 contiguous bytes.
+// balanced value, then (from the cache) for the split; 8 rows' 16-byte stores are 128 contiguous bytes.
 __global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nslab, const float2* __restrict__ A,
-                                                      int64_t lda, unsigned char* __restrict__ out,
-                                                      float* __restrict__ inv, int64_t rows_pad) {
+                                                      int64_t lda, const int* __restrict__ dk,
+                                                      unsigned char* __restrict__ out, float* __restrict__ inv,
+                                                      int64_t rows_pad) {
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5)) * 8 + (lane & 7);
   if (row >= rows_pad) return;  // (rows_pad is a multiple of 128: whole warps)
   const float2* a = A + row * lda;
   const bool ok = row < M;
-  unsigned mb = 0;
+  int e = kNone;
   for (int g = lane >> 3; g < 2 * nslab; g += 4) {
+    int d[8];
+    balance8(dk, 8 * g, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
       const float2 v = ok && k < K ? a[k] : make_float2(0.f, 0.f);
-      mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
+      e = max(e, value_exp(v) + d[i]);
     }
   }
-  mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, 8));
-  mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, 16));
-  float is;
-  const float s = split_scale(mb, is);
-  if (lane < 8) inv[row] = is;
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 8));
+  e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
+  const int sh = scale_exp(e);
+  if (lane < 8) inv[row] = pow2(-sh);
   unsigned char* base = out + (row / U_TM) * nslab * int64_t(U_ABYTES);
   for (int g = lane >> 3; g < 2 * nslab; g += 4) {
     float re[8], im[8];
+    int d[8];
+    balance8(dk, 8 * g, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
       const float2 v = ok && k < K ? a[k] : make_float2(0.f, 0.f);
-      re[i] = v.x;
-      im[i] = v.y;
+      re[i] = scale2(v.x, sh + d[i]);
+      im[i] = scale2(v.y, sh + d[i]);
     }
     uint4 rh, rl, ih, il;
-    split8(re, s, rh, rl);
-    split8(im, s, ih, il);
+    split8(re, rh, rl);
+    split8(im, ih, il);
     unsigned char* o = base + (g >> 1) * int64_t(U_ABYTES) + part_off(int(row % U_TM), (g & 1) * 8);
     *reinterpret_cast<uint4*>(o) = rh;
     *reinterpret_cast<uint4*>(o + U_PART) = rl;
@@ -219,44 +296,31 @@ __global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nsla
 }
 // B (K x N, ldb), K <= 256: out[(ct * nslab + s) * 24 KB + p * 4 KB + part_off(c, k)], parts
 // Br_h, Bi_h, -Br_h, Br_l, Bi_l, -Br_l; zero outside K x N; inv[col] the inverse scales.  A CTA per
-// 32 columns, lanes along the columns (coalesced), the warps sharing the groups of 8 values of k, first for the
-// columns' largest values, then for the split.
+// 32 columns, lanes along the columns (coalesced), the warps sharing the groups of 8 values of k.
 __global__ void __launch_bounds__(256) split_b_kernel(int64_t N, int K, int nslab, const float2* __restrict__ B,
-                                                      int64_t ldb, unsigned char* __restrict__ out,
+                                                      int64_t ldb, const int* __restrict__ ex,
+                                                      const int* __restrict__ dk, unsigned char* __restrict__ out,
                                                       float* __restrict__ inv) {
-  __shared__ unsigned s_mb[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t col = int64_t(blockIdx.x) * 32 + lane;
   const bool ok = col < N;
-  unsigned mb = 0;
-  for (int g = warp; g < 2 * nslab; g += 8) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int k = 8 * g + i;
-      const float2 v = ok && k < K ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
-      mb = max(mb, max(abs_bits(v.x), abs_bits(v.y)));
-    }
-  }
-  s_mb[warp][lane] = mb;
-  __syncthreads();
-#pragma unroll
-  for (int w = 0; w < 8; ++w) mb = max(mb, s_mb[w][lane]);
-  float is;
-  const float s = split_scale(mb, is);
-  if (warp == 0) inv[col] = is;
+  const int sh = scale_exp(ok ? ex[col] : kNone);
+  if (warp == 0) inv[col] = pow2(-sh);
   unsigned char* base = out + (col / U_TN) * nslab * int64_t(U_BBYTES);
   for (int g = warp; g < 2 * nslab; g += 8) {
     float re[8], im[8];
+    int d[8];
+    balance8(dk, 8 * g, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
       const float2 v = ok && k < K ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
-      re[i] = v.x;
-      im[i] = v.y;
+      re[i] = scale2(v.x, sh - d[i]);
+      im[i] = scale2(v.y, sh - d[i]);
     }
     uint4 rh, rl, ih, il;
-    split8(re, s, rh, rl);
-    split8(im, s, ih, il);
+    split8(re, rh, rl);
+    split8(im, ih, il);
     unsigned char* o = base + (g >> 1) * int64_t(U_BBYTES) + part_off(int(col % U_TN), (g & 1) * 8);
     *reinterpret_cast<uint4*>(o) = rh;
     *reinterpret_cast<uint4*>(o + U_PART) = ih;
@@ -508,12 +572,13 @@ inline unsigned ucdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); 
 
 }  // namespace
 
-// the image, then one scale per padded row or column
+// the image, then one scale per padded row or column; behind B's also the column and balance exponents
 size_t update_split_a_bytes(int64_t M) {
   return size_t((M + U_TM - 1) / U_TM) * (size_t(U_SLABS) * U_ABYTES + U_TM * sizeof(float));
 }
 size_t update_split_b_bytes(int64_t N) {
-  return size_t((N + U_TN - 1) / U_TN) * (size_t(U_SLABS) * U_BBYTES + U_TN * sizeof(float));
+  return size_t((N + U_TN - 1) / U_TN) * (size_t(U_SLABS) * U_BBYTES + U_TN * (sizeof(float) + sizeof(int))) +
+         U_KB * sizeof(int);
 }
 
 // C (M x N) -= A (M x K) B (K x N), complex64 row-major, K <= kLuBlock: split A and B once into
@@ -544,10 +609,14 @@ cudaError_t cgemm_update_tc_split(int64_t M, int64_t N, int64_t K, const void* A
   unsigned char* img_b = static_cast<unsigned char*>(ws_b);
   float* inv_a = reinterpret_cast<float*>(img_a + RT * nslab * int64_t(U_ABYTES));
   float* inv_b = reinterpret_cast<float*>(img_b + CT * nslab * int64_t(U_BBYTES));
-  split_a_kernel<<<ucdiv(rows_pad, 64), 256, 0, s>>>(M, int(K), nslab, static_cast<const float2*>(A), lda, img_a, inv_a,
-                                                     rows_pad);
-  split_b_kernel<<<ucdiv(cols_pad, 32), 256, 0, s>>>(N, int(K), nslab, static_cast<const float2*>(B), ldb, img_b, inv_b);
-  note_launches(2);
+  int* ex_b = reinterpret_cast<int*>(inv_b + cols_pad);
+  int* dk = ex_b + cols_pad;
+  const float2 *a = static_cast<const float2*>(A), *b = static_cast<const float2*>(B);
+  col_exp_kernel<<<ucdiv(cols_pad, 32), 1024, 0, s>>>(N, int(K), b, ldb, ex_b, dk);
+  row_balance_kernel<<<dim3(ucdiv(N, kBalCols), ucdiv(K, kBalRows)), 256, 0, s>>>(N, int(K), b, ldb, ex_b, dk);
+  split_a_kernel<<<ucdiv(rows_pad, 64), 256, 0, s>>>(M, int(K), nslab, a, lda, dk, img_a, inv_a, rows_pad);
+  split_b_kernel<<<ucdiv(cols_pad, 32), 256, 0, s>>>(N, int(K), nslab, b, ldb, ex_b, dk, img_b, inv_b);
+  note_launches(4);
   const unsigned grid = unsigned(std::min<int64_t>(RT * CT, std::max(nsm[dev], 1)));
   const int vec_ok = (reinterpret_cast<uintptr_t>(C) % 16 == 0) && (ldc % 2 == 0);
   cgemm_update_split_kernel<<<grid, U_THREADS, U_SMEM, s>>>(M, N, nslab, img_a, img_b, inv_a, inv_b,
