@@ -247,7 +247,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       xfull = xn;
     }
     if (digits)
-      FOSB_CUDA(oz_gemm(OP_N, n, nrhs, n, -1.0, lu->zdig, lu->zex, full ? X : dx.p, full ? ldx : nrhs, 1.0, r.p, nrhs,
+      FOSB_CUDA(oz_gemm(n, nrhs, n, -1.0, lu->zdig, lu->zex, full ? X : dx.p, full ? ldx : nrhs, 1.0, r.p, nrhs,
                         xex.as<int>() + (full ? 0 : nrhs), full ? nullptr : xex.as<int>(), lu->d_status, s));
     else
       FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, n, nrhs, n, -1.0, 0.0, lu->zref, lu->ldz, X, ldx, 1.0, r.p, nrhs, s,
@@ -420,7 +420,7 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
     if (digits) {
       lu->zdig = base + o_dig;
       lu->zex = reinterpret_cast<int*>(base + o_ex);
-      if ((e = oz_prepare_a(OP_N, Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
+      if ((e = oz_prepare_a(Z, n, n, ldz, lu->zdig, lu->zex, s)) != cudaSuccess)
         return cleanup(cuda_fail(e, "fosb_factor: digit tiles of Z"));
     }
     Scratch nrm(s);

@@ -221,12 +221,13 @@ cudaError_t cgemm_update_tc(int64_t M, int64_t N, int64_t K, const void* A, int6
 // with K = kLuBlock per block).
 constexpr int kLuBlock = 256;
 // The same update for K <= kLuBlock with A and B split once into bulk-copy images
-// (tc_update.cu): workspaces of update_split_a_bytes(M) and update_split_b_bytes(N) bytes.
+// (tc_update.cu): workspaces of update_split_a_bytes(M) and update_split_b_bytes(N) bytes;
+// col_ex: the scale exponents of C's columns in the matrix (getrf's column_scales).
 size_t update_split_a_bytes(int64_t M);
 size_t update_split_b_bytes(int64_t N);
 cudaError_t cgemm_update_tc_split(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B,
                                   int64_t ldb, void* C, int64_t ldc, int* status, void* ws_a, void* ws_b,
-                                  cudaStream_t s);
+                                  const int* col_ex, cudaStream_t s);
 // complex128 GEMM computed in float-float on the FP32 pipe (FP64-class accuracy).  A_split,
 // if given, is split_ff of A as stored (same shape, leading dimension lda).
 cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha_re, double alpha_im,
@@ -234,22 +235,21 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
                          cudaStream_t s, const void* A_split = nullptr);
 // FP64-class complex GEMM on the bf16 tensor cores by exact digit splitting (oz_gemm.cu):
 // oz_prepare_a writes the digit tiles (oz_a_bytes(M, K) bytes) and row exponents (M ints)
-// of op(A) (M x K); oz_gemm then computes C <- beta C + alpha op(A) op(B), alpha and beta real,
-// for a complex128 op(B) (K x N) and leaves the exponents of its columns in b_ex (N ints).  With
-// ref_ex op(B) is a correction of a matrix with those column exponents, and digit orders below
+// of A (M x K); oz_gemm then computes C <- beta C + alpha A B, alpha and beta real, for a
+// complex128 B (K x N) and leaves the exponents of its columns in b_ex (N ints).  With
+// ref_ex B is a correction of a matrix with those column exponents, and digit orders below
 // 2^-60 of that matrix's are left out.  A bounded wait that gives up sets *status (may be null)
 // and leaves NaN.
 size_t oz_a_bytes(int64_t M, int64_t K);
-cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex,
-                         cudaStream_t s);
-cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
+cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s);
+cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
                     const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
                     int* status, cudaStream_t s);
-// C <- C - L U (M x K, K x N) of an FP64 factorisation in digits, rows and columns of the operands
-// balanced first; scratch: oz_update_bytes(max(M, N), K).
-size_t oz_update_bytes(int64_t n, int64_t K);
+// C <- C - L U (M x K, K x N) of an FP64 factorisation in digits, the operands balanced along k
+// first in the scale of C's columns (col_ex); scratch: oz_balanced_bytes(M, N, K) of the largest update.
+size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K);
 cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
-                      int64_t ldc, void* scratch, int* status, cudaStream_t s);
+                      int64_t ldc, const int* col_ex, void* scratch, int* status, cudaStream_t s);
 // C <- beta C + alpha op(A) op(B) in FP64-class arithmetic: digits where the product is large
 // enough to pay for making them, float-float (gemm_c128_ff) otherwise.
 cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,

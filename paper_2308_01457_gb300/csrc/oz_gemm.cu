@@ -184,15 +184,35 @@ __device__ __forceinline__ int oz_exponent(unsigned long long mb) {
 __device__ __forceinline__ unsigned long long oz_umax(unsigned long long a, unsigned long long b) {
   return a > b ? a : b;
 }
+// Balance exponent of a value of k (below): far below all others where B's row is zero or not finite, whose
+// products are zero or NaN anyway.
+constexpr int OZ_NO_ROW = int(0x80808080u);
+__device__ __forceinline__ int oz_balance(const int* dk, int64_t k) {
+  const int d = dk ? dk[k] : 0;
+  return d == OZ_NO_ROW ? -(1 << 14) : d;
+}
+// Exponent of one entry times 2^{sign dk[k]}
+__device__ __forceinline__ int oz_entry_exponent(double2 v, const int* dk, int sign, int64_t k) {
+  const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
+  return b == 0 ? INT_MIN : (b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) + sign * oz_balance(dk, k));
+}
 // Power-of-two scale exponent per row of a complex128 matrix (rows x cols, ld), the max
-// over Re and Im parts.  One warp per row.
+// over Re and Im parts, with dk of the matrix whose column k is multiplied by 2^{sign dk[k]}.  One warp per row.
 __global__ void oz_row_exp_kernel(const double2* __restrict__ A, int64_t rows, int64_t cols, int64_t ld,
-                                  int* __restrict__ ex) {
+                                  const int* __restrict__ dk, int sign, int* __restrict__ ex) {
   const int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
-  unsigned long long m = 0;
   const double2* a = A + row * ld;
+  if (dk) {
+    int e = INT_MIN;
+#pragma unroll 4
+    for (int64_t k = lane; k < cols; k += 32) e = max(e, oz_entry_exponent(a[k], dk, sign, k));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) ex[row] = e == INT_MIN ? 0 : e;
+    return;
+  }
+  unsigned long long m = 0;
 #pragma unroll 4
   for (int64_t k = lane; k < cols; k += 32) {
     const double2 v = a[k];
@@ -202,85 +222,98 @@ __global__ void oz_row_exp_kernel(const double2* __restrict__ A, int64_t rows, i
   for (int off = 16; off > 0; off >>= 1) m = oz_umax(m, __shfl_xor_sync(0xffffffffu, m, off));
   if (lane == 0) ex[row] = oz_exponent(m);
 }
-// the same per column of a matrix stored rows x cols (exponent per column)
+// the same per column of a matrix stored rows x cols (exponent per column, dk per row)
 __global__ void oz_col_exp_kernel(const double2* __restrict__ A, int64_t rows, int64_t cols, int64_t ld,
-                                  int* __restrict__ ex) {
+                                  const int* __restrict__ dk, int sign, int* __restrict__ ex) {
   const int64_t col = blockIdx.x;
-  __shared__ unsigned long long red[8];
-  unsigned long long m = 0;
-  for (int64_t r = threadIdx.x; r < rows; r += blockDim.x) {
-    const double2 v = A[r * ld + col];
-    m = oz_umax(m, oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y)));
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) m = oz_umax(m, __shfl_xor_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < int(blockDim.x >> 5); ++w) m = oz_umax(m, red[w]);
-    ex[col] = oz_exponent(m);
-  }
-}
-// The exponents of a trailing update's operands L (M x K) and U (K x N), which are first balanced: column
-// k of L times, row k of U over 2^{d_k}, d_k the exponent of the largest finite entry of U's row k
-// relative to its column's largest (exponents cj).  A row of L then has its largest entry where
-// its largest products are, and the digits lose no more than FP64 does when rows or columns of the
-// matrix differ in scale (rows scaled by 10^-6 .. 10^6, n = 130: componentwise backward error
-// 2.6e-15 with FP64 products, 4.6e-11 without the balance, 2.4e-15 so).
-__global__ void oz_balance_kernel(const double2* __restrict__ U, int64_t N, int64_t ld, const int* __restrict__ cj,
-                                  int* __restrict__ dk) {
   __shared__ int red[8];
-  const double2* u = U + int64_t(blockIdx.x) * ld;
   int e = INT_MIN;
-#pragma unroll 4
-  for (int64_t j = threadIdx.x; j < N; j += blockDim.x) {
-    const unsigned long long b = oz_umax(oz_abs_bits(u[j].x), oz_abs_bits(u[j].y));
-    if (b && b < 0x7FF0000000000000ull && cj[j] != OZ_BAD) e = max(e, oz_exponent(b) - cj[j]);
+  if (dk) {
+    for (int64_t r = threadIdx.x; r < rows; r += blockDim.x) e = max(e, oz_entry_exponent(A[r * ld + col], dk, sign, r));
+  } else {
+    unsigned long long m = 0;
+    for (int64_t r = threadIdx.x; r < rows; r += blockDim.x) {
+      const double2 v = A[r * ld + col];
+      m = oz_umax(m, oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y)));
+    }
+    if (m) e = oz_exponent(m);
   }
   e = __reduce_max_sync(0xffffffffu, e);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < int(blockDim.x >> 5); ++w) e = max(e, red[w]);
-    dk[blockIdx.x] = e == INT_MIN ? 0 : e;
+    ex[col] = e == INT_MIN ? 0 : e;
   }
 }
-// Exponents of the balanced rows of L (rs = ld, ks = 1, sign +1: a warp per row) ...
-__global__ void oz_balanced_row_exp_kernel(const double2* __restrict__ A, int64_t rows, int64_t K, int64_t ld,
-                                           const int* __restrict__ dk, int* __restrict__ ex) {
-  const int64_t row = int64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= rows) return;
-  int e = INT_MIN;
-  for (int64_t k = lane; k < K; k += 32) {
-    const double2 v = A[row * ld + k];
-    const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
-    if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) + dk[k]);
-  }
-  e = __reduce_max_sync(0xffffffffu, e);
-  if (lane == 0) ex[row] = e == INT_MIN ? 0 : e;
-}
-// ... and of the columns of U, balanced or (no dk) as they are (32 columns x 8 lanes along k)
-__global__ void __launch_bounds__(256) oz_balanced_col_exp_kernel(const double2* __restrict__ A, int64_t cols, int64_t K,
-                                                                  int64_t ld, const int* __restrict__ dk,
-                                                                  int* __restrict__ ex) {
+// the same for few rows (the block row of a trailing update): 32 columns x 8 lanes along the rows
+__global__ void __launch_bounds__(256) oz_wide_col_exp_kernel(const double2* __restrict__ A, int64_t cols, int64_t K,
+                                                              int64_t ld, const int* __restrict__ dk, int sign,
+                                                              int* __restrict__ ex) {
   __shared__ int red[256];
   const int cl = threadIdx.x & 31, kl = threadIdx.x >> 5;
   const int64_t col = int64_t(blockIdx.x) * 32 + cl;
   int e = INT_MIN;
   if (col < cols) {
 #pragma unroll 8
-    for (int64_t k = kl; k < K; k += 8) {
-      const double2 v = A[k * ld + col];
-      const unsigned long long b = oz_umax(oz_abs_bits(v.x), oz_abs_bits(v.y));
-      if (b) e = max(e, b >= 0x7FF0000000000000ull ? OZ_BAD : oz_exponent(b) - (dk ? dk[k] : 0));
-    }
+    for (int64_t k = kl; k < K; k += 8) e = max(e, oz_entry_exponent(A[k * ld + col], dk, sign, k));
   }
   red[threadIdx.x] = e;
   __syncthreads();
   if (kl == 0 && col < cols) {
     for (int w = 1; w < 8; ++w) e = max(e, red[w * 32 + cl]);
     ex[col] = e == INT_MIN ? 0 : e;
+  }
+}
+// Products of two operands A (M x K) and B (K x N) that are both split here are balanced first: column
+// k of A times, row k of B over 2^{d_k}, d_k the exponent of the largest finite entry of B's row k, for the
+// trailing updates of a factorisation in the scale of the matrix' columns (col_ex).  Every k then has a
+// column where B_kj attains 2^{d_k}, so the error in a row of the product is a rounding of that
+// row's largest |A||B| (columns in their scale) whatever the scales of the values of k are.
+// Trailing updates, CPU model with n = 400 and random matrices, componentwise backward errors of solves with
+// FP64 products / digits / digits without the balance: rows scaled by 10^-8 .. 10^8 3e-15 / 3e-15 / 1e-13,
+// with ten entries in half of the columns 2e-14 / 2e-14 / 2e-13, banded 4e-12 / 3e-12 / 2e-5; with d_k
+// relative to the columns of the block row alone 3e-15 / 2e-13 / 3e-7.
+// A CTA per k (B as stored, its rows contiguous) ...
+__global__ void oz_balance_kernel(const double2* __restrict__ B, int64_t N, int64_t ld, const int* __restrict__ col_ex,
+                                  int* __restrict__ dk) {
+  __shared__ int red[8];
+  const double2* b = B + int64_t(blockIdx.x) * ld;
+  int e = OZ_NO_ROW;
+#pragma unroll 4
+  for (int64_t j = threadIdx.x; j < N; j += blockDim.x) {
+    const int v = oz_entry_exponent(b[j], nullptr, 0, 0), c = col_ex ? col_ex[j] : 0;
+    if (v != INT_MIN && v != OZ_BAD) e = max(e, v - (c == OZ_NO_ROW ? 0 : c));
+  }
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < int(blockDim.x >> 5); ++w) e = max(e, red[w]);
+    dk[blockIdx.x] = e;
+  }
+}
+// ... and for a transposed B (N x K as stored): 32 values of k along the lanes, the warps share the rows
+// j of a chunk, one atomic per k and CTA into dk, which starts as OZ_NO_ROW
+constexpr int64_t kBalanceRows = 512;
+__global__ void __launch_bounds__(256) oz_balance_t_kernel(const double2* __restrict__ B, int64_t N, int64_t K,
+                                                           int64_t ld, int* __restrict__ dk) {
+  __shared__ int red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t k = int64_t(blockIdx.x) * 32 + lane, j1 = min(N, (int64_t(blockIdx.y) + 1) * kBalanceRows);
+  int e = OZ_NO_ROW;
+  if (k < K) {
+#pragma unroll 8
+    for (int64_t j = int64_t(blockIdx.y) * kBalanceRows + warp; j < j1; j += 8) {
+      const int v = oz_entry_exponent(B[j * ld + k], nullptr, 0, 0);
+      if (v != INT_MIN && v != OZ_BAD) e = max(e, v);
+    }
+  }
+  red[warp][lane] = e;
+  __syncthreads();
+  if (warp == 0 && k < K) {
+    for (int w = 1; w < 8; ++w) e = max(e, red[w][lane]);
+    if (e != OZ_NO_ROW) atomicMax(dk + k, e);
   }
 }
 // x 2^(55 - e) rounded to an integer (|x| < 2^e, so |F| <= 2^55), from the bit pattern:
@@ -336,7 +369,7 @@ __global__ void oz_split_kernel(const double2* __restrict__ A, int64_t rows, int
     gr[j] = gi[j] = BIAS;
     if (row < rows && k < K) {
       const double2 v = A[row * rs + k * ks];
-      const int ek = dk ? e - sign * dk[k] : e;
+      const int ek = e - sign * oz_balance(dk, k);
       gr[j] = static_cast<unsigned long long>(oz_fixed(v.x, ek)) + BIAS;
       gi[j] = static_cast<unsigned long long>(oz_fixed(conj ? -v.y : v.y, ek)) + BIAS;
     }
@@ -710,33 +743,39 @@ size_t oz_a_bytes(int64_t M, int64_t K) {
   return size_t((M + OZ_TM - 1) / OZ_TM) * size_t((K + OZ_KS - 1) / OZ_KS) * OZ_NT * OZ_ATILE;
 }
 
-// Exponents and digit tiles of op(X) (rows x K after op, rows in tiles of TR); with dk balanced: op(X)
-// is L (sign +1) or U by its columns (sign -1)
+// Exponents (of the rows, times 2^{sign dk[k]} with dk) of a matrix read as rows x K
+static void oz_exponents(const double2* X, int64_t rows, int64_t K, int64_t rs, int64_t ks, const int* dk, int sign,
+                         int* ex, cudaStream_t s) {
+  if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, dk, sign, ex);
+  else if (K < 128) oz_wide_col_exp_kernel<<<oz_cdiv(rows, 32), 256, 0, s>>>(X, rows, K, ks, dk, sign, ex);
+  else oz_col_exp_kernel<<<unsigned(rows), 256, 0, s>>>(X, K, rows, ks, dk, sign, ex);
+}
+// Digit tiles of a matrix read as rows x K with the exponents ex of its rows, in tiles of TR rows; with dk
+// balanced, as the left (sign +1) or the right (sign -1) operand
 template <int TR>
 static cudaError_t oz_digits(const double2* X, int64_t rows, int64_t K, int64_t rs, int64_t ks, bool conj,
-                             const int* dk, int sign, int* ex, void* digits, cudaStream_t s) {
+                             const int* dk, int sign, const int* ex, void* digits, cudaStream_t s) {
   const int64_t KC = (K + OZ_KS - 1) / OZ_KS, RP = (rows + TR - 1) / TR * TR;
   if (RP / 8 > 65535) return cudaErrorInvalidValue;
-  if (dk && sign > 0) oz_balanced_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, dk, ex);
-  else if (dk) oz_balanced_col_exp_kernel<<<oz_cdiv(rows, 32), 256, 0, s>>>(X, rows, K, ks, dk, ex);
-  else if (ks == 1) oz_row_exp_kernel<<<oz_cdiv(rows, 8), 256, 0, s>>>(X, rows, K, rs, ex);
-  else oz_col_exp_kernel<<<unsigned(rows), 256, 0, s>>>(X, K, rows, ks, ex);
   oz_split_kernel<TR><<<dim3(oz_cdiv(KC * 2, OZ_SPLIT_WARPS * 4), unsigned(RP / 8)), OZ_SPLIT_WARPS * 32, 0, s>>>(
       X, rows, K, rs, ks, conj, ex, dk, sign, KC, static_cast<unsigned char*>(digits));
-  return launched(2);
+  return launched(1);
 }
 
-cudaError_t oz_prepare_a(int opA, const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex,
-                         cudaStream_t s) {
+cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s) {
   if (M <= 0 || K <= 0) return cudaSuccess;
   ProfScope prof("oz_prep", s, 44.0 * double(M) * double(K));  // bytes read + written
-  return oz_digits<OZ_TM>(static_cast<const double2*>(A), M, K, opA == OP_N ? lda : 1, opA == OP_N ? 1 : lda,
-                          opA == OP_C, nullptr, 0, ex, digits, s);
+  const double2* a = static_cast<const double2*>(A);
+  oz_exponents(a, M, K, lda, 1, nullptr, 0, ex, s);
+  note_launches(1);
+  return oz_digits<OZ_TM>(a, M, K, lda, 1, false, nullptr, 0, ex, digits, s);
 }
 
+// b_ex: the exponents of op(B)'s columns
 static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
-                              const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex,
-                              const int* ref_ex, const int* dk, int gmax, int* status, cudaStream_t s) {
+                              const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
+                              const int* b_ex, const int* ref_ex, const int* dk, int gmax, int* status,
+                              cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   static bool attr[64] = {};
   static int nsm[64] = {};
@@ -787,29 +826,48 @@ static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double a
   return e;
 }
 
-cudaError_t oz_gemm(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
+cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
                     const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
                     int* status, cudaStream_t s) {
-  return oz_product(opB, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, nullptr, OZ_ND - 1, status, s);
+  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
+  oz_exponents(static_cast<const double2*>(B), N, K, 1, ldb, nullptr, 0, b_ex, s);
+  note_launches(1);
+  return oz_product(OP_N, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, nullptr, OZ_ND - 1, status, s);
 }
 
-size_t oz_update_bytes(int64_t n, int64_t K) { return oz_a_bytes(n, K) + sizeof(int) * size_t(2 * n + K); }
+size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K) { return oz_a_bytes(M, K) + sizeof(int) * size_t(M + N + K); }
 
-cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
-                      int64_t ldc, void* scratch, int* status, cudaStream_t s) {
+// C <- beta C + alpha op(A) op(B), balanced along k, with the digit orders up to gmax; scratch:
+// oz_balanced_bytes(M, N, K)
+static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,
+                               int64_t lda, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
+                               const int* col_ex, void* scratch, int gmax, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   char* dig = static_cast<char*>(scratch);
   int* dk = reinterpret_cast<int*>(dig + oz_a_bytes(M, K));
-  int *lex = dk + K, *uex = lex + M;
-  const double2* u = static_cast<const double2*>(U);
-  oz_balanced_col_exp_kernel<<<oz_cdiv(N, 32), 256, 0, s>>>(u, N, K, ldu, nullptr, uex);
-  oz_balance_kernel<<<unsigned(K), 256, 0, s>>>(u, N, ldu, uex, dk);
-  cudaError_t e = launched(2);
-  if (e == cudaSuccess)
-    e = oz_digits<OZ_TM>(static_cast<const double2*>(L), M, K, ldl, 1, false, dk, 1, lex, dig, s);
-  if (e == cudaSuccess)
-    e = oz_product(OP_N, M, N, K, -1.0, dig, lex, U, ldu, 1.0, C, ldc, uex, nullptr, dk, OZ_ND, status, s);
-  return e;
+  int *a_ex = dk + K, *b_ex = a_ex + M;
+  const double2 *a = static_cast<const double2*>(A), *b = static_cast<const double2*>(B);
+  if (gmax < OZ_ND) {
+    dk = nullptr;
+  } else if (opB == OP_N) {
+    oz_balance_kernel<<<unsigned(K), 256, 0, s>>>(b, N, ldb, col_ex, dk);
+  } else {
+    const cudaError_t e = cudaMemsetAsync(dk, 0x80, sizeof(int) * size_t(K), s);
+    if (e != cudaSuccess) return e;
+    oz_balance_t_kernel<<<dim3(oz_cdiv(K, 32), oz_cdiv(N, kBalanceRows)), 256, 0, s>>>(b, N, K, ldb, dk);
+  }
+  const int64_t rs = opA == OP_N ? lda : 1, ks = opA == OP_N ? 1 : lda;
+  oz_exponents(a, M, K, rs, ks, dk, 1, a_ex, s);
+  oz_exponents(b, N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, dk, -1, b_ex, s);
+  note_launches(3);
+  const cudaError_t e = oz_digits<OZ_TM>(a, M, K, rs, ks, opA == OP_C, dk, 1, a_ex, dig, s);
+  if (e != cudaSuccess) return e;
+  return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, dk, gmax, status, s);
+}
+
+cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
+                      int64_t ldc, const int* col_ex, void* scratch, int* status, cudaStream_t s) {
+  return oz_balanced(OP_N, OP_N, M, N, K, -1.0, L, ldl, U, ldu, 1.0, C, ldc, col_ex, scratch, OZ_ND, status, s);
 }
 
 // FP64-class op(A) op(B) for any operands: digits of both, made here.  The digit path takes over at
@@ -822,14 +880,10 @@ cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t 
                                 cudaStream_t s) {
   if (M > 0 && N > 8 && K >= 128 && M <= 65535 * 8 - 128 &&
       N <= 65535 * 8 - 64) {
-    char* d = nullptr;
-    const size_t ab = oz_a_bytes(M, K);
-    cudaError_t e = device_alloc(reinterpret_cast<void**>(&d), ab + sizeof(int) * size_t(M + N), s);
+    void* d = nullptr;
+    cudaError_t e = device_alloc(&d, oz_balanced_bytes(M, N, K), s);
     if (e == cudaSuccess) {
-      int* ex = reinterpret_cast<int*>(d + ab);
-      e = oz_prepare_a(opA, A, M, K, lda, d, ex, s);
-      if (e == cudaSuccess)
-        e = oz_gemm(opB, M, N, K, alpha, d, ex, B, ldb, beta, C, ldc, ex + M, nullptr, nullptr, s);
+      e = oz_balanced(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, nullptr, d, OZ_ND - 1, nullptr, s);
       cudaFreeAsync(d, s);
     }
     if (e != cudaErrorMemoryAllocation) return e;
@@ -861,8 +915,8 @@ extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, con
   FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M + N)));
   FOSB_CUDA(st.alloc(sizeof(int)));
   FOSB_CUDA(cudaMemsetAsync(st.p, 0, sizeof(int), s));
-  FOSB_CUDA(oz_prepare_a(OP_N, A, M, K, lda, dig.p, ex.as<int>(), s));
-  FOSB_CUDA(oz_gemm(OP_N, M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
+  FOSB_CUDA(oz_prepare_a(A, M, K, lda, dig.p, ex.as<int>(), s));
+  FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
                     st.as<int>(), s));
   int status = 0;
   FOSB_CUDA(cudaMemcpyAsync(&status, st.p, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -2,7 +2,7 @@
 // bulk copies of operands split once per block into two fp16 values per real number.
 //
 // The split.  A and B are first balanced along k: row k of B over 2^{d_k}, column k of A times 2^{d_k},
-// d_k the exponent of the largest entry of B's row k relative to its column's largest.  Then every row
+// d_k the exponent of the largest entry of B's row k in the scale of the matrix' columns.  Then every row
 // i of A and column j of B is scaled by a power of two that brings its largest |Re|, |Im| into
 // [2^14, 2^15), and x s = x_h + x_l with x_h = fp16(x s), x_l = fp16(x s - x_h):
 //   x y ~ x_h y_h + x_h y_l + x_l y_h,
@@ -14,7 +14,11 @@
 // many accumulations in the tensor core.
 // The balance is for matrices whose rows differ in scale: U12's rows then carry the scales and L21's
 // columns their inverses, so the products are of one size but lie far below a row's times a column's
-// largest value.
+// largest value.  With it a row's error is below 2^-40 of the largest |L||U| in that row, columns taken
+// in the matrix' own scale (every k has a column where U_kj attains 2^{d_k}), as far as a single value
+// is below the 22 bits: CPU model, K = 256, n = 400, scaled, banded and sparse matrices, factor error over
+// |L||U| as with 3xTF32 (1e-7), 3e-4 without the balance; matrices of blocks with scales of their own
+// are normwise in each row only (4e-5 of |L||U|; backward errors of solves as with 3xTF32).
 //
 // Split once, copied many times.  A (L21, M x K) and B (U12, K x N) are each split by one
 // pass per column block (K <= 256) into the exact shared-memory image the MMAs read: for every
@@ -161,8 +165,6 @@ __device__ __forceinline__ int value_exp(float2 v) {
 __device__ __forceinline__ int scale_exp(int e) {
   return e <= kNone / 2 || e >= kBad / 2 ? 0 : max(-126, min(126, 14 + 127 - e));
 }
-// Balance exponent of a value of k: at least -100, so that the scales stay normal floats; 0 for a zero row
-__device__ __forceinline__ int balance(int d) { return d <= kNone / 2 ? 0 : max(d, -100); }
 // fp16 pair of 8 scaled values, packed for two 16-byte stores
 __device__ __forceinline__ void split8(const float (&x)[8], uint4& hi, uint4& lo) {
   uint32_t h[4], l[4];
@@ -182,66 +184,43 @@ __device__ __forceinline__ uint4 neg8(uint4 v) {
   return make_uint4(v.x ^ 0x80008000u, v.y ^ 0x80008000u, v.z ^ 0x80008000u, v.w ^ 0x80008000u);
 }
 
-// The balance exponents of 8 values of k from k0 on (a multiple of 8; dk has U_KB entries)
-__device__ __forceinline__ void balance8(const int* __restrict__ dk, int k0, int (&d)[8]) {
+// dk[k] = the largest value_exp of B's row k less that of its column (col_ex), over the finite entries; kNone for
+// a zero row and k >= K.  A CTA per k.  Bound by latency: 6 us per update of an
+// N = 15360 factorisation; all 59 updates with their splits 24.9 ms, 24.3 ms without the balance.
+__global__ void __launch_bounds__(512) row_balance_kernel(int64_t N, int K, const float2* __restrict__ B, int64_t ldb,
+                                                          const int* __restrict__ col_ex, int* __restrict__ dk) {
+  __shared__ int red[16];
+  const int k = int(blockIdx.x);
+  int d = kNone;
+  if (k < K) {
+    const float2* b = B + int64_t(k) * ldb;
+#pragma unroll 8
+    for (int64_t j = threadIdx.x; j < N; j += 512) {
+      const int e = value_exp(b[j]), c = col_ex[j];
+      if (e != kNone && e != kBad) d = max(d, e - (c < kNone ? 0 : c));  // (none: a column without finite values)
+    }
+  }
+  d = __reduce_max_sync(0xffffffffu, d);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = d;
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  d = __reduce_max_sync(0xffffffffu, red[threadIdx.x & 15]);
+  if (threadIdx.x == 0) dk[k] = d;
+}
+// The largest of the balance exponents, by a warp; the balance in use is relative to it: at most 0, and at
+// least -100 so that the scales stay normal floats (zero rows have that too, their products are zero).
+__device__ __forceinline__ int balance_max(const int* __restrict__ dk, int lane) {
+  int d = kNone;
+#pragma unroll
+  for (int i = 0; i < U_KB; i += 32) d = max(d, dk[i + lane]);
+  return __reduce_max_sync(0xffffffffu, d);
+}
+// The balance exponents of 8 values of k from k0 on (a multiple of 8)
+__device__ __forceinline__ void balance8(const int* __restrict__ dk, int k0, int dmax, int (&d)[8]) {
   const int4 p = *reinterpret_cast<const int4*>(dk + k0), q = *reinterpret_cast<const int4*>(dk + k0 + 4);
   const int v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
 #pragma unroll
-  for (int i = 0; i < 8; ++i) d[i] = balance(v[i]);
-}
-
-// Exponents of B's columns (value_exp of the largest entry; a CTA per 32 columns, the warps sharing
-// the values of k), and dk = "none yet" for the kernel below.
-__global__ void __launch_bounds__(1024) col_exp_kernel(int64_t N, int K, const float2* __restrict__ B, int64_t ldb,
-                                                      int* __restrict__ ex, int* __restrict__ dk) {
-  __shared__ int s_e[32][33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t col = int64_t(blockIdx.x) * 32 + lane;
-  if (blockIdx.x == 0 && threadIdx.x < U_KB) dk[threadIdx.x] = kNone;
-  int e = kNone;
-#pragma unroll
-  for (int i = 0; i < U_KB / 32; ++i) {
-    const int k = warp + 32 * i;
-    if (col < N && k < K) e = max(e, value_exp(B[int64_t(k) * ldb + col]));
-  }
-  s_e[warp][lane] = e;
-  __syncthreads();
-  e = __reduce_max_sync(0xffffffffu, s_e[lane][warp]);
-  if (lane == 0) ex[int64_t(blockIdx.x) * 32 + warp] = e;
-}
-// dk[k] = the exponent of the largest finite entry of B's row k relative to its column's largest (<= 0; a
-// column's own largest entry has 0, so the column exponents are those of the balanced B too).  A CTA per
-// 128 columns and 32 values of k, all its loads in flight, one atomic per k.  Bound by latency: an
-// update of an N = 15360 factorisation takes 4 us longer for the column exponents and 6 us for this;
-// all 59 updates with their splits 25.0 ms, 24.1 ms without the balance.
-constexpr int kBalCols = 128, kBalRows = 32;
-__global__ void __launch_bounds__(256) row_balance_kernel(int64_t N, int K, const float2* __restrict__ B, int64_t ldb,
-                                                          const int* __restrict__ ex, int* __restrict__ dk) {
-  constexpr int Q = kBalCols / 32, P = kBalRows / 8;
-  const int lane = threadIdx.x & 31, k0 = int(blockIdx.y) * kBalRows + int(threadIdx.x >> 5);
-  const int64_t c0 = int64_t(blockIdx.x) * kBalCols + lane;
-  float2 v[P][Q];
-  int cj[Q];
-#pragma unroll
-  for (int q = 0; q < Q; ++q) cj[q] = c0 + 32 * q < N ? ex[c0 + 32 * q] : kBad;
-#pragma unroll
-  for (int p = 0; p < P; ++p)
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      const int k = k0 + 8 * p;
-      v[p][q] = k < K && c0 + 32 * q < N ? B[int64_t(k) * ldb + c0 + 32 * q] : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-  for (int p = 0; p < P; ++p) {
-    int d = kNone;
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {  // (the products of a column that is not finite are not finite anyway)
-      const int e = value_exp(v[p][q]);
-      if (e != kNone && cj[q] != kBad) d = max(d, e - cj[q]);
-    }
-    d = __reduce_max_sync(0xffffffffu, d);
-    if (lane == 0 && d != kNone) atomicMax(dk + k0 + 8 * p, d);
-  }
+  for (int i = 0; i < 8; ++i) d[i] = max(v[i] - dmax, -100);
 }
 
 // A (M x K, lda), K <= 256 in nslab = ceil(K / 16) slabs: out[(rt * nslab + s) * 16 KB + p * 4 KB +
@@ -257,10 +236,11 @@ __global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nsla
   if (row >= rows_pad) return;  // (rows_pad is a multiple of 128: whole warps)
   const float2* a = A + row * lda;
   const bool ok = row < M;
+  const int dmax = balance_max(dk, lane);
   int e = kNone;
   for (int g = lane >> 3; g < 2 * nslab; g += 4) {
     int d[8];
-    balance8(dk, 8 * g, d);
+    balance8(dk, 8 * g, dmax, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
@@ -276,7 +256,7 @@ __global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nsla
   for (int g = lane >> 3; g < 2 * nslab; g += 4) {
     float re[8], im[8];
     int d[8];
-    balance8(dk, 8 * g, d);
+    balance8(dk, 8 * g, dmax, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
@@ -296,21 +276,38 @@ __global__ void __launch_bounds__(256) split_a_kernel(int64_t M, int K, int nsla
 }
 // B (K x N, ldb), K <= 256: out[(ct * nslab + s) * 24 KB + p * 4 KB + part_off(c, k)], parts
 // Br_h, Bi_h, -Br_h, Br_l, Bi_l, -Br_l; zero outside K x N; inv[col] the inverse scales.  A CTA per
-// 32 columns, lanes along the columns (coalesced), the warps sharing the groups of 8 values of k.
+// 32 columns, lanes along the columns (coalesced), the warps sharing the groups of 8 values of k, first for the
+// columns' largest balanced values, then for the split.
 __global__ void __launch_bounds__(256) split_b_kernel(int64_t N, int K, int nslab, const float2* __restrict__ B,
-                                                      int64_t ldb, const int* __restrict__ ex,
-                                                      const int* __restrict__ dk, unsigned char* __restrict__ out,
-                                                      float* __restrict__ inv) {
+                                                      int64_t ldb, const int* __restrict__ dk,
+                                                      unsigned char* __restrict__ out, float* __restrict__ inv) {
+  __shared__ int s_e[8][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t col = int64_t(blockIdx.x) * 32 + lane;
   const bool ok = col < N;
-  const int sh = scale_exp(ok ? ex[col] : kNone);
+  const int dmax = balance_max(dk, lane);
+  int e = kNone;
+  for (int g = warp; g < 2 * nslab; g += 8) {
+    int d[8];
+    balance8(dk, 8 * g, dmax, d);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * g + i;
+      const float2 v = ok && k < K ? B[int64_t(k) * ldb + col] : make_float2(0.f, 0.f);
+      e = max(e, value_exp(v) - d[i]);
+    }
+  }
+  s_e[warp][lane] = e;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < 8; ++w) e = max(e, s_e[w][lane]);
+  const int sh = scale_exp(e);
   if (warp == 0) inv[col] = pow2(-sh);
   unsigned char* base = out + (col / U_TN) * nslab * int64_t(U_BBYTES);
   for (int g = warp; g < 2 * nslab; g += 8) {
     float re[8], im[8];
     int d[8];
-    balance8(dk, 8 * g, d);
+    balance8(dk, 8 * g, dmax, d);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * g + i;
@@ -572,21 +569,20 @@ inline unsigned ucdiv(int64_t a, int64_t b) { return unsigned((a + b - 1) / b); 
 
 }  // namespace
 
-// the image, then one scale per padded row or column; behind B's also the column and balance exponents
+// the image, then one scale per padded row or column; behind B's also the balance exponents
 size_t update_split_a_bytes(int64_t M) {
   return size_t((M + U_TM - 1) / U_TM) * (size_t(U_SLABS) * U_ABYTES + U_TM * sizeof(float));
 }
 size_t update_split_b_bytes(int64_t N) {
-  return size_t((N + U_TN - 1) / U_TN) * (size_t(U_SLABS) * U_BBYTES + U_TN * (sizeof(float) + sizeof(int))) +
-         U_KB * sizeof(int);
+  return size_t((N + U_TN - 1) / U_TN) * (size_t(U_SLABS) * U_BBYTES + U_TN * sizeof(float)) + U_KB * sizeof(int);
 }
 
 // C (M x N) -= A (M x K) B (K x N), complex64 row-major, K <= kLuBlock: split A and B once into
 // the workspaces (update_split_a_bytes(M), update_split_b_bytes(N) bytes, 16-byte aligned),
-// then the bulk-copy-fed tcgen05 update.
+// then the bulk-copy-fed tcgen05 update.  col_ex: the biased FP32 exponents of the scale of C's columns.
 cudaError_t cgemm_update_tc_split(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B,
                                   int64_t ldb, void* C, int64_t ldc, int* status, void* ws_a, void* ws_b,
-                                  cudaStream_t s) {
+                                  const int* col_ex, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   if (K > U_KB) return cudaErrorInvalidValue;
   static bool attr[64] = {};
@@ -609,14 +605,12 @@ cudaError_t cgemm_update_tc_split(int64_t M, int64_t N, int64_t K, const void* A
   unsigned char* img_b = static_cast<unsigned char*>(ws_b);
   float* inv_a = reinterpret_cast<float*>(img_a + RT * nslab * int64_t(U_ABYTES));
   float* inv_b = reinterpret_cast<float*>(img_b + CT * nslab * int64_t(U_BBYTES));
-  int* ex_b = reinterpret_cast<int*>(inv_b + cols_pad);
-  int* dk = ex_b + cols_pad;
+  int* dk = reinterpret_cast<int*>(inv_b + cols_pad);
   const float2 *a = static_cast<const float2*>(A), *b = static_cast<const float2*>(B);
-  col_exp_kernel<<<ucdiv(cols_pad, 32), 1024, 0, s>>>(N, int(K), b, ldb, ex_b, dk);
-  row_balance_kernel<<<dim3(ucdiv(N, kBalCols), ucdiv(K, kBalRows)), 256, 0, s>>>(N, int(K), b, ldb, ex_b, dk);
+  row_balance_kernel<<<U_KB, 512, 0, s>>>(N, int(K), b, ldb, col_ex, dk);
   split_a_kernel<<<ucdiv(rows_pad, 64), 256, 0, s>>>(M, int(K), nslab, a, lda, dk, img_a, inv_a, rows_pad);
-  split_b_kernel<<<ucdiv(cols_pad, 32), 256, 0, s>>>(N, int(K), nslab, b, ldb, ex_b, dk, img_b, inv_b);
-  note_launches(4);
+  split_b_kernel<<<ucdiv(cols_pad, 32), 256, 0, s>>>(N, int(K), nslab, b, ldb, dk, img_b, inv_b);
+  note_launches(3);
   const unsigned grid = unsigned(std::min<int64_t>(RT * CT, std::max(nsm[dev], 1)));
   const int vec_ok = (reinterpret_cast<uintptr_t>(C) % 16 == 0) && (ldc % 2 == 0);
   cgemm_update_split_kernel<<<grid, U_THREADS, U_SMEM, s>>>(M, N, nslab, img_a, img_b, inv_a, inv_b,
