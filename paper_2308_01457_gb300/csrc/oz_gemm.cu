@@ -274,6 +274,8 @@ __global__ void __launch_bounds__(256) oz_wide_col_exp_kernel(const double2* __r
 // FP64 products / digits / digits without the balance: rows scaled by 10^-8 .. 10^8 3e-15 / 3e-15 / 1e-13,
 // with ten entries in half of the columns 2e-14 / 2e-14 / 2e-13, banded 4e-12 / 3e-12 / 2e-5; with d_k
 // relative to the columns of the block row alone 3e-15 / 2e-13 / 3e-7.
+// Products of stored factors graded by 2^-16 .. 2^16 against each other, K = 300, error over |A||B|: float-float
+// 3.6e-14, digits without the balance 9e-8, with it 9e-17.
 // A CTA per k (B as stored, its rows contiguous) ...
 __global__ void oz_balance_kernel(const double2* __restrict__ B, int64_t N, int64_t ld, const int* __restrict__ col_ex,
                                   int* __restrict__ dk) {
@@ -847,9 +849,7 @@ static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K
   int* dk = reinterpret_cast<int*>(dig + oz_a_bytes(M, K));
   int *a_ex = dk + K, *b_ex = a_ex + M;
   const double2 *a = static_cast<const double2*>(A), *b = static_cast<const double2*>(B);
-  if (gmax < OZ_ND) {
-    dk = nullptr;
-  } else if (opB == OP_N) {
+  if (opB == OP_N) {
     oz_balance_kernel<<<unsigned(K), 256, 0, s>>>(b, N, ldb, col_ex, dk);
   } else {
     const cudaError_t e = cudaMemsetAsync(dk, 0x80, sizeof(int) * size_t(K), s);
