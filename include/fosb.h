@@ -492,10 +492,11 @@ fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, const void* A,
  * Every spin-wait of the library's kernels gives up after a number of polls, sets the
  * status word of the call to FOSB_ERR_TIMEOUT and returns, so the call reports
  * FOSB_ERR_TIMEOUT and the context stays usable.  This sets that number for the LU panel
- * grid barriers and the streaming triangular sweeps' waits on the current device (polls <= 0
- * restores the default 2^26, about 2 s); failure-detection tests use a tiny limit to make
- * the waits run out.  The tensor-core and cluster-panel kernels keep their own limits.  A factorisation whose
- * wait ran out leaves its outputs unspecified; destroy and recreate its handle. */
+ * grid barriers, the streaming triangular sweeps' waits and those of the digit products
+ * (fosb_zgemm_fp64class) on the current device (polls <= 0 restores the defaults, 2^26 and for the
+ * digits 2^24, about 2 s); failure-detection tests use a tiny limit to make the waits run out.  The
+ * LU update and cluster-panel kernels keep their own limits.  A factorisation whose wait ran
+ * out leaves its outputs unspecified; destroy and recreate its handle. */
 fosb_status fosb_debug_set_wait_limit(int64_t polls);
 
 /* Throughput microbenchmarks of the execution units the kernels are bound by (diagnostics

@@ -670,6 +670,7 @@ fosb_status fosb_farfield_moments(fosb_mesh m1, fosb_mesh m2, double k, const do
 fosb_status fosb_debug_set_wait_limit(int64_t polls) {
   FOSB_CUDA(set_wait_limit_panels(polls));
   FOSB_CUDA(set_wait_limit_sweeps(polls));
+  FOSB_CUDA(set_wait_limit_digits(polls));
   return FOSB_OK;
 }
 

@@ -315,6 +315,7 @@ cudaError_t zaxpy(int64_t n, double ar, double ai, const void* x, int64_t incx, 
 // panel grid barriers (linalg.cu) and streaming-sweep flags (trsv_stream.cu).
 cudaError_t set_wait_limit_panels(long long polls);
 cudaError_t set_wait_limit_sweeps(long long polls);
+cudaError_t set_wait_limit_digits(long long polls);
 // Largest n that the external-scratch panel path can factor with at most max_ctas CTAs on
 // the current device (co-resident panel CTAs x rows a CTA can hold).
 fosb_status getrf_external_max_n(int64_t max_ctas, int64_t* max_n);

@@ -61,6 +61,10 @@ constexpr int OZ_FLUSH = 8 * 32;
 constexpr int OZ_HN = OZ_TN / 2;                               // columns per flush thread
 constexpr int OZ_TMEM_COLS = 512;                              // 7 or 8 orders x 64 columns
 constexpr long long kOzSpinLimit = 1ll << 24;
+// Poll limit of the waits between the roles on this device (kOzSpinLimit unless changed by
+// fosb_debug_set_wait_limit).  The waits for copies and MMAs in flight before the kernel leaves keep
+// kOzSpinLimit.
+__device__ long long g_oz_wait_limit = kOzSpinLimit;
 static_assert(OZ_SMEM <= 226 * 1024, "digit stages and the barriers do not fit shared memory");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -127,12 +131,21 @@ __device__ __forceinline__ uint32_t oz_test(uint32_t mbar, uint32_t parity) {
   return done;
 }
 template <bool SLEEP = false>
-__device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity) {
-  for (long long spins = 0; spins < kOzSpinLimit; ++spins) {
+__device__ __forceinline__ bool oz_wait(uint32_t mbar, uint32_t parity, long long limit = kOzSpinLimit) {
+  for (long long spins = 0; spins < limit; ++spins) {
     if (oz_test(mbar, parity)) return true;
     if (SLEEP) __nanosleep(32);
   }
   return false;
+}
+// barrier of the eight flush warps; true where any of their threads passed true
+__device__ __forceinline__ bool oz_any(bool x) {
+  uint32_t any;
+  asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n bar.red.or.pred p, 1, 256, q;\n selp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(any)
+               : "r"(uint32_t(x))
+               : "memory");
+  return any != 0;
 }
 __device__ __forceinline__ void oz_init(uint32_t a, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count));
@@ -451,6 +464,7 @@ struct OzMma {
   uint64_t *full, *empty;  // full by stage; empty by stage and digit of Z, digit 0 also for the digits of X
   uint32_t phase;          // phase of the full barriers, a bit per stage
   uint32_t ready;          // the next stage was seen full
+  long long limit;         // polls of a wait
 };
 // The MMAs of one k step with the orders 0 .. G out of stage P, from digit S of Z on, part IM (0 Re,
 // 1 Im).  A wait that has nothing to wait for still takes 80 cycles, and few MMAs queue up behind
@@ -475,7 +489,7 @@ __device__ __forceinline__ void oz_step(OzMma& m, uint32_t tmem, uint32_t smem, 
 }
 template <int G, int IM, int P>
 __device__ __forceinline__ bool oz_stage(OzMma& m, uint32_t tmem, uint32_t smem, uint32_t acc) {
-  if (!m.ready && !oz_wait(smem_u32(&m.full[P]), m.phase >> P & 1)) return false;
+  if (!m.ready && !oz_wait(smem_u32(&m.full[P]), m.phase >> P & 1, m.limit)) return false;
   asm volatile("tcgen05.fence::after_thread_sync;");
   m.phase ^= 1u << P;
   oz_step<G, IM, P, 0>(m, tmem, smem, acc);
@@ -488,7 +502,7 @@ __device__ __forceinline__ bool oz_tile(OzMma& m, uint32_t tmem, uint32_t smem, 
   m.ready = 0;
   for (int64_t c = c0; c < c1; ++c, ++chunks) {
     // the order accumulators are free once the flush warps have read the last chunk
-    if (chunks > 0 && !oz_wait(smem_u32(acce), uint32_t((chunks - 1) & 1))) return false;
+    if (chunks > 0 && !oz_wait(smem_u32(acce), uint32_t((chunks - 1) & 1), m.limit)) return false;
     asm volatile("tcgen05.fence::after_thread_sync;");
     const int steps = int(std::min<int64_t>(KC - c * OZ_KCH, OZ_KCH));
     for (int k = 0; k < steps; k += 2) {  // a chunk starts at an even step
@@ -524,7 +538,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   __shared__ uint64_t bar_accf, bar_acce, bar_drain;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
-  __shared__ volatile int fl_stop;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t CT = (N + OZ_TN - 1) / OZ_TN;
   const int64_t nch = (KC + OZ_KCH - 1) / OZ_KCH;  // chunks per tile
@@ -541,8 +554,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_init(smem_u32(&bar_drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
     abort_sh = 0;
-    fl_stop = 0;
   }
+  const long long limit = g_oz_wait_limit;
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
@@ -574,7 +587,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
           const int p = int(kc & 1);
           const uint32_t turn = p ? fills1 : fills0;
           bool ok = !abort_sh;
-          if (ok && s <= G && turn > 0 && !oz_wait(smem_u32(&empty[p * OZ_ND + s]), (turn - 1) & 1)) {
+          if (ok && s <= G && turn > 0 && !oz_wait(smem_u32(&empty[p * OZ_ND + s]), (turn - 1) & 1, limit)) {
             fail();
             ok = false;
           }
@@ -598,7 +611,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   } else if (warp == 1) {
     // ---------------------------------------------------------- MMA issuer
     if (oz_elect()) {
-      OzMma m = {full, empty, 0u, 0u};
+      OzMma m = {full, empty, 0u, 0u, limit};
       const uint32_t stage0 = smem_u32(smem);
       int64_t chunks = 0;
       for (int64_t w = blockIdx.x; w < items && !abort_sh; w += gridDim.x) {
@@ -649,12 +662,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         t[j] = 0.f;
       }
       for (int64_t c = item.c0; c < item.c1 && !stopped; ++c, ++chunks) {
-        if (!oz_wait<true>(smem_u32(&bar_accf), uint32_t(chunks & 1))) {
-          fail();
-          fl_stop = 1;
-        }
-        asm volatile("bar.sync 1, 256;");  // the stop decision is the same in all eight warps
-        stopped = fl_stop;
+        const bool full_in_time = oz_wait<true>(smem_u32(&bar_accf), uint32_t(chunks & 1), limit);
+        if (!full_in_time) fail();
+        // the stop decision is the same in all eight warps: the barrier itself hands out the OR (a flag
+        // read behind it could already be the next chunk's)
+        stopped = oz_any(!full_in_time);
         if (stopped) break;
         asm volatile("tcgen05.fence::after_thread_sync;");
         // eight columns of two orders at a time, the next ones on their way during the arithmetic
@@ -893,6 +905,12 @@ cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t 
 }
 
 }  // namespace fosb
+
+// Sets the poll limit of the digit kernel's waits on the current device (polls <= 0: the default).
+cudaError_t fosb::set_wait_limit_digits(long long polls) {
+  const long long v = polls > 0 ? polls : kOzSpinLimit;
+  return cudaMemcpyToSymbol(g_oz_wait_limit, &v, sizeof(v));
+}
 
 extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, const void* A, int64_t lda, const void* B,
                                             int64_t ldb, void* C, int64_t ldc, int method, void* stream) {
