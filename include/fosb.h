@@ -347,7 +347,8 @@ fosb_status fosb_farfield_pmchwt(fosb_mesh mesh, double k0, const double* dirs, 
  *   M = Y1 op(Y2), op = ^H (pseudo = 0) or ^T (pseudo = 1, the pseudo-covariance), the mirror
  *   added when hermitian_mirror = 1 (a block with l1 != l2 of the CT sum, Section IV-B).
  *   Y1, Y2 : device nd3 x r (ldy1, ldy2 >= r); out : device nd3 x nd3 (ldo >= nd3).
- *   Enqueued on `stream`. */
+ *   Enqueued on `stream`; FOSB_MIXED products with r >= 128 are waited for (FOSB_ERR_TIMEOUT), unless
+ *   the stream is being captured, where they run in float-float. */
 fosb_status fosb_kernel_lowrank(const fosb_mesh* meshes, int64_t nmesh, const fosb_cov_kernel* kernel, double tol,
                                 int64_t max_rank, double* R, int64_t ldr, int64_t* rank, double* trace_err,
                                 void* stream);

@@ -525,15 +525,16 @@ fosb_status fosb_covariance(fosb_mesh m1, fosb_lu lu1, const void* u1, fosb_mesh
   }
   FOSB_TRY(solve_internal(lu1, y1.p, r, r, y1.p, r, ropt, nullptr, s));
   FOSB_TRY(solve_internal(lu2, y2.p, r, r, y2.p, r, ropt, nullptr, s));
+  DigitStatus st(s);
   cudaError_t e;
   if (c64)
     e = gemm<float>(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, 0.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
   else if (prec == FOSB_MIXED)
-    e = gemm_c128_fp64class(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
+    e = gemm_c128_fp64class(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, st, s);
   else
     e = gemm<double>(OP_N, pseudo ? OP_T : OP_C, d1.ne, d2.ne, r, 1.0, 0.0, y1.p, r, y2.p, r, 0.0, Sigma, lds, s);
   FOSB_CUDA(e);
-  return FOSB_OK;
+  return st.check("fosb_covariance");
 }
 
 fosb_status fosb_kernel_lowrank(const fosb_mesh* meshes, int64_t nmesh, const fosb_cov_kernel* kernel, double tol,
@@ -562,9 +563,10 @@ fosb_status fosb_kernel_lowrank(const fosb_mesh* meshes, int64_t nmesh, const fo
 
 namespace {
 cudaError_t gemm_prec(int prec, int opA, int opB, int64_t M, int64_t N, int64_t K, double ar, const void* A, int64_t lda,
-                      const void* B, int64_t ldb, double beta, void* C, int64_t ldc, cudaStream_t s) {
+                      const void* B, int64_t ldb, double beta, void* C, int64_t ldc, DigitStatus& st,
+                      cudaStream_t s) {
   if (is_c64(prec)) return gemm<float>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
-  if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, s);
+  if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, st, s);
   return gemm<double>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
 }
 }  // namespace
@@ -594,9 +596,10 @@ fosb_status fosb_covariance_lowrank(fosb_mesh mesh, fosb_lu lu, const void* u, d
   FOSB_CUDA(a.alloc(elem * nd3 * N));
   FOSB_CUDA(cudaMemsetAsync(a.p, 0, elem * nd3 * N, s));
   FOSB_CUDA(launch_farfield_matrix(d, k, ddirs.as<double>(), n_dir, c64, a.p, s));
-  FOSB_CUDA(gemm_prec(prec, OP_N, OP_N, nd3, r, N, 1.0, a.p, N, w.p, r, 0.0, Y, ldy, s));
+  DigitStatus st(s);
+  FOSB_CUDA(gemm_prec(prec, OP_N, OP_N, nd3, r, N, 1.0, a.p, N, w.p, r, 0.0, Y, ldy, st, s));
   FOSB_CUDA(cudaStreamSynchronize(s));
-  return FOSB_OK;
+  return st.check("fosb_covariance_lowrank");
 }
 
 fosb_status fosb_lowrank_combine(int64_t nd3, int64_t r, const void* Y1, int64_t ldy1, const void* Y2, int64_t ldy2,
@@ -607,15 +610,16 @@ fosb_status fosb_lowrank_combine(int64_t nd3, int64_t r, const void* Y1, int64_t
   FOSB_TRY(check_prec(prec));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int op = pseudo ? OP_T : OP_C;
+  DigitStatus st(s);
   if (!hermitian_mirror) {
-    FOSB_CUDA(gemm_prec(prec, OP_N, op, nd3, nd3, r, weight, Y1, ldy1, Y2, ldy2, accumulate ? 1.0 : 0.0, out, ldo, s));
-    return FOSB_OK;
+    FOSB_CUDA(gemm_prec(prec, OP_N, op, nd3, nd3, r, weight, Y1, ldy1, Y2, ldy2, accumulate ? 1.0 : 0.0, out, ldo, st, s));
+    return st.check("fosb_lowrank_combine");
   }
   Scratch mm(s);
   FOSB_CUDA(mm.alloc((is_c64(prec) ? 8 : 16) * nd3 * nd3));
-  FOSB_CUDA(gemm_prec(prec, OP_N, op, nd3, nd3, r, 1.0, Y1, ldy1, Y2, ldy2, 0.0, mm.p, nd3, s));
+  FOSB_CUDA(gemm_prec(prec, OP_N, op, nd3, nd3, r, 1.0, Y1, ldy1, Y2, ldy2, 0.0, mm.p, nd3, st, s));
   FOSB_CUDA(add_mirrored(mm.p, nd3, nd3, op, weight, accumulate != 0, is_c64(prec), out, ldo, s));
-  return FOSB_OK;
+  return st.check("fosb_lowrank_combine");
 }
 
 fosb_status fosb_farfield_moments(fosb_mesh m1, fosb_mesh m2, double k, const double* dirs, int64_t n_dir,
@@ -637,16 +641,17 @@ fosb_status fosb_farfield_moments(fosb_mesh m1, fosb_mesh m2, double k, const do
   FOSB_CUDA(a1.alloc(elem * nd3 * m1->d.ne));
   FOSB_CUDA(cudaMemsetAsync(a1.p, 0, elem * nd3 * m1->d.ne, s));
   FOSB_CUDA(launch_farfield_matrix(m1->d, k, ddirs.as<double>(), n_dir, c64, a1.p, s));
+  DigitStatus st(s);
   auto G = [&](int opA, int opB, int64_t M, int64_t N, int64_t K, double ar, const void* A, int64_t lda,
                const void* B, int64_t ldb, double beta, void* C, int64_t ldc) {
     if (c64) return gemm<float>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
-    if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, s);
+    if (prec == FOSB_MIXED) return gemm_c128_fp64class(opA, opB, M, N, K, ar, A, lda, B, ldb, beta, C, ldc, st, s);
     return gemm<double>(opA, opB, M, N, K, ar, 0.0, A, lda, B, ldb, beta, C, ldc, s);
   };
   if (!m2) {
     FOSB_CUDA(G(OP_N, OP_N, nd3, ncols, m1->d.ne, weight, a1.p, m1->d.ne, X, ldx, accumulate ? 1.0 : 0.0, out, ldo));
     FOSB_CUDA(cudaStreamSynchronize(s));
-    return FOSB_OK;
+    return st.check("fosb_farfield_moments");
   }
   const int64_t N1 = m1->d.ne, N2 = m2->d.ne;
   FOSB_CUDA(a2.alloc(elem * nd3 * N2));
@@ -664,7 +669,7 @@ fosb_status fosb_farfield_moments(fosb_mesh m1, fosb_mesh m2, double k, const do
     FOSB_CUDA(add_mirrored(mm.p, nd3, nd3, pseudo ? OP_T : OP_C, weight, accumulate != 0, c64, out, ldo, s));
   }
   FOSB_CUDA(cudaStreamSynchronize(s));
-  return FOSB_OK;
+  return st.check("fosb_farfield_moments");
 }
 
 fosb_status fosb_debug_set_wait_limit(int64_t polls) {
@@ -700,10 +705,12 @@ fosb_status fosb_rcs_monostatic(fosb_mesh mesh, fosb_lu lu, double k, const fosb
   FOSB_CUDA(cudaMemsetAsync(A.p, 0, 16 * nd3 * N, s));
   FOSB_CUDA(launch_farfield_matrix(d, k, dxh.as<double>(), n, false, A.p, s));
   FOSB_CUDA(FA.alloc(16 * nd3 * n));
-  FOSB_CUDA(gemm_c128_fp64class(OP_N, OP_N, nd3, n, N, 1.0, A.p, N, U, ldu, 0.0, FA.p, n, s));
+  DigitStatus st(s);
+  FOSB_CUDA(gemm_c128_fp64class(OP_N, OP_N, nd3, n, N, 1.0, A.p, N, U, ldu, 0.0, FA.p, n, st, s));
   std::vector<double> fa(2 * nd3 * n);
   FOSB_CUDA(cudaMemcpyAsync(fa.data(), FA.p, 16 * nd3 * n, cudaMemcpyDeviceToHost, s));
   FOSB_CUDA(cudaStreamSynchronize(s));
+  FOSB_TRY(st.check("fosb_rcs_monostatic"));
   // F_i = (A u_i) at xh_i: rows 3i..3i+2 of column i;  sigma_i = |F_i|^2 / (4 pi)
   std::vector<double> sig(n), Fr(3 * n), Fi(3 * n);
   for (int64_t i = 0; i < n; ++i) {
@@ -761,7 +768,8 @@ fosb_status fosb_rcs_monostatic(fosb_mesh mesh, fosb_lu lu, double k, const fosb
   FOSB_CUDA(dC.alloc(16 * nd3 * n));
   FOSB_CUDA(cudaMemcpyAsync(dC.p, Cm.data(), 16 * nd3 * n, cudaMemcpyHostToDevice, s));
   FOSB_CUDA(lam.alloc(16 * N * n));
-  FOSB_CUDA(gemm_c128_fp64class(OP_T, OP_N, N, n, nd3, 1.0, A.p, N, dC.p, n, 0.0, lam.p, n, s));
+  FOSB_CUDA(gemm_c128_fp64class(OP_T, OP_N, N, n, nd3, 1.0, A.p, N, dC.p, n, 0.0, lam.p, n, st, s));
+  FOSB_TRY(st.check("fosb_rcs_monostatic"));
   FOSB_TRY(solve_internal(lu, lam.p, n, n, lam.p, n, nullptr, nullptr, s));
   FOSB_CUDA(dpw.alloc(sizeof(double) * 11 * 2 * n));
   FOSB_CUDA(cudaMemcpyAsync(dpw.p, pw.data(), sizeof(double) * 11 * 2 * n, cudaMemcpyHostToDevice, s));

@@ -250,11 +250,23 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a
 size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K);
 cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
                       int64_t ldc, const int* col_ex, void* scratch, int* status, cudaStream_t s);
+// Status word of a call's digit products, made at the first of them; check() waits for them and
+// reports a wait that gave up (nothing to wait for where the call had none).
+class DigitStatus {
+ public:
+  explicit DigitStatus(cudaStream_t s) : word_(s) {}
+  cudaError_t get(int** p);
+  fosb_status check(const char* call);
+
+ private:
+  Scratch word_;
+};
 // C <- beta C + alpha op(A) op(B) in FP64-class arithmetic: digits where the product is large
-// enough to pay for making them, float-float (gemm_c128_ff) otherwise.
+// enough to pay for making them, float-float (gemm_c128_ff) otherwise and while the stream is being
+// captured, where no status could be read.  The caller checks st before it returns or uses C on the host.
 cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,
                                 int64_t lda, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
-                                cudaStream_t s);
+                                DigitStatus& st, cudaStream_t s);
 // dst (rows x cols float4, ldd) = (hi, lo) float split of the complex128 src
 cudaError_t split_ff(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd,
                      cudaStream_t s);

@@ -882,6 +882,25 @@ cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ld
   return oz_balanced(OP_N, OP_N, M, N, K, -1.0, L, ldl, U, ldu, 1.0, C, ldc, col_ex, scratch, OZ_ND, status, s);
 }
 
+cudaError_t DigitStatus::get(int** p) {
+  if (!word_.p) {
+    cudaError_t e = word_.alloc(sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(word_.p, 0, sizeof(int), word_.s);
+    if (e != cudaSuccess) return e;
+  }
+  *p = word_.as<int>();
+  return cudaSuccess;
+}
+
+fosb_status DigitStatus::check(const char* call) {
+  if (!word_.p) return FOSB_OK;
+  int status = 0;
+  FOSB_CUDA(cudaMemcpyAsync(&status, word_.p, sizeof(int), cudaMemcpyDeviceToHost, word_.s));
+  FOSB_CUDA(cudaStreamSynchronize(word_.s));
+  if (status == FOSB_ERR_TIMEOUT) return fail(FOSB_ERR_TIMEOUT, std::string(call) + ": tensor-core wait timed out");
+  return FOSB_OK;
+}
+
 // FP64-class op(A) op(B) for any operands: digits of both, made here.  The digit path takes over at
 // K = 128: below, the passes over the outputs are most of either (digits / float-float, us: 1000 x
 // 1000 x 64 158 / 164, 3000 x 3000 x 32 707 / 650, 1000 x 1000 x 16 148 / 72), above it wins at any
@@ -889,15 +908,18 @@ cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ld
 // x 1089 980 / 5708, 7503 x 7503 x 642 9685 / 61614).
 cudaError_t gemm_c128_fp64class(int opA, int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* A,
                                 int64_t lda, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
-                                cudaStream_t s) {
+                                DigitStatus& st, cudaStream_t s) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) cudaGetLastError();
   if (M > 0 && N > 8 && K >= 128 && M <= 65535 * 8 - 128 &&
-      N <= 65535 * 8 - 64) {
+      N <= 65535 * 8 - 64 && capture == cudaStreamCaptureStatusNone) {
     void* d = nullptr;
-    cudaError_t e = device_alloc(&d, oz_balanced_bytes(M, N, K), s);
-    if (e == cudaSuccess) {
-      e = oz_balanced(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, nullptr, d, OZ_ND - 1, nullptr, s);
-      cudaFreeAsync(d, s);
-    }
+    int* status = nullptr;
+    cudaError_t e = st.get(&status);
+    if (e == cudaSuccess) e = device_alloc(&d, oz_balanced_bytes(M, N, K), s);
+    if (e == cudaSuccess)
+      e = oz_balanced(opA, opB, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, nullptr, d, OZ_ND - 1, status, s);
+    if (d) cudaFreeAsync(d, s);
     if (e != cudaErrorMemoryAllocation) return e;
     cudaGetLastError();  // no room for the digits (28 bytes per entry): float-float needs 16
   }
@@ -928,18 +950,15 @@ extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, con
     FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, M, N, K, 1.0, 0.0, A, lda, B, ldb, 0.0, C, ldc, s));
     return FOSB_OK;
   }
-  Scratch dig(s), ex(s), st(s);
+  Scratch dig(s), ex(s);
+  DigitStatus st(s);
+  int* status = nullptr;
   FOSB_CUDA(dig.alloc(oz_a_bytes(M, K)));
   FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M + N)));
-  FOSB_CUDA(st.alloc(sizeof(int)));
-  FOSB_CUDA(cudaMemsetAsync(st.p, 0, sizeof(int), s));
+  FOSB_CUDA(st.get(&status));
   FOSB_CUDA(oz_prepare_a(A, M, K, lda, dig.p, ex.as<int>(), s));
   FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
-                    st.as<int>(), s));
-  int status = 0;
-  FOSB_CUDA(cudaMemcpyAsync(&status, st.p, sizeof(int), cudaMemcpyDeviceToHost, s));
-  FOSB_CUDA(cudaStreamSynchronize(s));
-  if (status == FOSB_ERR_TIMEOUT) return fail(FOSB_ERR_TIMEOUT, "fosb_zgemm_fp64class: tensor-core wait timed out");
-  return FOSB_OK;
+                    status, s));
+  return st.check("fosb_zgemm_fp64class");
 }
 
