@@ -86,7 +86,8 @@ typedef struct {
   int max_iters;     /* iterative-refinement steps (default 10) */
   double tol;        /* stop when ||b - Z x||_inf / (||Z||_inf ||x||_inf + ||b||_inf) <= tol per column;
                         tol <= 0 selects the default max(64, 8 sqrt(n)) * 2^-52.  Refinement also stops
-                        when a step gains less than a factor 2 below 1e-13 (rounding floor reached) */
+                        when a step gains less than a factor 2 below 1e-13 (rounding floor reached), and
+                        with the default tries one more step from a backward error in (tol/16, tol] */
   int solver;        /* FOSB_REFINE_AUTO (0): refinement, then GMRES-IR for the columns it left above tol;
                         FOSB_REFINE_IR (1): refinement only; FOSB_REFINE_GMRES (2): GMRES-IR from the start */
 } fosb_refine_opts;

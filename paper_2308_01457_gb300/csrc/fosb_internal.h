@@ -238,13 +238,13 @@ cudaError_t gemm_c128_ff(int opA, int opB, int64_t M, int64_t N, int64_t K, doub
 // of A (M x K); oz_gemm then computes C <- beta C + alpha A B, alpha and beta real, for a
 // complex128 B (K x N) and leaves the exponents of its columns in b_ex (N ints).  With
 // ref_ex B is a correction of a matrix with those column exponents, and digit orders below
-// 2^-60 of that matrix's are left out.  A bounded wait that gives up sets *status (may be null)
+// 2^-bits of that matrix's are left out.  A bounded wait that gives up sets *status (may be null)
 // and leaves NaN.
 size_t oz_a_bytes(int64_t M, int64_t K);
 cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void* digits, int* ex, cudaStream_t s);
 cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
                     const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
-                    int* status, cudaStream_t s);
+                    int bits, int* status, cudaStream_t s);
 // C <- C - L U (M x K, K x N) of an FP64 factorisation in digits, the operands balanced along k
 // first in the scale of C's columns (col_ex); scratch: oz_balanced_bytes(M, N, K) of the largest update.
 size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K);

@@ -412,14 +412,14 @@ constexpr int OZ_SPLIT_WARPS = 8;  // a block covers 8 rows x 8 warps x 4 groups
 // The highest order kept in each tile of 64 columns: gmax without ref.  With ref the
 // operand is a correction of a matrix whose columns have the exponents ref, and what matters is
 // the error against that matrix: dropping the orders above g leaves 2^{-8(g+1)} sigma tau per
-// product, which is at most 2^-60 sigma 2^ref (1/16 of what the product with the matrix itself
-// leaves) once 8 (g + 1) >= 60 - (ref - ex).  One warp per tile.
-__global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restrict__ ref, int64_t N, int gmax,
+// product, which is at most 2^-bits sigma 2^ref (60: 1/16 of what the product with the matrix itself
+// leaves) once 8 (g + 1) >= bits - (ref - ex).  One warp per tile.
+__global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restrict__ ref, int bits, int64_t N, int gmax,
                                  int* __restrict__ orders) {
   int g = ref ? 0 : gmax;
   for (int q = threadIdx.x; ref && q < OZ_TN; q += 32) {
     const int64_t c = int64_t(blockIdx.x) * OZ_TN + q;
-    if (c < N) g = max(g, min(OZ_ND - 1, (59 - min(59, max(0, ref[c] - ex[c]))) / 8));
+    if (c < N) g = max(g, min(OZ_ND - 1, (bits - 1 - min(bits - 1, max(0, ref[c] - ex[c]))) / 8));
   }
   g = __reduce_max_sync(0xffffffffu, g);
   if (threadIdx.x == 0) orders[blockIdx.x] = g;
@@ -788,7 +788,7 @@ cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void*
 // b_ex: the exponents of op(B)'s columns
 static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
                               const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
-                              const int* b_ex, const int* ref_ex, const int* dk, int gmax, int* status,
+                              const int* b_ex, const int* ref_ex, int bits, const int* dk, int gmax, int* status,
                               cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   static bool attr[64] = {};
@@ -825,7 +825,7 @@ static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double a
     cudaFreeAsync(bd, s);
     return e;
   }
-  oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, N, gmax, orders);
+  oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, bits, N, gmax, orders);
   {
     ProfScope prof("gemm_oz", s, 8.0 * double(M) * double(N) * double(K));
     oz_gemm_kernel<<<unsigned(std::min(items, sms)), OZ_THREADS, OZ_SMEM, s>>>(
@@ -842,11 +842,12 @@ static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double a
 
 cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
                     const void* B, int64_t ldb, double beta, void* C, int64_t ldc, int* b_ex, const int* ref_ex,
-                    int* status, cudaStream_t s) {
+                    int bits, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   oz_exponents(static_cast<const double2*>(B), N, K, 1, ldb, nullptr, 0, b_ex, s);
   note_launches(1);
-  return oz_product(OP_N, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, nullptr, OZ_ND - 1, status, s);
+  return oz_product(OP_N, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, bits, nullptr, OZ_ND - 1, status,
+                    s);
 }
 
 size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K) { return oz_a_bytes(M, K) + sizeof(int) * size_t(M + N + K); }
@@ -874,7 +875,7 @@ static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K
   note_launches(3);
   const cudaError_t e = oz_digits<OZ_TM>(a, M, K, rs, ks, opA == OP_C, dk, 1, a_ex, dig, s);
   if (e != cudaSuccess) return e;
-  return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, dk, gmax, status, s);
+  return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, 0, dk, gmax, status, s);
 }
 
 cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
@@ -957,7 +958,7 @@ extern "C" fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, con
   FOSB_CUDA(ex.alloc(sizeof(int) * size_t(M + N)));
   FOSB_CUDA(st.get(&status));
   FOSB_CUDA(oz_prepare_a(A, M, K, lda, dig.p, ex.as<int>(), s));
-  FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr,
+  FOSB_CUDA(oz_gemm(M, N, K, 1.0, dig.p, ex.as<int>(), B, ldb, 0.0, C, ldc, ex.as<int>() + M, nullptr, 0,
                     status, s));
   return st.check("fosb_zgemm_fp64class");
 }
