@@ -210,7 +210,8 @@ fosb_status fosb_factor(const void* Z, int64_t n, int64_t ldz, int prec, fosb_lu
  * tensor cores for more (n >= 256); both are accurate to a few units of 2^-52 of
  * |b| + |Z||x|.  Triangular sweeps of complex64 factors run as one persistent kernel per sweep, or
  * with many right-hand sides as one per 512 rows with tensor-core updates between them.
- * Errors: FOSB_ERR_NOT_CONVERGED (best iterate written). */
+ * Errors: FOSB_ERR_NOT_CONVERGED (best iterate written; also where a column of B or X has infinities
+ * or NaN, after the refinement of the others). */
 fosb_status fosb_solve(fosb_lu lu, char op, const void* B, int64_t nrhs, int64_t ldb, void* X, int64_t ldx,
                        const fosb_refine_opts* ropt, fosb_solve_stats* stats, void* stream);
 

@@ -48,6 +48,13 @@ fosb_status col_norms(const void* A, int64_t rows, int64_t cols, int64_t lda, do
   return FOSB_OK;
 }
 
+// Normwise backward error of a column with residual norm r and ||Z|| ||x|| + ||b|| = size; infinite
+// where either is not finite.
+double backward_error(double r, double size) {
+  if (!std::isfinite(r) || !std::isfinite(size)) return INFINITY;
+  return size > 0 ? r / size : (r == 0 ? 0.0 : INFINITY);
+}
+
 // GMRES-based iterative refinement of one column (contiguous device n-vectors bc, xc; see
 // FOSB_REFINE_GMRES in fosb.h): outer steps r = b - Z x (FP64-class), berr test, then the
 // correction d from GMRES on M^-1 Z d = M^-1 r (M the complex64 factors) with FP64 Arnoldi
@@ -99,9 +106,8 @@ fosb_status gmres_ir_column(fosb_lu lu, const void* bc, void* xc, double bnorm, 
     FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, n, 1, n, -1.0, 0.0, lu->zref, lu->ldz, xc, 1, 1.0, r.p, 1, s, lu->zff));
     FOSB_TRY(col_norms(r.p, n, 1, 1, nb.as<double>(), rn, s));
     FOSB_TRY(col_norms(xc, n, 1, 1, nb.as<double>(), xn, s));
-    const double den = lu->znorm_inf * xn[0] + bnorm;
-    berr = den > 0 ? rn[0] / den : 0.0;
-    if (berr <= tol || outer >= max_outer) break;
+    berr = backward_error(rn[0], lu->znorm_inf * xn[0] + bnorm);
+    if (berr <= tol || outer >= max_outer || !std::isfinite(berr)) break;
     // GMRES on M^-1 Z d = M^-1 r, d = 0 initially
     FOSB_TRY(precond(r.p, w.p));
     double beta = 0.0;
@@ -240,6 +246,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
   int it = 0;
   Scratch xkeep(s);  // the iterate that met the tolerance, while the correction after it is tried
   double berr_kept = INFINITY;
+  bool lost = false;  // a column with infinities or NaN
   for (; solver != FOSB_REFINE_GMRES;) {
     FOSB_TRY(col_norms(X, n, nrhs, ldx, nb.as<double>(), xn, s));
     bool full = !dx.p || it == 0;
@@ -257,9 +264,14 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
                              lu->zff));
     FOSB_TRY(col_norms(r.p, n, nrhs, nrhs, nb.as<double>(), rn, s));
     berr = res = 0.0;
+    lost = false;
     for (int64_t c = 0; c < nrhs; ++c) {
-      double den = lu->znorm_inf * xn[c] + bn[c];
-      berr = std::max(berr, den > 0 ? rn[c] / den : 0.0);
+      const double e = backward_error(rn[c], lu->znorm_inf * xn[c] + bn[c]);
+      if (!std::isfinite(e)) {  // no step helps such a column; the others go on
+        lost = true;
+        continue;
+      }
+      berr = std::max(berr, e);
       res = std::max(res, bn[c] > 0 ? rn[c] / bn[c] : rn[c]);
     }
     if (it == 0) res0 = res;
@@ -316,6 +328,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       berr = std::max(berr, bc_err);
     }
   }
+  if (lost) berr = INFINITY;
   if (stats) {
     stats->iters = it;
     stats->backward_error = berr;
