@@ -502,6 +502,11 @@ fosb_status fosb_zgemm_fp64class(int64_t M, int64_t N, int64_t K, const void* A,
  * out leaves its outputs unspecified; destroy and recreate its handle. */
 fosb_status fosb_debug_set_wait_limit(int64_t polls);
 
+/* Lets the `after` next scratch allocations of the calling thread's library calls succeed and the
+ * one behind them fail as if device memory had run out (once; after < 0: none); tests of what calls do
+ * at scratch limits.  A handle's own storage is not counted. */
+fosb_status fosb_debug_fail_allocation(int64_t after);
+
 /* Throughput microbenchmarks of the execution units the kernels are bound by (diagnostics
  * for roofline denominators).  kind 0: FP32 FMA pipe; 1: FP64 FMA pipe; 2: tcgen05.mma
  * kind::tf32 (M = 128, N = 256, K = 8) back to back from shared memory, one CTA per SM; 3: the

@@ -73,7 +73,8 @@ def lib():
                      "fosb_assemble_efie", "fosb_factor", "fosb_solve", "fosb_lu_info", "fosb_lu_destroy",
                      "fosb_covariance", "fosb_farfield_moments", "fosb_rcs_monostatic",
                      "fosb_getrf_static", "fosb_profile_enable", "fosb_profile_read", "fosb_rcs_moments",
-                     "fosb_debug_set_wait_limit", "fosb_peak_microbench", "fosb_assemble_efie_batched",
+                     "fosb_debug_set_wait_limit", "fosb_debug_fail_allocation", "fosb_peak_microbench",
+                     "fosb_assemble_efie_batched",
                      "fosb_solve_batched", "fosb_field_samples", "fosb_mesh_perturb", "fosb_mc_moments",
                      "fosb_zgemm_fp64class", "fosb_kernel_lowrank", "fosb_covariance_lowrank",
                      "fosb_lowrank_combine", "fosb_assemble_pmchwt", "fosb_farfield_pmchwt"):
@@ -371,6 +372,11 @@ def debug_set_wait_limit(polls: int):
     """fosb_debug_set_wait_limit: poll limit of the bounded panel-barrier and sweep-flag
     waits on the current device (polls <= 0 restores the default)."""
     _check(lib().fosb_debug_set_wait_limit(ctypes.c_int64(polls)))
+
+
+def debug_fail_allocation(after: int):
+    """fosb_debug_fail_allocation: the scratch allocation after the `after` next ones of this thread fails."""
+    _check(lib().fosb_debug_fail_allocation(ctypes.c_int64(after)))
 
 
 def peak_microbench(kind: str) -> float:

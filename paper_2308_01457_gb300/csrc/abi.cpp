@@ -706,6 +706,11 @@ fosb_status fosb_debug_set_wait_limit(int64_t polls) {
   return FOSB_OK;
 }
 
+fosb_status fosb_debug_fail_allocation(int64_t after) {
+  tl_fail_allocation = after;
+  return FOSB_OK;
+}
+
 fosb_status fosb_rcs_monostatic(fosb_mesh mesh, fosb_lu lu, double k, const fosb_quad_opts* opts, const double* inc,
                                 int64_t n_inc, const void* U, int64_t ldu, const double* weights, int db, double* sigma,
                                 double* grad, void* stream) {

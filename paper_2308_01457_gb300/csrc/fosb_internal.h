@@ -50,7 +50,9 @@ class ProfScope {
 // Stream-ordered device memory of the calling thread: from the device's default pool, or from the
 // pool that a call has given its worker threads (fosb_solve_batched).
 extern thread_local cudaMemPool_t tl_pool;
+extern thread_local int64_t tl_fail_allocation;  // allocations until one fails (fosb_debug_fail_allocation), < 0: none
 inline cudaError_t device_alloc(void** p, size_t bytes, cudaStream_t s) {
+  if (tl_fail_allocation >= 0 && tl_fail_allocation-- == 0) return cudaErrorMemoryAllocation;
   return tl_pool ? cudaMallocFromPoolAsync(p, bytes, tl_pool, s) : cudaMallocAsync(p, bytes, s);
 }
 

@@ -15,6 +15,7 @@ namespace fosb {
 
 static thread_local std::string g_last_error;
 thread_local cudaMemPool_t tl_pool = nullptr;
+thread_local int64_t tl_fail_allocation = -1;
 static std::atomic<uint64_t> g_launches{0};
 
 void note_launches(uint64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }

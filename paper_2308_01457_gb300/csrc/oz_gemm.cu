@@ -785,11 +785,16 @@ cudaError_t oz_prepare_a(const void* A, int64_t M, int64_t K, int64_t lda, void*
   return oz_digits<OZ_TM>(a, M, K, lda, 1, false, nullptr, 0, ex, digits, s);
 }
 
-// b_ex: the exponents of op(B)'s columns
+// Digit tiles and orders of an N-column right operand
+static size_t oz_right_bytes(int64_t N, int64_t K) {
+  return size_t((N + OZ_TN - 1) / OZ_TN) * (size_t((K + OZ_KS - 1) / OZ_KS) * OZ_BSLOT + sizeof(int));
+}
+
+// b_ex: the exponents of op(B)'s columns; right: oz_right_bytes(N, K) of scratch, or null to allocate
 static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits,
                               const int* a_ex, const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
                               const int* b_ex, const int* ref_ex, int bits, const int* dk, int gmax, int* status,
-                              cudaStream_t s) {
+                              void* right, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   static bool attr[64] = {};
   static int nsm[64] = {};
@@ -811,20 +816,21 @@ static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double a
   const int pieces = rem ? int(std::max<int64_t>(1, std::min<int64_t>(sms / rem, nch / 8))) : 1;
   const int64_t items = whole + rem * pieces;
   const int unit = K <= (1 << 15) ? 32 : 24;  // of the integer sums (oz_store)
-  // digit tiles of B, then the pieces' sums, then the orders
+  // the pieces' sums, then digit tiles of B, then the orders
   const size_t bbytes = size_t(CT) * size_t(KC) * OZ_BSLOT;
   const size_t pbytes = pieces > 1 ? sizeof(OzPart) * size_t(rem * pieces) * OZ_TM * OZ_TN : 0;
-  unsigned char* bd = nullptr;
-  cudaError_t e = device_alloc(reinterpret_cast<void**>(&bd), bbytes + pbytes + sizeof(int) * size_t(CT), s);
-  if (e != cudaSuccess) return e;
-  OzPart* part = reinterpret_cast<OzPart*>(bd + bbytes);
-  int* orders = reinterpret_cast<int*>(bd + bbytes + pbytes);
-  e = oz_digits<OZ_TN>(static_cast<const double2*>(B), N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, opB == OP_C,
-                       dk, -1, b_ex, bd, s);
-  if (e != cudaSuccess) {
-    cudaFreeAsync(bd, s);
-    return e;
+  Scratch own(s);
+  if (!right || pieces > 1) {
+    const cudaError_t e = own.alloc(pbytes + oz_right_bytes(N, K));
+    if (e != cudaSuccess) return e;
+    right = static_cast<char*>(own.p) + pbytes;
   }
+  OzPart* part = static_cast<OzPart*>(own.p);
+  unsigned char* bd = static_cast<unsigned char*>(right);
+  int* orders = reinterpret_cast<int*>(bd + bbytes);
+  cudaError_t e = oz_digits<OZ_TN>(static_cast<const double2*>(B), N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, opB == OP_C,
+                       dk, -1, b_ex, bd, s);
+  if (e != cudaSuccess) return e;
   oz_orders_kernel<<<unsigned(CT), 32, 0, s>>>(b_ex, ref_ex, bits, N, gmax, orders);
   {
     ProfScope prof("gemm_oz", s, 8.0 * double(M) * double(N) * double(K));
@@ -835,9 +841,7 @@ static cudaError_t oz_product(int opB, int64_t M, int64_t N, int64_t K, double a
       oz_reduce_kernel<<<dim3(unsigned(rem), OZ_TM * OZ_TN / 256), 256, 0, s>>>(
           M, N, whole, pieces, part, a_ex, b_ex, unit, alpha, beta, static_cast<double*>(C), ldc);
   }
-  e = launched(pieces > 1 ? 3 : 2);
-  cudaFreeAsync(bd, s);
-  return e;
+  return launched(pieces > 1 ? 3 : 2);
 }
 
 cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a_digits, const int* a_ex,
@@ -847,10 +851,13 @@ cudaError_t oz_gemm(int64_t M, int64_t N, int64_t K, double alpha, const void* a
   oz_exponents(static_cast<const double2*>(B), N, K, 1, ldb, nullptr, 0, b_ex, s);
   note_launches(1);
   return oz_product(OP_N, M, N, K, alpha, a_digits, a_ex, B, ldb, beta, C, ldc, b_ex, ref_ex, bits, nullptr, OZ_ND - 1, status,
-                    s);
+                    nullptr, s);
 }
 
-size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K) { return oz_a_bytes(M, K) + sizeof(int) * size_t(M + N + K); }
+// All the memory of a balanced product that is not cut into pieces along k (K <= 64 is one chunk)
+size_t oz_balanced_bytes(int64_t M, int64_t N, int64_t K) {
+  return oz_a_bytes(M, K) + (oz_right_bytes(N, K) + 15) / 16 * 16 + sizeof(int) * size_t(M + N + K);
+}
 
 // C <- beta C + alpha op(A) op(B), balanced along k, with the digit orders up to gmax; scratch:
 // oz_balanced_bytes(M, N, K)
@@ -859,7 +866,8 @@ static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K
                                const int* col_ex, void* scratch, int gmax, int* status, cudaStream_t s) {
   if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
   char* dig = static_cast<char*>(scratch);
-  int* dk = reinterpret_cast<int*>(dig + oz_a_bytes(M, K));
+  char* right = dig + oz_a_bytes(M, K);
+  int* dk = reinterpret_cast<int*>(right + (oz_right_bytes(N, K) + 15) / 16 * 16);
   int *a_ex = dk + K, *b_ex = a_ex + M;
   const double2 *a = static_cast<const double2*>(A), *b = static_cast<const double2*>(B);
   if (opB == OP_N) {
@@ -875,7 +883,7 @@ static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K
   note_launches(3);
   const cudaError_t e = oz_digits<OZ_TM>(a, M, K, rs, ks, opA == OP_C, dk, 1, a_ex, dig, s);
   if (e != cudaSuccess) return e;
-  return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, 0, dk, gmax, status, s);
+  return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, 0, dk, gmax, status, right, s);
 }
 
 cudaError_t oz_update(int64_t M, int64_t N, int64_t K, const void* L, int64_t ldl, const void* U, int64_t ldu, void* C,
