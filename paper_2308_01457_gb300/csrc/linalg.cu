@@ -1626,33 +1626,46 @@ cudaError_t getrs(const void* LUv, int64_t n, int64_t ldlu, const int32_t* perm,
   using V = typename C2<T>::type;
   const V* LU = static_cast<const V*>(LUv);
   V* X = static_cast<V*>(Xv);
-  V* tmp = nullptr;
   ProfScope prof("getrs", s, 8.0 * double(n) * double(n) * double(nrhs));
-  // complex64 rows start on 16 bytes: the tensor-core updates then move two values at a time
-  // (163 columns at N = 7503, one sweep by superblocks 1.57 ms with rows of 163, 1.28 ms with rows of 164)
-  const int64_t ldt = sizeof(T) == 4 ? nrhs + (nrhs & 1) : nrhs;
-  cudaError_t e = device_alloc(reinterpret_cast<void**>(&tmp), sizeof(V) * n * ldt, s);
-  if (e != cudaSuccess) return e;
-  gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, ldt);
   if constexpr (sizeof(T) == 4) {
-    // persistent streaming kernels, tmp -> y -> tmp; the tickets lie behind y
-    if (!status || !dinv) e = cudaErrorInvalidValue;
-    char* y = nullptr;
-    const size_t ybytes = sizeof(V) * size_t(n) * size_t(ldt);
-    if (e == cudaSuccess) e = device_alloc(reinterpret_cast<void**>(&y), ybytes + 4 * trsv_stream_tickets(n) + 16, s);
-    int* tickets = reinterpret_cast<int*>(y + ybytes);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nrhs, ldt, 0, direct, tickets, status, s);
-    if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nrhs, ldt, 1, direct, tickets, status, s);
-    if (y) cudaFreeAsync(y, s);
-    if (e != cudaSuccess) {
-      cudaFreeAsync(tmp, s);
-      return e;
+    // persistent streaming kernels, tmp -> y -> tmp; the tickets lie behind y.  Where the two copies of
+    // the right-hand sides do not fit, half as many columns at a time.
+    if (!status || !dinv) return cudaErrorInvalidValue;
+    cudaError_t e = cudaSuccess;
+    for (int64_t c0 = 0, w = nrhs; c0 < nrhs && e == cudaSuccess;) {
+      const int64_t nc = std::min(w, nrhs - c0);
+      // rows start on 16 bytes: the tensor-core updates then move two values at a time
+      // (163 columns at N = 7503, one sweep by superblocks 1.57 ms with rows of 163, 1.28 ms with rows of 164)
+      const int64_t ldt = nc + (nc & 1);
+      const size_t bytes = sizeof(V) * size_t(n) * size_t(ldt);
+      Scratch both(s);
+      e = both.alloc(2 * bytes + 4 * trsv_stream_tickets(n) + 16);
+      if (e == cudaErrorMemoryAllocation && nc > 1) {
+        both.p = nullptr;
+        cudaGetLastError();
+        e = cudaSuccess;
+        w = (nc + 1) / 2;
+        continue;
+      }
+      if (e != cudaSuccess) return e;
+      V* tmp = static_cast<V*>(both.p);
+      char* y = static_cast<char*>(both.p) + bytes;
+      int* tickets = reinterpret_cast<int*>(y + bytes);
+      gather_rows_kernel<T><<<cdiv(n * nc, 256), 256, 0, s>>>(X + c0, ldx, perm, n, nc, tmp, ldt);
+      e = trsv_stream_c64(LU, n, ldlu, dinv, tmp, y, nc, ldt, 0, direct, tickets, status, s);
+      if (e == cudaSuccess) e = trsv_stream_c64(LU, n, ldlu, dinv, y, tmp, nc, ldt, 1, direct, tickets, status, s);
+      if (e != cudaSuccess) return e;
+      copy_kernel<V><<<cdiv(n * nc, 256), 256, 0, s>>>(tmp, n, nc, ldt, X + c0, ldx);
+      note_launches(2);  // gather + copy back
+      e = cudaGetLastError();
+      c0 += nc;
     }
-    copy_kernel<V><<<cdiv(n * nrhs, 256), 256, 0, s>>>(tmp, n, nrhs, ldt, X, ldx);
-    note_launches(2);  // gather + final copy
-    cudaFreeAsync(tmp, s);
-    return cudaGetLastError();
+    return e;
   } else {
+  V* tmp = nullptr;
+  cudaError_t e = device_alloc(reinterpret_cast<void**>(&tmp), sizeof(V) * n * nrhs, s);
+  if (e != cudaSuccess) return e;
+  gather_rows_kernel<T><<<cdiv(n * nrhs, 256), 256, 0, s>>>(X, ldx, perm, n, nrhs, tmp, nrhs);
   const int nb = 64;
   auto diag = [&](int64_t i0, int ib, int upper) {
     trsv_block<T>(LU + i0 * ldlu + i0, ldlu, ib, upper, tmp + i0 * nrhs, nrhs, nrhs, s);

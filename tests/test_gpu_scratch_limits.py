@@ -40,3 +40,19 @@ def test_fp64_factorisation_without_digits(F, after):
     X = torch.empty_like(B)
     F.solve(lu, B, X)
     assert _backward_error(Z, X, B) <= n * 2.0**-52
+
+
+@pytest.mark.parametrize("n,r", [(200, 1), (200, 7), (130, 1100), (700, 1501)])
+def test_complex64_sweeps_in_parts(F, n, r):
+    """The sweeps' copies of the right-hand sides do not fit at the first attempt."""
+    Z, B = _system(n, r, torch.complex64)
+    lu = F.factor(Z, prec=F.FP32)
+    X = torch.empty_like(B)
+    F.debug_fail_allocation(0)
+    if r == 1:  # one column cannot be halved
+        with pytest.raises(F.FosbError) as e:
+            F.solve(lu, B, X)
+        assert e.value.status == F.FOSB_ERR_OOM
+    F.solve(lu, B, X)
+    F.debug_fail_allocation(-1)
+    assert _backward_error(Z, X, B) <= 3 * n * 2.0**-24
