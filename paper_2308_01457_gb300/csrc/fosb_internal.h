@@ -277,7 +277,8 @@ cudaError_t split_ff(const void* src, int64_t rows, int64_t cols, int64_t lds, v
 template <typename T>
 fosb_status getrf(void* A, int64_t n, int64_t lda, int32_t* ipiv, int* d_status, cudaStream_t s);
 size_t getrf_scratch_bytes(int64_t max_ctas, bool c128);
-// Tournament-pivoting factorisation of one complex64 panel (m x jb at Ap, jb <= 64, m >= jb)
+// Tournament-pivoting factorisation of one complex64 panel (m x jb at Ap, jb <= 64, m >= jb; with
+// jb < 64 at most 2048 rows)
 // with scratch of tslu_scratch_bytes(n_max) bytes (n_max >= m): permutes the panel's own rows
 // and leaves the moves in the scratch for tslu_swap.
 size_t tslu_scratch_bytes(int64_t n_max);

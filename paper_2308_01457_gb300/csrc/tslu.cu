@@ -739,6 +739,9 @@ cudaError_t tslu_panel(void* Ap, int64_t m, int jb, int64_t lda, void* scratch, 
   int* last = idx[1] + groups_max * kTsluCols;  // [2]
   int* sel = last + 2;
   if (max_clusters(128) < 1 || max_clusters(256) < 1) return cudaErrorInvalidConfiguration;
+  // A group has 64 places for nominees and the next level reads them all, but a panel narrower than
+  // that fills only jb of them: its rows have to fit one level (the last panel of a matrix has m = jb).
+  if (jb < kTsluCols && plan_level(m).clusters > 1) return cudaErrorInvalidValue;
   uint64_t nl = 0;
   int64_t rows = m;
   int groups = 0, cur = 0;
