@@ -244,11 +244,11 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
     return fail(FOSB_ERR_INVALID_ARG, "fosb_solve: unknown refinement solver");
   double prev = INFINITY, prev2 = INFINITY, berr = INFINITY, res = INFINITY, res0 = INFINITY;
   int it = 0;
-  Scratch xkeep(s);  // the iterate that met the tolerance, while the correction after it is tried
-  double berr_kept = INFINITY;
+  double berr_kept = INFINITY;  // of the iterate that met the tolerance, while the correction after it is tried
   bool lost = false;  // a column with infinities or NaN
   for (; solver != FOSB_REFINE_GMRES;) {
-    FOSB_TRY(col_norms(X, n, nrhs, ldx, nb.as<double>(), xn, s));
+    const bool last = std::isfinite(berr_kept);
+    if (!last) FOSB_TRY(col_norms(X, n, nrhs, ldx, nb.as<double>(), xn, s));  // (the norms of x stand by then)
     bool full = !dx.p || it == 0;
     for (int64_t c = 0; c < nrhs && !full; ++c) full = !(xn[c] >= 0.5 * xfull[c]);
     if (full) {
@@ -257,7 +257,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
     }
     if (digits)
       FOSB_CUDA(oz_gemm(n, nrhs, n, -1.0, lu->zdig, lu->zex, full ? X : dx.p, full ? ldx : nrhs, 1.0, r.p, nrhs,
-                        xex.as<int>() + (full ? 0 : nrhs), full ? nullptr : xex.as<int>(), xkeep.p ? 50 : 60,
+                        xex.as<int>() + (full ? 0 : nrhs), full ? nullptr : xex.as<int>(), last ? 50 : 60,
                         lu->d_status, s));
     else
       FOSB_CUDA(gemm_c128_ff(OP_N, OP_N, n, nrhs, n, -1.0, 0.0, lu->zref, lu->ldz, X, ldx, 1.0, r.p, nrhs, s,
@@ -275,9 +275,9 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       res = std::max(res, bn[c] > 0 ? rn[c] / bn[c] : rn[c]);
     }
     if (it == 0) res0 = res;
-    if (xkeep.p) {  // the correction below the tolerance stands only if it is one
+    if (last) {  // the correction below the tolerance stands only if it is one
       if (!(berr <= berr_kept)) {
-        FOSB_CUDA(copy_matrix(xkeep.p, n, nrhs, nrhs, X, ldx, 16, s));
+        FOSB_CUDA(axpy_c64_into_c128(d.p, n, nrhs, nrhs, X, ldx, nullptr, s, -1.0));
         berr = berr_kept;
         --it;
       }
@@ -287,13 +287,7 @@ fosb_status solve_internal(fosb_lu lu, const void* B, int64_t nrhs, int64_t ldb,
       // just below the default tolerance, whose last factor of 16 is above the rounding floor: the
       // correction that this residual gives is worth its sweep (a better factorisation may stop a
       // step earlier and must not end further off); its residual needs to be right to a few per cent of
-      // the tolerance only, and without room for the iterate before it, that one is returned
-      if (xkeep.alloc(sizeof(double) * 2 * n * nrhs) != cudaSuccess) {
-        xkeep.p = nullptr;
-        cudaGetLastError();
-        break;
-      }
-      FOSB_CUDA(copy_matrix(X, n, nrhs, ldx, xkeep.p, nrhs, 16, s));
+      // the tolerance only
       berr_kept = berr;
     } else if (berr <= tol || it >= max_iters || (berr >= prev && prev >= prev2) ||  // no decrease over two steps
                (berr < 1e-13 && berr > 0.5 * prev)) {  // at the rounding floor: progress has stalled

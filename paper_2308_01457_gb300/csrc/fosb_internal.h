@@ -318,7 +318,7 @@ cudaError_t convert_c64_to_c128(const void* src, int64_t rows, int64_t cols, int
 cudaError_t copy_matrix(const void* src, int64_t rows, int64_t cols, int64_t lds, void* dst, int64_t ldd, size_t elem,
                         cudaStream_t s);
 cudaError_t axpy_c64_into_c128(const void* d, int64_t rows, int64_t cols, int64_t ldd, void* x, int64_t ldx,
-                               void* change, cudaStream_t s);
+                               void* change, cudaStream_t s, double sign = 1.0);
 // out = (accumulate ? out : 0) + w (M + op(M)) for a square n x n matrix M (op = OP_T or OP_C)
 cudaError_t add_mirrored(const void* M, int64_t n, int64_t ldm, int op, double w, bool accumulate, bool c64, void* out,
                          int64_t ldo, cudaStream_t s);

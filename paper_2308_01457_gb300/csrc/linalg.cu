@@ -999,12 +999,12 @@ __global__ void c64_to_c128_kernel(const float2* s, int64_t rows, int64_t cols, 
   d[i * ldd + j] = make_double2(v.x, v.y);
 }
 __global__ void axpy_kernel(const float2* dlt, int64_t rows, int64_t cols, int64_t ldd, double2* x, int64_t ldx,
-                            double2* change) {
+                            double2* change, double sign) {
   int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
   if (e >= rows * cols) return;
   int64_t i = e / cols, j = e % cols;
   float2 v = dlt[i * ldd + j];
-  const double2 o = x[i * ldx + j], w = make_double2(o.x + v.x, o.y + v.y);
+  const double2 o = x[i * ldx + j], w = make_double2(o.x + sign * v.x, o.y + sign * v.y);
   x[i * ldx + j] = w;
   if (change) change[e] = make_double2(w.x - o.x, w.y - o.y);
 }
@@ -1729,10 +1729,10 @@ cudaError_t copy_matrix(const void* src, int64_t rows, int64_t cols, int64_t lds
   return cudaMemcpy2DAsync(dst, ldd * elem, src, lds * elem, cols * elem, rows, cudaMemcpyDeviceToDevice, s);
 }
 cudaError_t axpy_c64_into_c128(const void* d, int64_t rows, int64_t cols, int64_t ldd, void* x, int64_t ldx,
-                               void* change, cudaStream_t s) {
+                               void* change, cudaStream_t s, double sign) {
   if (rows * cols == 0) return cudaSuccess;
   axpy_kernel<<<cdiv(rows * cols, 256), 256, 0, s>>>(static_cast<const float2*>(d), rows, cols, ldd,
-                                                     static_cast<double2*>(x), ldx, static_cast<double2*>(change));
+                                                     static_cast<double2*>(x), ldx, static_cast<double2*>(change), sign);
   return launched();
 }
 cudaError_t add_mirrored(const void* M, int64_t n, int64_t ldm, int op, double w, bool accumulate, bool c64, void* out,

@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstdint>
+#include <thread>
 #include <type_traits>
 
 #include "fosb_internal.h"
@@ -905,7 +906,10 @@ fosb_status DigitStatus::check(const char* call) {
   if (!word_.p) return FOSB_OK;
   int status = 0;
   FOSB_CUDA(cudaMemcpyAsync(&status, word_.p, sizeof(int), cudaMemcpyDeviceToHost, word_.s));
-  FOSB_CUDA(cudaStreamSynchronize(word_.s));
+  // (polled: a synchronisation would also give the pool's free memory back, which the next call maps again)
+  cudaError_t e;
+  while ((e = cudaStreamQuery(word_.s)) == cudaErrorNotReady) std::this_thread::yield();
+  FOSB_CUDA(e);
   if (status == FOSB_ERR_TIMEOUT) return fail(FOSB_ERR_TIMEOUT, std::string(call) + ": tensor-core wait timed out");
   return FOSB_OK;
 }
