@@ -311,6 +311,26 @@ __global__ void oz_balance_kernel(const double2* __restrict__ B, int64_t N, int6
 }
 // ... and for a transposed B (N x K as stored): 32 values of k along the lanes, the warps share the rows
 // j of a chunk, one atomic per k and CTA into dk, which starts as OZ_NO_ROW
+// Both leave raw exponents; this makes them relative to the largest and leaves rows of B down to 2^-T of it
+// alone (T = kFreeBinades): where rows of U are small without columns of L being large, a balance only raises
+// the scales.  Forward errors of FP64 solves, EFIE matrices of 1920 unknowns, geometric means: 1.23e-14 with T = 0,
+// 1.20e-14, 1.19e-14 and 1.20e-14 with 2, 3 and 5 (1.55e-14 with FP64 products); row-scaled random
+// matrices n = 640, backward error 4e-15 up to 3, 6.5e-15 with 5.
+constexpr int kFreeBinades = 3;
+__global__ void __launch_bounds__(256) oz_balance_limit_kernel(int64_t K, int* __restrict__ dk) {
+  __shared__ int red[8];
+  int m = OZ_NO_ROW;
+  for (int64_t k = threadIdx.x; k < K; k += 256) m = max(m, dk[k]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = red[0];
+  for (int w = 1; w < 8; ++w) m = max(m, red[w]);
+  for (int64_t k = threadIdx.x; k < K; k += 256) {
+    const int d = dk[k];
+    if (d != OZ_NO_ROW) dk[k] = min(d - m + kFreeBinades, 0);
+  }
+}
 constexpr int64_t kBalanceRows = 512;
 __global__ void __launch_bounds__(256) oz_balance_t_kernel(const double2* __restrict__ B, int64_t N, int64_t K,
                                                            int64_t ld, int* __restrict__ dk) {
@@ -878,10 +898,11 @@ static cudaError_t oz_balanced(int opA, int opB, int64_t M, int64_t N, int64_t K
     if (e != cudaSuccess) return e;
     oz_balance_t_kernel<<<dim3(oz_cdiv(K, 32), oz_cdiv(N, kBalanceRows)), 256, 0, s>>>(b, N, K, ldb, dk);
   }
+  oz_balance_limit_kernel<<<1, 256, 0, s>>>(K, dk);
   const int64_t rs = opA == OP_N ? lda : 1, ks = opA == OP_N ? 1 : lda;
   oz_exponents(a, M, K, rs, ks, dk, 1, a_ex, s);
   oz_exponents(b, N, K, opB == OP_N ? 1 : ldb, opB == OP_N ? ldb : 1, dk, -1, b_ex, s);
-  note_launches(3);
+  note_launches(4);
   const cudaError_t e = oz_digits<OZ_TM>(a, M, K, rs, ks, opA == OP_C, dk, 1, a_ex, dig, s);
   if (e != cudaSuccess) return e;
   return oz_product(opB, M, N, K, alpha, dig, a_ex, B, ldb, beta, C, ldc, b_ex, nullptr, 0, dk, gmax, status, right, s);

@@ -207,8 +207,11 @@ __global__ void __launch_bounds__(512) row_balance_kernel(int64_t N, int K, cons
   d = __reduce_max_sync(0xffffffffu, red[threadIdx.x & 15]);
   if (threadIdx.x == 0) dk[k] = d;
 }
-// The largest of the balance exponents, by a warp; the balance in use is relative to it: at most 0, and at
-// least -100 so that the scales stay normal floats (zero rows have that too, their products are zero).
+// The largest of the balance exponents, by a warp.  The balance in use is relative to it: rows of B down to
+// 2^-kFreeBinades of the largest are left alone (the split carries them, and where rows of U are small without
+// columns of L being large a balance only raises the scales), and none is below -100 so that the scales
+// stay normal floats (zero rows have that too, their products are zero).
+constexpr int kFreeBinades = 8;
 __device__ __forceinline__ int balance_max(const int* __restrict__ dk, int lane) {
   int d = kNone;
 #pragma unroll
@@ -220,7 +223,7 @@ __device__ __forceinline__ void balance8(const int* __restrict__ dk, int k0, int
   const int4 p = *reinterpret_cast<const int4*>(dk + k0), q = *reinterpret_cast<const int4*>(dk + k0 + 4);
   const int v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
 #pragma unroll
-  for (int i = 0; i < 8; ++i) d[i] = max(v[i] - dmax, -100);
+  for (int i = 0; i < 8; ++i) d[i] = max(min(v[i] - dmax + kFreeBinades, 0), -100);
 }
 
 // A (M x K, lda), K <= 256 in nslab = ceil(K / 16) slabs: out[(rt * nslab + s) * 16 KB + p * 4 KB +
