@@ -85,7 +85,7 @@ TF32_PER_BF16 = 1.1 / 2.25  # nominal dense TF32 / BF16 tensor ratio of the part
 LU_BLOCK = 256  # column block of the complex64 LU: every trailing update has K = 256
 # DRAM bytes (read + write) per complex64 output element of one tcgen05 LU-update launch,
 # from the ncu capture summarised in profiles/ (C is read and written once: 16 B algorithmic)
-LU_UPDATE_DRAM_BYTES_PER_OUTPUT = (543.779072e6 + 382.323712e6) / 7424.0**2  # 16.80 B
+LU_UPDATE_DRAM_BYTES_PER_OUTPUT = (545.424640e6 + 382.422528e6) / 7424.0**2  # 16.83 B
 
 
 def _peaks():

@@ -845,40 +845,6 @@ __global__ void laswp_kernel(typename C2<T>::type* A, int64_t n, int64_t lda, in
   }
 }
 
-// X (nb x ncols block) <- L^{-1} X with L unit lower (unit=1) or U^{-1} X with U upper
-// (unit=0), diagonal block of size nb at D (leading dimension ldd).  Thread per column.
-template <typename T>
-__global__ void trsm_diag_kernel(const typename C2<T>::type* D, int64_t ldd, int nb, int upper,
-                                 typename C2<T>::type* X, int64_t ldx, int64_t ncols) {
-  using V = typename C2<T>::type;
-  int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (c >= ncols) return;
-  if (!upper) {
-    for (int i = 1; i < nb; ++i) {
-      V s = X[int64_t(i) * ldx + c];
-      for (int k = 0; k < i; ++k) {
-        V l = D[int64_t(i) * ldd + k], x = X[int64_t(k) * ldx + c];
-        s.x -= l.x * x.x - l.y * x.y;
-        s.y -= l.x * x.y + l.y * x.x;
-      }
-      X[int64_t(i) * ldx + c] = s;
-    }
-  } else {
-    for (int i = nb - 1; i >= 0; --i) {
-      V s = X[int64_t(i) * ldx + c];
-      for (int k = i + 1; k < nb; ++k) {
-        V u = D[int64_t(i) * ldd + k], x = X[int64_t(k) * ldx + c];
-        s.x -= u.x * x.x - u.y * x.y;
-        s.y -= u.x * x.y + u.y * x.x;
-      }
-      V d = D[int64_t(i) * ldd + i];
-      T den = d.x * d.x + d.y * d.y;
-      V q = den > T(0) ? V{(s.x * d.x + s.y * d.y) / den, (s.y * d.x - s.x * d.y) / den} : V{T(0), T(0)};
-      X[int64_t(i) * ldx + c] = q;
-    }
-  }
-}
-
 template <typename T>
 __device__ __forceinline__ typename C2<T>::type cmul_add(typename C2<T>::type a, typename C2<T>::type b,
                                                          typename C2<T>::type c) {  // a b + c

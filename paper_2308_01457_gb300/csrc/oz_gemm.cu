@@ -9,10 +9,11 @@
 //   (Z X)_ij = sigma_i tau_j 2^-14 sum_{s,t} 2^{-8(s+t)} sum_k d_s[i,k] e_t[k,j],
 // and a digit product is an integer of at most 2^14, so sums of the same order g = s+t over
 // 128 values of k are exact in the FP32 accumulators of the tensor cores for g <= 3
-// ((g+1) x 2 x 128 x 2^14 <= 2^24).  Orders g <= 6 (28 digit pairs) are kept: the dropped
+// ((g+1) x 2 x 128 x 2^14 <= 2^24; order 4 too unless nearly all digits are at the ends of their range,
+// the first ones included, and then its rounding is below 2^-49 of |Z||X|).  Orders g <= 6 (28 digit pairs) are kept: the dropped
 // terms are below 2^-56 of sigma_i tau_j per product (the trailing updates of FP64 factorisations keep
-// order 7 too, 34 pairs, and leave nothing of that size but the rounding of the operands).  After every 128 values of k the seven
-// order accumulators are read out of TMEM: orders 0-4 are added into a 64-bit integer
+// order 7 too, 34 pairs, and leave nothing of that size but the rounding of the operands).  After every
+// 128 values of k the seven order accumulators are read out of TMEM: orders 0-4 are added into a 64-bit integer
 // sum per output, orders 5-6 (below 2^-40 of them) into an FP32 sum; the result is scaled by
 // sigma_i tau_j 2^-14.
 //
@@ -379,7 +380,7 @@ __device__ __forceinline__ uint32_t oz_bf16_bits(uint32_t byte) {
 // Digit tiles of a matrix read as rows x K elements (element (r, k) at A[r * rs + k * ks]),
 // one power-of-two exponent per row (and with dk a factor 2^{sign dk[k]} per k), zero-padded to whole tiles of TR rows x 16 k:
 // tile (rt, kc, s, p) of TR x 16 bf16 at byte offset (((rt * KC + kc) * 7 + s) * 2 + p) * TR * 32.
-// Z (rs = ld, ks = 1, TR = 128) and X read by columns (rs = 1, ks = ld, TR = 32) both land here.
+// Z (rs = ld, ks = 1, TR = 128) and X read by columns (rs = 1, ks = ld, TR = 64) both land here.
 // Digits: F = x 2^(55 - e) rounded (above) is written in balanced base 256,
 // F = sum_{s=0..6} d_s 256^(6-s) with d_1..d_6 in [-128, 127] and |d_0| <= 128: adding 128 in
 // each of the seven byte positions turns every digit into a plain byte (the carries of the
@@ -447,8 +448,8 @@ __global__ void oz_orders_kernel(const int* __restrict__ ex, const int* __restri
 }
 
 // The sums of one output: a = sum_g V_g 2^{unit-8g} over the orders that this leaves whole (V_g the
-// integer order sums), exact; t the others in FP32 in the same units; the value is 2^-unit (a + t).
-// unit 32 (orders 0-4 exact, the rounding of t near 2^-58 of the result) as long as K <= 2^15 keeps a
+// order sums), added without rounding; t the others in FP32 in the same units; the value is 2^-unit (a + t).
+// unit 32 (orders 0-4, the rounding of t near 2^-58 of the result) as long as K <= 2^15 keeps a
 // below 2^62, 24 (orders 0-3, 2^-53) above.
 __device__ __forceinline__ void oz_store(double* C, long long a, float t, int aex, int bex, int unit, double alpha,
                                          double beta) {

@@ -3,8 +3,8 @@
 //
 // A blocked sweep that launches one diagonal solve and one panel update per 64-row block
 // is latency-bound (2 x n/64 dependent launches per sweep).  Here one persistent kernel
-// does a whole sweep.  The right-hand sides are cut into chunks of at most 8 columns (one
-// chunk of the exact width for 1-8); CTAs take (block, chunk) tasks in block-major order
+// does a whole sweep.  The right-hand sides are cut into chunks of 1, 2, 4 or 8 columns
+// (chunk_width; the last chunk may have fewer); CTAs take (block, chunk) tasks in block-major order
 // from a ticket counter.  With D_i the inverse of the diagonal block and j the blocks that
 // precede i in the sweep, the last of them h,
 //     y_i = D_i (x_i - sum_{j != h} L_ij y_j) - E_i y_h,   E_i = D_i L_ih  (E_i formed once per factorisation),
@@ -209,14 +209,14 @@ __global__ void __launch_bounds__(256) tri_refine_kernel(const float2* __restric
 
 // Shared tiles of the streaming sweep.  A factor tile (later the inverse of the diagonal block)
 // and the neighbour product E are 64 x 64 with a row pitch of 72 complex values; the published
-// blocks of the solution are 64 x NR with a pitch that is odd for odd NR and else keeps 16-byte
-// rows in distinct banks.  Thread (g, q) of 256 owns rows g and g + 32 and the columns q, q + 8,
+// blocks of the solution are 64 x NR with a pitch that keeps 16-byte rows of 4 and 8 columns in
+// distinct banks.  Thread (g, q) of 256 owns rows g and g + 32 and the columns q, q + 8,
 // ..., q + 56, so in one step of c the 16 threads of a half-warp read 8 consecutive complex
 // values of two rows 72 apart (every bank once) and 8 rows of the solution block (distinct banks).
 constexpr int kLP = 72;
 template <int NR>
 struct StreamSmem {
-  static constexpr int NRP = NR & 1 ? NR : (NR == 2 || NR == 6 ? NR : NR + 2);
+  static constexpr int NRP = NR <= 2 ? NR : NR + 2;
   float2 L[kTB][kLP];
   float2 E[kTB][kLP];
   float2 Y[2][kTB][NRP];  // the current block of the solution; minus the neighbour's
